@@ -546,19 +546,13 @@ def measure(args, w, dev, world, rank, local):
 
 def _sgd_kernel_name(K):
     """The SGD launches of one clock that the profile events bracket."""
-    if 32 < K <= 64:
-        return "sgd_work16_kernel (+ user_copy_kernel, and heavy_merge_kernel when some user is heavy)"
-    if 64 < K <= 128:
-        return "sgd_users32_kernel (+ sgd_chunks_kernel / heavy_merge_kernel when some user is heavy)"
-    return "sgd_users_kernel (+ sgd_chunks_kernel / heavy_merge_kernel when some user is heavy)"
+    return "sgd_stream_kernel (+ heavy_merge_kernel when some user is heavy)"
 
 
 def _sgd_launches(K, heavy: bool) -> int:
     """Kernels of one clock's SGD phase plus the item merge (which also
     computes the next schedule)."""
-    if 32 < K <= 64:  # forward copy, work list, heavy merge
-        return 2 + int(heavy) + 1
-    return 1 + 2 * int(heavy) + 1
+    return 1 + int(heavy) + 1
 
 
 def run_gpu(args, w):

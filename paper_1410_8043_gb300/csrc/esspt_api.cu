@@ -18,6 +18,7 @@ struct esspt_ctx {
   int32_t K = 0, P = 0, s = 0, nslots = 0, dmax = 0;
   float* ring = nullptr;
   int32_t* v = nullptr;
+  int32_t* vslot = nullptr;  // [P] ring slot of each read version
   uint32_t* status = nullptr;
   uint32_t* thr = nullptr;
   uint32_t* vap_norm = nullptr;  // [s+1] VAP in-transit norms of the current clock
@@ -30,20 +31,22 @@ struct esspt_ctx {
   int64_t n_users = 0, n_items = 0, n_obs = 0;
   int32_t F = 0;
   int32_t *rec_u = nullptr, *rec_j = nullptr, *uoff = nullptr, *item_cnt = nullptr, *worker = nullptr;
-  int32_t *item_rep = nullptr, *rec_dst = nullptr;
+  int32_t *item_rep = nullptr, *hot_item = nullptr;
+  int4* rec = nullptr;                // records of the SGD kernel
   float *rec_D = nullptr, *dR = nullptr, *dL = nullptr;
   int32_t* rowver = nullptr;     // row-granular SSP: [P][n_rows] cached versions, -1 = never read
   int32_t* user_slot = nullptr;  // row-granular SSP: [n_users] per-clock ring slot of each user row
   int32_t* rec_row = nullptr;    // row-granular SSP: per-clock ring row of each entry's item row
   int4 *chunk = nullptr, *heavy = nullptr;
   std::vector<int64_t> mb_base, chunk_base, heavy_base;
+  int32_t* part = nullptr;            // split of each minibatch's work items over the warps
+  std::vector<int64_t> part_base;     // [F+1] first word of each minibatch's split
   cudaEvent_t ev_before = nullptr, ev_after = nullptr;
-  // Work-list path: last clock that changed each user row, and the last clock
-  // at which every idle row is still copied forward (after an INC or a
-  // sequential clock, whose writes are not tracked per row).
+  // Last clock that changed each user row, and the last clock at which every
+  // idle row is still copied forward (after an INC or a sequential clock,
+  // whose writes are not tracked per row).
   int32_t* chg = nullptr;
   int32_t copy_all_until = 0;
-  int32_t* hot_item = nullptr;   // work-list path: [F][kHot] hot items of each minibatch
 };
 
 namespace {
@@ -96,7 +99,7 @@ int32_t delay_max(const esspt_config* c) {
 }
 
 struct Carve {
-  size_t ring, v, status, thr, vap, rowver, total;
+  size_t ring, v, vslot, status, thr, vap, rowver, total;
 };
 
 Carve carve(const esspt_config* c) {
@@ -105,6 +108,8 @@ Carve carve(const esspt_config* c) {
   k.ring = o;
   o += align256((size_t)(c->staleness + 2) * (size_t)c->n_rows * (size_t)c->row_width * sizeof(float));
   k.v = o;
+  o += align256(sizeof(int32_t) * (size_t)c->num_workers);
+  k.vslot = o;
   o += align256(sizeof(int32_t) * (size_t)c->num_workers);
   k.status = o;
   o += 256;
@@ -170,11 +175,13 @@ esspt_status advance(esspt_ctx* c, bool scheduled = false) {
 ScheduleArgs schedule_args(const esspt_ctx* c, int32_t clock) {
   ScheduleArgs a{};
   a.v = c->v;
+  a.vslot = c->vslot;
   a.status = c->status;
   a.thr = c->thr;
   a.P = c->P;
   a.c = clock;
   a.s = c->s;
+  a.nslots = c->nslots;
   a.model = c->cfg.model;
   a.phased = c->cfg.phased;
   a.dmax = c->dmax;
@@ -194,9 +201,9 @@ bool is_host_ptr(const void* p) {
 }
 
 struct MfCarve {
-  size_t rec_u, rec_j, rec_D, rec_dst, uoff, mb_base, item_cnt, item_rep, dR, worker, chunk, chunk_base, heavy, heavy_base, dL,
-      user_slot, rec_row, chg, hot_item, total;
-  int64_t max_chunks, max_heavy, dR_rows, dL_rows;
+  size_t rec_u, rec_j, rec_D, rec, uoff, mb_base, item_cnt, item_rep, dR, worker, chunk, chunk_base, heavy, heavy_base, dL,
+      user_slot, rec_row, chg, hot_item, part, total;
+  int64_t max_chunks, max_heavy, dR_rows, dL_rows, part_rows;
 };
 
 // Persistent MF workspace: entries laid out by (minibatch, user), per-minibatch
@@ -204,7 +211,7 @@ struct MfCarve {
 // zero-initialised delta replicas dR (items) and dL (heavy users).
 MfCarve mf_carve(int64_t n_obs, int64_t n_users, int64_t n_items, int32_t F, int32_t K, bool row_mode) {
   MfCarve k{};
-  k.max_chunks = layout_max_chunks(n_obs, F, n_users, uses_work16(K));
+  k.max_chunks = layout_max_chunks(n_obs, F, n_users);
   k.max_heavy = layout_max_heavy(n_obs, F);
   k.dR_rows = layout_max_item_reps(n_obs, n_items);
   k.dL_rows = n_users + layout_max_user_reps(n_obs);
@@ -218,7 +225,7 @@ MfCarve mf_carve(int64_t n_obs, int64_t n_users, int64_t n_items, int32_t F, int
   k.rec_u = take(sizeof(int32_t) * (n_obs + 4));
   k.rec_j = take(sizeof(int32_t) * (n_obs + 4));
   k.rec_D = take(sizeof(float) * (n_obs + 4));
-  k.rec_dst = take(sizeof(int32_t) * (n_obs + 4));
+  k.rec = take(sizeof(int4) * n_obs);
   k.uoff = take(sizeof(int32_t) * (size_t)F * (n_users + 1));
   k.mb_base = take(sizeof(int64_t) * (F + 1));
   k.item_cnt = take(sizeof(int32_t) * (size_t)F * n_items);
@@ -234,9 +241,12 @@ MfCarve mf_carve(int64_t n_obs, int64_t n_users, int64_t n_items, int32_t F, int
   // holds at most n_obs entries).
   k.user_slot = row_mode ? take(sizeof(int32_t) * n_users) : o;
   k.rec_row = row_mode ? take(sizeof(int32_t) * (n_obs + 4)) : o;
-  // Work-list path: the clock that last changed each user row.
-  k.chg = uses_work16(K) ? take(sizeof(int32_t) * n_users) : o;
+  // The clock that last changed each user row.
+  k.chg = take(sizeof(int32_t) * n_users);
   k.hot_item = uses_hot(K) ? take(sizeof(int32_t) * (size_t)F * kHot) : o;
+  // A minibatch uses at most one warp per work item.
+  k.part_rows = std::min((int64_t)F * (stream_max_warps(K) + 1), k.max_chunks + F);
+  k.part = take(sizeof(int32_t) * (size_t)k.part_rows);
   k.total = o;
   return k;
 }
@@ -245,11 +255,11 @@ bool mf_sizes_ok(const esspt_ctx* c, int64_t n_obs, int64_t n_users, int32_t F) 
   if (!(c && n_obs >= 0 && n_obs < (int64_t)INT32_MAX && n_users > 0 && n_users < c->n_rows && F >= 1 && F <= 255 &&
         (int64_t)F * n_users < (int64_t)INT32_MAX))
     return false;
-  // The SGD kernels offset item rows and item replica rows by 32-bit float4
-  // products (item * K/4, replica row * row stride).
+  // Item rows (item * K/4 float4) and item replica rows (in whole 32-byte
+  // sectors) stay below 2^31 float4; the merge splits the first with 32 bits.
   const int64_t n_items = c->n_rows - n_users;
   return n_items * (c->K / 4) < (int64_t)INT32_MAX &&
-         layout_max_item_reps(n_obs, n_items) * dR_stride4(c->K) < (int64_t)INT32_MAX;
+         layout_max_item_reps(n_obs, n_items) * ((c->K + 7) / 8 * 2) < (int64_t)INT32_MAX;
 }
 
 }  // namespace
@@ -312,6 +322,7 @@ esspt_status esspt_create(const esspt_config* cfg, void* d_workspace, size_t byt
   char* w = static_cast<char*>(d_workspace);
   c->ring = reinterpret_cast<float*>(w + k.ring);
   c->v = reinterpret_cast<int32_t*>(w + k.v);
+  c->vslot = reinterpret_cast<int32_t*>(w + k.vslot);
   c->status = reinterpret_cast<uint32_t*>(w + k.status);
   c->thr = reinterpret_cast<uint32_t*>(w + k.thr);
   if (cfg->model == ESSPT_VAP) c->vap_norm = reinterpret_cast<uint32_t*>(w + k.vap);
@@ -500,14 +511,13 @@ esspt_status esspt_mf_load(esspt_ctx* c, const int32_t* d_i, const int32_t* d_j,
   b.mb_base = reinterpret_cast<int64_t*>(w + k.mb_base);
   b.item_cnt = reinterpret_cast<int32_t*>(w + k.item_cnt);
   b.item_rep = reinterpret_cast<int32_t*>(w + k.item_rep);
-  b.rec_dst = reinterpret_cast<int32_t*>(w + k.rec_dst);
+  b.rec = reinterpret_cast<int4*>(w + k.rec);
+  b.hot_item = uses_hot(c->K) ? reinterpret_cast<int32_t*>(w + k.hot_item) : nullptr;
   b.chunk = reinterpret_cast<int4*>(w + k.chunk);
   b.chunk_base = reinterpret_cast<int64_t*>(w + k.chunk_base);
   b.heavy = reinterpret_cast<int4*>(w + k.heavy);
   b.heavy_base = reinterpret_cast<int64_t*>(w + k.heavy_base);
   b.max_chunks = k.max_chunks;
-  b.light_items = uses_work16(c->K);
-  b.hot_item = uses_hot(c->K) ? reinterpret_cast<int32_t*>(w + k.hot_item) : nullptr;
   b.max_heavy = k.max_heavy;
   b.scratch = d_scratch;
   b.scratch_bytes = scratch_bytes;
@@ -542,6 +552,20 @@ esspt_status esspt_mf_load(esspt_ctx* c, const int32_t* d_i, const int32_t* d_j,
     ESSPT_CUDA(c, cudaMemsetAsync(c->status, 0, sizeof(uint32_t), c->st));
     return fail(c, ESSPT_ECUDA, "internal: chunk list overflow");
   }
+  // Split each minibatch's work items over the warps of the SGD kernel.
+  const int gpw = stream_groups_per_warp(c->K);
+  std::vector<int64_t> ptb((size_t)F + 1, 0);
+  int32_t* part = reinterpret_cast<int32_t*>(w + k.part);
+  for (int32_t f = 0; f < F; ++f) {
+    const int64_t items = chb[f + 1] - chb[f];
+    const int64_t warps = std::min(stream_max_warps(c->K), (items + gpw - 1) / gpw);
+    ptb[f + 1] = ptb[f] + warps + 1;
+    if (ptb[f + 1] > k.part_rows) return fail(c, ESSPT_ECUDA, "internal: work split overflow");
+    ESSPT_CUDA(c, launch_stream_partition(b.pre + chb[f], items, warps, part + ptb[f], c->st));
+  }
+  ESSPT_CUDA(c, cudaStreamSynchronize(c->st));
+  c->part = part;
+  c->part_base = ptb;
   c->n_users = n_users;
   c->n_items = n_items;
   c->n_obs = n_obs;
@@ -557,19 +581,16 @@ esspt_status esspt_mf_load(esspt_ctx* c, const int32_t* d_i, const int32_t* d_j,
   c->item_cnt = b.item_cnt;
   c->worker = worker;
   c->item_rep = b.item_rep;
-  c->rec_dst = b.rec_dst;
+  c->rec = b.rec;
+  c->hot_item = b.hot_item;
   c->dR = dR;
   c->dL = dL;
   c->chunk = b.chunk;
   c->heavy = b.heavy;
-  c->chg = nullptr;
-  c->hot_item = b.hot_item;
-  if (uses_work16(c->K)) {
-    c->chg = reinterpret_cast<int32_t*>(w + k.chg);
-    ESSPT_CUDA(c, cudaMemsetAsync(c->chg, 0, sizeof(int32_t) * (size_t)n_users, c->st));
-    // rows changed before this load are not tracked
-    c->copy_all_until = c->clock + c->s + 1;
-  }
+  c->chg = reinterpret_cast<int32_t*>(w + k.chg);
+  ESSPT_CUDA(c, cudaMemsetAsync(c->chg, 0, sizeof(int32_t) * (size_t)n_users, c->st));
+  // rows changed before this load are not tracked
+  c->copy_all_until = c->clock + c->s + 1;
   c->mb_base = mbb;
   c->chunk_base = chb;
   c->heavy_base = hvb;
@@ -596,14 +617,8 @@ esspt_status esspt_mf_sgd_clock(esspt_ctx* c, float eta, float lambda, int32_t c
   a.nslots = c->nslots;
   a.slot_base = slot_base;
   a.slot_out = slot_out;
-  a.n_b = (int32_t)(c->mb_base[b + 1] - c->mb_base[b]);
-  a.v = c->v;
-  a.worker = c->worker;
+  a.vslot = c->vslot;
   a.uoff = c->uoff + (int64_t)b * (c->n_users + 1);
-  a.rec_j = c->rec_j + c->mb_base[b];
-  a.rec_D = c->rec_D + c->mb_base[b];
-  a.rec_dst = c->rec_dst + c->mb_base[b];
-  a.item_rep = c->item_rep;
   a.dR = c->dR;
   a.dR_ld = dR_stride4(c->K);
   a.eta = eta;
@@ -611,21 +626,20 @@ esspt_status esspt_mf_sgd_clock(esspt_ctx* c, float eta, float lambda, int32_t c
   a.cap = cap;
   a.sq_loss = d_sq_loss;
   a.chg = c->chg;
-  a.clock = c->clock;
+  a.item_rep = c->item_rep;
   a.hot_item = c->hot_item ? c->hot_item + (int64_t)b * kHot : nullptr;
+  a.clock = c->clock;
   a.copy_all_until = c->copy_all_until;
   if (c->rowver) {
     // Row-granular SSP: refresh the rows read this clock; the kernels then
     // take each user's slot and each entry's item ring row from the refresh.
     RowRefreshArgs r{};
     r.rowver = c->rowver;
-    r.worker = c->worker;
-    r.uoff = a.uoff;
-    r.rec_u = c->rec_u + c->mb_base[b];
-    r.rec_j = a.rec_j;
+    r.items = c->chunk + c->chunk_base[b];
+    r.n_items = c->chunk_base[b + 1] - c->chunk_base[b];
+    r.rec = c->rec + c->mb_base[b];
     r.n_rows = c->n_rows;
     r.n_users = a.n_users;
-    r.n_b = a.n_b;
     r.c = c->clock;
     r.s = c->s;
     r.nslots = c->nslots;
@@ -634,25 +648,18 @@ esspt_status esspt_mf_sgd_clock(esspt_ctx* c, float eta, float lambda, int32_t c
     ESSPT_CUDA(c, launch_row_refresh(r, c->st));
     a.row_mode = 1;
     a.user_slot = c->user_slot;
-    a.rec_j = c->rec_row;
+    a.rec_row = c->rec_row;
   }
-  const int64_t nch = c->chunk_base[b + 1] - c->chunk_base[b];
   const int64_t nhv = c->heavy_base[b + 1] - c->heavy_base[b];
   if (c->ev_before) ESSPT_CUDA(c, cudaEventRecord(c->ev_before, c->st));
-  ChunkArgs ch{};
-  ch.a = a;
-  ch.chunk = c->chunk + c->chunk_base[b];
-  ch.n_chunks = nch;
-  ch.dL = c->dL;
-  if (uses_work16(c->K)) {
-    // Work-list path: users without entries are copied forward; every other
-    // user (and every chunk of a heavy user) is one item of the work kernel.
-    ESSPT_CUDA(c, launch_user_copy(a, c->st));
-    ESSPT_CUDA(c, launch_sgd_work16(ch, c->st));
-  } else {
-    if (nch > 0) ESSPT_CUDA(c, launch_sgd_chunks(ch, c->st));
-    ESSPT_CUDA(c, launch_sgd_users(a, c->st));
-  }
+  StreamArgs sa{};
+  sa.a = a;
+  sa.items = c->chunk + c->chunk_base[b];
+  sa.part = c->part + c->part_base[b];
+  sa.n_warps = c->part_base[b + 1] - c->part_base[b] - 1;
+  sa.rec = c->rec + c->mb_base[b];
+  sa.dL = c->dL;
+  ESSPT_CUDA(c, launch_sgd_stream(sa, c->st));
   if (nhv > 0) {
     HeavyMergeArgs h{};
     h.ring = c->ring;
@@ -813,6 +820,7 @@ esspt_status esspt_mf_stage_minibatch(esspt_ctx* c, int32_t b, const int32_t* h_
   ESSPT_CUDA(c, cudaMemcpyAsync(su, h_u, sizeof(int32_t) * n, cudaMemcpyHostToDevice, st));
   ESSPT_CUDA(c, cudaMemcpyAsync(sj, h_j, sizeof(int32_t) * n, cudaMemcpyHostToDevice, st));
   ESSPT_CUDA(c, cudaMemcpyAsync(suoff, h_uoff, sizeof(int32_t) * (c->n_users + 1), cudaMemcpyHostToDevice, st));
+  ESSPT_CUDA(c, launch_refill(c->rec + base, c->rec_D + base, n, st));
   ESSPT_CUDA(c, launch_stage_check(su, sj, suoff, c->rec_u + base, c->rec_j + base, ruoff, n, c->n_users + 1,
                                    c->status, st));
   return ESSPT_OK;

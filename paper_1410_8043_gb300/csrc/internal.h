@@ -24,9 +24,15 @@ constexpr uint64_t kStreamPhase = 101u;
 constexpr uint64_t kStreamDelay = 102u;
 
 // Users with more than kHeavy entries in a minibatch are split in chunks of
-// kChunk entries, processed apart from the per-user kernel.
+// kChunk entries, each a work item of its own.
 constexpr int32_t kHeavy = 96;
 constexpr int32_t kChunk = 64;
+// The work list is sorted by length within tiles of 2^kTileBits users: the
+// items that a warp takes together then have (nearly) one length, and a tile's
+// rows stay close in memory.
+constexpr int kTileBits = 8;
+// Cost of an item in a warp's share: its entries plus kItemCost.
+constexpr int32_t kItemCost = 5;
 // Replica accumulators: an item gets one delta row per kItemRep entries
 // (largest minibatch count, rounded up to a power of two); a heavy user one
 // per kUserRep chunks.  Replicas spread the fp32 reductions of popular rows
@@ -41,36 +47,29 @@ constexpr int32_t kUserRep = 64;
 #endif
 constexpr int32_t kMaxRep = ESSPT_MAX_REP;
 
-// Rows of 36..64 values (9..16 float4 slices) take the work-list path: every
-// user with 1..kHeavy entries in a minibatch is one work item beside the
-// chunks of the heavy users, processed by one kernel, and the users without
-// entries are copied forward by a streaming kernel.
-inline bool uses_work16(int32_t K) { return K > 32 && K <= 64; }
-// Work-list path: the kHot items with the most entries of each minibatch have
-// their updates summed per warp in shared memory and added to the replica
-// rows once per warp instead of once per entry (0 = off).  An entry of hot
-// slot h carries rec_dst = -1 - h.
-#ifndef ESSPT_W16_HOT
-#define ESSPT_W16_HOT 2
-#endif
-constexpr int kHot = ESSPT_W16_HOT;
-inline bool uses_hot(int32_t K) { return kHot > 0 && uses_work16(K); }
-// Resident blocks per SM that the launches of the forward copy and of the
-// work kernel ask for (the occupancy limit caps the second).
-constexpr int kCopyBlocksPerSm = 8;
-constexpr int kWorkBlocksPerSm = 8;
+// Rows of 36..64 values: the kHot items with the most entries of each minibatch
+// have their updates summed per row group in shared memory and added to the
+// replica rows once per warp instead of once per entry.
+constexpr int kHot = 2;
+inline bool uses_hot(int32_t K) { return K > 32 && K <= 64; }
 
 // Row stride (in float4) of the item delta replicas: K rounded up to a whole
-// number of 32-byte sectors, so that a row's reductions touch the fewest sectors.
-inline int32_t dR_stride4(int32_t K) { return ((K + 7) / 8) * 2; }
+// number of 128-byte lines where that adds at most a third, so that eight
+// lanes' 128 bytes of a reduction are one request, else to 32-byte sectors, so
+// that they touch the fewest.
+inline int32_t dR_stride4(int32_t K) {
+  const int32_t lines = (K + 31) / 32 * 8;
+  return 3 * lines <= K ? lines : (K + 7) / 8 * 2;
+}
 
 struct ScheduleArgs {
   int32_t* v;              // [P] read versions (in: v(c-1), out: v(c))
+  int32_t* vslot;          // [P] out: ring slot v mod nslots of each read version
   uint32_t* status;        // latched error bits
   const uint32_t* thr;     // [dmax+1] ESSP delay thresholds, thr[k] = floor((1-p)^k 2^32)
   const uint32_t* vap_norm;  // [s+1] VAP: bits of |X[c-1] - X[c-1-k]|_inf (fp32, >= 0)
   double vap_bound;        // VAP: v0 / sqrt(c)
-  int32_t P, c, s, model, phased, dmax;
+  int32_t P, c, s, nslots, model, phased, dmax;
   uint64_t seed;
 };
 
@@ -83,39 +82,39 @@ struct SgdArgs {
   int32_t nslots;           // s + 2
   int32_t slot_base;        // slot merged from (c-1, or c if INCs already landed there)
   int32_t slot_out;         // slot of version c
-  int32_t n_b;              // entries of minibatch b
-  const int32_t* v;         // [P] read versions
-  const int32_t* worker;    // [n_users]
+  const int32_t* vslot;     // [P] ring slots of the read versions
   const int32_t* uoff;      // [n_users+1] entry offsets of minibatch b (relative)
-  const int32_t* rec_j;     // item of each entry of minibatch b; in row mode the ring row
-                            // (slot * n_rows + N + item) of the item's cached version
-  const float* rec_D;       // value of each entry of minibatch b
-  const int32_t* rec_dst;   // replica row in dR that each entry's item update adds into
-  const int32_t* item_rep;  // [M+1] prefix of extra replicas: replica 0 of item j is row j of dR,
-                            // replica r > 0 row M + item_rep[j] + r - 1
+  const int32_t* rec_row;   // row mode: ring row (slot * n_rows + N + item) of each record's item
   float* dR;                // item delta replicas (all zero between clocks)
-  int32_t dR_ld;            // float4 per dR row (K rounded up to whole 32-byte sectors)
+  int32_t dR_ld;            // float4 per dR row (dR_stride4)
+  const int32_t* item_rep;  // see ItemMergeArgs; hot_item: [kHot] hot items of minibatch b, -1 if unused
+  const int32_t* hot_item;
   float eta, lambda;
   int32_t cap;
   double* sq_loss;          // optional
   int32_t row_mode;         // row-granular SSP: per-user slots and per-entry ring rows
   const int32_t* user_slot; // [n_users] row mode: ring slot of each user's cached row
-  // Work-list path: chg[u] = last clock that changed user row u (written with
-  // every user row that changes); an idle row whose slot already holds its
-  // current value is not copied forward: clock > copy_all_until and
-  // clock - chg[u] >= nslots (unchanged over the whole ring).
+  // chg[u] = last clock that changed user row u (written with every user row
+  // that changes); an idle row whose slot already holds its current value is
+  // not copied forward: clock > copy_all_until and clock - chg[u] >= nslots
+  // (unchanged over the whole ring).
   int32_t* chg;
   int32_t clock, copy_all_until;
-  const int32_t* hot_item;  // [kHot] work-list path: item of each hot slot of minibatch b, -1 if unused
 };
 
-// Chunks of heavy users: x = user, y = begin, z = end (relative), w = replica row in dL.
-// On the work-list path a user with 1..kHeavy entries is one item with w = -1
-// (its row of version c is written directly).
-struct ChunkArgs {
+// The work list of minibatch b: x = user, y = first entry, z = replica row
+// in dL of a heavy user's chunk, or -1 for a user with 1..kHeavy entries (its
+// row of version c is written directly), w = entries << 16 | worker; sorted
+// by length within tiles of 2^kTileBits users.  Records: x = item, y = replica
+// row in dR that the item's update adds into, or -1 - h for hot slot h, z =
+// value (fp32), w unused (16 bytes are one aligned copy).
+// Warp w takes items [part[w], part[w+1]).
+struct StreamArgs {
   SgdArgs a;
-  const int4* chunk;
-  int64_t n_chunks;
+  const int4* items;
+  const int4* rec;
+  const int32_t* part;
+  int64_t n_warps;
   float* dL;                // heavy-user delta replicas (all zero between clocks)
 };
 
@@ -129,7 +128,7 @@ struct HeavyMergeArgs {
   float* dL;
   float eta;
   int32_t cap;
-  int32_t* chg;             // work-list path: set chg[user] = clock (see SgdArgs)
+  int32_t* chg;             // set chg[user] = clock (see SgdArgs)
   int32_t clock;
 };
 
@@ -138,7 +137,8 @@ struct ItemMergeArgs {
   float* ring;
   int64_t n_rows;
   int32_t K, n_users, n_items, slot_base, slot_out;
-  const int32_t* item_rep;
+  const int32_t* item_rep;  // [M+1] prefix of extra replicas: replica 0 of item j is row j of dR,
+                            // replica r > 0 row M + item_rep[j] + r - 1
   float* dR;
   int32_t dR_ld;
   const int32_t* item_cnt;  // [M] entries per item in minibatch b
@@ -163,21 +163,27 @@ cudaError_t launch_get(const float* ring, int64_t n_rows, int32_t K, int32_t nsl
                        int32_t* rowver, int32_t c, int32_t s, int32_t* vmin, cudaStream_t st);
 cudaError_t launch_inc(float* slot, int64_t n_rows, int32_t K, const int32_t* ids, const float* d, int64_t n,
                        uint32_t* status, cudaStream_t st);
-cudaError_t launch_sgd_users(const SgdArgs& a, cudaStream_t st);
+// The SGD kernel of one clock; the warps it can use at row width K on this
+// device and the items a warp takes at a time; and the split of a minibatch's
+// n_items work items over n_warps of them (pre: see LayoutBuild).
+cudaError_t launch_sgd_stream(const StreamArgs& a, cudaStream_t st);
+int64_t stream_max_warps(int32_t K);
+int stream_groups_per_warp(int32_t K);
+cudaError_t launch_stream_partition(const int64_t* pre, int64_t n_items, int64_t n_warps, int32_t* part,
+                                    cudaStream_t st);
 // Row-granular SSP, before the SGD kernels of clock c: refresh the cached
 // version of every row a worker reads (rowver[p * n_rows + r], -1 = never
 // read) to c-1 where it is missing or older than c-1-s, and write the ring
 // slot of each user's row and the ring row of each entry's item row.
 struct RowRefreshArgs {
   int32_t* rowver;
-  const int32_t* worker;   // [n_users]
-  const int32_t* uoff;     // [n_users+1] of minibatch b
-  const int32_t* rec_u;    // [n_b] user of each entry
-  const int32_t* rec_j;    // [n_b] item of each entry
+  const int4* items;       // work list of minibatch b
+  int64_t n_items;
+  const int4* rec;         // its records
   int64_t n_rows;
-  int32_t n_users, n_b, c, s, nslots;
-  int32_t* user_slot;      // out [n_users]
-  int32_t* rec_row;        // out [n_b]
+  int32_t n_users, c, s, nslots;
+  int32_t* user_slot;      // out [n_users], for the users of the work list
+  int32_t* rec_row;        // out, one per record
 };
 cudaError_t launch_row_refresh(const RowRefreshArgs& a, cudaStream_t st);
 
@@ -199,11 +205,6 @@ struct SeqArgs {
   double* sq_loss;          // optional
 };
 cudaError_t launch_seq_clock(const SeqArgs& a, cudaStream_t st);
-cudaError_t launch_sgd_chunks(const ChunkArgs& a, cudaStream_t st);
-// Work-list path (uses_work16): the items of minibatch b (light users and
-// heavy-user chunks) and the forward copy of the users without entries.
-cudaError_t launch_sgd_work16(const ChunkArgs& a, cudaStream_t st);
-cudaError_t launch_user_copy(const SgdArgs& a, cudaStream_t st);
 cudaError_t launch_heavy_merge(const HeavyMergeArgs& a, cudaStream_t st);
 cudaError_t launch_item_merge(const ItemMergeArgs& a, cudaStream_t st);
 cudaError_t launch_objective(const float* slot, int64_t n_users, int32_t K, const int32_t* rec_u,
@@ -223,30 +224,32 @@ struct LayoutBuild {
   int32_t* rec_u;
   int32_t* rec_j;
   float* rec_D;
-  int32_t* rec_dst;     // replica row of each entry's item update
+  int4* rec;            // [n_obs] records of the SGD kernel (see StreamArgs)
+  int32_t* hot_item;    // [F][kHot] hot items of each minibatch, or null
   int32_t* uoff;        // [F][n_users+1]
   int64_t* mb_base;     // [F+1]
   int32_t* item_cnt;    // [F][n_items]
   int32_t* item_rep;    // [n_items+1]
-  int4* chunk;          // [max_chunks]
+  int4* chunk;          // [max_chunks] work items (see StreamArgs)
   int64_t* chunk_base;  // [F+1]
   int4* heavy;          // [max_heavy]
   int64_t* heavy_base;  // [F+1]
   int64_t max_chunks, max_heavy;
-  bool light_items;     // also list every user with 1..kHeavy entries (work-list path)
-  int32_t* hot_item;    // [F][kHot] work-list path with kHot > 0: the hot items of each minibatch
   // scratch
   void* scratch;
   size_t scratch_bytes;
+  const int64_t* pre;   // out, in the scratch: [items+1] summed cost of the items before each
   uint32_t* status;
 };
 
 size_t layout_scratch_bytes(int64_t n_obs, int64_t n_users, int64_t n_items, int32_t F);
-int64_t layout_max_chunks(int64_t n_obs, int32_t F, int64_t n_users, bool light_items);
+int64_t layout_max_chunks(int64_t n_obs, int32_t F, int64_t n_users);
 int64_t layout_max_heavy(int64_t n_obs, int32_t F);
 int64_t layout_max_item_reps(int64_t n_obs, int64_t n_items);
 int64_t layout_max_user_reps(int64_t n_obs);
-cudaError_t build_layout(const LayoutBuild& b, cudaStream_t st);
+cudaError_t build_layout(LayoutBuild& b, cudaStream_t st);
+// New values of n records from those of their entries.
+cudaError_t launch_refill(int4* rec, const float* D, int64_t n, cudaStream_t st);
 cudaError_t launch_validate(const LayoutBuild& b, cudaStream_t st);
 // Staged minibatch check: su/sj (n entries) and suoff (n_off offsets) against
 // the resident ru/rj/ruoff; a difference latches kErrInput.

@@ -81,8 +81,7 @@ __global__ void gather_kernel(const uint32_t* __restrict__ perm, int64_t n_obs, 
 // per (b, u): chunks, heavy flag and extra replica rows.
 __global__ void offsets_kernel(const int64_t* __restrict__ off, int64_t n_users, int32_t F, int32_t* __restrict__ uoff,
                                int64_t* __restrict__ mb_base, const int32_t* __restrict__ cnt,
-                               int32_t* __restrict__ nch, int32_t* __restrict__ hflag, int32_t* __restrict__ hextra,
-                               bool light_items) {
+                               int32_t* __restrict__ nch, int32_t* __restrict__ hflag, int32_t* __restrict__ hextra) {
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   const int64_t total = (int64_t)F * (n_users + 1);
   for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < total; x += stride) {
@@ -93,7 +92,7 @@ __global__ void offsets_kernel(const int64_t* __restrict__ off, int64_t n_users,
     if (u < n_users) {
       const int32_t n = cnt[b * n_users + u];
       const int32_t c = n > kHeavy ? (n + kChunk - 1) / kChunk : 0;
-      nch[b * n_users + u] = c + (light_items && n > 0 && c == 0 ? 1 : 0);
+      nch[b * n_users + u] = c + (n > 0 && c == 0 ? 1 : 0);
       hflag[b * n_users + u] = c > 0 ? 1 : 0;
       hextra[b * n_users + u] = c > 0 ? user_reps(c) - 1 : 0;
     }
@@ -101,17 +100,24 @@ __global__ void offsets_kernel(const int64_t* __restrict__ off, int64_t n_users,
   if (blockIdx.x == 0 && threadIdx.x == 0) mb_base[F] = off[(int64_t)F * n_users];
 }
 
-// Chunk descriptors (user, begin, end, replica row) and heavy-user
-// descriptors (user, first extra replica row, replicas, entries).  Replica 0
-// of heavy user u is row u of dL; replicas 1.. are rows n_users + hext[...].
+// Work items (see StreamArgs) and heavy-user descriptors (user, first extra
+// replica row, replicas, entries).  Replica 0 of heavy user u is row u of dL;
+// replicas 1.. are rows n_users + hext[...].
 __global__ void heavy_kernel(const int64_t* __restrict__ choff, const int32_t* __restrict__ nch,
                              const int64_t* __restrict__ hoff, const int64_t* __restrict__ hext,
-                             const int32_t* __restrict__ uoff, int64_t n_users, int32_t F, int4* __restrict__ chunk,
+                             const int32_t* __restrict__ uoff, const int32_t* __restrict__ worker, int64_t n_users,
+                             int32_t F, int4* __restrict__ chunk,
+                             uint32_t* __restrict__ key, uint32_t* __restrict__ val, int64_t n_tiles,
                              int64_t* __restrict__ chunk_base, int64_t max_chunks, int4* __restrict__ heavy,
                              int64_t* __restrict__ heavy_base, int64_t max_heavy, int64_t max_user_reps,
                              uint32_t* status) {
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   const int64_t total = (int64_t)F * n_users;
+  auto put = [&](int64_t at, int64_t b, int64_t u, int32_t beg, int32_t dst, int32_t n) {
+    chunk[at] = make_int4((int32_t)u, beg, dst, n << 16 | worker[u]);
+    key[at] = (uint32_t)(b * n_tiles + (u >> kTileBits)) << 7 | (uint32_t)(127 - n);
+    val[at] = (uint32_t)at;
+  };
   for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < total; x += stride) {
     const int32_t nc = nch[x];
     if (nc == 0) continue;
@@ -122,7 +128,7 @@ __global__ void heavy_kernel(const int64_t* __restrict__ choff, const int32_t* _
         atomicOr(status, kErrInput);
         continue;
       }
-      chunk[choff[x]] = make_int4((int32_t)u, beg, end, -1);
+      put(choff[x], b, u, beg, -1, end - beg);
       continue;
     }
     const int32_t reps = user_reps(nc);
@@ -136,7 +142,7 @@ __global__ void heavy_kernel(const int64_t* __restrict__ choff, const int32_t* _
     for (int32_t t = 0; t < nc; ++t) {
       const int32_t r = t & (reps - 1);
       const int32_t dst = r == 0 ? (int32_t)u : (int32_t)(extra0 + r - 1);
-      chunk[choff[x] + t] = make_int4((int32_t)u, beg + t * kChunk, min(end, beg + (t + 1) * kChunk), dst);
+      put(choff[x] + t, b, u, beg + t * kChunk, dst, min(kChunk, end - beg - t * kChunk));
     }
   }
   for (int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; b <= F; b += stride) {
@@ -161,15 +167,30 @@ __global__ void item_reps_kernel(const int32_t* __restrict__ item_cnt, int64_t n
   }
 }
 
-// Replica row of every entry's item update: entry t (position within its
+// The work list in its final order, and each item's cost.
+__global__ void place_items_kernel(const int4* __restrict__ raw, const uint32_t* __restrict__ perm, int64_t n,
+                                   int4* __restrict__ items, int32_t* __restrict__ cost) {
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x <= n; x += stride) {
+    if (x == n) {
+      cost[x] = 0;
+      continue;
+    }
+    const int4 it = raw[perm[x]];
+    items[x] = it;
+    cost[x] = (it.w >> 16) + kItemCost;
+  }
+}
+
+// The records of the SGD kernel, one per entry.  Replica row of an entry's
+// item update: entry t (position within its
 // minibatch) of item j adds into replica (t mod replicas of j): replica 0 is
-// row j, replica r > 0 row n_items + item_rep[j] + r - 1.
-// With hot_item (work-list path, kHot > 0) an entry of hot slot h of its
-// minibatch gets -1 - h instead.
-__global__ void dst_kernel(const uint32_t* __restrict__ key, const int64_t* __restrict__ mb_base,
-                           const int32_t* __restrict__ rec_j, const int32_t* __restrict__ item_rep, int64_t n_obs,
-                           int64_t n_users, int64_t n_items, const int32_t* __restrict__ hot_item,
-                           int32_t* __restrict__ rec_dst) {
+// row j, replica r > 0 row n_items + item_rep[j] + r - 1.  With hot_item an
+// entry of hot slot h of its minibatch gets -1 - h instead.
+__global__ void records_kernel(const uint32_t* __restrict__ key, const int64_t* __restrict__ mb_base,
+                               const int32_t* __restrict__ rec_j, const float* __restrict__ rec_D,
+                               const int32_t* __restrict__ item_rep, int64_t n_obs, int64_t n_users,
+                               int64_t n_items, const int32_t* __restrict__ hot_item, int4* __restrict__ rec) {
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n_obs; k += stride) {
     const int64_t b = (int64_t)key[k] / n_users;
@@ -177,18 +198,18 @@ __global__ void dst_kernel(const uint32_t* __restrict__ key, const int64_t* __re
     const int32_t j = rec_j[k];
     const int32_t e0 = item_rep[j], e1 = item_rep[j + 1];  // extra replicas of j: e1 - e0 (reps - 1)
     const int32_t r = (int32_t)(t & (int64_t)(e1 - e0));    // reps is a power of two
-    int32_t d = r == 0 ? j : (int32_t)(n_items + e0 + r - 1);
+    int32_t dst = r == 0 ? j : (int32_t)(n_items + e0 + r - 1);
     if (hot_item != nullptr)
       for (int h = 0; h < kHot; ++h)
-        if (hot_item[b * kHot + h] == j) d = -1 - h;
-    rec_dst[k] = d;
+        if (hot_item[b * kHot + h] == j) dst = -1 - h;
+    rec[k] = make_int4(j, dst, __float_as_int(rec_D[k]), 0);
   }
 }
 
 // The kHot items with the most entries of each minibatch (at least 2), most
 // popular first, ties by id; -1 for unused slots.  Host side, at setup.
 cudaError_t build_hot(const LayoutBuild& b, cudaStream_t st) {
-  if (kHot <= 0 || b.hot_item == nullptr) return cudaSuccess;
+  if (b.hot_item == nullptr) return cudaSuccess;
   const size_t FM = (size_t)b.F * (size_t)b.n_items;
   std::vector<int32_t> cnt(FM), hot((size_t)b.F * kHot, -1), idx((size_t)b.n_items);
   cudaError_t e = cudaMemcpyAsync(cnt.data(), b.item_cnt, sizeof(int32_t) * FM, cudaMemcpyDeviceToHost, st);
@@ -205,6 +226,12 @@ cudaError_t build_hot(const LayoutBuild& b, cudaStream_t st) {
   e = cudaMemcpyAsync(b.hot_item, hot.data(), sizeof(int32_t) * hot.size(), cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   return e;
+}
+
+__global__ void refill_kernel(int4* __restrict__ rec, const float* __restrict__ D, int64_t n) {
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += stride)
+    rec[k].z = __float_as_int(D[k]);
 }
 
 // A staged minibatch against the loaded one: every user id, item id and
@@ -230,28 +257,30 @@ int blocks_for(int64_t n) {
 }
 
 struct ScratchPlan {
-  size_t key_in, key_out, val_in, val_out, cnt, off, nch, choff, hflag, hoff, hextra, hext, ireps, cub, total;
+  size_t key_in, key_out, val_in, val_out, cnt, off, nch, choff, hflag, hoff, hextra, hext, ireps, raw, pre, cub, total;
   size_t cub_bytes;
 };
 
 ScratchPlan plan(int64_t n_obs, int64_t n_users, int64_t n_items, int32_t F) {
   ScratchPlan p{};
   const int64_t keys = (int64_t)F * n_users;
-  size_t sort_bytes = 0, scan_bytes = 0, scan2_bytes = 0;
+  const int64_t items = std::min(n_obs, layout_max_chunks(n_obs, F, n_users));  // an item holds an entry or more
+  size_t sort_bytes = 0, scan_bytes = 0, scan2_bytes = 0, scan3_bytes = 0;
   cub::DeviceRadixSort::SortPairs(nullptr, sort_bytes, (const uint32_t*)nullptr, (uint32_t*)nullptr,
                                   (const uint32_t*)nullptr, (uint32_t*)nullptr, (int)std::max<int64_t>(n_obs, 1), 0,
                                   32);
   cub::DeviceScan::ExclusiveSum(nullptr, scan_bytes, (const int32_t*)nullptr, (int64_t*)nullptr, (int)(keys + 1));
   cub::DeviceScan::ExclusiveSum(nullptr, scan2_bytes, (const int32_t*)nullptr, (int32_t*)nullptr,
                                 (int)(n_items + 1));
-  p.cub_bytes = std::max(sort_bytes, std::max(scan_bytes, scan2_bytes));
+  cub::DeviceScan::ExclusiveSum(nullptr, scan3_bytes, (const int32_t*)nullptr, (int64_t*)nullptr, (int)(items + 1));
+  p.cub_bytes = std::max(std::max(sort_bytes, scan3_bytes), std::max(scan_bytes, scan2_bytes));
   size_t o = 0;
   auto take = [&o](size_t bytes) {
     const size_t at = o;
     o += align256(bytes);
     return at;
   };
-  p.key_in = take(sizeof(uint32_t) * n_obs);
+  p.key_in = take(sizeof(uint32_t) * (n_obs + 1));
   p.key_out = take(sizeof(uint32_t) * n_obs);
   p.val_in = take(sizeof(uint32_t) * n_obs);
   p.val_out = take(sizeof(uint32_t) * n_obs);
@@ -264,6 +293,8 @@ ScratchPlan plan(int64_t n_obs, int64_t n_users, int64_t n_items, int32_t F) {
   p.hextra = take(sizeof(int32_t) * (keys + 1));
   p.hext = take(sizeof(int64_t) * (keys + 1));
   p.ireps = take(sizeof(int32_t) * (n_items + 1));
+  p.raw = take(sizeof(int4) * items);
+  p.pre = take(sizeof(int64_t) * (items + 1));
   p.cub = take(p.cub_bytes);
   p.total = o;
   return p;
@@ -282,9 +313,9 @@ size_t layout_scratch_bytes(int64_t n_obs, int64_t n_users, int64_t n_items, int
 }
 
 // A heavy segment has n > kHeavy >= kChunk entries and ceil(n/kChunk) < 2n/kChunk chunks.
-// On the work-list path every user with entries in a minibatch adds one more item.
-int64_t layout_max_chunks(int64_t n_obs, int32_t F, int64_t n_users, bool light_items) {
-  return 2 * n_obs / kChunk + F + 1 + (light_items ? std::min(n_obs, (int64_t)F * n_users) : 0);
+// Every other user with entries in a minibatch adds one item.
+int64_t layout_max_chunks(int64_t n_obs, int32_t F, int64_t n_users) {
+  return 2 * n_obs / kChunk + F + 1 + std::min(n_obs, (int64_t)F * n_users);
 }
 
 int64_t layout_max_heavy(int64_t n_obs, int32_t F) { return n_obs / (kHeavy + 1) + F + 1; }
@@ -295,7 +326,7 @@ int64_t layout_max_item_reps(int64_t n_obs, int64_t n_items) { return n_items + 
 // Extra replica rows of heavy users: reps - 1 < 3 nch / (2 kUserRep), sum nch < 2 n_obs / kChunk.
 int64_t layout_max_user_reps(int64_t n_obs) { return 3 * n_obs / (kChunk * kUserRep) + 2; }
 
-cudaError_t build_layout(const LayoutBuild& b, cudaStream_t st) {
+cudaError_t build_layout(LayoutBuild& b, cudaStream_t st) {
   const ScratchPlan p = plan(b.n_obs, b.n_users, b.n_items, b.F);
   if (b.scratch_bytes < p.total) return cudaErrorInvalidValue;
   char* s = static_cast<char*>(b.scratch);
@@ -333,8 +364,7 @@ cudaError_t build_layout(const LayoutBuild& b, cudaStream_t st) {
   size_t tb = p.cub_bytes;
   if ((e = cub::DeviceScan::ExclusiveSum(cub_tmp, tb, cnt, off, (int)(keys + 1), st)) != cudaSuccess) return e;
   offsets_kernel<<<blocks_for((int64_t)b.F * (b.n_users + 1)), 256, 0, st>>>(off, b.n_users, b.F, b.uoff, b.mb_base,
-                                                                            cnt, nch, hflag, hextra,
-                                                                            b.light_items);
+                                                                            cnt, nch, hflag, hextra);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   tb = p.cub_bytes;
   if ((e = cub::DeviceScan::ExclusiveSum(cub_tmp, tb, nch, choff, (int)(keys + 1), st)) != cudaSuccess) return e;
@@ -342,19 +372,46 @@ cudaError_t build_layout(const LayoutBuild& b, cudaStream_t st) {
   if ((e = cub::DeviceScan::ExclusiveSum(cub_tmp, tb, hflag, hoff, (int)(keys + 1), st)) != cudaSuccess) return e;
   tb = p.cub_bytes;
   if ((e = cub::DeviceScan::ExclusiveSum(cub_tmp, tb, hextra, hext, (int)(keys + 1), st)) != cudaSuccess) return e;
-  heavy_kernel<<<blocks_for(keys + 1), 256, 0, st>>>(choff, nch, hoff, hext, b.uoff, b.n_users, b.F, b.chunk,
-                                                     b.chunk_base, b.max_chunks, b.heavy, b.heavy_base, b.max_heavy,
-                                                     layout_max_user_reps(b.n_obs), b.status);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
   item_reps_kernel<<<blocks_for(b.n_items + 1), 256, 0, st>>>(b.item_cnt, b.n_items, b.F, ireps);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   tb = p.cub_bytes;
   if ((e = cub::DeviceScan::ExclusiveSum(cub_tmp, tb, ireps, b.item_rep, (int)(b.n_items + 1), st)) != cudaSuccess)
     return e;
-  if (b.n_obs == 0) return cudaSuccess;
-  if ((e = build_hot(b, st)) != cudaSuccess) return e;
-  dst_kernel<<<blocks_for(b.n_obs), 256, 0, st>>>(key_out, b.mb_base, b.rec_j, b.item_rep, b.n_obs, b.n_users,
-                                                  b.n_items, kHot > 0 ? b.hot_item : nullptr, b.rec_dst);
+  if (b.n_obs > 0) {
+    if ((e = build_hot(b, st)) != cudaSuccess) return e;
+    records_kernel<<<blocks_for(b.n_obs), 256, 0, st>>>(key_out, b.mb_base, b.rec_j, b.rec_D, b.item_rep, b.n_obs,
+                                                        b.n_users, b.n_items, b.hot_item, b.rec);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  }
+  // The work list, then its order: by tile of users and length, ties in user
+  // order (the sort is stable).  The sort buffers of the entries are free now.
+  int4* raw = reinterpret_cast<int4*>(s + p.raw);
+  int64_t* pre = reinterpret_cast<int64_t*>(s + p.pre);
+  const int64_t n_tiles = (b.n_users >> kTileBits) + 1;
+  heavy_kernel<<<blocks_for(keys + 1), 256, 0, st>>>(
+      choff, nch, hoff, hext, b.uoff, b.worker, b.n_users, b.F, raw, key_in, val_in, n_tiles, b.chunk_base,
+      std::min(b.n_obs, b.max_chunks), b.heavy, b.heavy_base, b.max_heavy, layout_max_user_reps(b.n_obs), b.status);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  int64_t n = 0;
+  if ((e = cudaMemcpyAsync(&n, choff + keys, sizeof n, cudaMemcpyDeviceToHost, st)) != cudaSuccess) return e;
+  if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return e;
+  if (n > std::min(b.n_obs, b.max_chunks)) return cudaErrorInvalidValue;
+  b.pre = pre;
+  if (n > 0) {
+    tb = p.cub_bytes;
+    e = cub::DeviceRadixSort::SortPairs(cub_tmp, tb, key_in, key_out, val_in, val_out, (int)n, 0,
+                                        bits_for((uint64_t)b.F * n_tiles << 7), st);
+    if (e != cudaSuccess) return e;
+  }
+  place_items_kernel<<<blocks_for(n + 1), 256, 0, st>>>(raw, val_out, n, b.chunk, reinterpret_cast<int32_t*>(key_in));
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  tb = p.cub_bytes;
+  return cub::DeviceScan::ExclusiveSum(cub_tmp, tb, reinterpret_cast<int32_t*>(key_in), pre, (int)(n + 1), st);
+}
+
+cudaError_t launch_refill(int4* rec, const float* D, int64_t n, cudaStream_t st) {
+  if (n <= 0) return cudaSuccess;
+  refill_kernel<<<blocks_for(n), 256, 0, st>>>(rec, D, n);
   return cudaGetLastError();
 }
 

@@ -1,5 +1,5 @@
-// Small inline-PTX helpers: vector loads/stores with L2 eviction hints and
-// vector fp32 reductions into global memory (sm_90 and later).
+// Small inline-PTX helpers: vector loads/stores with L2 eviction hints, packed
+// fp32 arithmetic, and vector fp32 reductions into global memory.
 #pragma once
 
 #include <stdint.h>
@@ -10,37 +10,6 @@ __device__ __forceinline__ uint64_t policy_evict_first() {
   uint64_t p;
   asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
   return p;
-}
-
-__device__ __forceinline__ uint64_t policy_evict_last() {
-  uint64_t p;
-  asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(p));
-  return p;
-}
-
-// Streaming load: skip L1, mark the L2 lines for early eviction.
-__device__ __forceinline__ float4 ld_stream(const float4* p, uint64_t pol) {
-  float4 r;
-  asm volatile("ld.global.L1::no_allocate.L2::cache_hint.v4.f32 {%0,%1,%2,%3}, [%4], %5;"
-               : "=f"(r.x), "=f"(r.y), "=f"(r.z), "=f"(r.w)
-               : "l"(p), "l"(pol));
-  return r;
-}
-
-// Load that keeps the line in L2 (hot, reused rows).
-__device__ __forceinline__ float4 ld_keep(const float4* p, uint64_t pol) {
-  float4 r;
-  asm volatile("ld.global.L2::cache_hint.v4.f32 {%0,%1,%2,%3}, [%4], %5;"
-               : "=f"(r.x), "=f"(r.y), "=f"(r.z), "=f"(r.w)
-               : "l"(p), "l"(pol));
-  return r;
-}
-
-__device__ __forceinline__ void st_stream(float4* p, float4 v, uint64_t pol) {
-  asm volatile("st.global.L1::no_allocate.L2::cache_hint.v4.f32 [%0], {%1,%2,%3,%4}, %5;"
-               :
-               : "l"(p), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "l"(pol)
-               : "memory");
 }
 
 // Predicated forms: the access happens only when `pred` is true, without a
@@ -65,45 +34,99 @@ __device__ __forceinline__ void st_stream_if(float4* p, float4 v, uint64_t pol, 
       : "memory");
 }
 
-// out[0..3] += v when `pred`, performed at L2 (vector reduction, sm_90 and
-// later), predicated inside the asm so that no branch surrounds it.
-__device__ __forceinline__ void red_add_v4_if(float4* p, float4 v, bool pred) {
-  asm volatile("{\n .reg .pred q;\n setp.ne.b32 q, %5, 0;\n @q red.global.add.v4.f32 [%0], {%1,%2,%3,%4};\n}" ::"l"(p),
-               "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "r"((int)pred)
+// 16-byte asynchronous global -> shared copy (bypassing L1) with an L2
+// eviction-priority policy for the source lines, and a 4-byte one; nothing
+// happens when `pred` is false.
+__device__ __forceinline__ void cp_async16_hint_if(void* smem, const void* gmem, bool pred, uint64_t pol) {
+  const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
+  asm volatile(
+      "{\n .reg .pred q;\n setp.ne.b32 q, %2, 0;\n"
+      " @q cp.async.cg.shared.global.L2::cache_hint [%0], [%1], 16, %3;\n}" ::"r"(s),
+      "l"(gmem), "r"((int)pred), "l"(pol)
+      : "memory");
+}
+__device__ __forceinline__ void cp_async4_if(void* smem, const void* gmem, bool pred) {
+  const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
+  asm volatile("{\n .reg .pred q;\n setp.ne.b32 q, %2, 0;\n @q cp.async.ca.shared.global [%0], [%1], 4;\n}" ::"r"(s),
+               "l"(gmem), "r"((int)pred)
                : "memory");
 }
 
-// 16-byte asynchronous global -> shared copy (bypassing L1); when `pred` is
-// false the 16 shared bytes are zero-filled and nothing is read.
-__device__ __forceinline__ void cp_async16(void* smem, const void* gmem, bool pred) {
-  const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(s), "l"(gmem), "r"(pred ? 16 : 0) : "memory");
-}
-// The same with an L2 eviction-priority policy for the source lines.
-__device__ __forceinline__ void cp_async16_hint(void* smem, const void* gmem, bool pred, uint64_t pol) {
-  const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
-  asm volatile("cp.async.cg.shared.global.L2::cache_hint [%0], [%1], 16, %2, %3;" ::"r"(s), "l"(gmem),
-               "r"(pred ? 16 : 0), "l"(pol)
-               : "memory");
-}
-
-// Streaming 32-bit loads (entries read once per clock): skip L1, evict-first in L2.
+// Streaming 32-bit load (read once per clock): skip L1, evict-first in L2.
 __device__ __forceinline__ int32_t ld_stream_i32(const int32_t* p, uint64_t pol) {
   int32_t r;
   asm volatile("ld.global.L1::no_allocate.L2::cache_hint.b32 %0, [%1], %2;" : "=r"(r) : "l"(p), "l"(pol));
   return r;
 }
-__device__ __forceinline__ float ld_stream_f32(const float* p, uint64_t pol) {
-  float r;
-  asm volatile("ld.global.L1::no_allocate.L2::cache_hint.f32 %0, [%1], %2;" : "=f"(r) : "l"(p), "l"(pol));
-  return r;
-}
-
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 
 // out[0..3] += v, performed at L2 (no return value).
 __device__ __forceinline__ void red_add_v4(float4* p, float4 v) { atomicAdd(p, v); }
+
+// One float4 slice as two packed fp32 pairs, the operands of the packed fp32
+// instructions (sm_100 and later): two IEEE fp32 operations per instruction,
+// each rounded as its scalar form.
+typedef unsigned long long u64;
+struct f2x2 {
+  u64 lo, hi;
+};
+__device__ __forceinline__ u64 pack2(float x, float y) {
+  u64 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+  return r;
+}
+__device__ __forceinline__ float sum2(u64 v) {
+  float x, y;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(v));
+  return x + y;
+}
+__device__ __forceinline__ u64 mul2(u64 a, u64 b) {
+  u64 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ u64 add2(u64 a, u64 b) {
+  u64 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ u64 fma2(u64 a, u64 b, u64 c) {
+  u64 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+// r = *p when `pred`, else r as it was; through L1, for memory that no kernel
+// in flight writes.
+__device__ __forceinline__ void ldg_f2x2_if(f2x2& r, const float4* p, bool pred) {
+  asm volatile("{\n .reg .pred q;\n setp.ne.b32 q, %3, 0;\n @q ld.global.nc.v2.b64 {%0, %1}, [%2];\n}"
+               : "+l"(r.lo), "+l"(r.hi)
+               : "l"(p), "r"((int)pred));
+}
+__device__ __forceinline__ f2x2 lds_f2x2(const float4* p) {
+  const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(p);
+  return f2x2{v.x, v.y};
+}
+__device__ __forceinline__ void sts_f2x2(float4* p, u64 lo, u64 hi) {
+  *reinterpret_cast<ulonglong2*>(p) = make_ulonglong2(lo, hi);
+}
+__device__ __forceinline__ void st_stream_f2x2_if(float4* p, u64 lo, u64 hi, uint64_t pol, bool pred) {
+  asm volatile(
+      "{\n .reg .pred q;\n setp.ne.b32 q, %4, 0;\n"
+      " @q st.global.L1::no_allocate.L2::cache_hint.v2.b64 [%0], {%1, %2}, %3;\n}" ::"l"(p),
+      "l"(lo), "l"(hi), "l"(pol), "r"((int)pred)
+      : "memory");
+}
+// p[0..3] += (lo, hi) when `pred`, performed at L2 (vector reduction, sm_90
+// and later), predicated inside the asm so that no branch surrounds it.
+__device__ __forceinline__ void red_add_f2x2_if(float4* p, u64 lo, u64 hi, bool pred) {
+  float a, b, c, d;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(lo));
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(c), "=f"(d) : "l"(hi));
+  asm volatile("{\n .reg .pred q;\n setp.ne.b32 q, %5, 0;\n @q red.global.add.v4.f32 [%0], {%1,%2,%3,%4};\n}" ::"l"(p),
+               "f"(a), "f"(b), "f"(c), "f"(d), "r"((int)pred)
+               : "memory");
+}
 
 // SplitMix64 (Steele, Lea and Flood, OOPSLA 2014): output n of the sequence
 // whose state starts at s0 is mix64(s0 + n * 0x9E3779B97F4A7C15).

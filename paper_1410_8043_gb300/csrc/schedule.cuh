@@ -47,6 +47,7 @@ __device__ __forceinline__ void schedule_worker(const ScheduleArgs& a, int32_t p
   // ESSPT_EXTERNAL: v was written by the host; only the check below runs.
   if (v < lo || v > a.c - 1) atomicOr(a.status, kErrStale);
   a.v[p] = v;
+  a.vslot[p] = v % a.nslots;
 }
 
 }  // namespace esspt
