@@ -32,14 +32,17 @@ struct esspt_ctx {
   int32_t F = 0;
   int32_t *rec_u = nullptr, *rec_j = nullptr, *uoff = nullptr, *item_cnt = nullptr, *worker = nullptr;
   int32_t *item_rep = nullptr, *hot_item = nullptr;
-  int4* rec = nullptr;                // records of the SGD kernel
+  // The SGD kernel's stream: its geometry, words and places (see StreamArgs),
+  // and the first place of each minibatch.
+  StreamGeometry geo{1, 1};
+  uint32_t *sx = nullptr, *syz = nullptr, *place = nullptr, *row_x = nullptr;
+  std::vector<int64_t> stream_base;
   float *rec_D = nullptr, *dR = nullptr, *dL = nullptr;
   int32_t* rowver = nullptr;     // row-granular SSP: [P][n_rows] cached versions, -1 = never read
   int32_t* user_slot = nullptr;  // row-granular SSP: [n_users] per-clock ring slot of each user row
-  int32_t* rec_row = nullptr;    // row-granular SSP: per-clock ring row of each entry's item row
   int4 *chunk = nullptr, *heavy = nullptr;
   std::vector<int64_t> mb_base, chunk_base, heavy_base;
-  int32_t* part = nullptr;            // split of each minibatch's work items over the warps
+  int4* part = nullptr;               // split of each minibatch's work items over the warps
   std::vector<int64_t> part_base;     // [F+1] first word of each minibatch's split
   cudaEvent_t ev_before = nullptr, ev_after = nullptr;
   // Last clock that changed each user row, and the last clock at which every
@@ -201,9 +204,9 @@ bool is_host_ptr(const void* p) {
 }
 
 struct MfCarve {
-  size_t rec_u, rec_j, rec_D, rec, uoff, mb_base, item_cnt, item_rep, dR, worker, chunk, chunk_base, heavy, heavy_base, dL,
-      user_slot, rec_row, chg, hot_item, part, total;
-  int64_t max_chunks, max_heavy, dR_rows, dL_rows, part_rows;
+  size_t rec_u, rec_j, rec_D, sx, syz, place, steps, uoff, mb_base, item_cnt, item_rep, dR, worker, chunk, chunk_base, heavy, heavy_base, dL,
+      user_slot, row_x, chg, hot_item, part, total;
+  int64_t max_chunks, max_heavy, dR_rows, dL_rows, part_rows, max_places;
 };
 
 // Persistent MF workspace: entries laid out by (minibatch, user), per-minibatch
@@ -225,7 +228,11 @@ MfCarve mf_carve(int64_t n_obs, int64_t n_users, int64_t n_items, int32_t F, int
   k.rec_u = take(sizeof(int32_t) * (n_obs + 4));
   k.rec_j = take(sizeof(int32_t) * (n_obs + 4));
   k.rec_D = take(sizeof(float) * (n_obs + 4));
-  k.rec = take(sizeof(int4) * n_obs);
+  k.max_places = layout_max_places(n_obs, n_users, F, stream_geometry(K), stream_max_warps(K));
+  k.sx = take(sizeof(uint32_t) * k.max_places);
+  k.syz = take(2 * sizeof(uint32_t) * k.max_places);
+  k.place = take(sizeof(uint32_t) * k.max_chunks);
+  k.steps = take(sizeof(int32_t) * F);
   k.uoff = take(sizeof(int32_t) * (size_t)F * (n_users + 1));
   k.mb_base = take(sizeof(int64_t) * (F + 1));
   k.item_cnt = take(sizeof(int32_t) * (size_t)F * n_items);
@@ -237,16 +244,15 @@ MfCarve mf_carve(int64_t n_obs, int64_t n_users, int64_t n_items, int32_t F, int
   k.heavy = take(sizeof(int4) * k.max_heavy);
   k.heavy_base = take(sizeof(int64_t) * (F + 1));
   k.dL = take(sizeof(float) * (size_t)k.dL_rows * K);
-  // Row-granular SSP: per-clock user slots and entry ring rows (a minibatch
-  // holds at most n_obs entries).
+  // Row-granular SSP: per-clock user slots and x words of the stream.
   k.user_slot = row_mode ? take(sizeof(int32_t) * n_users) : o;
-  k.rec_row = row_mode ? take(sizeof(int32_t) * (n_obs + 4)) : o;
+  k.row_x = row_mode ? take(sizeof(uint32_t) * k.max_places) : o;
   // The clock that last changed each user row.
   k.chg = take(sizeof(int32_t) * n_users);
   k.hot_item = uses_hot(K) ? take(sizeof(int32_t) * (size_t)F * kHot) : o;
   // A minibatch uses at most one warp per work item.
-  k.part_rows = std::min((int64_t)F * (stream_max_warps(K) + 1), k.max_chunks + F);
-  k.part = take(sizeof(int32_t) * (size_t)k.part_rows);
+  k.part_rows = std::min((int64_t)F * stream_max_warps(K), k.max_chunks);
+  k.part = take(sizeof(int4) * (size_t)k.part_rows);
   k.total = o;
   return k;
 }
@@ -511,7 +517,6 @@ esspt_status esspt_mf_load(esspt_ctx* c, const int32_t* d_i, const int32_t* d_j,
   b.mb_base = reinterpret_cast<int64_t*>(w + k.mb_base);
   b.item_cnt = reinterpret_cast<int32_t*>(w + k.item_cnt);
   b.item_rep = reinterpret_cast<int32_t*>(w + k.item_rep);
-  b.rec = reinterpret_cast<int4*>(w + k.rec);
   b.hot_item = uses_hot(c->K) ? reinterpret_cast<int32_t*>(w + k.hot_item) : nullptr;
   b.chunk = reinterpret_cast<int4*>(w + k.chunk);
   b.chunk_base = reinterpret_cast<int64_t*>(w + k.chunk_base);
@@ -553,15 +558,39 @@ esspt_status esspt_mf_load(esspt_ctx* c, const int32_t* d_i, const int32_t* d_j,
     return fail(c, ESSPT_ECUDA, "internal: chunk list overflow");
   }
   // Split each minibatch's work items over the warps of the SGD kernel.
-  const int gpw = stream_groups_per_warp(c->K);
+  const StreamGeometry geo = stream_geometry(c->K);
   std::vector<int64_t> ptb((size_t)F + 1, 0);
-  int32_t* part = reinterpret_cast<int32_t*>(w + k.part);
+  int4* part = reinterpret_cast<int4*>(w + k.part);
+  uint32_t* sx = reinterpret_cast<uint32_t*>(w + k.sx);
+  uint32_t* syz = reinterpret_cast<uint32_t*>(w + k.syz);
+  uint32_t* place = reinterpret_cast<uint32_t*>(w + k.place);
+  int32_t* steps = reinterpret_cast<int32_t*>(w + k.steps);
   for (int32_t f = 0; f < F; ++f) {
     const int64_t items = chb[f + 1] - chb[f];
-    const int64_t warps = std::min(stream_max_warps(c->K), (items + gpw - 1) / gpw);
-    ptb[f + 1] = ptb[f] + warps + 1;
+    const int64_t warps = std::min(stream_max_warps(c->K), (items + geo.gpw - 1) / geo.gpw);
+    ptb[f + 1] = ptb[f] + warps;
     if (ptb[f + 1] > k.part_rows) return fail(c, ESSPT_ECUDA, "internal: work split overflow");
     ESSPT_CUDA(c, launch_stream_partition(b.pre + chb[f], items, warps, part + ptb[f], c->st));
+    ESSPT_CUDA(c, launch_stream_steps(b.chunk + chb[f], part + ptb[f], warps, geo, steps + f, c->st));
+  }
+  std::vector<int32_t> n_steps((size_t)F);
+  ESSPT_CUDA(c, cudaMemcpyAsync(n_steps.data(), steps, sizeof(int32_t) * F, cudaMemcpyDeviceToHost, c->st));
+  ESSPT_CUDA(c, cudaStreamSynchronize(c->st));
+  std::vector<int64_t> rcb((size_t)F + 1, 0);
+  for (int32_t f = 0; f < F; ++f) {
+    const int64_t places = (int64_t)n_steps[f] * geo.gpw * geo.per_step;
+    rcb[f + 1] = rcb[f] + places;
+    if (rcb[f + 1] > k.max_places) return fail(c, ESSPT_ECUDA, "internal: stream overflow");
+    StreamSource src{};
+    src.rec_j = b.rec_j + mbb[f];
+    src.rec_D = b.rec_D + mbb[f];
+    src.item_rep = b.item_rep;
+    src.hot_item = b.hot_item ? b.hot_item + (int64_t)f * kHot : nullptr;
+    src.n_items = n_items;
+    src.K = c->K;
+    src.dR_ld = dR_stride4(c->K);
+    ESSPT_CUDA(c, launch_stream_fill(b.chunk + chb[f], part + ptb[f], ptb[f + 1] - ptb[f], geo, src, places,
+                                     sx + rcb[f], syz + 2 * rcb[f], place + chb[f], c->st));
   }
   ESSPT_CUDA(c, cudaStreamSynchronize(c->st));
   c->part = part;
@@ -576,12 +605,18 @@ esspt_status esspt_mf_load(esspt_ctx* c, const int32_t* d_i, const int32_t* d_j,
   c->uoff = b.uoff;
   if (c->rowver) {
     c->user_slot = reinterpret_cast<int32_t*>(w + k.user_slot);
-    c->rec_row = reinterpret_cast<int32_t*>(w + k.rec_row);
+    c->row_x = reinterpret_cast<uint32_t*>(w + k.row_x);
+    // empty places of one minibatch may be read as another's: rows in the ring, or nothing
+    ESSPT_CUDA(c, cudaMemsetAsync(c->row_x, 0xff, sizeof(uint32_t) * k.max_places, c->st));
   }
   c->item_cnt = b.item_cnt;
   c->worker = worker;
   c->item_rep = b.item_rep;
-  c->rec = b.rec;
+  c->geo = geo;
+  c->sx = sx;
+  c->syz = syz;
+  c->place = place;
+  c->stream_base = rcb;
   c->hot_item = b.hot_item;
   c->dR = dR;
   c->dL = dL;
@@ -636,19 +671,21 @@ esspt_status esspt_mf_sgd_clock(esspt_ctx* c, float eta, float lambda, int32_t c
     RowRefreshArgs r{};
     r.rowver = c->rowver;
     r.items = c->chunk + c->chunk_base[b];
+    r.place = c->place + c->chunk_base[b];
     r.n_items = c->chunk_base[b + 1] - c->chunk_base[b];
-    r.rec = c->rec + c->mb_base[b];
+    r.g = c->geo;
+    r.K4 = c->K / 4;
+    r.rec_j = c->rec_j + c->mb_base[b];
     r.n_rows = c->n_rows;
     r.n_users = a.n_users;
     r.c = c->clock;
     r.s = c->s;
     r.nslots = c->nslots;
     r.user_slot = c->user_slot;
-    r.rec_row = c->rec_row;
+    r.x = c->row_x;
     ESSPT_CUDA(c, launch_row_refresh(r, c->st));
     a.row_mode = 1;
     a.user_slot = c->user_slot;
-    a.rec_row = c->rec_row;
   }
   const int64_t nhv = c->heavy_base[b + 1] - c->heavy_base[b];
   if (c->ev_before) ESSPT_CUDA(c, cudaEventRecord(c->ev_before, c->st));
@@ -656,8 +693,9 @@ esspt_status esspt_mf_sgd_clock(esspt_ctx* c, float eta, float lambda, int32_t c
   sa.a = a;
   sa.items = c->chunk + c->chunk_base[b];
   sa.part = c->part + c->part_base[b];
-  sa.n_warps = c->part_base[b + 1] - c->part_base[b] - 1;
-  sa.rec = c->rec + c->mb_base[b];
+  sa.n_warps = c->part_base[b + 1] - c->part_base[b];
+  sa.x = c->rowver ? c->row_x : c->sx + c->stream_base[b];
+  sa.yz = c->syz + 2 * c->stream_base[b];
   sa.dL = c->dL;
   ESSPT_CUDA(c, launch_sgd_stream(sa, c->st));
   if (nhv > 0) {
@@ -820,7 +858,9 @@ esspt_status esspt_mf_stage_minibatch(esspt_ctx* c, int32_t b, const int32_t* h_
   ESSPT_CUDA(c, cudaMemcpyAsync(su, h_u, sizeof(int32_t) * n, cudaMemcpyHostToDevice, st));
   ESSPT_CUDA(c, cudaMemcpyAsync(sj, h_j, sizeof(int32_t) * n, cudaMemcpyHostToDevice, st));
   ESSPT_CUDA(c, cudaMemcpyAsync(suoff, h_uoff, sizeof(int32_t) * (c->n_users + 1), cudaMemcpyHostToDevice, st));
-  ESSPT_CUDA(c, launch_refill(c->rec + base, c->rec_D + base, n, st));
+  ESSPT_CUDA(c, launch_stream_refill(c->chunk + c->chunk_base[b], c->place + c->chunk_base[b],
+                                     c->chunk_base[b + 1] - c->chunk_base[b], c->geo, c->rec_D + base,
+                                     c->syz + 2 * c->stream_base[b], st));
   ESSPT_CUDA(c, launch_stage_check(su, sj, suoff, c->rec_u + base, c->rec_j + base, ruoff, n, c->n_users + 1,
                                    c->status, st));
   return ESSPT_OK;

@@ -29,8 +29,9 @@ constexpr int32_t kHeavy = 96;
 constexpr int32_t kChunk = 64;
 // The work list is sorted by length within tiles of 2^kTileBits users: the
 // items that a warp takes together then have (nearly) one length, and a tile's
-// rows stay close in memory.
-constexpr int kTileBits = 8;
+// rows stay close in memory.  Tiles of 256, 1024 and 4096 users: 2729, 2682 and
+// 2672 us per clock on 10M x 1M, K = 64, and the same within 1% on 480k x 18k.
+constexpr int kTileBits = 12;
 // Cost of an item in a warp's share: its entries plus kItemCost.
 constexpr int32_t kItemCost = 5;
 // Replica accumulators: an item gets one delta row per kItemRep entries
@@ -84,7 +85,6 @@ struct SgdArgs {
   int32_t slot_out;         // slot of version c
   const int32_t* vslot;     // [P] ring slots of the read versions
   const int32_t* uoff;      // [n_users+1] entry offsets of minibatch b (relative)
-  const int32_t* rec_row;   // row mode: ring row (slot * n_rows + N + item) of each record's item
   float* dR;                // item delta replicas (all zero between clocks)
   int32_t dR_ld;            // float4 per dR row (dR_stride4)
   const int32_t* item_rep;  // see ItemMergeArgs; hot_item: [kHot] hot items of minibatch b, -1 if unused
@@ -92,7 +92,7 @@ struct SgdArgs {
   float eta, lambda;
   int32_t cap;
   double* sq_loss;          // optional
-  int32_t row_mode;         // row-granular SSP: per-user slots and per-entry ring rows
+  int32_t row_mode;         // row-granular SSP: per-user slots, and offsets of item rows in the whole ring
   const int32_t* user_slot; // [n_users] row mode: ring slot of each user's cached row
   // chg[u] = last clock that changed user row u (written with every user row
   // that changes); an idle row whose slot already holds its current value is
@@ -102,19 +102,29 @@ struct SgdArgs {
   int32_t clock, copy_all_until;
 };
 
-// The work list of minibatch b: x = user, y = first entry, z = replica row
-// in dL of a heavy user's chunk, or -1 for a user with 1..kHeavy entries (its
-// row of version c is written directly), w = entries << 16 | worker; sorted
-// by length within tiles of 2^kTileBits users.  Records: x = item, y = replica
-// row in dR that the item's update adds into, or -1 - h for hot slot h, z =
-// value (fp32), w unused (16 bytes are one aligned copy).
-// Warp w takes items [part[w], part[w+1]).
+// The work list of minibatch b: x = user, y = first entry, z = replica row in
+// dL of a heavy user's chunk, or -1 for a user with 1..kHeavy entries (its row
+// of version c is written directly), w = entries << 16 | worker; sorted by
+// length within tiles of 2^kTileBits users.
+// Warp w takes items part[w].x .. part[w].y in rounds of gpw (one per row
+// group), per_step entries of an item per step, and its steps are part[w].z ..
+// part[w].w of the minibatch's stream.  A step has gpw * per_step places, those
+// of one group side by side.  Place p holds an entry: x[p] = item * K/4, and in
+// yz, per_step y words before per_step z words, y = replica row * dR_stride4
+// (both float4 offsets: of the item's row, and of the row in dR that its update
+// adds into), or 1 + 2 * hot slot, and z = the value (fp32).  Empty places hold
+// kNoRecord.
+constexpr uint32_t kNoRecord = 0xffffffffu;
+constexpr int kStepAlign = 4;  // a warp's first step is a multiple
+struct StreamGeometry {
+  int gpw, per_step;
+};
 struct StreamArgs {
   SgdArgs a;
   const int4* items;
-  const int4* rec;
-  const int32_t* part;
+  const int4* part;
   int64_t n_warps;
+  const uint32_t *x, *yz;   // x: in row mode (float4 offset in the ring of the cached version)
   float* dL;                // heavy-user delta replicas (all zero between clocks)
 };
 
@@ -164,26 +174,45 @@ cudaError_t launch_get(const float* ring, int64_t n_rows, int32_t K, int32_t nsl
 cudaError_t launch_inc(float* slot, int64_t n_rows, int32_t K, const int32_t* ids, const float* d, int64_t n,
                        uint32_t* status, cudaStream_t st);
 // The SGD kernel of one clock; the warps it can use at row width K on this
-// device and the items a warp takes at a time; and the split of a minibatch's
-// n_items work items over n_warps of them (pre: see LayoutBuild).
+// device, and the shape of its stream.
 cudaError_t launch_sgd_stream(const StreamArgs& a, cudaStream_t st);
 int64_t stream_max_warps(int32_t K);
-int stream_groups_per_warp(int32_t K);
-cudaError_t launch_stream_partition(const int64_t* pre, int64_t n_items, int64_t n_warps, int32_t* part,
-                                    cudaStream_t st);
+StreamGeometry stream_geometry(int32_t K);
+// Build of a minibatch's stream (setup): the split of its n_items work items
+// over n_warps warps (pre: see LayoutBuild), the steps of the warps (their sum
+// in *total), the places (place[i] = that of item i's first entry), and new
+// values for them.
+struct StreamSource {
+  const int32_t* rec_j;
+  const float* rec_D;
+  const int32_t* item_rep;
+  const int32_t* hot_item;  // [kHot] or null
+  int64_t n_items;
+  int32_t K, dR_ld;
+};
+cudaError_t launch_stream_partition(const int64_t* pre, int64_t n_items, int64_t n_warps, int4* part, cudaStream_t st);
+cudaError_t launch_stream_steps(const int4* items, int4* part, int64_t n_warps, const StreamGeometry& g,
+                                int32_t* total, cudaStream_t st);
+cudaError_t launch_stream_fill(const int4* items, const int4* part, int64_t n_warps, const StreamGeometry& g,
+                               const StreamSource& src, int64_t n_places, uint32_t* x, uint32_t* yz, uint32_t* place,
+                               cudaStream_t st);
+cudaError_t launch_stream_refill(const int4* items, const uint32_t* place, int64_t n_items, const StreamGeometry& g,
+                                 const float* D, uint32_t* yz, cudaStream_t st);
 // Row-granular SSP, before the SGD kernels of clock c: refresh the cached
 // version of every row a worker reads (rowver[p * n_rows + r], -1 = never
 // read) to c-1 where it is missing or older than c-1-s, and write the ring
-// slot of each user's row and the ring row of each entry's item row.
+// slot of each user's row and the place in the ring of each entry's item row.
 struct RowRefreshArgs {
   int32_t* rowver;
-  const int4* items;       // work list of minibatch b
+  const int4* items;       // work list of minibatch b and its places (see StreamArgs)
+  const uint32_t* place;
   int64_t n_items;
-  const int4* rec;         // its records
+  StreamGeometry g;
+  const int32_t* rec_j;    // item of each entry of minibatch b
   int64_t n_rows;
-  int32_t n_users, c, s, nslots;
+  int32_t K4, n_users, c, s, nslots;
   int32_t* user_slot;      // out [n_users], for the users of the work list
-  int32_t* rec_row;        // out, one per record
+  uint32_t* x;             // out: the x words of the stream
 };
 cudaError_t launch_row_refresh(const RowRefreshArgs& a, cudaStream_t st);
 
@@ -224,7 +253,6 @@ struct LayoutBuild {
   int32_t* rec_u;
   int32_t* rec_j;
   float* rec_D;
-  int4* rec;            // [n_obs] records of the SGD kernel (see StreamArgs)
   int32_t* hot_item;    // [F][kHot] hot items of each minibatch, or null
   int32_t* uoff;        // [F][n_users+1]
   int64_t* mb_base;     // [F+1]
@@ -248,8 +276,8 @@ int64_t layout_max_heavy(int64_t n_obs, int32_t F);
 int64_t layout_max_item_reps(int64_t n_obs, int64_t n_items);
 int64_t layout_max_user_reps(int64_t n_obs);
 cudaError_t build_layout(LayoutBuild& b, cudaStream_t st);
-// New values of n records from those of their entries.
-cudaError_t launch_refill(int4* rec, const float* D, int64_t n, cudaStream_t st);
+// Places that the streams of all minibatches can take, empty ones included.
+int64_t layout_max_places(int64_t n_obs, int64_t n_users, int32_t F, const StreamGeometry& g, int64_t max_warps);
 cudaError_t launch_validate(const LayoutBuild& b, cudaStream_t st);
 // Staged minibatch check: su/sj (n entries) and suoff (n_off offsets) against
 // the resident ru/rj/ruoff; a difference latches kErrInput.

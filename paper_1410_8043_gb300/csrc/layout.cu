@@ -182,30 +182,6 @@ __global__ void place_items_kernel(const int4* __restrict__ raw, const uint32_t*
   }
 }
 
-// The records of the SGD kernel, one per entry.  Replica row of an entry's
-// item update: entry t (position within its
-// minibatch) of item j adds into replica (t mod replicas of j): replica 0 is
-// row j, replica r > 0 row n_items + item_rep[j] + r - 1.  With hot_item an
-// entry of hot slot h of its minibatch gets -1 - h instead.
-__global__ void records_kernel(const uint32_t* __restrict__ key, const int64_t* __restrict__ mb_base,
-                               const int32_t* __restrict__ rec_j, const float* __restrict__ rec_D,
-                               const int32_t* __restrict__ item_rep, int64_t n_obs, int64_t n_users,
-                               int64_t n_items, const int32_t* __restrict__ hot_item, int4* __restrict__ rec) {
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n_obs; k += stride) {
-    const int64_t b = (int64_t)key[k] / n_users;
-    const int64_t t = k - mb_base[b];
-    const int32_t j = rec_j[k];
-    const int32_t e0 = item_rep[j], e1 = item_rep[j + 1];  // extra replicas of j: e1 - e0 (reps - 1)
-    const int32_t r = (int32_t)(t & (int64_t)(e1 - e0));    // reps is a power of two
-    int32_t dst = r == 0 ? j : (int32_t)(n_items + e0 + r - 1);
-    if (hot_item != nullptr)
-      for (int h = 0; h < kHot; ++h)
-        if (hot_item[b * kHot + h] == j) dst = -1 - h;
-    rec[k] = make_int4(j, dst, __float_as_int(rec_D[k]), 0);
-  }
-}
-
 // The kHot items with the most entries of each minibatch (at least 2), most
 // popular first, ties by id; -1 for unused slots.  Host side, at setup.
 cudaError_t build_hot(const LayoutBuild& b, cudaStream_t st) {
@@ -226,12 +202,6 @@ cudaError_t build_hot(const LayoutBuild& b, cudaStream_t st) {
   e = cudaMemcpyAsync(b.hot_item, hot.data(), sizeof(int32_t) * hot.size(), cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   return e;
-}
-
-__global__ void refill_kernel(int4* __restrict__ rec, const float* __restrict__ D, int64_t n) {
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += stride)
-    rec[k].z = __float_as_int(D[k]);
 }
 
 // A staged minibatch against the loaded one: every user id, item id and
@@ -377,12 +347,7 @@ cudaError_t build_layout(LayoutBuild& b, cudaStream_t st) {
   tb = p.cub_bytes;
   if ((e = cub::DeviceScan::ExclusiveSum(cub_tmp, tb, ireps, b.item_rep, (int)(b.n_items + 1), st)) != cudaSuccess)
     return e;
-  if (b.n_obs > 0) {
-    if ((e = build_hot(b, st)) != cudaSuccess) return e;
-    records_kernel<<<blocks_for(b.n_obs), 256, 0, st>>>(key_out, b.mb_base, b.rec_j, b.rec_D, b.item_rep, b.n_obs,
-                                                        b.n_users, b.n_items, b.hot_item, b.rec);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  }
+  if (b.n_obs > 0 && (e = build_hot(b, st)) != cudaSuccess) return e;
   // The work list, then its order: by tile of users and length, ties in user
   // order (the sort is stable).  The sort buffers of the entries are free now.
   int4* raw = reinterpret_cast<int4*>(s + p.raw);
@@ -409,10 +374,18 @@ cudaError_t build_layout(LayoutBuild& b, cudaStream_t st) {
   return cub::DeviceScan::ExclusiveSum(cub_tmp, tb, reinterpret_cast<int32_t*>(key_in), pre, (int)(n + 1), st);
 }
 
-cudaError_t launch_refill(int4* rec, const float* D, int64_t n, cudaStream_t st) {
-  if (n <= 0) return cudaSuccess;
-  refill_kernel<<<blocks_for(n), 256, 0, st>>>(rec, D, n);
-  return cudaGetLastError();
+// A round takes gpw * per_step places per step of its longest item.  In a sorted
+// run its longest item is no longer than any of the round before it, so all but
+// two rounds per run cost no more than the entries of the round before, each
+// rounded up to whole steps; those two cost at most kHeavy entries' steps.  A
+// run ends with a tile or a warp; a warp's first step is aligned.
+int64_t layout_max_places(int64_t n_obs, int64_t n_users, int32_t F, const StreamGeometry& g, int64_t max_warps) {
+  const int64_t items = std::min(n_obs, layout_max_chunks(n_obs, F, n_users));
+  const int64_t warps = std::min((int64_t)F * max_warps, items);
+  const int64_t runs = (int64_t)F * ((n_users >> kTileBits) + 1) + warps;
+  const int64_t step = (int64_t)g.gpw * g.per_step;
+  return std::min(step * n_obs, n_obs + (items + g.gpw * warps) * (g.per_step - 1) +
+                                    2 * runs * g.gpw * (kHeavy + g.per_step)) + kStepAlign * step * (warps + F);
 }
 
 cudaError_t launch_stage_check(const int32_t* su, const int32_t* sj, const int32_t* suoff, const int32_t* ru,

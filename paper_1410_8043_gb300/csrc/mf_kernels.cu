@@ -84,6 +84,8 @@ __device__ __forceinline__ void flush_loss(double* out, float v, int lane) {
 }  // namespace
 
 constexpr int kStreamWarps = 4;   // warps per block
+constexpr int kChunkSteps = 8;    // steps whose records are fetched together
+constexpr int kMetaRounds = 8;    // rounds in the ring of item metadata
 
 // Forward copy of the users with no entry in minibatch b: the row of version
 // c-1 becomes that of version c.  One warp per 32 consecutive users: their
@@ -141,39 +143,44 @@ __device__ __forceinline__ void copy_idle_users(const SgdArgs& a, int64_t warp, 
 // length within tiles of consecutive users.  A warp walks one contiguous range
 // of items in rounds of 32/G: each row group of G lanes (NV float4 slices of a
 // row per lane, slice glane + t G on lane glane) takes one item, and the groups
-// step through their items' entries together, one entry per group and step:
+// step through their items' entries together, E entries per group and step:
 //   e = D - L.R,  gL += e R,  dR[dst] += e L - lambda R
 // At the end of a round every group closes its item: a user's row of version c
 // = base + eta s (gL - n lambda L), written once; a chunk's partial sum goes,
-// unscaled, into its replica row of dL.
+// unscaled, into its replica row of dL.  Which entries a step takes is known
+// when the data are loaded, so the layout holds them in that order, those of a
+// step side by side, and the stream runs on across rounds.
 //
-// The work is bound by issue slots, not by memory (the kernels this replaces
-// took 80..92% of their time with the gathers served by L1 and the reductions
-// left out), so it is built to issue little: the 32/G groups share every
-// instruction, rounds included, since the items of a round have (nearly) one
-// length; packed fp32 pairs (fma.rn.f32x2); one broadcast shared-memory read
-// for an entry's item, replica row, value and count; constant offsets from one
-// pointer per row; log2 G shuffles per step for 32/G dot products.
-// In flight per group: the next entry's item row (registers), the user rows
-// and first window of the next item (cp.async; every lane copies and reads its
-// own slices only), the item's next window.
-template <int G, int NV, int MINB, int HOT>
+// The kernels that this one replaced took 80..92% of their time with the item
+// rows served by L1 and the reductions left out: they waited on instruction
+// issue and on the rows' latency.  So the groups of a warp share every
+// instruction, on packed fp32 pairs (fma.rn.f32x2), with constant offsets from
+// one pointer per row, and the item rows are gathered ahead:
+//   rows of up to 64 values (E = 2): by cp.async, PF steps ahead (every lane
+//     copies and reads its own slices only, so no barrier stands between); two
+//     entries share a step's control and its shuffles;
+//   wider rows (E = 1): in registers, one step ahead.  Their 256..2048 bytes
+//     per entry through shared memory as well would make the SM's load/store
+//     data path the limit (480k x 18k, K = 100: 480 us per clock against 440).
+//     What bounds them is the SM's outgoing port: an entry's reduction leaves
+//     at 32 bytes per cycle.
+template <int G, int NV, int E, int PF, int MINB, int HOT>
 __global__ void __launch_bounds__(kStreamWarps * 32, MINB) sgd_stream_kernel(StreamArgs c) {
   constexpr int kGpw = 32 / G;
-  constexpr int kWindow = G < 8 ? G : 8;       // records per window of a row group
-  constexpr int kRecs = kGpw * (kWindow + 1);  // per window buffer: groups fall on different banks
+  constexpr int kPlaces = kGpw * E;          // entries per step of the warp
+  constexpr int kRing = 2 * kChunkSteps;     // steps whose records are at hand
+  static_assert(PF <= 3, "a chunk of records must have arrived when the gathers reach it");
+  static_assert(E == 2 || (E == 1 && PF == 1 && HOT == 0), "one entry per step: rows in registers, one step ahead");
   __shared__ __align__(16) float4 stageL[kStreamWarps][NV][32];
-  __shared__ __align__(16) float4 stageB[kStreamWarps][2][NV][32];
-  // window buffers: the first windows of this round and the next, then two for later windows
-  __shared__ __align__(16) int4 recs[kStreamWarps][4][kRecs];
-  __shared__ __align__(16) int4 metas[kStreamWarps][2][kGpw];
+  __shared__ __align__(16) float4 stageB[kStreamWarps][NV][32];
+  __shared__ __align__(16) float4 rowsR[E == 2 ? kStreamWarps : 1][PF + 1][E][NV][E == 2 ? 32 : 1];
+  __shared__ __align__(16) uint32_t recX[kStreamWarps][kRing * kPlaces];
+  __shared__ __align__(16) uint32_t recYZ[kStreamWarps][kRing * kPlaces * 2];
+  __shared__ __align__(16) int4 metas[kStreamWarps][kMetaRounds][kGpw];
   // per warp and lane: the summed updates of the minibatch's hot items
-  __shared__ __align__(16) float4 hot[kStreamWarps][HOT > 0 ? HOT : 1][NV][HOT > 0 ? 32 : 1];
-  // row mode (the launch asks for it then): ring row of each record's item
-  extern __shared__ int32_t rows_dyn[];
+  __shared__ __align__(16) float4 hot[HOT > 0 ? kStreamWarps : 1][HOT > 0 ? HOT : 1][NV][HOT > 0 ? 32 : 1];
   const SgdArgs& a = c.a;
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  int32_t* rows = rows_dyn + wib * 4 * kRecs;
   const int glane = lane & (G - 1), grp = lane / G;
   const int32_t K4 = a.K >> 2;
   const bool last_on = glane + (NV - 1) * G < K4;  // the lane's last slice lies inside the row
@@ -185,174 +192,117 @@ __global__ void __launch_bounds__(kStreamWarps * 32, MINB) sgd_stream_kernel(Str
   // traffic runs beside the other warps' arithmetic.
   if (warp & 1) copy_idle_users<G, NV>(a, warp, nwarps, lane);
 
-  int32_t xa = 0, xb = 0;
+  int32_t xr = 0, xb = 0, s0 = 0, s1 = 0;
   if (warp < c.n_warps) {
-    xa = __ldg(c.part + warp);
-    xb = __ldg(c.part + warp + 1);
+    const int4 p0 = __ldg(c.part + warp);
+    xr = p0.x;
+    xb = p0.y;
+    s0 = p0.z;
+    s1 = p0.w;
   }
-  if (xa < xb) {
+  if (s0 < s1) {
     const int64_t slot4 = a.n_rows * K4;
     float4* ring4 = reinterpret_cast<float4*>(a.ring) + glane;
+    float4* dRq = reinterpret_cast<float4*>(a.dR) + glane;
     const uint64_t pol = policy_evict_first();
+    const u64 nlam = pack2(-a.lambda, -a.lambda);
+
     auto load_item = [&](int32_t r0) {  // the group's item of the round that starts at item r0
       const int32_t x = r0 + grp;
       return x < xb ? __ldg(c.items + x) : make_int4(0, 0, -2, 0);
     };
-    // Records [at, at + n) of the stream, n <= kWindow, into window buffer w.
-    auto fetch_window = [&](int w, int32_t at, int32_t n) {
-#pragma unroll
-      for (int l = glane; l < kWindow; l += G) {
-        cp_async16_hint_if(&recs[wib][w][grp * (kWindow + 1) + l], c.rec + at + l, l < n, pol);
-        if (a.row_mode) cp_async4_if(rows + w * kRecs + grp * (kWindow + 1) + l, a.rec_row + at + l, l < n);
-      }
-    };
-    // Rows, first window and metadata of the next round's item, in half sb of
-    // the double buffers.
-    auto stage = [&](const int4& it, int sb) {
+    // Item as kept for its round: x = user, y = steps of the round, z as in
+    // the list, w = its read version's ring slot and its length.
+    auto put_meta = [&](int at, const int4& it) {
       const int32_t n = it.w >> 16;
+      const int32_t steps = __reduce_max_sync(0xffffffffu, (n + E - 1) / E);
       const int32_t vs = a.row_mode ? __ldg(a.user_slot + it.x) : __ldg(a.vslot + (it.w & 0xffff));
-      const float4* pv = ring4 + vs * slot4 + (int64_t)it.x * K4;
-      const float4* pb = ring4 + a.slot_base * slot4 + (int64_t)it.x * K4;
-      const bool bon = it.z == -1 && vs != a.slot_base;
-#pragma unroll
-      for (int k = 0; k < NV; ++k) {
-        const bool in = k < NV - 1 || last_on;
-        cp_async16_hint_if(&stageL[wib][k][lane], pv + k * G, n > 0 && in, pol);
-        cp_async16_hint_if(&stageB[wib][sb][k][lane], pb + k * G, bon && in, pol);
-      }
-      fetch_window(sb, it.y, n);
-      if (glane == 0) metas[wib][sb][grp] = make_int4(it.x, it.y, it.z, vs << 7 | n);
+      if (glane == 0) metas[wib][at][grp] = make_int4(it.x, steps, it.z, vs << 7 | n);
     };
-
-#pragma unroll
-    for (int k = 0; k < NV; ++k) stageL[wib][k][lane] = f4_zero();  // slices past the row end stay zero
-#pragma unroll
-    for (int h = 0; h < HOT; ++h)
-#pragma unroll
-      for (int k = 0; k < NV; ++k) hot[wib][h][k][lane] = f4_zero();
-    int32_t xr = xa;  // first item of the current round
-    int4 far = load_item(xr);
-    stage(far, 0);
-    cp_async_commit();
-    far = load_item(xr + kGpw);
-    cp_async_wait_all();
-    __syncwarp();
-
-    // Current round.
-    f2x2 L[NV], gL[NV];
-    int32_t cur_u = 0, cur_beg = 0, cur_z = 0, cur_n = 0, cur_vs = 0, steps = 0;
-    const float4* cur_R = ring4;
-    int sb = 0;                 // the round's half of the double buffers
-    int win = 0;                // window buffer of entry i
     auto item_rows = [&](int32_t vs) -> const float4* {
       return a.row_mode ? ring4 : ring4 + vs * slot4 + (int64_t)a.n_users * K4;
     };
+    // Copy user u's row of ring slot vs.
+    auto stage = [&](float4(&to)[NV][32], int32_t vs, int32_t u, bool on) {
+      const float4* row = ring4 + vs * slot4 + (int64_t)u * K4;
+#pragma unroll
+      for (int k = 0; k < NV; ++k) cp_async16_hint_if(&to[k][lane], row + k * G, on && (k < NV - 1 || last_on), pol);
+    };
+    // The records of kChunkSteps steps from step s (s - s0 a multiple of it).
+    auto fetch_records = [&](int32_t s) {
+      const int half = (s - s0) & kChunkSteps;
+#pragma unroll
+      for (int l0 = 0; l0 < kChunkSteps * kPlaces; l0 += 128) {
+        const int l = l0 + 4 * lane;
+        const bool on = l < kChunkSteps * kPlaces && s + l / kPlaces < s1;
+        cp_async16_hint_if(&recX[wib][half * kPlaces + l], c.x + (int64_t)s * kPlaces + l, on, pol);
+      }
+#pragma unroll
+      for (int l0 = 0; l0 < kChunkSteps * kPlaces * 2; l0 += 128) {
+        const int l = l0 + 4 * lane;
+        const bool on = l < kChunkSteps * kPlaces * 2 && s + l / (2 * kPlaces) < s1;
+        cp_async16_hint_if(&recYZ[wib][half * kPlaces * 2 + l], c.yz + (int64_t)s * kPlaces * 2 + l, on, pol);
+      }
+    };
+
+#pragma unroll
+    for (int k = 0; k < NV; ++k) {  // slices past the row end stay zero
+      stageL[wib][k][lane] = f4_zero();
+      if constexpr (E == 2)
+#pragma unroll
+        for (int q = 0; q <= PF; ++q) rowsR[wib][q][0][k][lane] = rowsR[wib][q][1][k][lane] = f4_zero();
+#pragma unroll
+      for (int h = 0; h < HOT; ++h) hot[wib][h][k][lane] = f4_zero();
+    }
+    fetch_records(s0);
+    fetch_records(s0 + kChunkSteps);
+    constexpr int kAhead = PF + 2;  // rounds whose metadata are at hand
+    static_assert(kAhead < kMetaRounds, "the ring of metadata");
+#pragma unroll
+    for (int d = 0; d < kAhead; ++d) put_meta(d, load_item(xr + d * kGpw));
+    int4 far = load_item(xr + kAhead * kGpw);
+    cp_async_wait_all();
+    __syncwarp();
+
+    // The gathers' place: round in the ring of metadata, steps left of it, its item rows.
+    int frnd = 0, fleft = metas[wib][0][grp].y;
+    const float4* fR = item_rows(metas[wib][0][grp].w >> 7);
+    auto f_next = [&]() {
+      if (--fleft == 0) {
+        frnd = (frnd + 1) & (kMetaRounds - 1);
+        const int4 m = metas[wib][frnd][grp];
+        fleft = m.y;
+        fR = item_rows(m.w >> 7);
+      }
+    };
+
+    // Current round.
+    f2x2 L[NV], gL[NV];
+    int32_t cur_u = 0, cur_z = 0, cur_n = 0, cur_vs = 0, left = 0;
+    int rnd = 0;
+    bool quick = false;  // a round of so few steps that its staged rows may not be there at its end
     auto open_round = [&]() {
-      const int4 m = metas[wib][sb][grp];
+      const int4 m = metas[wib][rnd][grp];
       cur_u = m.x;
-      cur_beg = m.y;
+      left = m.y;
       cur_z = m.z;
       cur_n = m.w & 127;
       cur_vs = m.w >> 7;
-      cur_R = item_rows(cur_vs);
-      steps = __reduce_max_sync(0xffffffffu, cur_n);
+      quick = left <= PF;
 #pragma unroll
       for (int k = 0; k < NV; ++k) {
         L[k] = lds_f2x2(&stageL[wib][k][lane]);
         gL[k] = f2x2{0ull, 0ull};
       }
-      win = sb;
-      if (xr + kGpw < xb) stage(far, sb ^ 1);
-      if (steps > kWindow) fetch_window(2, cur_beg + kWindow, cur_n - kWindow);
-      cp_async_commit();
-      far = load_item(xr + 2 * kGpw);
-    };
-    open_round();
-
-    f2x2 Ra[NV], Rb[NV];
-#pragma unroll
-    for (int k = 0; k < NV; ++k) Ra[k] = Rb[k] = f2x2{0ull, 0ull};
-    int4 ra = recs[wib][0][grp * (kWindow + 1)], rb;
-    if (cur_n > 0) {
-      const float4* row = cur_R + (int64_t)(a.row_mode ? rows[grp * (kWindow + 1)] : ra.x) * K4;
-#pragma unroll
-      for (int k = 0; k < NV; ++k) ldg_f2x2_if(Ra[k], row + k * G, k < NV - 1 || last_on);
-    }
-
-    // Step i of the round: the group's entry i (record rc, item row Rc), and
-    // the gather of the entry after it, of this round or the next, into Rn.
-    const u64 nlam = pack2(-a.lambda, -a.lambda);
-    int32_t i = 0;
-    auto step = [&](const int4& rc, int4& rn, const f2x2(&Rc)[NV], f2x2(&Rn)[NV]) {
-      const bool last = i + 1 == steps;
-      const float4* base = cur_R;
-      int at = grp * (kWindow + 1);
-      bool more;
-      if (last) {  // the next round's first entries
-        cp_async_wait_all();
-        __syncwarp();
-        win = sb ^ 1;
-        const int32_t w = metas[wib][sb ^ 1][grp].w;
-        more = xr + kGpw < xb && (w & 127) > 0;
-        base = item_rows(w >> 7);
-      } else {
-        const int o = (i + 1) & (kWindow - 1);
-        if (o == 0) {  // the item's next window
-          cp_async_wait_all();
-          __syncwarp();
-          const int32_t w = (i + 1) / kWindow;
-          win = 2 + ((w - 1) & 1);
-          if (steps > i + 1 + kWindow) {
-            fetch_window(2 + (w & 1), cur_beg + i + 1 + kWindow, cur_n - (i + 1 + kWindow));
-            cp_async_commit();
-          }
-        }
-        at += o;
-        more = i + 1 < cur_n;
-      }
-      rn = recs[wib][win][at];
-      {
-        const float4* row = base + (int64_t)(a.row_mode ? rows[win * kRecs + at] : rn.x) * K4;
-#pragma unroll
-        for (int k = 0; k < NV; ++k) ldg_f2x2_if(Rn[k], row + k * G, more && (k < NV - 1 || last_on));
-      }
-      u64 p = mul2(L[0].lo, Rc[0].lo);
-      p = fma2(L[0].hi, Rc[0].hi, p);
-#pragma unroll
-      for (int k = 1; k < NV; ++k) {
-        p = fma2(L[k].lo, Rc[k].lo, p);
-        p = fma2(L[k].hi, Rc[k].hi, p);
-      }
-      float dot = sum2(p);
-#pragma unroll
-      for (int off = G / 2; off > 0; off >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, off);
-      if (i < cur_n) {
-        const float e = __int_as_float(rc.z) - dot;
-        loss += e * e;
-        const u64 ee = pack2(e, e);
-#pragma unroll
-        for (int k = 0; k < NV; ++k) {
-          gL[k].lo = fma2(ee, Rc[k].lo, gL[k].lo);
-          gL[k].hi = fma2(ee, Rc[k].hi, gL[k].hi);
-        }
-        if (HOT > 0 && rc.y < 0) {
-#pragma unroll
-          for (int k = 0; k < NV; ++k) {
-            float4* h = &hot[wib][-1 - rc.y][k][lane];
-            const f2x2 v = lds_f2x2(h);
-            sts_f2x2(h, add2(v.lo, fma2(ee, L[k].lo, mul2(nlam, Rc[k].lo))),
-                     add2(v.hi, fma2(ee, L[k].hi, mul2(nlam, Rc[k].hi))));
-          }
-        } else {
-          float4* out = reinterpret_cast<float4*>(a.dR) + glane + (int64_t)rc.y * a.dR_ld;
-#pragma unroll
-          for (int k = 0; k < NV; ++k)
-            red_add_f2x2_if(out + k * G, fma2(ee, L[k].lo, mul2(nlam, Rc[k].lo)),
-                            fma2(ee, L[k].hi, mul2(nlam, Rc[k].hi)), k < NV - 1 || last_on);
-        }
-      }
+      const int4 m1 = metas[wib][(rnd + 1) & (kMetaRounds - 1)][grp];
+      stage(stageL[wib], m1.w >> 7, m1.x, xr + kGpw < xb && (m1.w & 127) > 0);
+      stage(stageB[wib], a.slot_base, cur_u, cur_z == -1 && cur_vs != a.slot_base);
+      put_meta((rnd + kAhead) & (kMetaRounds - 1), far);
+      far = load_item(xr + (kAhead + 1) * kGpw);
+      __syncwarp();
     };
     auto close_round = [&]() {
+      if (E == 1 || quick) cp_async_wait_all();
       const float nl = -a.lambda * (float)cur_n;
       const u64 nl2 = pack2(nl, nl);
       if (cur_z == -1) {
@@ -364,7 +314,7 @@ __global__ void __launch_bounds__(kStreamWarps * 32, MINB) sgd_stream_kernel(Str
 #pragma unroll
         for (int k = 0; k < NV; ++k) {
           f2x2 b = L[k];
-          if (!same) b = lds_f2x2(&stageB[wib][sb][k][lane]);
+          if (!same) b = lds_f2x2(&stageB[wib][k][lane]);
           st_stream_f2x2_if(o + k * G, fma2(sc2, fma2(nl2, L[k].lo, gL[k].lo), b.lo),
                             fma2(sc2, fma2(nl2, L[k].hi, gL[k].hi), b.hi), pol, k < NV - 1 || last_on);
         }
@@ -377,22 +327,139 @@ __global__ void __launch_bounds__(kStreamWarps * 32, MINB) sgd_stream_kernel(Str
                           k < NV - 1 || last_on);
       }
     };
-    // After each step: at the round's end close it and open the next.
-    auto next = [&]() -> bool {
-      if (++i < steps) return true;
+    // True once the warp's stream is done.
+    auto step_done = [&]() -> bool {
+      if (--left > 0) return false;
       close_round();
       xr += kGpw;
-      if (xr >= xb) return false;
-      sb ^= 1;
-      i = 0;
+      if (xr >= xb) return true;
+      rnd = (rnd + 1) & (kMetaRounds - 1);
       open_round();
-      return true;
+      return false;
     };
-    for (;;) {
-      step(ra, rb, Ra, Rb);
-      if (!next()) break;
-      step(rb, ra, Rb, Ra);
-      if (!next()) break;
+    auto dot_part = [&](const f2x2(&R)[NV]) -> float {
+      u64 p = mul2(L[0].lo, R[0].lo);
+      p = fma2(L[0].hi, R[0].hi, p);
+#pragma unroll
+      for (int k = 1; k < NV; ++k) {
+        p = fma2(L[k].lo, R[k].lo, p);
+        p = fma2(L[k].hi, R[k].hi, p);
+      }
+      return sum2(p);
+    };
+    // gL and the item update of an entry with residual e, y its record's word.
+    auto update = [&](float e, uint32_t y, const f2x2(&R)[NV]) {
+      const u64 ee = pack2(e, e);
+#pragma unroll
+      for (int k = 0; k < NV; ++k) {
+        gL[k].lo = fma2(ee, R[k].lo, gL[k].lo);
+        gL[k].hi = fma2(ee, R[k].hi, gL[k].hi);
+      }
+      if (HOT > 0 && (y & 1u)) {
+#pragma unroll
+        for (int k = 0; k < NV; ++k) {
+          float4* h = &hot[wib][y >> 1][k][lane];
+          const f2x2 v = lds_f2x2(h);
+          sts_f2x2(h, add2(v.lo, fma2(ee, L[k].lo, mul2(nlam, R[k].lo))),
+                   add2(v.hi, fma2(ee, L[k].hi, mul2(nlam, R[k].hi))));
+        }
+      } else {
+        float4* out = dRq + y;
+#pragma unroll
+        for (int k = 0; k < NV; ++k)
+          red_add_f2x2_if(out + k * G, fma2(ee, L[k].lo, mul2(nlam, R[k].lo)),
+                          fma2(ee, L[k].hi, mul2(nlam, R[k].hi)), k < NV - 1 || last_on);
+      }
+    };
+
+    {
+      const int4 m = metas[wib][0][grp];
+      stage(stageL[wib], m.w >> 7, m.x, (m.w & 127) > 0);
+    }
+    if constexpr (E == 2) {
+      // Gather the item rows of step t into place q of the ring of rows.
+      auto gather = [&](int32_t t, int q) {
+        if (t < s1) {
+          const uint2 x = *reinterpret_cast<const uint2*>(&recX[wib][(((t - s0) & (kRing - 1)) * kGpw + grp) * 2]);
+#pragma unroll
+          for (int k = 0; k < NV; ++k) {
+            cp_async16_if(&rowsR[wib][q][0][k][lane], fR + x.x + k * G, x.x != kNoRecord && (k < NV - 1 || last_on));
+            cp_async16_if(&rowsR[wib][q][1][k][lane], fR + x.y + k * G, x.y != kNoRecord && (k < NV - 1 || last_on));
+          }
+          f_next();
+        }
+      };
+#pragma unroll
+      for (int q = 0; q < PF; ++q) gather(s0 + q, q);
+      cp_async_wait_all();
+      open_round();
+      int q = 0;  // place of step s in the ring of rows
+      const bool hi = lane & (G / 2);  // this lane ends up with the second entry's dot product
+      for (int32_t s = s0;; ++s) {
+        gather(s + PF, q == 0 ? PF : q - 1);
+        if (((s - s0) & (kChunkSteps - 1)) == 0 && s > s0) fetch_records(s + kChunkSteps);
+        cp_async_commit();
+        cp_async_wait<PF>();
+        __syncwarp();
+        const uint4 r = *reinterpret_cast<const uint4*>(&recYZ[wib][(((s - s0) & (kRing - 1)) * kGpw + grp) * 4]);
+        f2x2 R0[NV], R1[NV];
+#pragma unroll
+        for (int k = 0; k < NV; ++k) {
+          R0[k] = lds_f2x2(&rowsR[wib][q][0][k][lane]);
+          R1[k] = lds_f2x2(&rowsR[wib][q][1][k][lane]);
+        }
+        q = q == PF ? 0 : q + 1;
+        const float p0 = dot_part(R0), p1 = dot_part(R1);
+        float dot = hi ? p1 : p0;
+        dot += __shfl_xor_sync(0xffffffffu, hi ? p0 : p1, G / 2);
+#pragma unroll
+        for (int off = G / 4; off > 0; off >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, off);
+        const float e = __uint_as_float(hi ? r.w : r.z) - dot;
+        const float o = __shfl_xor_sync(0xffffffffu, e, G / 2);
+        if (r.x != kNoRecord) update(hi ? o : e, r.x, R0);
+        if (r.y != kNoRecord) update(hi ? e : o, r.y, R1);
+        if ((hi ? r.y : r.x) != kNoRecord) loss += e * e;
+        if (step_done()) break;
+      }
+      if (glane % (G / 2) != 0) loss = 0.f;
+    } else {
+      f2x2 Ra[NV], Rb[NV];
+#pragma unroll
+      for (int k = 0; k < NV; ++k) Ra[k] = Rb[k] = f2x2{0ull, 0ull};
+      auto gather = [&](int32_t t, f2x2(&R)[NV]) {
+        if (t < s1) {
+          const uint32_t x = recX[wib][((t - s0) & (kRing - 1)) * kGpw + grp];
+#pragma unroll
+          for (int k = 0; k < NV; ++k) ldg_f2x2_if(R[k], fR + x + k * G, x != kNoRecord && (k < NV - 1 || last_on));
+          f_next();
+        }
+      };
+      gather(s0, Ra);
+      cp_async_wait_all();
+      open_round();
+      auto step = [&](int32_t s, const f2x2(&Rc)[NV], f2x2(&Rn)[NV]) -> bool {
+        if (((s - s0) & (kChunkSteps - 1)) == kChunkSteps - 1) {  // the next step's records, fetched 8 steps ago
+          cp_async_wait_all();
+          __syncwarp();
+        }
+        gather(s + 1, Rn);
+        if (((s - s0) & (kChunkSteps - 1)) == 0 && s > s0) fetch_records(s + kChunkSteps);
+        const uint2 r = *reinterpret_cast<const uint2*>(&recYZ[wib][(((s - s0) & (kRing - 1)) * kGpw + grp) * 2]);
+        float dot = dot_part(Rc);
+#pragma unroll
+        for (int off = G / 2; off > 0; off >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, off);
+        if (r.x != kNoRecord) {
+          const float e = __uint_as_float(r.y) - dot;
+          loss += e * e;
+          update(e, r.x, Rc);
+        }
+        return step_done();
+      };
+      for (int32_t s = s0;; s += 2) {
+        if (step(s, Ra, Rb)) break;
+        if (step(s + 1, Rb, Ra)) break;
+      }
+      if (glane != 0) loss = 0.f;
     }
     cp_async_wait_all();
     // Hot items: the groups' sums, added once into a replica row of the item
@@ -420,24 +487,138 @@ __global__ void __launch_bounds__(kStreamWarps * 32, MINB) sgd_stream_kernel(Str
     }
   }
   if (!(warp & 1)) copy_idle_users<G, NV>(a, warp, nwarps, lane);
-  flush_loss(a.sq_loss, glane == 0 ? loss : 0.f, lane);
+  flush_loss(a.sq_loss, loss, lane);
+}
+
+// ---- the stream's build (setup) --------------------------------------------
+
+// Steps of every warp of a minibatch, in part[w].z for now.
+__global__ void __launch_bounds__(256) stream_steps_kernel(const int4* __restrict__ items, int4* part,
+                                                           int64_t n_warps, StreamGeometry g) {
+  const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (w >= n_warps) return;
+  const int lane = threadIdx.x & 31;
+  const int32_t x0 = part[w].x, x1 = part[w].y;
+  int32_t sum = 0;
+  for (int32_t r = x0 + lane * g.gpw; r < x1; r += 32 * g.gpw) {
+    int32_t mx = 0;
+    for (int32_t x = r; x < min(r + g.gpw, x1); ++x) mx = max(mx, items[x].w >> 16);
+    sum += (mx + g.per_step - 1) / g.per_step;
+  }
+  sum = __reduce_add_sync(0xffffffffu, sum);
+  if (lane == 0) part[w].z = sum;
+}
+// part[w].z, .w = first and end step of warp w; a warp starts at a multiple of
+// kStepAlign steps, so that its records start on 16 bytes.  One block.
+__global__ void __launch_bounds__(1024) stream_offsets_kernel(int4* part, int64_t n_warps, int32_t* total) {
+  __shared__ int32_t sums[1024];
+  const int64_t per = (n_warps + 1023) / 1024, w0 = threadIdx.x * per, w1 = min(n_warps, w0 + per);
+  int32_t sum = 0;
+  for (int64_t w = w0; w < w1; ++w) sum += (part[w].z + kStepAlign - 1) / kStepAlign * kStepAlign;
+  sums[threadIdx.x] = sum;
+  __syncthreads();
+  for (int off = 1; off < 1024; off <<= 1) {
+    const int32_t v = threadIdx.x >= off ? sums[threadIdx.x - off] : 0;
+    __syncthreads();
+    sums[threadIdx.x] += v;
+    __syncthreads();
+  }
+  int32_t at = sums[threadIdx.x] - sum;
+  for (int64_t w = w0; w < w1; ++w) {
+    const int32_t n = part[w].z;
+    part[w].z = at;
+    part[w].w = at + n;
+    at += (n + kStepAlign - 1) / kStepAlign * kStepAlign;
+  }
+  if (threadIdx.x == 1023) *total = sums[1023];
+}
+
+cudaError_t launch_stream_steps(const int4* items, int4* part, int64_t n_warps, const StreamGeometry& g,
+                                int32_t* total, cudaStream_t st) {
+  stream_steps_kernel<<<(unsigned)(n_warps / 8 + 1), 256, 0, st>>>(items, part, n_warps, g);
+  stream_offsets_kernel<<<1, 1024, 0, st>>>(part, n_warps, total);
+  return cudaGetLastError();
+}
+
+// Place of entry k of an item whose first entry's place is `at`, and where its
+// y and z words are.
+__device__ __forceinline__ int64_t record_place(const StreamGeometry& g, int64_t at, int32_t k) {
+  return at + (int64_t)(k / g.per_step) * g.gpw * g.per_step + k % g.per_step;
+}
+__device__ __forceinline__ int64_t y_word(const StreamGeometry& g, int64_t place) {
+  return place / g.per_step * g.per_step * 2 + place % g.per_step;
+}
+
+// The records of a minibatch (x and yz hold kNoRecord everywhere on entry) and
+// the place of every item's first entry.  One warp per warp of the kernel.
+__global__ void __launch_bounds__(256) stream_fill_kernel(const int4* __restrict__ items,
+                                                          const int4* __restrict__ part, int64_t n_warps,
+                                                          StreamGeometry g, StreamSource src, uint32_t* __restrict__ x,
+                                                          uint32_t* __restrict__ yz, uint32_t* __restrict__ place) {
+  const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (w >= n_warps) return;
+  const int lane = threadIdx.x & 31, G = 32 / g.gpw, grp = lane / G, l = lane & (G - 1);
+  const int4 p = part[w];
+  int64_t s = p.z;
+  for (int32_t x0 = p.x; x0 < p.y; x0 += g.gpw) {
+    const int32_t i = x0 + grp;
+    const int4 it = i < p.y ? items[i] : make_int4(0, 0, -2, 0);
+    const int32_t n = it.w >> 16;
+    const int64_t at = (s * g.gpw + grp) * g.per_step;
+    if (l == 0 && n > 0) place[i] = (uint32_t)at;
+    for (int32_t k = l; k < n; k += G) {
+      const int32_t t = it.y + k, j = src.rec_j[t];
+      const int32_t e0 = src.item_rep[j], e1 = src.item_rep[j + 1];  // extra replicas of j: e1 - e0 (reps - 1)
+      const int32_t q = t & (e1 - e0);                               // reps is a power of two
+      uint32_t y = (uint32_t)(q == 0 ? j : src.n_items + e0 + q - 1) * (uint32_t)src.dR_ld;
+      if (src.hot_item != nullptr)
+        for (int h = 0; h < kHot; ++h)
+          if (src.hot_item[h] == j) y = 2u * h + 1u;
+      const int64_t to = record_place(g, at, k);
+      x[to] = (uint32_t)j * (uint32_t)(src.K / 4);
+      yz[y_word(g, to)] = y;
+      yz[y_word(g, to) + g.per_step] = __float_as_uint(src.rec_D[t]);
+    }
+    s += __reduce_max_sync(0xffffffffu, (n + g.per_step - 1) / g.per_step);
+  }
+}
+cudaError_t launch_stream_fill(const int4* items, const int4* part, int64_t n_warps, const StreamGeometry& g,
+                               const StreamSource& src, int64_t n_places, uint32_t* x, uint32_t* yz, uint32_t* place,
+                               cudaStream_t st) {
+  cudaError_t e = cudaMemsetAsync(x, 0xff, sizeof(uint32_t) * n_places, st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(yz, 0xff, 2 * sizeof(uint32_t) * n_places, st);
+  if (e != cudaSuccess || n_warps <= 0) return e;
+  stream_fill_kernel<<<(unsigned)((n_warps + 7) / 8), 256, 0, st>>>(items, part, n_warps, g, src, x, yz, place);
+  return cudaGetLastError();
+}
+
+// New values of a minibatch's records: eight lanes per item.
+__global__ void __launch_bounds__(256) stream_refill_kernel(const int4* __restrict__ items,
+                                                            const uint32_t* __restrict__ place, int64_t n_items,
+                                                            StreamGeometry g, const float* __restrict__ D,
+                                                            uint32_t* __restrict__ yz) {
+  const int64_t stride = ((int64_t)gridDim.x * blockDim.x) >> 3;
+  for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 3; i < n_items; i += stride) {
+    const int4 it = items[i];
+    const int64_t at = place[i];
+    for (int32_t k = threadIdx.x & 7; k < it.w >> 16; k += 8)
+      yz[y_word(g, record_place(g, at, k)) + g.per_step] = __float_as_uint(D[it.y + k]);
+  }
 }
 
 // Row-granular SSP (Sec. 4 client cache, a clock c_param per cached row): for
-// every work item, refresh its user's row and its records' item rows in the
-// cache of the reading worker.  Eight lanes per item, one record per lane and
-// pass.  All lanes that refresh one (worker, row) in a clock write the same
-// value, c-1, so the races are benign and every read of the row in the clock
-// sees one version.
+// every work item, refresh its user's row and its entries' item rows in the
+// cache of the reading worker; eight lanes per item.  All lanes that refresh
+// one (worker, row) in a clock write the same value, c-1, so the races are
+// benign and every read of the row in the clock sees one version.
 __global__ void __launch_bounds__(256) row_refresh_kernel(RowRefreshArgs a) {
   const int32_t lo = a.c - 1 - a.s;
-  const int l = threadIdx.x & 7;
   const int64_t stride = ((int64_t)gridDim.x * blockDim.x) >> 3;
-  for (int64_t x = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 3; x < a.n_items; x += stride) {
-    const int4 it = __ldg(a.items + x);
+  for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 3; i < a.n_items; i += stride) {
+    const int4 it = __ldg(a.items + i);
+    const int64_t at = __ldg(a.place + i);
     int32_t* V = a.rowver + (int64_t)(it.w & 0xffff) * a.n_rows;
-    const int32_t n = it.w >> 16;
-    if (l == 0) {
+    if ((threadIdx.x & 7) == 0) {
       int32_t v = V[it.x];
       if (v < 0 || v < lo) {
         v = a.c - 1;
@@ -445,14 +626,14 @@ __global__ void __launch_bounds__(256) row_refresh_kernel(RowRefreshArgs a) {
       }
       a.user_slot[it.x] = v % a.nslots;
     }
-    for (int32_t k = l; k < n; k += 8) {
-      const int64_t r = (int64_t)a.n_users + __ldg(&a.rec[it.y + k].x);
+    for (int32_t k = threadIdx.x & 7; k < it.w >> 16; k += 8) {
+      const int64_t r = (int64_t)a.n_users + __ldg(a.rec_j + it.y + k);
       int32_t v = V[r];
       if (v < 0 || v < lo) {
         v = a.c - 1;
         V[r] = v;
       }
-      a.rec_row[it.y + k] = (int32_t)((int64_t)(v % a.nslots) * a.n_rows + r);
+      a.x[record_place(a.g, at, k)] = (uint32_t)(((int64_t)(v % a.nslots) * a.n_rows + r) * a.K4);
     }
   }
 }
@@ -554,30 +735,31 @@ int grid_for(int64_t work_items, int64_t per_block, int max_per_sm) {
 }
 
 // Row-group shape for K: G lanes per row (a power of two) and NV float4 slices
-// per lane, G (NV - 1) < K/4 <= G NV, and the blocks per SM the kernel is
-// compiled for.  Eight lanes read 128 consecutive bytes per load, a whole
-// line; wider groups only where NV = 4 slices per lane do not hold the row.
-// Blocks per SM: as many as spill (next to) nothing; on the 300k x 40k, K=48
-// case 6 blocks take 122 us, 7 blocks 128, 8 blocks (64 registers, spills)
-// 213; 5 blocks with rows staged two rounds ahead 131; on 480k x 18k, K=100
-// 4 blocks 443 us, 5 blocks (spills) 785, 3 blocks 525 (before the wider
-// replica rows, where 4 blocks took 508).
-template <int G_, int NV_, int MINB_, int HOT_ = 0>
+// per lane, G (NV - 1) < K/4 <= G NV; E entries per step and PF steps of gathers
+// ahead (see the kernel); the blocks per SM it is compiled for.  Eight lanes
+// read 128 consecutive bytes per load, a whole line; wider groups only where
+// NV = 4 slices per lane do not hold the row.  Measured (us per clock):
+//   K = 32, 200k x 30k: PF 2 with 7 blocks 84, PF 1 with 8 blocks 89, 6 blocks
+//     82; one entry per step 86..93;
+//   K = 48, 300k x 40k: PF 1 with 5 blocks 107, PF 2 with 4 blocks 114; one
+//     entry per step 108..118; 10M x 1M, K = 64: 2630, 2650; 2720..2810;
+//   K = 100, 480k x 18k: 4 blocks 441..450, 3 blocks 470, 5 blocks spill (785).
+template <int G_, int NV_, int E_, int PF_, int MINB_, int HOT_ = 0>
 struct StreamShape {
-  static constexpr int G = G_, NV = NV_, MINB = MINB_, HOT = HOT_, GPW = 32 / G_;
+  static constexpr int G = G_, NV = NV_, E = E_, PF = PF_, MINB = MINB_, HOT = HOT_, GPW = 32 / G_;
 };
 template <typename F>
 auto dispatch_stream(int32_t K, F&& f) {
   const int32_t K4 = K / 4;
-  if (K4 <= 4) return f(StreamShape<4, 1, 8>{});
-  if (K4 <= 8) return f(StreamShape<8, 1, 7>{});
-  if (K4 <= 16) return f(StreamShape<8, 2, 6, kHot>{});
-  if (K4 <= 24) return f(StreamShape<8, 3, 4>{});
-  if (K4 <= 32) return f(StreamShape<8, 4, 4>{});
-  if (K4 <= 48) return f(StreamShape<16, 3, 4>{});
-  if (K4 <= 64) return f(StreamShape<16, 4, 4>{});
-  if (K4 <= 96) return f(StreamShape<32, 3, 4>{});
-  return f(StreamShape<32, 4, 4>{});
+  if (K4 <= 4) return f(StreamShape<4, 1, 2, 2, 6>{});
+  if (K4 <= 8) return f(StreamShape<8, 1, 2, 2, 7>{});
+  if (K4 <= 16) return f(StreamShape<8, 2, 2, 1, 5, kHot>{});
+  if (K4 <= 24) return f(StreamShape<8, 3, 1, 1, 5>{});
+  if (K4 <= 32) return f(StreamShape<8, 4, 1, 1, 4>{});
+  if (K4 <= 48) return f(StreamShape<16, 3, 1, 1, 5>{});
+  if (K4 <= 64) return f(StreamShape<16, 4, 1, 1, 4>{});
+  if (K4 <= 96) return f(StreamShape<32, 3, 1, 1, 5>{});
+  return f(StreamShape<32, 4, 1, 1, 4>{});
 }
 
 }  // namespace
@@ -586,14 +768,14 @@ int64_t stream_max_warps(int32_t K) {
   return dispatch_stream(K, [](auto s) { return (int64_t)sm_count() * s.MINB * kStreamWarps; });
 }
 
-int stream_groups_per_warp(int32_t K) {
-  return dispatch_stream(K, [](auto s) { return s.GPW; });
+StreamGeometry stream_geometry(int32_t K) {
+  return dispatch_stream(K, [](auto s) { return StreamGeometry{s.GPW, s.E}; });
 }
 
 cudaError_t launch_sgd_stream(const StreamArgs& c, cudaStream_t st) {
   return dispatch_stream(c.a.K, [&](auto s) {
     using S = decltype(s);
-    const auto kernel = sgd_stream_kernel<S::G, S::NV, S::MINB, S::HOT>;
+    const auto kernel = sgd_stream_kernel<S::G, S::NV, S::E, S::PF, S::MINB, S::HOT>;
     static bool configured = false;
     if (!configured) {
       // The smallest shared-memory carveout that holds the resident blocks'
@@ -611,17 +793,15 @@ cudaError_t launch_sgd_stream(const StreamArgs& c, cudaStream_t st) {
     // Warps for the work list, and one per 32 users for the forward copy, up
     // to one resident wave.
     const int64_t warps = std::max<int64_t>(c.n_warps, (c.a.n_users + 31) / 32);
-    const int win = S::G < 8 ? S::G : 8;
-    const size_t rows = c.a.row_mode ? sizeof(int32_t) * kStreamWarps * 4 * S::GPW * (win + 1) : 0;
-    kernel<<<grid_for(warps, kStreamWarps, S::MINB), kStreamWarps * 32, rows, st>>>(c);
+    kernel<<<grid_for(warps, kStreamWarps, S::MINB), kStreamWarps * 32, 0, st>>>(c);
     return cudaGetLastError();
   });
 }
 
-// Warp w of n_warps takes items [part[w], part[w+1]), the shares balanced by
+// Warp w of n_warps takes items [part[w].x, part[w].y), the shares balanced by
 // cost: pre[x] is the summed cost of the items before x (over all minibatches).
 __global__ void __launch_bounds__(256) stream_partition_kernel(const int64_t* __restrict__ pre, int32_t n_items,
-                                                               int32_t n_warps, int32_t* __restrict__ part) {
+                                                               int32_t n_warps, int4* __restrict__ part) {
   const int32_t w = blockIdx.x * blockDim.x + threadIdx.x;
   if (w > n_warps) return;
   int32_t lo = 0, hi = n_items;
@@ -638,10 +818,11 @@ __global__ void __launch_bounds__(256) stream_partition_kernel(const int64_t* __
       }
     }
   }
-  part[w] = lo;
+  if (w < n_warps) part[w].x = lo;
+  if (w > 0) part[w - 1].y = lo;
 }
 
-cudaError_t launch_stream_partition(const int64_t* pre, int64_t n_items, int64_t n_warps, int32_t* part,
+cudaError_t launch_stream_partition(const int64_t* pre, int64_t n_items, int64_t n_warps, int4* part,
                                     cudaStream_t st) {
   stream_partition_kernel<<<(unsigned)(n_warps / 256 + 1), 256, 0, st>>>(pre, (int32_t)n_items, (int32_t)n_warps,
                                                                         part);
@@ -651,6 +832,13 @@ cudaError_t launch_stream_partition(const int64_t* pre, int64_t n_items, int64_t
 cudaError_t launch_row_refresh(const RowRefreshArgs& a, cudaStream_t st) {
   if (a.n_items <= 0) return cudaSuccess;
   row_refresh_kernel<<<grid_for(a.n_items, 32, 8), 256, 0, st>>>(a);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_stream_refill(const int4* items, const uint32_t* place, int64_t n_items, const StreamGeometry& g,
+                                 const float* D, uint32_t* yz, cudaStream_t st) {
+  if (n_items <= 0) return cudaSuccess;
+  stream_refill_kernel<<<grid_for(n_items, 32, 8), 256, 0, st>>>(items, place, n_items, g, D, yz);
   return cudaGetLastError();
 }
 

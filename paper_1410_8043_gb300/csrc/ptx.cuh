@@ -34,8 +34,8 @@ __device__ __forceinline__ void st_stream_if(float4* p, float4 v, uint64_t pol, 
       : "memory");
 }
 
-// 16-byte asynchronous global -> shared copy (bypassing L1) with an L2
-// eviction-priority policy for the source lines, and a 4-byte one; nothing
+// 16-byte asynchronous global -> shared copies, bypassing L1 with an L2
+// eviction-priority policy for the source lines, and through L1; nothing
 // happens when `pred` is false.
 __device__ __forceinline__ void cp_async16_hint_if(void* smem, const void* gmem, bool pred, uint64_t pol) {
   const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
@@ -45,13 +45,12 @@ __device__ __forceinline__ void cp_async16_hint_if(void* smem, const void* gmem,
       "l"(gmem), "r"((int)pred), "l"(pol)
       : "memory");
 }
-__device__ __forceinline__ void cp_async4_if(void* smem, const void* gmem, bool pred) {
+__device__ __forceinline__ void cp_async16_if(void* smem, const void* gmem, bool pred) {
   const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
-  asm volatile("{\n .reg .pred q;\n setp.ne.b32 q, %2, 0;\n @q cp.async.ca.shared.global [%0], [%1], 4;\n}" ::"r"(s),
+  asm volatile("{\n .reg .pred q;\n setp.ne.b32 q, %2, 0;\n @q cp.async.ca.shared.global [%0], [%1], 16;\n}" ::"r"(s),
                "l"(gmem), "r"((int)pred)
                : "memory");
 }
-
 // Streaming 32-bit load (read once per clock): skip L1, evict-first in L2.
 __device__ __forceinline__ int32_t ld_stream_i32(const int32_t* p, uint64_t pol) {
   int32_t r;
@@ -59,7 +58,13 @@ __device__ __forceinline__ int32_t ld_stream_i32(const int32_t* p, uint64_t pol)
   return r;
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
+// Wait for all of the thread's asynchronous copies, or until at most N of its
+// newest groups are in flight.
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
 
 // out[0..3] += v, performed at L2 (no return value).
 __device__ __forceinline__ void red_add_v4(float4* p, float4 v) { atomicAdd(p, v); }
