@@ -42,6 +42,7 @@ struct esspt_ctx {
   int32_t* user_slot = nullptr;  // row-granular SSP: [n_users] per-clock ring slot of each user row
   int4 *chunk = nullptr, *heavy = nullptr;
   std::vector<int64_t> mb_base, chunk_base, heavy_base;
+  int64_t *d_mb_base = nullptr, *d_chunk_base = nullptr;
   int4* part = nullptr;               // split of each minibatch's work items over the warps
   std::vector<int64_t> part_base;     // [F+1] first word of each minibatch's split
   cudaEvent_t ev_before = nullptr, ev_after = nullptr;
@@ -272,23 +273,24 @@ bool mf_sizes_ok(const esspt_ctx* c, int64_t n_obs, int64_t n_users, int32_t F) 
 
 namespace esspt {
 
-esspt_status mf_view(esspt_ctx* c, int32_t version, const float** slot, int64_t* n_users, int32_t* K,
-                     const int32_t** rec_u, const int32_t** rec_j, const float** rec_D, const int32_t** worker,
-                     int64_t* n_obs, int32_t* P, cudaStream_t* st) {
+esspt_status mf_view(esspt_ctx* c, int32_t version, ObjectiveArgs* a, cudaStream_t* st) {
   esspt_status s = need_init(c);
   if (s != ESSPT_OK) return s;
   if (!c->mf) return fail(c, ESSPT_ESTATE, "no MF data loaded (call esspt_mf_load)");
   const int32_t lo = c->clock - 1 - c->s > 0 ? c->clock - 1 - c->s : 0;
   if (version < lo || version > c->clock - 1) return fail(c, ESSPT_EINVAL, "version outside the live window");
-  *slot = slot_ptr(c, version);
-  *n_users = c->n_users;
-  *K = c->K;
-  *rec_u = c->rec_u;
-  *rec_j = c->rec_j;
-  *rec_D = c->rec_D;
-  *worker = c->worker;
-  *n_obs = c->n_obs;
-  *P = c->P;
+  *a = ObjectiveArgs{};
+  a->slot = slot_ptr(c, version);
+  a->n_users = c->n_users;
+  a->K = c->K;
+  a->F = c->F;
+  a->P = c->P;
+  a->items = c->chunk;
+  a->n_items = c->chunk_base[c->F];
+  a->item_base = c->d_chunk_base;
+  a->entry_base = c->d_mb_base;
+  a->rec_j = c->rec_j;
+  a->rec_D = c->rec_D;
   *st = c->st;
   return ESSPT_OK;
 }
@@ -627,6 +629,8 @@ esspt_status esspt_mf_load(esspt_ctx* c, const int32_t* d_i, const int32_t* d_j,
   // rows changed before this load are not tracked
   c->copy_all_until = c->clock + c->s + 1;
   c->mb_base = mbb;
+  c->d_mb_base = b.mb_base;
+  c->d_chunk_base = b.chunk_base;
   c->chunk_base = chb;
   c->heavy_base = hvb;
   c->mf = true;
@@ -789,14 +793,15 @@ esspt_status esspt_mf_sgd_clock_sequential(esspt_ctx* c, float eta, float lambda
 
 esspt_status esspt_mf_objective(esspt_ctx* c, int32_t version, float lambda, double* d_scratch, double* h_sq,
                                 double* h_pen) {
-  esspt_status s = need_init(c);
+  if (c && c->clock >= 1 && c->mf && (!d_scratch || !h_sq || !h_pen)) return fail(c, ESSPT_EINVAL, "null pointer");
+  ObjectiveArgs a;
+  cudaStream_t st = nullptr;
+  const esspt_status s = mf_view(c, version, &a, &st);
   if (s != ESSPT_OK) return s;
-  if (!c->mf) return fail(c, ESSPT_ESTATE, "no MF data loaded (call esspt_mf_load)");
-  if (!d_scratch || !h_sq || !h_pen) return fail(c, ESSPT_EINVAL, "null pointer");
-  const int32_t lo = c->clock - 1 - c->s > 0 ? c->clock - 1 - c->s : 0;
-  if (version < lo || version > c->clock - 1) return fail(c, ESSPT_EINVAL, "version outside the live window");
-  ESSPT_CUDA(c, launch_objective(slot_ptr(c, version), c->n_users, c->K, c->rec_u, c->rec_j, c->rec_D, c->n_obs,
-                                 lambda, d_scratch, c->st));
+  a.lambda = lambda;
+  a.out = d_scratch;
+  a.out_stride = 1;
+  ESSPT_CUDA(c, launch_objective(a, st));
   double out[2] = {0.0, 0.0};
   ESSPT_CUDA(c, cudaMemcpyAsync(out, d_scratch, sizeof out, cudaMemcpyDeviceToHost, c->st));
   ESSPT_CUDA(c, cudaStreamSynchronize(c->st));

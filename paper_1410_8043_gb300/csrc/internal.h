@@ -236,9 +236,25 @@ struct SeqArgs {
 cudaError_t launch_seq_clock(const SeqArgs& a, cudaStream_t st);
 cudaError_t launch_heavy_merge(const HeavyMergeArgs& a, cudaStream_t st);
 cudaError_t launch_item_merge(const ItemMergeArgs& a, cudaStream_t st);
-cudaError_t launch_objective(const float* slot, int64_t n_users, int32_t K, const int32_t* rec_u,
-                             const int32_t* rec_j, const float* rec_D, int64_t n_obs, float lambda,
-                             double* out2, cudaStream_t st);
+// Objective at one table version over the work lists of all F minibatches:
+// item_base and entry_base (device, [F+1]) hold each one's first item and entry.
+// out[0] = sum e^2 and out[out_stride] = penalised sum; by worker (P at most,
+// sums added to what out holds) at out[p] and out[out_stride + p].
+struct ObjectiveArgs {
+  const float* slot;
+  int64_t n_users;
+  int32_t K, F, P;
+  const int4* items;
+  int64_t n_items;
+  const int64_t *item_base, *entry_base;
+  const int32_t* rec_j;
+  const float* rec_D;
+  float lambda;
+  double* out;
+  int64_t out_stride;
+};
+cudaError_t launch_objective(const ObjectiveArgs& a, cudaStream_t st);
+cudaError_t launch_worker_objective(const ObjectiveArgs& a, cudaStream_t st);
 
 // MF layout build (setup, not per clock).
 struct LayoutBuild {
@@ -285,12 +301,11 @@ cudaError_t launch_stage_check(const int32_t* su, const int32_t* sj, const int32
                                const int32_t* rj, const int32_t* ruoff, int64_t n, int64_t n_off, uint32_t* status,
                                cudaStream_t st);
 
-// Read-only view of a context's loaded MF entries and of table version
-// `version` (checked against the live window), for entry points defined in
-// other translation units; and the context's error setter.
-esspt_status mf_view(esspt_ctx* ctx, int32_t version, const float** slot, int64_t* n_users, int32_t* K,
-                     const int32_t** rec_u, const int32_t** rec_j, const float** rec_D, const int32_t** worker,
-                     int64_t* n_obs, int32_t* P, cudaStream_t* st);
+// The objective's inputs for a context's loaded entries and table version
+// `version` (checked against the live window), all but out and lambda, for
+// entry points defined in other translation units; and the context's error
+// setter.
+esspt_status mf_view(esspt_ctx* ctx, int32_t version, ObjectiveArgs* a, cudaStream_t* st);
 esspt_status mf_fail(esspt_ctx* ctx, esspt_status code, const char* msg);
 
 }  // namespace esspt

@@ -22,17 +22,7 @@ namespace esspt {
 
 namespace {
 
-// Sum over the G lanes of a row group (G a power of two, <= 32).
-template <int G>
-__device__ __forceinline__ float group_sum(float x, unsigned mask) {
-#pragma unroll
-  for (int off = G / 2; off > 0; off >>= 1) x += __shfl_xor_sync(mask, x, off, G);
-  return x;
-}
-
 __device__ __forceinline__ float4 f4_zero() { return make_float4(0.f, 0.f, 0.f, 0.f); }
-
-__device__ __forceinline__ float dot4(float4 a, float4 b) { return a.x * b.x + a.y * b.y + a.z * b.z + a.w * b.w; }
 
 __device__ __forceinline__ float4 f4_axpy(float s, float4 x, float4 y) {  // y + s x
   return make_float4(y.x + s * x.x, y.y + s * x.y, y.z + s * x.z, y.w + s * x.w);
@@ -360,7 +350,7 @@ __global__ void __launch_bounds__(kStreamWarps * 32, MINB) sgd_stream_kernel(Str
         for (int k = 0; k < NV; ++k) {
           float4* h = &hot[wib][y >> 1][k][lane];
           const f2x2 v = lds_f2x2(h);
-          sts_f2x2(h, add2(v.lo, fma2(ee, L[k].lo, mul2(nlam, R[k].lo))),
+          st_f2x2(h, add2(v.lo, fma2(ee, L[k].lo, mul2(nlam, R[k].lo))),
                    add2(v.hi, fma2(ee, L[k].hi, mul2(nlam, R[k].hi))));
         }
       } else {
@@ -856,67 +846,6 @@ cudaError_t launch_item_merge(const ItemMergeArgs& a, cudaStream_t st) {
   // flight per thread beat more threads with one each (0.019 against
   // 0.029 ms per clock on mid; 74 against 207 us on a 200k-item table).
   item_merge_kernel<8><<<(unsigned)std::min<int64_t>((work + 2047) / 2048, (int64_t)1 << 30), 256, 0, st>>>(a);
-  return cudaGetLastError();
-}
-
-// ---------------------------------------------------------------------------
-// Objective (Sec. 3.1, Sec. 5) over all entries: sum e^2 and
-// sum [e^2 + lambda(|L_i|^2 + |R_j|^2)], fp32 residuals, fp64 sums.
-// One warp per entry.
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) objective_kernel(const float* __restrict__ slot, int64_t n_users, int32_t K,
-                                                        const int32_t* __restrict__ rec_u,
-                                                        const int32_t* __restrict__ rec_j,
-                                                        const float* __restrict__ rec_D, int64_t n_obs, float lambda,
-                                                        double* out2) {
-  const int lane = threadIdx.x & 31;
-  const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  const int32_t K4 = K >> 2;
-  const float4* t4 = reinterpret_cast<const float4*>(slot);
-  double s1 = 0.0, s2 = 0.0;
-  for (int64_t k = warp; k < n_obs; k += nwarps) {
-    const float4* L = t4 + (int64_t)rec_u[k] * K4;
-    const float4* R = t4 + (n_users + rec_j[k]) * K4;
-    float dot = 0.f, nl = 0.f, nr = 0.f;
-    for (int32_t q = lane; q < K4; q += 32) {
-      const float4 l = L[q], r = R[q];
-      dot += dot4(l, r);
-      nl += dot4(l, l);
-      nr += dot4(r, r);
-    }
-    dot = group_sum<32>(dot, 0xffffffffu);
-    nl = group_sum<32>(nl, 0xffffffffu);
-    nr = group_sum<32>(nr, 0xffffffffu);
-    if (lane == 0) {
-      const double e = (double)(rec_D[k] - dot);
-      s1 += e * e;
-      s2 += e * e + (double)lambda * ((double)nl + (double)nr);
-    }
-  }
-  __shared__ double sh[2][8];
-  const int w = threadIdx.x >> 5;
-  if (lane == 0) {
-    sh[0][w] = s1;
-    sh[1][w] = s2;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double x = 0.0, y = 0.0;
-    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) {
-      x += sh[0][i];
-      y += sh[1][i];
-    }
-    atomicAdd(out2, x);
-    atomicAdd(out2 + 1, y);
-  }
-}
-
-cudaError_t launch_objective(const float* slot, int64_t n_users, int32_t K, const int32_t* rec_u, const int32_t* rec_j,
-                             const float* rec_D, int64_t n_obs, float lambda, double* out2, cudaStream_t st) {
-  cudaError_t err = cudaMemsetAsync(out2, 0, 2 * sizeof(double), st);
-  if (err != cudaSuccess || n_obs == 0) return err;
-  objective_kernel<<<grid_for(n_obs, 8, 16), 256, 0, st>>>(slot, n_users, K, rec_u, rec_j, rec_D, n_obs, lambda, out2);
   return cudaGetLastError();
 }
 

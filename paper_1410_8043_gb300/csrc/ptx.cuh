@@ -81,9 +81,12 @@ __device__ __forceinline__ u64 pack2(float x, float y) {
   asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
   return r;
 }
+__device__ __forceinline__ void unpack2(u64 v, float& x, float& y) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(v));
+}
 __device__ __forceinline__ float sum2(u64 v) {
   float x, y;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(v));
+  unpack2(v, x, y);
   return x + y;
 }
 __device__ __forceinline__ u64 mul2(u64 a, u64 b) {
@@ -112,7 +115,7 @@ __device__ __forceinline__ f2x2 lds_f2x2(const float4* p) {
   const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(p);
   return f2x2{v.x, v.y};
 }
-__device__ __forceinline__ void sts_f2x2(float4* p, u64 lo, u64 hi) {
+__device__ __forceinline__ void st_f2x2(float4* p, u64 lo, u64 hi) {
   *reinterpret_cast<ulonglong2*>(p) = make_ulonglong2(lo, hi);
 }
 __device__ __forceinline__ void st_stream_f2x2_if(float4* p, u64 lo, u64 hi, uint64_t pol, bool pred) {
