@@ -30,7 +30,8 @@ struct esspt_ctx {
   bool mf = false;
   int64_t n_users = 0, n_items = 0, n_obs = 0;
   int32_t F = 0;
-  int32_t *rec_u = nullptr, *rec_j = nullptr, *uoff = nullptr, *item_cnt = nullptr, *worker = nullptr;
+  int32_t *rec_u = nullptr, *rec_j = nullptr, *uoff = nullptr, *item_cnt = nullptr;
+  int32_t *wuser = nullptr, *wbase = nullptr;  // users by worker
   int32_t *item_rep = nullptr, *hot_item = nullptr;
   // The SGD kernel's stream: its geometry, words and places (see StreamArgs),
   // and the first place of each minibatch.
@@ -47,8 +48,8 @@ struct esspt_ctx {
   std::vector<int64_t> part_base;     // [F+1] first word of each minibatch's split
   cudaEvent_t ev_before = nullptr, ev_after = nullptr;
   // Last clock that changed each user row, and the last clock at which every
-  // idle row is still copied forward (after an INC or a sequential clock,
-  // whose writes are not tracked per row).
+  // idle row is still copied forward (after an INC, whose writes are not
+  // tracked per row).
   int32_t* chg = nullptr;
   int32_t copy_all_until = 0;
 };
@@ -205,7 +206,7 @@ bool is_host_ptr(const void* p) {
 }
 
 struct MfCarve {
-  size_t rec_u, rec_j, rec_D, sx, syz, place, steps, uoff, mb_base, item_cnt, item_rep, dR, worker, chunk, chunk_base, heavy, heavy_base, dL,
+  size_t rec_u, rec_j, rec_D, sx, syz, place, steps, uoff, mb_base, item_cnt, item_rep, dR, wuser, wbase, chunk, chunk_base, heavy, heavy_base, dL,
       user_slot, row_x, chg, hot_item, part, total;
   int64_t max_chunks, max_heavy, dR_rows, dL_rows, part_rows, max_places;
 };
@@ -213,7 +214,7 @@ struct MfCarve {
 // Persistent MF workspace: entries laid out by (minibatch, user), per-minibatch
 // user offsets and item counts, item replica rows, heavy-user lists and the
 // zero-initialised delta replicas dR (items) and dL (heavy users).
-MfCarve mf_carve(int64_t n_obs, int64_t n_users, int64_t n_items, int32_t F, int32_t K, bool row_mode) {
+MfCarve mf_carve(int64_t n_obs, int64_t n_users, int64_t n_items, int32_t F, int32_t K, int32_t P, bool row_mode) {
   MfCarve k{};
   k.max_chunks = layout_max_chunks(n_obs, F, n_users);
   k.max_heavy = layout_max_heavy(n_obs, F);
@@ -239,7 +240,8 @@ MfCarve mf_carve(int64_t n_obs, int64_t n_users, int64_t n_items, int32_t F, int
   k.item_cnt = take(sizeof(int32_t) * (size_t)F * n_items);
   k.item_rep = take(sizeof(int32_t) * (n_items + 1));
   k.dR = take(sizeof(float4) * (size_t)k.dR_rows * dR_stride4(K));
-  k.worker = take(sizeof(int32_t) * n_users);
+  k.wuser = take(sizeof(int32_t) * n_users);
+  k.wbase = take(sizeof(int32_t) * (P + 1));
   k.chunk = take(sizeof(int4) * k.max_chunks);
   k.chunk_base = take(sizeof(int64_t) * (F + 1));
   k.heavy = take(sizeof(int4) * k.max_heavy);
@@ -477,7 +479,7 @@ esspt_status esspt_read_table(esspt_ctx* c, int32_t version, float* out) {
 
 size_t esspt_mf_workspace_bytes(const esspt_ctx* c, int64_t n_obs, int64_t n_users, int32_t F) {
   if (!mf_sizes_ok(c, n_obs, n_users, F)) return 0;
-  return mf_carve(n_obs, n_users, c->n_rows - n_users, F, c->K, c->rowver != nullptr).total;
+  return mf_carve(n_obs, n_users, c->n_rows - n_users, F, c->K, c->P, c->rowver != nullptr).total;
 }
 
 size_t esspt_mf_scratch_bytes(const esspt_ctx* c, int64_t n_obs, int64_t n_users, int32_t F) {
@@ -495,7 +497,7 @@ esspt_status esspt_mf_load(esspt_ctx* c, const int32_t* d_i, const int32_t* d_j,
   if ((reinterpret_cast<uintptr_t>(d_ws) & 255u) || (reinterpret_cast<uintptr_t>(d_scratch) & 255u))
     return fail(c, ESSPT_EINVAL, "MF buffers must be 256-byte aligned");
   const int64_t n_items = c->n_rows - n_users;
-  const MfCarve k = mf_carve(n_obs, n_users, n_items, F, c->K, c->rowver != nullptr);
+  const MfCarve k = mf_carve(n_obs, n_users, n_items, F, c->K, c->P, c->rowver != nullptr);
   if (bytes < k.total) return fail(c, ESSPT_ENOSPC, "MF workspace too small");
   if (scratch_bytes < layout_scratch_bytes(n_obs, n_users, n_items, F))
     return fail(c, ESSPT_ENOSPC, "MF scratch too small");
@@ -526,6 +528,8 @@ esspt_status esspt_mf_load(esspt_ctx* c, const int32_t* d_i, const int32_t* d_j,
   b.heavy_base = reinterpret_cast<int64_t*>(w + k.heavy_base);
   b.max_chunks = k.max_chunks;
   b.max_heavy = k.max_heavy;
+  b.wuser = reinterpret_cast<int32_t*>(w + k.wuser);
+  b.wbase = reinterpret_cast<int32_t*>(w + k.wbase);
   b.scratch = d_scratch;
   b.scratch_bytes = scratch_bytes;
   b.status = c->status;
@@ -539,8 +543,6 @@ esspt_status esspt_mf_load(esspt_ctx* c, const int32_t* d_i, const int32_t* d_j,
     ESSPT_CUDA(c, cudaMemsetAsync(c->status, 0, sizeof(uint32_t), c->st));
     return fail(c, ESSPT_EINVAL, "an MF input index is out of range");
   }
-  int32_t* worker = reinterpret_cast<int32_t*>(w + k.worker);
-  ESSPT_CUDA(c, cudaMemcpyAsync(worker, d_worker, sizeof(int32_t) * n_users, cudaMemcpyDeviceToDevice, c->st));
   float* dR = reinterpret_cast<float*>(w + k.dR);
   float* dL = reinterpret_cast<float*>(w + k.dL);
   ESSPT_CUDA(c, cudaMemsetAsync(dR, 0, sizeof(float4) * (size_t)k.dR_rows * dR_stride4(c->K), c->st));
@@ -612,7 +614,8 @@ esspt_status esspt_mf_load(esspt_ctx* c, const int32_t* d_i, const int32_t* d_j,
     ESSPT_CUDA(c, cudaMemsetAsync(c->row_x, 0xff, sizeof(uint32_t) * k.max_places, c->st));
   }
   c->item_cnt = b.item_cnt;
-  c->worker = worker;
+  c->wuser = b.wuser;
+  c->wbase = b.wbase;
   c->item_rep = b.item_rep;
   c->geo = geo;
   c->sx = sx;
@@ -760,33 +763,36 @@ esspt_status esspt_mf_sgd_clock_sequential(esspt_ctx* c, float eta, float lambda
   if (!d_work || (reinterpret_cast<uintptr_t>(d_work) & 15u)) return fail(c, ESSPT_EINVAL, "work must be 16-byte aligned");
   if (work_bytes < need) return fail(c, ESSPT_ENOSPC, "sequential work buffer too small");
   const int32_t b = (c->clock - 1) % c->F;
-  SeqArgs a{};
+  SeqArgs q{};
+  SgdArgs& a = q.a;
   a.ring = c->ring;
   a.n_rows = c->n_rows;
   a.K = c->K;
   a.n_users = (int32_t)c->n_users;
-  a.n_items = (int32_t)c->n_items;
   a.nslots = c->nslots;
   a.slot_out = c->clock % c->nslots;
   a.slot_base = c->acc_ready ? a.slot_out : (c->clock - 1) % c->nslots;
-  a.P = c->P;
-  a.v = c->v;
-  a.worker = c->worker;
   a.uoff = c->uoff + (int64_t)b * (c->n_users + 1);
-  a.rec_j = c->rec_j + c->mb_base[b];
-  a.rec_D = c->rec_D + c->mb_base[b];
-  a.item_cnt = c->item_cnt + (int64_t)b * c->n_items;
-  a.mine = static_cast<float*>(d_work);
   a.eta = eta;
   a.lambda = lambda;
   a.cap = cap;
   a.sq_loss = d_sq_loss;
+  a.chg = c->chg;
+  a.clock = c->clock;
+  a.copy_all_until = c->copy_all_until;
+  q.P = c->P;
+  q.n_items = (int32_t)c->n_items;
+  q.v = c->v;
+  q.wuser = c->wuser;
+  q.wbase = c->wbase;
+  q.rec_j = c->rec_j + c->mb_base[b];
+  q.rec_D = c->rec_D + c->mb_base[b];
+  q.item_cnt = c->item_cnt + (int64_t)b * c->n_items;
+  q.mine = static_cast<float*>(d_work);
   ESSPT_CUDA(c, cudaMemsetAsync(d_work, 0, need, c->st));
   if (c->ev_before) ESSPT_CUDA(c, cudaEventRecord(c->ev_before, c->st));
-  ESSPT_CUDA(c, launch_seq_clock(a, c->st));
+  ESSPT_CUDA(c, launch_seq_clock(q, c->st));
   if (c->ev_after) ESSPT_CUDA(c, cudaEventRecord(c->ev_after, c->st));
-  // the sequential kernels' row writes are not tracked per row
-  c->copy_all_until = std::max(c->copy_all_until, c->clock + c->s + 1);
   c->acc_ready = true;
   return advance(c);
 }

@@ -219,19 +219,15 @@ cudaError_t launch_row_refresh(const RowRefreshArgs& a, cudaStream_t st);
 // Sequential (read-my-writes) SGD of one clock over minibatch b: the users
 // kernel writes every user row of version c, the item merge every item row.
 struct SeqArgs {
-  float* ring;
-  int64_t n_rows;
-  int32_t K, n_users, n_items, nslots, slot_base, slot_out, P;
+  SgdArgs a;                // ring, slots, offsets, step sizes (no vslot, dR or work list)
+  int32_t P, n_items;
   const int32_t* v;         // [P] read versions
-  const int32_t* worker;    // [n_users]
-  const int32_t* uoff;      // [n_users+1] entry offsets of minibatch b
+  const int32_t* wuser;     // [n_users] users by worker, ascending within a worker
+  const int32_t* wbase;     // [P+1] first of each worker's users
   const int32_t* rec_j;     // item of each entry of minibatch b
   const float* rec_D;
   const int32_t* item_cnt;  // [n_items] entries per item in minibatch b (hot-row cap)
   float* mine;              // [P][n_items][K] each worker's item changes this clock (zero on entry)
-  float eta, lambda;
-  int32_t cap;
-  double* sq_loss;          // optional
 };
 cudaError_t launch_seq_clock(const SeqArgs& a, cudaStream_t st);
 cudaError_t launch_heavy_merge(const HeavyMergeArgs& a, cudaStream_t st);
@@ -278,6 +274,8 @@ struct LayoutBuild {
   int64_t* chunk_base;  // [F+1]
   int4* heavy;          // [max_heavy]
   int64_t* heavy_base;  // [F+1]
+  int32_t* wuser;       // [n_users] users by worker, ascending within a worker
+  int32_t* wbase;       // [P+1] first of each worker's users
   int64_t max_chunks, max_heavy;
   // scratch
   void* scratch;

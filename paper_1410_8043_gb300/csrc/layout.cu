@@ -167,6 +167,28 @@ __global__ void item_reps_kernel(const int32_t* __restrict__ item_cnt, int64_t n
   }
 }
 
+// wbase[p] = first place of worker p among the sorted workers of the users.
+__global__ void worker_bases_kernel(const uint32_t* __restrict__ sorted, int64_t n_users, int32_t P,
+                                    int32_t* __restrict__ wbase) {
+  const int32_t p = blockIdx.x * blockDim.x + threadIdx.x;
+  if (p > P) return;
+  int64_t lo = 0, hi = n_users;
+  while (lo < hi) {
+    const int64_t m = (lo + hi) / 2;
+    if (sorted[m] >= (uint32_t)p) {
+      hi = m;
+    } else {
+      lo = m + 1;
+    }
+  }
+  wbase[p] = (int32_t)lo;
+}
+
+__global__ void iota_kernel(uint32_t* __restrict__ val, int64_t n) {
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += stride) val[k] = (uint32_t)k;
+}
+
 // The work list in its final order, and each item's cost.
 __global__ void place_items_kernel(const int4* __restrict__ raw, const uint32_t* __restrict__ perm, int64_t n,
                                    int4* __restrict__ items, int32_t* __restrict__ cost) {
@@ -237,7 +259,7 @@ ScratchPlan plan(int64_t n_obs, int64_t n_users, int64_t n_items, int32_t F) {
   const int64_t items = std::min(n_obs, layout_max_chunks(n_obs, F, n_users));  // an item holds an entry or more
   size_t sort_bytes = 0, scan_bytes = 0, scan2_bytes = 0, scan3_bytes = 0;
   cub::DeviceRadixSort::SortPairs(nullptr, sort_bytes, (const uint32_t*)nullptr, (uint32_t*)nullptr,
-                                  (const uint32_t*)nullptr, (uint32_t*)nullptr, (int)std::max<int64_t>(n_obs, 1), 0,
+                                  (const uint32_t*)nullptr, (uint32_t*)nullptr, (int)std::max<int64_t>(std::max(n_obs, n_users), 1), 0,
                                   32);
   cub::DeviceScan::ExclusiveSum(nullptr, scan_bytes, (const int32_t*)nullptr, (int64_t*)nullptr, (int)(keys + 1));
   cub::DeviceScan::ExclusiveSum(nullptr, scan2_bytes, (const int32_t*)nullptr, (int32_t*)nullptr,
@@ -362,6 +384,16 @@ cudaError_t build_layout(LayoutBuild& b, cudaStream_t st) {
   if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return e;
   if (n > std::min(b.n_obs, b.max_chunks)) return cudaErrorInvalidValue;
   b.pre = pre;
+  // Users by worker (cnt and nch, [F n_users + 1] each, are free now).
+  uint32_t* ids = reinterpret_cast<uint32_t*>(cnt);
+  uint32_t* sorted = reinterpret_cast<uint32_t*>(nch);
+  iota_kernel<<<blocks_for(b.n_users), 256, 0, st>>>(ids, b.n_users);
+  tb = p.cub_bytes;
+  e = cub::DeviceRadixSort::SortPairs(cub_tmp, tb, reinterpret_cast<const uint32_t*>(b.worker), sorted, ids,
+                                      reinterpret_cast<uint32_t*>(b.wuser), (int)b.n_users, 0, bits_for(b.P), st);
+  if (e != cudaSuccess) return e;
+  worker_bases_kernel<<<b.P / 256 + 1, 256, 0, st>>>(sorted, b.n_users, b.P, b.wbase);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if (n > 0) {
     tb = p.cub_bytes;
     e = cub::DeviceRadixSort::SortPairs(cub_tmp, tb, key_in, key_out, val_in, val_out, (int)n, 0,
