@@ -21,7 +21,7 @@ struct esspt_ctx {
   int32_t* vslot = nullptr;  // [P] ring slot of each read version
   uint32_t* status = nullptr;
   uint32_t* thr = nullptr;
-  uint32_t* vap_norm = nullptr;  // [s+1] VAP in-transit norms of the current clock
+  uint32_t* vap_norm = nullptr;  // [s+1] VAP in-transit norms of the current clock, then [s+1] words of their scan
   int32_t clock = 0;      // clock in progress (0 = table not initialised)
   bool acc_ready = false; // slot of version `clock` holds version clock-1 + INCs so far
   bool sched_set = false; // ESSPT_EXTERNAL: v_p(clock) supplied
@@ -121,7 +121,7 @@ Carve carve(const esspt_config* c) {
   k.thr = o;
   o += align256(sizeof(uint32_t) * (size_t)(delay_max(c) + 1));
   k.vap = o;
-  o += c->model == ESSPT_VAP ? align256(sizeof(uint32_t) * (size_t)(c->staleness + 1)) : 0;
+  o += c->model == ESSPT_VAP ? align256(2 * sizeof(uint32_t) * (size_t)(c->staleness + 1)) : 0;
   k.rowver = o;
   o += c->model == ESSPT_SSP_ROW ? align256(sizeof(int32_t) * (size_t)c->num_workers * (size_t)c->n_rows) : 0;
   k.total = o;
@@ -149,11 +149,13 @@ ScheduleArgs schedule_args(const esspt_ctx* c, int32_t clock);
 
 esspt_status run_schedule(esspt_ctx* c) {
   if (c->cfg.model == ESSPT_VAP) {
-    // In-transit norms of the candidate versions against version clock-1.
+    // In-transit norms of the candidate versions against version clock-1, from the stalest down.
     const int32_t kmax = std::min(c->s, c->clock - 1);
-    ESSPT_CUDA(c, cudaMemsetAsync(c->vap_norm, 0, sizeof(uint32_t) * (size_t)(c->s + 1), c->st));
+    ESSPT_CUDA(c, cudaMemsetAsync(c->vap_norm, 0, 2 * sizeof(uint32_t) * (size_t)(c->s + 1), c->st));
     if (kmax > 0)
-      ESSPT_CUDA(c, launch_vap_norms(c->ring, c->n_rows * c->K, c->nslots, c->clock, kmax, c->vap_norm, c->st));
+      ESSPT_CUDA(c, launch_vap(c->ring, c->n_rows * c->K, c->nslots, c->clock, kmax,
+                                    c->cfg.vap_v0 / std::sqrt((double)c->clock), c->vap_norm,
+                                    c->vap_norm + c->s + 1, c->st));
   }
   ESSPT_CUDA(c, launch_schedule(schedule_args(c, c->clock), c->st));
   return ESSPT_OK;

@@ -68,7 +68,7 @@ struct ScheduleArgs {
   int32_t* vslot;          // [P] out: ring slot v mod nslots of each read version
   uint32_t* status;        // latched error bits
   const uint32_t* thr;     // [dmax+1] ESSP delay thresholds, thr[k] = floor((1-p)^k 2^32)
-  const uint32_t* vap_norm;  // [s+1] VAP: bits of |X[c-1] - X[c-1-k]|_inf (fp32, >= 0)
+  const uint32_t* vap_norm;  // [s+1] VAP: see launch_vap
   double vap_bound;        // VAP: v0 / sqrt(c)
   int32_t P, c, s, nslots, model, phased, dmax;
   uint64_t seed;
@@ -160,10 +160,12 @@ struct ItemMergeArgs {
 
 // Launchers (return the launch error, if any).
 cudaError_t launch_schedule(const ScheduleArgs& a, cudaStream_t st);
-// VAP: norm[k] = bits of max |X[c-1] - X[c-1-k]| over the table, k = 1..kmax
-// (norm must be zero on entry; a NaN difference gives +inf).
-cudaError_t launch_vap_norms(const float* ring, int64_t slot_floats, int32_t nslots, int32_t c, int32_t kmax,
-                             uint32_t* norm, cudaStream_t st);
+// VAP: norm[k], k = 1..kmax, is within the bound (as fp32 bits) exactly where
+// max |X[c-1] - X[c-1-k]| over the table is, down to the stalest such k: the
+// norm itself, or 0 / +inf (norm and words, s+1 each, must be zero on entry; a
+// NaN difference counts as +inf).
+cudaError_t launch_vap(const float* ring, int64_t slot_floats, int32_t nslots, int32_t c, int32_t kmax,
+                            double bound, uint32_t* norm, uint32_t* words, cudaStream_t st);
 cudaError_t launch_copy_rows(float* dst, const float* src, int64_t n_floats, cudaStream_t st);
 // GET; with rowver non-null (row-granular SSP at clock c) each row is read at
 // the worker's cached version, refreshed to c-1 first where it is missing or

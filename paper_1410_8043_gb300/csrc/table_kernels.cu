@@ -1,6 +1,7 @@
 // Table kernels: the read-version schedule, the Clock() copy-forward of the
 // version ring, and the generic GET / INC row kernels.
 #include <algorithm>
+#include <cmath>
 
 #include "internal.h"
 #include "ptx.cuh"
@@ -32,7 +33,7 @@ cudaError_t launch_schedule(const ScheduleArgs& a, cudaStream_t st) {
 // value).  Candidates are taken 8 at a time so that each pass reads X[c-1]
 // once for 8 older versions.
 // ---------------------------------------------------------------------------
-constexpr int kVapBatch = 8;
+constexpr int kVapBatch = 8;  // candidates per launch
 
 __device__ __forceinline__ float vap_absdiff_max(float m, float4 a, float4 b) {
   const float d0 = fabsf(a.x - b.x), d1 = fabsf(a.y - b.y), d2 = fabsf(a.z - b.z), d3 = fabsf(a.w - b.w);
@@ -75,16 +76,110 @@ __global__ void __launch_bounds__(256) vap_norms_kernel(const float4* __restrict
   }
 }
 
-cudaError_t launch_vap_norms(const float* ring, int64_t slot_floats, int32_t nslots, int32_t c, int32_t kmax,
-                             uint32_t* norm, cudaStream_t st) {
+// ---------------------------------------------------------------------------
+// The same on large tables: which of the versions c-1-k, k = k0 .. k1, have an
+// in-transit max-norm |X[c-1] - X[c-1-k]| (over the table, fp32) within the
+// bound; norm[k] stays 0 if so and becomes +inf if not.  Only the stalest one within the bound
+// is read, so the candidates are taken from the stalest down, each until an
+// element breaks the bound, and none after one has been scanned whole: two
+// tables are read where all candidates at once would take k1 + 1 of them (s = 3
+// on a 498k x 100 table: 160 us with each norm taken in full).
+//
+// The work is one sequence of pieces, candidate by candidate, that the blocks
+// draw from a ticket (words[0]); a broken bound moves the ticket on to the next
+// candidate.  A block never waits: while a candidate's last pieces are with
+// other blocks it takes pieces of the next one, which may turn out needless.
+// words[k] counts the scanned pieces of candidate k.
+// ---------------------------------------------------------------------------
+constexpr int kVapLoads = 8;  // float4 of each version per thread and piece
+constexpr int64_t kVapPiece = 256 * kVapLoads;
+
+// A NaN difference counts as +inf.
+__device__ __forceinline__ bool vap_breaks(float4 a, float4 b, float bound) {
+  const float d0 = fabsf(a.x - b.x), d1 = fabsf(a.y - b.y), d2 = fabsf(a.z - b.z), d3 = fabsf(a.w - b.w);
+  const float m = fmaxf(fmaxf(d0, d1), fmaxf(d2, d3));  // drops NaN
+  const bool nan = (d0 != d0) || (d1 != d1) || (d2 != d2) || (d3 != d3);
+  return m > bound || (nan && bound < __int_as_float(0x7f800000));
+}
+
+__global__ void __launch_bounds__(256) vap_scan_kernel(const float4* __restrict__ ring, int64_t slot4, int32_t nslots,
+                                                       int32_t c, int32_t k0, int32_t k1, int32_t kmax, float bound,
+                                                       uint32_t pieces, uint32_t* norm, uint32_t* words) {
+  __shared__ uint32_t ticket;
+  volatile uint32_t* vnorm = norm;
+  volatile uint32_t* vwords = words;
+  if (k1 < kmax && vnorm[k1 + 1] == 0u) return;  // an earlier launch found the version
+  const uint32_t last = (uint32_t)(k1 - k0 + 1) * pieces;
+  const float4* cur = ring + (int64_t)((c - 1) % nslots) * slot4;
+  for (;;) {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      uint32_t t = atomicAdd(words, 1u);
+      // A candidate before this one that is scanned whole within its bound ends the search.
+      if (t < last)
+        for (int32_t k = k1; k > k1 - (int32_t)(t / pieces); --k)
+          if (vnorm[k] == 0u && vwords[k] == pieces) t = last;
+      ticket = t;
+    }
+    __syncthreads();
+    const uint32_t t = ticket;
+    if (t >= last) return;
+    const int32_t k = k1 - (int32_t)(t / pieces);
+    const float4* old = ring + (int64_t)((c - 1 - k) % nslots) * slot4;
+    const int64_t q0 = (int64_t)(t % pieces) * kVapPiece + threadIdx.x;
+    bool breaks = false;
+    float4 x[kVapLoads], y[kVapLoads];
+#pragma unroll
+    for (int i = 0; i < kVapLoads; ++i) {
+      const int64_t q = min(q0 + 256 * i, slot4 - 1);
+      x[i] = cur[q];
+      y[i] = old[q];
+    }
+#pragma unroll
+    for (int i = 0; i < kVapLoads; ++i) breaks |= vap_breaks(x[i], y[i], bound);
+    breaks = __syncthreads_or(breaks);
+    if (threadIdx.x == 0) {
+      if (breaks) {
+        vnorm[k] = 0x7f800000u;
+        atomicMax(words, (t / pieces + 1u) * pieces);
+      } else {
+        __threadfence();
+        atomicAdd(words + k, 1u);
+      }
+    }
+  }
+}
+
+cudaError_t launch_vap(const float* ring, int64_t slot_floats, int32_t nslots, int32_t c, int32_t kmax,
+                            double bound, uint32_t* norm, uint32_t* words, cudaStream_t st) {
   int dev = 0, sms = 148;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int64_t slot4 = slot_floats / 4;
-  const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((slot4 + 255) / 256, (int64_t)sms * 8));
-  for (int32_t k0 = 1; k0 <= kmax; k0 += kVapBatch) {
-    const int32_t nk = std::min(kVapBatch, kmax - k0 + 1);
-    vap_norms_kernel<<<blocks, 256, 0, st>>>(reinterpret_cast<const float4*>(ring), slot4, nslots, c, k0, nk, norm);
+  // The largest fp32 value within the bound: fp32 norms compare with it as with the bound.
+  float fb = (float)bound;
+  if ((double)fb > bound) fb = std::nextafterf(fb, 0.f);
+  const int64_t slot4 = slot_floats / 4, pieces = (slot4 + kVapPiece - 1) / kVapPiece;
+  // The scan saves up to kmax - 1 tables of traffic and costs its tickets, about
+  // 10 us (4 MB table, kmax = 6: 17 us against 7 for all norms at once).
+  if ((kmax - 1) * slot_floats * 4 < (128 << 20)) {
+    const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((slot4 + 255) / 256, (int64_t)sms * 8));
+    for (int32_t k0 = 1; k0 <= kmax; k0 += kVapBatch) {
+      vap_norms_kernel<<<blocks, 256, 0, st>>>(reinterpret_cast<const float4*>(ring), slot4, nslots, c, k0,
+                                               std::min(kVapBatch, kmax - k0 + 1), norm);
+      const cudaError_t e = cudaGetLastError();
+      if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+  }
+  for (int32_t k1 = kmax; k1 >= 1; k1 -= kVapBatch) {
+    const int32_t k0 = std::max(1, k1 - kVapBatch + 1);
+    if (k1 < kmax) {
+      const cudaError_t e = cudaMemsetAsync(words, 0, sizeof(uint32_t), st);
+      if (e != cudaSuccess) return e;
+    }
+    const int blocks = (int)std::min<int64_t>(pieces * (k1 - k0 + 1), (int64_t)sms * 8);
+    vap_scan_kernel<<<blocks, 256, 0, st>>>(reinterpret_cast<const float4*>(ring), slot4, nslots, c, k0, k1, kmax, fb,
+                                            (uint32_t)pieces, norm, words);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
