@@ -189,11 +189,12 @@ class FloorModel:
     clock's merge just wrote them).  Counted with torch on `device` (the
     distinct pairs by sorting), one minibatch at a time.
 
-    On the work-list path (32 < K <= 64) an idle user row unchanged over the
-    last s+2 clocks is not merged (its ring slot already holds it), and each
-    user has a 4-byte change-clock word, read for idle users and written for
-    active ones.  `bytes` must then see every clock from the table's version
-    0 in order."""
+    An idle user row unchanged over the last s+2 clocks is not merged (its ring
+    slot already holds it), and each user has a 4-byte change-clock word, read
+    for idle users and written for active ones: counted for 32 < K <= 64, where
+    the workloads have many idle users (at other widths the count is an upper
+    bound: mid has 14 of 480k idle).  `bytes` must then see every clock from the
+    table's version 0 in order."""
 
     def __init__(self, w, data, wp, mb, device="cpu"):
         import torch
@@ -205,43 +206,33 @@ class FloorModel:
         self.mb = torch.as_tensor(np.ascontiguousarray(mb)).to(self.dev)
         self.wp = torch.as_tensor(np.ascontiguousarray(wp)).to(self.dev).long()
         self._b = None
-        self._per_b = {}
         self.skip = 32 < w.K <= 64
         self.chg = torch.zeros(w.n_users, dtype=torch.int64, device=self.dev) if self.skip else None
         self.last_c = 0
 
     def _minibatch(self, b):
         """(entries, worker of each user with entries, distinct worker*M + item
-        pairs, some user has more than 96 entries) of minibatch b."""
+        pairs, users with entries) of minibatch b."""
         import torch
 
         if self._b != b:
             idx = torch.nonzero(self.mb == b).squeeze(1)
             ui = self.i[idx].long()
             jj = self.j[idx].long()
-            users, cnt = torch.unique(ui, return_counts=True)
+            users = torch.unique(ui)
             uw = self.wp[users]
             pj = torch.unique(self.wp[ui] * self.w.n_items + jj)
-            heavy = bool(cnt.numel() and int(cnt.max()) > 96)
-            self._cache = (int(idx.numel()), uw, pj, heavy, users)
+            self._cache = (int(idx.numel()), uw, pj, users)
             self._b = b
-            del idx, ui, jj, users, cnt
+            del idx, ui, jj, users
         return self._cache
-
-    def heavy(self, b) -> bool:
-        """Whether minibatch b has a user with more than 96 entries (those go
-        through the chunk and heavy-merge kernels)."""
-        if b not in self._per_b:
-            self._per_b[b] = self._minibatch(b)[3]
-        return self._per_b[b]
 
     def bytes(self, c, v):
         import torch
 
         w = self.w
         b = (c - 1) % w.F
-        n, uw, pj, heavy, active = self._minibatch(b)
-        self._per_b[b] = heavy
+        n, uw, pj, active = self._minibatch(b)
         vt = torch.as_tensor(np.ascontiguousarray(v, dtype=np.int64)).to(self.dev)
         stale = vt != (c - 1)
         users = int(stale[uw].sum())
@@ -411,7 +402,6 @@ def measure(args, w, dev, world, rank, local):
             stale += np.bincount(c - 1 - v, minlength=w.s + 1)[: w.s + 1]
         t.mf_sgd_clock(w.eta, w.lam, w.cap)
     t.poll()
-    heavy = {b: model.heavy(b) for b in {(c - 1) % w.F for c in range(W + 1, W + K + 1)}}
     del model
     torch.cuda.empty_cache()
 
@@ -527,10 +517,9 @@ def measure(args, w, dev, world, rank, local):
         "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": h2d // K, "d2h_bytes_per_step": d2h // K,
                 "copies": "minibatch of clock c+1 staged on a second stream while clock c runs",
                 "host_memory": host_kind},
-        # per clock: the SGD kernels and the item merge (which also computes the
+        # per clock: the SGD kernel and the Clock() merge (which also computes the
         # next schedule), plus the read model's own kernels
-        "gpu_launches": int(sum(_sgd_launches(w.K, heavy[(c - 1) % w.F]) + _model_launches(w, c)
-                                for c in range(W + 1, W + K + 1))),
+        "gpu_launches": int(sum(_sgd_launches() + _model_launches(w, c) for c in range(W + 1, W + K + 1))),
         "clocks": clocks,
         "objective": {"clock": c_final, "sq_loss": sq, "penalised": pen},
         # Fig. 1 (left) quantity: clock differential v_p(c) - c of every read in
@@ -546,13 +535,13 @@ def measure(args, w, dev, world, rank, local):
 
 def _sgd_kernel_name(K):
     """The SGD launches of one clock that the profile events bracket."""
-    return "sgd_stream_kernel (+ heavy_merge_kernel when some user is heavy)"
+    return "sgd_stream_kernel"
 
 
-def _sgd_launches(K, heavy: bool) -> int:
-    """Kernels of one clock's SGD phase plus the item merge (which also
+def _sgd_launches() -> int:
+    """Kernels of one clock: the SGD stream and the Clock() merge (which also
     computes the next schedule)."""
-    return 1 + int(heavy) + 1
+    return 2
 
 
 def run_gpu(args, w):

@@ -41,16 +41,17 @@ struct esspt_ctx {
   float *rec_D = nullptr, *dR = nullptr, *dL = nullptr;
   int32_t* rowver = nullptr;     // row-granular SSP: [P][n_rows] cached versions, -1 = never read
   int32_t* user_slot = nullptr;  // row-granular SSP: [n_users] per-clock ring slot of each user row
-  int4 *chunk = nullptr, *heavy = nullptr;
+  int4 *chunk = nullptr, *heavy = nullptr, *popular = nullptr;
+  int64_t n_popular = 0;
   std::vector<int64_t> mb_base, chunk_base, heavy_base;
   int64_t *d_mb_base = nullptr, *d_chunk_base = nullptr;
   int4* part = nullptr;               // split of each minibatch's work items over the warps
   std::vector<int64_t> part_base;     // [F+1] first word of each minibatch's split
   cudaEvent_t ev_before = nullptr, ev_after = nullptr;
-  // Last clock that changed each user row, and the last clock at which every
-  // idle row is still copied forward (after an INC, whose writes are not
+  // Last clock that changed each user and item row, and the last clock at which
+  // every idle row is still copied forward (after an INC, whose writes are not
   // tracked per row).
-  int32_t* chg = nullptr;
+  int32_t *chg = nullptr, *chg_item = nullptr;
   int32_t copy_all_until = 0;
 };
 
@@ -209,7 +210,7 @@ bool is_host_ptr(const void* p) {
 
 struct MfCarve {
   size_t rec_u, rec_j, rec_D, sx, syz, place, steps, uoff, mb_base, item_cnt, item_rep, dR, wuser, wbase, chunk, chunk_base, heavy, heavy_base, dL,
-      user_slot, row_x, chg, hot_item, part, total;
+      user_slot, row_x, chg, chg_item, popular, n_popular, hot_item, part, total;
   int64_t max_chunks, max_heavy, dR_rows, dL_rows, part_rows, max_places;
 };
 
@@ -252,8 +253,11 @@ MfCarve mf_carve(int64_t n_obs, int64_t n_users, int64_t n_items, int32_t F, int
   // Row-granular SSP: per-clock user slots and x words of the stream.
   k.user_slot = row_mode ? take(sizeof(int32_t) * n_users) : o;
   k.row_x = row_mode ? take(sizeof(uint32_t) * k.max_places) : o;
-  // The clock that last changed each user row.
+  // The clock that last changed each user and item row; items with extra replicas.
   k.chg = take(sizeof(int32_t) * n_users);
+  k.chg_item = take(sizeof(int32_t) * n_items);
+  k.popular = take(sizeof(int4) * layout_max_popular(n_obs));
+  k.n_popular = take(sizeof(uint32_t));
   k.hot_item = uses_hot(K) ? take(sizeof(int32_t) * (size_t)F * kHot) : o;
   // A minibatch uses at most one warp per work item.
   k.part_rows = std::min((int64_t)F * stream_max_warps(K), k.max_chunks);
@@ -380,6 +384,7 @@ esspt_status esspt_table_init(esspt_ctx* c, const float* rows) {
   c->sched_set = false;
   if (c->chg) {  // every row is version 0's: unchanged since clock 0
     ESSPT_CUDA(c, cudaMemsetAsync(c->chg, 0, sizeof(int32_t) * (size_t)c->n_users, c->st));
+    ESSPT_CUDA(c, cudaMemsetAsync(c->chg_item, 0, sizeof(int32_t) * (size_t)c->n_items, c->st));
     c->copy_all_until = 0;
   }
   if (c->cfg.model != ESSPT_EXTERNAL) return run_schedule(c);
@@ -527,6 +532,8 @@ esspt_status esspt_mf_load(esspt_ctx* c, const int32_t* d_i, const int32_t* d_j,
   b.chunk = reinterpret_cast<int4*>(w + k.chunk);
   b.chunk_base = reinterpret_cast<int64_t*>(w + k.chunk_base);
   b.heavy = reinterpret_cast<int4*>(w + k.heavy);
+  b.popular = reinterpret_cast<int4*>(w + k.popular);
+  b.n_popular = reinterpret_cast<uint32_t*>(w + k.n_popular);
   b.heavy_base = reinterpret_cast<int64_t*>(w + k.heavy_base);
   b.max_chunks = k.max_chunks;
   b.max_heavy = k.max_heavy;
@@ -556,6 +563,8 @@ esspt_status esspt_mf_load(esspt_ctx* c, const int32_t* d_i, const int32_t* d_j,
   std::vector<int64_t> mbb((size_t)F + 1), chb((size_t)F + 1), hvb((size_t)F + 1);
   ESSPT_CUDA(c, cudaMemcpyAsync(mbb.data(), b.mb_base, sizeof(int64_t) * (F + 1), cudaMemcpyDeviceToHost, c->st));
   ESSPT_CUDA(c, cudaMemcpyAsync(chb.data(), b.chunk_base, sizeof(int64_t) * (F + 1), cudaMemcpyDeviceToHost, c->st));
+  uint32_t n_popular = 0;
+  ESSPT_CUDA(c, cudaMemcpyAsync(&n_popular, b.n_popular, sizeof n_popular, cudaMemcpyDeviceToHost, c->st));
   ESSPT_CUDA(c, cudaMemcpyAsync(hvb.data(), b.heavy_base, sizeof(int64_t) * (F + 1), cudaMemcpyDeviceToHost, c->st));
   ESSPT_CUDA(c, cudaMemcpyAsync(&bits, c->status, sizeof bits, cudaMemcpyDeviceToHost, c->st));
   ESSPT_CUDA(c, cudaStreamSynchronize(c->st));
@@ -631,6 +640,10 @@ esspt_status esspt_mf_load(esspt_ctx* c, const int32_t* d_i, const int32_t* d_j,
   c->heavy = b.heavy;
   c->chg = reinterpret_cast<int32_t*>(w + k.chg);
   ESSPT_CUDA(c, cudaMemsetAsync(c->chg, 0, sizeof(int32_t) * (size_t)n_users, c->st));
+  c->chg_item = reinterpret_cast<int32_t*>(w + k.chg_item);
+  ESSPT_CUDA(c, cudaMemsetAsync(c->chg_item, 0, sizeof(int32_t) * (size_t)n_items, c->st));
+  c->popular = b.popular;
+  c->n_popular = n_popular;
   // rows changed before this load are not tracked
   c->copy_all_until = c->clock + c->s + 1;
   c->mb_base = mbb;
@@ -696,7 +709,6 @@ esspt_status esspt_mf_sgd_clock(esspt_ctx* c, float eta, float lambda, int32_t c
     a.row_mode = 1;
     a.user_slot = c->user_slot;
   }
-  const int64_t nhv = c->heavy_base[b + 1] - c->heavy_base[b];
   if (c->ev_before) ESSPT_CUDA(c, cudaEventRecord(c->ev_before, c->st));
   StreamArgs sa{};
   sa.a = a;
@@ -707,43 +719,36 @@ esspt_status esspt_mf_sgd_clock(esspt_ctx* c, float eta, float lambda, int32_t c
   sa.yz = c->syz + 2 * c->stream_base[b];
   sa.dL = c->dL;
   ESSPT_CUDA(c, launch_sgd_stream(sa, c->st));
-  if (nhv > 0) {
-    HeavyMergeArgs h{};
-    h.ring = c->ring;
-    h.n_rows = c->n_rows;
-    h.K = c->K;
-    h.nslots = c->nslots;
-    h.slot_base = slot_base;
-    h.slot_out = slot_out;
-    h.heavy = c->heavy + c->heavy_base[b];
-    h.n_heavy = nhv;
-    h.dL = c->dL;
-    h.eta = eta;
-    h.cap = cap;
-    h.chg = c->chg;
-    h.clock = c->clock;
-    ESSPT_CUDA(c, launch_heavy_merge(h, c->st));
-  }
   if (c->ev_after) ESSPT_CUDA(c, cudaEventRecord(c->ev_after, c->st));
-  ItemMergeArgs m{};
+  MergeArgs m{};
   m.ring = c->ring;
   m.n_rows = c->n_rows;
   m.K = c->K;
   m.n_users = (int32_t)c->n_users;
   m.n_items = (int32_t)c->n_items;
+  m.nslots = c->nslots;
   m.slot_base = slot_base;
   m.slot_out = slot_out;
   m.item_rep = c->item_rep;
   m.dR = c->dR;
   m.dR_ld = dR_stride4(c->K);
   m.item_cnt = c->item_cnt + (int64_t)b * c->n_items;
+  m.popular = c->popular;
+  m.n_popular = c->n_popular;
+  m.heavy = c->heavy + c->heavy_base[b];
+  m.n_heavy = c->heavy_base[b + 1] - c->heavy_base[b];
+  m.dL = c->dL;
   m.eta = eta;
   m.cap = cap;
+  m.chg = c->chg;
+  m.chg_item = c->chg_item;
+  m.clock = c->clock;
+  m.copy_all_until = c->copy_all_until;
   // SSP and ESSP schedules need only the previous read versions, so the merge
   // computes them; VAP needs version c complete, so it runs after the merge.
   m.do_schedule = c->cfg.model == ESSPT_SSP_LAZY || c->cfg.model == ESSPT_ESSP_EAGER || c->cfg.model == ESSPT_SSP_ROW;
   m.sched = schedule_args(c, c->clock + 1);
-  ESSPT_CUDA(c, launch_item_merge(m, c->st));
+  ESSPT_CUDA(c, launch_clock_merge(m, c->st));
   c->acc_ready = true;
   return advance(c, m.do_schedule != 0);
 }
@@ -790,6 +795,7 @@ esspt_status esspt_mf_sgd_clock_sequential(esspt_ctx* c, float eta, float lambda
   q.rec_j = c->rec_j + c->mb_base[b];
   q.rec_D = c->rec_D + c->mb_base[b];
   q.item_cnt = c->item_cnt + (int64_t)b * c->n_items;
+  q.chg_item = c->chg_item;
   q.mine = static_cast<float*>(d_work);
   ESSPT_CUDA(c, cudaMemsetAsync(d_work, 0, need, c->st));
   if (c->ev_before) ESSPT_CUDA(c, cudaEventRecord(c->ev_before, c->st));

@@ -87,7 +87,7 @@ struct SgdArgs {
   const int32_t* uoff;      // [n_users+1] entry offsets of minibatch b (relative)
   float* dR;                // item delta replicas (all zero between clocks)
   int32_t dR_ld;            // float4 per dR row (dR_stride4)
-  const int32_t* item_rep;  // see ItemMergeArgs; hot_item: [kHot] hot items of minibatch b, -1 if unused
+  const int32_t* item_rep;  // see MergeArgs; hot_item: [kHot] hot items of minibatch b, -1 if unused
   const int32_t* hot_item;
   float eta, lambda;
   int32_t cap;
@@ -97,7 +97,7 @@ struct SgdArgs {
   // chg[u] = last clock that changed user row u (written with every user row
   // that changes); an idle row whose slot already holds its current value is
   // not copied forward: clock > copy_all_until and clock - chg[u] >= nslots
-  // (unchanged over the whole ring).
+  // (unchanged over the whole ring).  chg_item likewise for item rows.
   int32_t* chg;
   int32_t clock, copy_all_until;
 };
@@ -128,32 +128,26 @@ struct StreamArgs {
   float* dL;                // heavy-user delta replicas (all zero between clocks)
 };
 
-// Merge of heavy user rows: x = user, y = first replica row, z = replicas, w = entries.
-struct HeavyMergeArgs {
+// The Clock() merge of the item rows, R^c_j = R^base_j + eta s_j sum of
+// replicas, and of the heavy users' rows.
+struct MergeArgs {
   float* ring;
   int64_t n_rows;
-  int32_t K, nslots, slot_base, slot_out;
-  const int4* heavy;
-  int64_t n_heavy;
-  float* dL;
-  float eta;
-  int32_t cap;
-  int32_t* chg;             // set chg[user] = clock (see SgdArgs)
-  int32_t clock;
-};
-
-// Clock() merge of the item rows: R^c_j = R^base_j + eta s_j sum of replicas.
-struct ItemMergeArgs {
-  float* ring;
-  int64_t n_rows;
-  int32_t K, n_users, n_items, slot_base, slot_out;
+  int32_t K, n_users, n_items, nslots, slot_base, slot_out;
   const int32_t* item_rep;  // [M+1] prefix of extra replicas: replica 0 of item j is row j of dR,
                             // replica r > 0 row M + item_rep[j] + r - 1
   float* dR;
   int32_t dR_ld;
   const int32_t* item_cnt;  // [M] entries per item in minibatch b
+  // Rows with several replicas: x = item or user (and its first replica row),
+  // y = second replica row, z = replicas; of a heavy user w = entries.
+  const int4 *popular, *heavy;
+  int64_t n_popular, n_heavy;
+  float* dL;
   float eta;
   int32_t cap;
+  int32_t *chg, *chg_item;  // see SgdArgs
+  int32_t clock, copy_all_until;
   int32_t do_schedule;      // also compute the next clock's read versions
   ScheduleArgs sched;
 };
@@ -229,11 +223,11 @@ struct SeqArgs {
   const int32_t* rec_j;     // item of each entry of minibatch b
   const float* rec_D;
   const int32_t* item_cnt;  // [n_items] entries per item in minibatch b (hot-row cap)
+  int32_t* chg_item;        // see SgdArgs
   float* mine;              // [P][n_items][K] each worker's item changes this clock (zero on entry)
 };
 cudaError_t launch_seq_clock(const SeqArgs& a, cudaStream_t st);
-cudaError_t launch_heavy_merge(const HeavyMergeArgs& a, cudaStream_t st);
-cudaError_t launch_item_merge(const ItemMergeArgs& a, cudaStream_t st);
+cudaError_t launch_clock_merge(const MergeArgs& a, cudaStream_t st);
 // Objective at one table version over the work lists of all F minibatches:
 // item_base and entry_base (device, [F+1]) hold each one's first item and entry.
 // out[0] = sum e^2 and out[out_stride] = penalised sum; by worker (P at most,
@@ -272,6 +266,8 @@ struct LayoutBuild {
   int64_t* mb_base;     // [F+1]
   int32_t* item_cnt;    // [F][n_items]
   int32_t* item_rep;    // [n_items+1]
+  int4* popular;        // [max_popular] items with extra replicas (see MergeArgs), in no order
+  uint32_t* n_popular;  // their number
   int4* chunk;          // [max_chunks] work items (see StreamArgs)
   int64_t* chunk_base;  // [F+1]
   int4* heavy;          // [max_heavy]
@@ -289,6 +285,7 @@ struct LayoutBuild {
 size_t layout_scratch_bytes(int64_t n_obs, int64_t n_users, int64_t n_items, int32_t F);
 int64_t layout_max_chunks(int64_t n_obs, int32_t F, int64_t n_users);
 int64_t layout_max_heavy(int64_t n_obs, int32_t F);
+int64_t layout_max_popular(int64_t n_obs);
 int64_t layout_max_item_reps(int64_t n_obs, int64_t n_items);
 int64_t layout_max_user_reps(int64_t n_obs);
 cudaError_t build_layout(LayoutBuild& b, cudaStream_t st);

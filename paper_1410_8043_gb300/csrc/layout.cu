@@ -204,6 +204,22 @@ __global__ void place_items_kernel(const int4* __restrict__ raw, const uint32_t*
   }
 }
 
+// The items with extra replicas.
+__global__ void popular_kernel(const int32_t* __restrict__ item_rep, int64_t n_items, int64_t max_popular,
+                               int4* __restrict__ popular, uint32_t* __restrict__ n_popular, uint32_t* status) {
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < n_items; j += stride) {
+    const int32_t e0 = item_rep[j], extra = item_rep[j + 1] - e0;
+    if (extra == 0) continue;
+    const uint32_t at = atomicAdd(n_popular, 1u);
+    if (at < max_popular) {
+      popular[at] = make_int4((int32_t)j, (int32_t)(n_items + e0), extra + 1, 0);
+    } else {  // cannot be: see layout_max_popular
+      atomicOr(status, kErrInput);
+    }
+  }
+}
+
 // The kHot items with the most entries of each minibatch (at least 2), most
 // popular first, ties by id; -1 for unused slots.  Host side, at setup.
 cudaError_t build_hot(const LayoutBuild& b, cudaStream_t st) {
@@ -310,6 +326,9 @@ int64_t layout_max_chunks(int64_t n_obs, int32_t F, int64_t n_users) {
   return 2 * n_obs / kChunk + F + 1 + std::min(n_obs, (int64_t)F * n_users);
 }
 
+// An item with extra replicas has more than kItemRep entries.
+int64_t layout_max_popular(int64_t n_obs) { return n_obs / (kItemRep + 1) + 1; }
+
 int64_t layout_max_heavy(int64_t n_obs, int32_t F) { return n_obs / (kHeavy + 1) + F + 1; }
 
 // Replica rows: one per item plus the extra ones, sum (reps - 1) with reps - 1 < 3 mx / (2 kItemRep).
@@ -369,6 +388,10 @@ cudaError_t build_layout(LayoutBuild& b, cudaStream_t st) {
   tb = p.cub_bytes;
   if ((e = cub::DeviceScan::ExclusiveSum(cub_tmp, tb, ireps, b.item_rep, (int)(b.n_items + 1), st)) != cudaSuccess)
     return e;
+  if ((e = cudaMemsetAsync(b.n_popular, 0, sizeof(uint32_t), st)) != cudaSuccess) return e;
+  popular_kernel<<<blocks_for(b.n_items), 256, 0, st>>>(b.item_rep, b.n_items, layout_max_popular(b.n_obs), b.popular,
+                                                       b.n_popular, b.status);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if (b.n_obs > 0 && (e = build_hot(b, st)) != cudaSuccess) return e;
   // The work list, then its order: by tile of users and length, ties in user
   // order (the sort is stable).  The sort buffers of the entries are free now.

@@ -5,8 +5,8 @@
 //                       the rows of users without entries, carried from
 //                       version c-1 to version c unless the ring already
 //                       holds them;
-//   heavy_merge_kernel  rows of the very active users (if any);
-//   item_merge_kernel   the Clock() merge of the item rows.
+//   clock_merge_kernel  the Clock() merge of the item rows and of the rows of
+//                       the very active users.
 // Item-row (and heavy-user) deltas are summed, unscaled, into zero-initialised
 // replica rows so that popular rows spread their fp32 reductions over many
 // L2 addresses; the merges apply eta, the hot-row scale and the sum of the
@@ -40,28 +40,6 @@ __device__ __noinline__ float capped_scale(int32_t cap, int32_t n) { return (flo
 
 __device__ __forceinline__ float4 f4_add(float4 a, float4 b) {
   return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
-}
-
-// Sum of n replica slices p[0], p[stride], ..., each cleared after reading;
-// eight independent loads in flight per lane.
-__device__ __forceinline__ float4 sum_and_clear(float4* p, int32_t n, int32_t stride) {
-  float4 acc = f4_zero();
-  int32_t r = 0;
-  for (; r + 8 <= n; r += 8) {
-    float4 x[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) x[k] = p[(int64_t)(r + k) * stride];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      p[(int64_t)(r + k) * stride] = f4_zero();
-      acc = f4_add(acc, x[k]);
-    }
-  }
-  for (; r < n; ++r) {
-    acc = f4_add(acc, p[(int64_t)r * stride]);
-    p[(int64_t)r * stride] = f4_zero();
-  }
-  return acc;
 }
 
 __device__ __forceinline__ void flush_loss(double* out, float v, int lane) {
@@ -578,80 +556,124 @@ __global__ void __launch_bounds__(256) row_refresh_kernel(RowRefreshArgs a) {
   }
 }
 
-// Heavy user rows: L^c = L^base + eta s sum of the user's replica rows (row u
-// of dL, then rows hv.y .. hv.y + hv.z - 2); the replicas are cleared for the
-// next clock.  One warp per heavy user.
-__global__ void __launch_bounds__(256) heavy_merge_kernel(HeavyMergeArgs a) {
-  const int lane = threadIdx.x & 31;
-  const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  const int32_t K4 = a.K >> 2;
-  const int64_t slot4 = a.n_rows * K4;
-  float4* ring4 = reinterpret_cast<float4*>(a.ring);
-  float4* dL4 = reinterpret_cast<float4*>(a.dL);
-  for (int64_t h = warp; h < a.n_heavy; h += nwarps) {
-    const int4 hv = a.heavy[h];
-    const float sc = a.eta * cap_scale(a.cap, hv.w);
-    for (int32_t q = lane; q < K4; q += 32) {
-      float4* p0 = dL4 + (int64_t)hv.x * K4 + q;
-      float4 acc = *p0;
-      *p0 = f4_zero();
-      acc = f4_add(acc, sum_and_clear(dL4 + (int64_t)hv.y * K4 + q, hv.z - 1, K4));
-      const float4 b = ring4[(int64_t)a.slot_base * slot4 + (int64_t)hv.x * K4 + q];
-      ring4[(int64_t)a.slot_out * slot4 + (int64_t)hv.x * K4 + q] = f4_axpy(sc, acc, b);
-    }
-    if (lane == 0) a.chg[hv.x] = a.clock;
-  }
-}
-
-// Clock() merge of the item rows (Sec. 2.1 additive updates, Sec. 4 server
-// clock): R^c_j = R^base_j + eta s_j sum of j's replica rows; replicas
-// cleared.  Each thread merges U (item, float4 slice) pairs.  Replica 0 of
-// item j is row j of dR, so the common single-replica item needs no index
-// load before its data loads: every load of a thread is issued at once.  With do_schedule the
-// first P threads also compute the next clock's read versions (the SGD
-// kernels of this clock, the only readers of v, have finished).
-template <int U>  // (item, slice) pairs per thread per round, the loads of all in flight
-__global__ void __launch_bounds__(256) item_merge_kernel(ItemMergeArgs a) {
+// The Clock() merge (Sec. 2.1 additive updates, Sec. 4 server clock):
+//   R^c_j = R^base_j + eta s_j (sum of j's replica rows of dR)
+// and, for the heavy users, L^c_i likewise from dL; replicas are cleared for
+// the next clock.  Warps take three kinds of task, the long ones first:
+//   an item with extra replicas or a heavy user: the row groups of the warp
+//     split its replica rows, each with all its loads of a pass in flight;
+//   kUnit other items: base row and replica row of each, read and written once;
+//     an item without entries is only copied forward, and not even that when
+//     the ring already holds it (as for idle users).
+// With do_schedule the first P threads also compute the next clock's read
+// versions (the SGD kernel of this clock, the only reader of v, has finished).
+// DRAM bounds the third kind: 1M items of 64 values move 1.0 GB.  One thread
+// per slice with the extra replicas in line, eight slices in flight at one
+// block per SM, took 353 us there and a launch for the heavy users 50 more.
+template <int G, int NV>
+__global__ void __launch_bounds__(256, 3) clock_merge_kernel(MergeArgs a) {
+  constexpr int kGpw = 32 / G;
+  constexpr int kBatch = NV >= 3 ? 1 : 4 / NV;  // items per group in flight
+  constexpr int kUnit = kGpw * kBatch;          // items per task, <= 32
+  constexpr int kRows = kBatch;                 // replica rows per group in flight
   const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t nth = (int64_t)gridDim.x * blockDim.x;
   if (a.do_schedule)
     for (int64_t p = tid; p < a.sched.P; p += nth) schedule_worker(a.sched, (int32_t)p);
+  const int lane = threadIdx.x & 31, glane = lane & (G - 1), grp = lane / G;
   const int32_t K4 = a.K >> 2;
-  const int64_t slot4 = a.n_rows * K4;
-  float4* ring4 = reinterpret_cast<float4*>(a.ring);
-  float4* dR4 = reinterpret_cast<float4*>(a.dR);
-  // n_items * K/4 < 2^31 (checked at load), so the (item, slice) split is a
-  // 32-bit division
-  const int64_t total = (int64_t)a.n_items * K4;
-  for (int64_t x0 = tid; x0 < total; x0 += U * nth) {
-    float4 first[U], base[U];
-    int32_t e0[U], e1[U], cnt[U];
-    int64_t row[U], dofs[U];
+  const bool last_on = glane + (NV - 1) * G < K4;
+  float4* ring4 = reinterpret_cast<float4*>(a.ring) + glane;
+  const float4* base4 = ring4 + (int64_t)a.slot_base * a.n_rows * K4;
+  float4* out4 = ring4 + (int64_t)a.slot_out * a.n_rows * K4;
+  const int64_t nwarps = nth >> 5, lists = a.n_popular + a.n_heavy;
+  int64_t task = tid >> 5;
+
+  for (; task < lists; task += nwarps) {
+    const bool item = task < a.n_popular;
+    const int4 d = __ldg(item ? a.popular + task : a.heavy + (task - a.n_popular));
+    float4* rows = reinterpret_cast<float4*>(item ? a.dR : a.dL) + glane;
+    const int64_t ld = item ? a.dR_ld : K4, row = item ? (int64_t)a.n_users + d.x : (int64_t)d.x;
+    const int32_t n = item ? __ldg(a.item_cnt + d.x) : d.w;
+    float4 acc[NV];
 #pragma unroll
-    for (int k = 0; k < U; ++k) {
-      const int64_t x = min(x0 + k * nth, total - 1);
-      const uint32_t j = (uint32_t)x / (uint32_t)K4;
-      const int32_t q = (int32_t)((uint32_t)x - j * (uint32_t)K4);
-      row[k] = ((int64_t)a.n_users + j) * K4 + q;
-      dofs[k] = (int64_t)j * a.dR_ld + q;
-      first[k] = dR4[dofs[k]];
-      base[k] = ring4[(int64_t)a.slot_base * slot4 + row[k]];
-      e0[k] = __ldg(a.item_rep + j);
-      e1[k] = __ldg(a.item_rep + j + 1);
-      cnt[k] = __ldg(a.item_cnt + j);
+    for (int k = 0; k < NV; ++k) acc[k] = f4_zero();
+    for (int32_t r0 = grp; r0 < d.z; r0 += kRows * kGpw) {
+      float4 x[kRows][NV];
+#pragma unroll
+      for (int u = 0; u < kRows; ++u) {
+        const int32_t r = r0 + u * kGpw;
+        const float4* p = rows + (r == 0 ? (int64_t)d.x : (int64_t)d.y + r - 1) * ld;
+#pragma unroll
+        for (int k = 0; k < NV; ++k) x[u][k] = r < d.z && (k < NV - 1 || last_on) ? p[k * G] : f4_zero();
+      }
+#pragma unroll
+      for (int u = 0; u < kRows; ++u) {
+        const int32_t r = r0 + u * kGpw;
+        float4* p = rows + (r == 0 ? (int64_t)d.x : (int64_t)d.y + r - 1) * ld;
+#pragma unroll
+        for (int k = 0; k < NV; ++k) {
+          acc[k] = f4_add(acc[k], x[u][k]);
+          if (r < d.z && (k < NV - 1 || last_on)) p[k * G] = f4_zero();
+        }
+      }
+    }
+    const float sc = a.eta * cap_scale(a.cap, n);
+#pragma unroll
+    for (int k = 0; k < NV; ++k) {
+#pragma unroll
+      for (int off = G; off < 32; off <<= 1) {
+        acc[k].x += __shfl_xor_sync(0xffffffffu, acc[k].x, off);
+        acc[k].y += __shfl_xor_sync(0xffffffffu, acc[k].y, off);
+        acc[k].z += __shfl_xor_sync(0xffffffffu, acc[k].z, off);
+        acc[k].w += __shfl_xor_sync(0xffffffffu, acc[k].w, off);
+      }
+      if (grp == 0 && (k < NV - 1 || last_on)) out4[row * K4 + k * G] = f4_axpy(sc, acc[k], base4[row * K4 + k * G]);
+    }
+    if (lane == 0 && n > 0) (item ? a.chg_item : a.chg)[d.x] = a.clock;
+  }
+
+  float4* dR4 = reinterpret_cast<float4*>(a.dR) + glane;
+  const bool may_skip = a.clock > a.copy_all_until;
+  const int64_t units = ((int64_t)a.n_items + kUnit - 1) / kUnit;
+  // What to do with this lane's item of a unit: nothing (it has extra replicas,
+  // or the ring holds its row), copy it (-1: no entries), or merge n entries.
+  auto look = [&](int64_t unit) -> int32_t {
+    const int64_t j = unit * kUnit + lane;
+    if (lane >= kUnit || j >= a.n_items || __ldg(a.item_rep + j + 1) > __ldg(a.item_rep + j)) return 0;
+    const int32_t n = __ldg(a.item_cnt + j);
+    if (n > 0) return n;
+    return may_skip && a.clock - a.chg_item[j] >= a.nslots ? 0 : -1;
+  };
+  int64_t unit = task - lists;
+  int32_t todo = unit < units ? look(unit) : 0;
+  for (; unit < units; unit += nwarps) {
+    const int32_t now = todo;
+    todo = unit + nwarps < units ? look(unit + nwarps) : 0;
+    if (now > 0) a.chg_item[unit * kUnit + lane] = a.clock;
+    float4 x[kBatch][NV], b[kBatch][NV];
+#pragma unroll
+    for (int u = 0; u < kBatch; ++u) {
+      const int32_t n = __shfl_sync(0xffffffffu, now, u * kGpw + grp);
+      const int64_t j = unit * kUnit + u * kGpw + grp;
+#pragma unroll
+      for (int k = 0; k < NV; ++k) {
+        const bool in = k < NV - 1 || last_on;
+        x[u][k] = n > 0 && in ? dR4[j * a.dR_ld + k * G] : f4_zero();
+        b[u][k] = n != 0 && in ? base4[(a.n_users + j) * K4 + k * G] : f4_zero();
+      }
     }
 #pragma unroll
-    for (int k = 0; k < U; ++k) {
-      if (x0 + k * nth >= total) break;
-      dR4[dofs[k]] = f4_zero();
-      float4 acc = first[k];
-      if (e1[k] > e0[k]) {
-        const int32_t q = (int32_t)(dofs[k] % a.dR_ld);
-        acc = f4_add(acc, sum_and_clear(dR4 + ((int64_t)a.n_items + e0[k]) * a.dR_ld + q, e1[k] - e0[k], a.dR_ld));
+    for (int u = 0; u < kBatch; ++u) {
+      const int32_t n = __shfl_sync(0xffffffffu, now, u * kGpw + grp);
+      const int64_t j = unit * kUnit + u * kGpw + grp;
+      const float sc = a.eta * cap_scale(a.cap, n);
+#pragma unroll
+      for (int k = 0; k < NV; ++k) {
+        const bool in = k < NV - 1 || last_on;
+        if (n > 0 && in) dR4[j * a.dR_ld + k * G] = f4_zero();
+        if (n != 0 && in) out4[(a.n_users + j) * K4 + k * G] = f4_axpy(sc, x[u][k], b[u][k]);
       }
-      const float sc = a.eta * cap_scale(a.cap, cnt[k]);
-      ring4[(int64_t)a.slot_out * slot4 + row[k]] = f4_axpy(sc, acc, base[k]);
     }
   }
 }
@@ -782,21 +804,15 @@ cudaError_t launch_stream_refill(const int4* items, const uint32_t* place, int64
   return cudaGetLastError();
 }
 
-cudaError_t launch_heavy_merge(const HeavyMergeArgs& a, cudaStream_t st) {
-  if (a.n_heavy <= 0) return cudaSuccess;
-  heavy_merge_kernel<<<grid_for(a.n_heavy, 8, 8), 256, 0, st>>>(a);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_item_merge(const ItemMergeArgs& a, cudaStream_t st) {
-  const int64_t work = std::max<int64_t>((int64_t)a.n_items * (a.K >> 2), a.do_schedule ? a.sched.P : 0);
-  if (work <= 0) return cudaSuccess;
-  // Every thread's loads are independent, so the whole merge is one set of
-  // in-flight requests.  Eight (item, slice) pairs per thread: more loads in
-  // flight per thread beat more threads with one each (0.019 against
-  // 0.029 ms per clock on mid; 74 against 207 us on a 200k-item table).
-  item_merge_kernel<8><<<(unsigned)std::min<int64_t>((work + 2047) / 2048, (int64_t)1 << 30), 256, 0, st>>>(a);
-  return cudaGetLastError();
+cudaError_t launch_clock_merge(const MergeArgs& a, cudaStream_t st) {
+  return dispatch_stream(a.K, [&](auto s) {
+    using S = decltype(s);
+    const int64_t unit = S::GPW * (S::NV >= 3 ? 1 : 4 / S::NV);
+    const int64_t warps = a.n_popular + a.n_heavy + (a.n_items + unit - 1) / unit;
+    const int64_t most = std::max<int64_t>(warps, a.do_schedule ? (a.sched.P + 31) / 32 : 0);
+    clock_merge_kernel<S::G, S::NV><<<grid_for(most, 8, 3), 256, 0, st>>>(a);
+    return cudaGetLastError();
+  });
 }
 
 }  // namespace esspt

@@ -267,7 +267,9 @@ __global__ void __launch_bounds__(256) seq_item_merge_kernel(SeqArgs s) {
       const float4 m = __ldg(mine + (int64_t)p * n + x);
       sum = make_float4(sum.x + m.x, sum.y + m.y, sum.z + m.z, sum.w + m.w);
     }
-    const float sc = seq_cap_scale(a.cap, __ldg(s.item_cnt + x / K4));
+    const int32_t entries = __ldg(s.item_cnt + x / K4);
+    if (entries > 0 && x % K4 == 0) s.chg_item[x / K4] = a.clock;
+    const float sc = seq_cap_scale(a.cap, entries);
     const float4 b = base[x];
     out[x] = make_float4(b.x + sc * sum.x, b.y + sc * sum.y, b.z + sc * sum.z, b.w + sc * sum.w);
   }
