@@ -19,12 +19,11 @@ namespace {
 // 400 bytes per entry out of L2).  One warp per entry, which it replaces, read
 // both rows and reduced three sums per entry: 11.0 ms on 20M entries, K = 100.
 //
-// The squares of U entries are added in fp32, their sums with the rounding error
-// kept beside them (two-sum, Knuth, TAOCP vol. 2, 4.2.2): as good as adding each
-// entry in fp64, whose units are few, since an entry's fp32 residual carries
-// more error than U - 1 additions.  On the 20M entries, K = 100: 0.75 ms with
-// plain fp32 sums per item (4.5e-9 off by worker where this is 5e-10), 1.09 ms
-// with a two-sum per entry.
+// The squares of up to eight entries are added in fp32, their sums with the
+// rounding error kept beside them (two-sum, Knuth, TAOCP vol. 2, 4.2.2) and only
+// at the end in fp64, whose units are few: an fp64 sum per item takes 1.05 ms
+// there.  An entry's fp32 residual carries more error than the eight additions.
+constexpr float kHuge = 1e36f;
 struct Sum2 {  // two packed fp32 sums and what they lost
   u64 sum = 0ull, lost = 0ull;
   __device__ __forceinline__ void add(u64 x, u64 minus1) {
@@ -33,17 +32,19 @@ struct Sum2 {  // two packed fp32 sums and what they lost
     sum = s;
     lost = add2(lost, d);
   }
-  __device__ __forceinline__ double total() const {
+  // The second sum, and the first (an infinite or NaN sum has no rounding error).
+  __device__ __forceinline__ double total(double& first) const {
     float a, b, c, d;
     unpack2(sum, a, b);
     unpack2(lost, c, d);
-    return ((double)a + (double)c) + ((double)b + (double)d);
+    first = isfinite(a) ? (double)a + (double)c : (double)a;
+    return isfinite(b) ? (double)b + (double)d : (double)b;
   }
 };
 
 template <int G, int NV, bool BY_WORKER>
 __global__ void __launch_bounds__(256) objective_kernel(ObjectiveArgs a) {
-  constexpr int kGpw = 32 / G, U = NV == 1 ? 8 : NV == 2 ? 4 : 2;
+  constexpr int kGpw = 32 / G, U = NV >= 3 ? 2 : NV == 2 || G == 4 ? 4 : 8;
   extern __shared__ double sums[];  // BY_WORKER: sum e^2 at [p], penalised sum at [P + p]
   if (BY_WORKER) {
     for (int k = threadIdx.x; k < 2 * a.P; k += blockDim.x) sums[k] = 0.0;
@@ -59,21 +60,25 @@ __global__ void __launch_bounds__(256) objective_kernel(ObjectiveArgs a) {
   const float* rec_D = a.rec_D + e_base;
   const int64_t step = (((int64_t)gridDim.x * blockDim.x) >> 5) * kGpw;
   const u64 minus1 = pack2(-1.f, -1.f);
-  double s1 = 0.0, s2 = 0.0;
+  // e^2 and what the rows' squares add up to; by worker, of the item at hand.
+  Sum2 sums2;  // (e^2, this lane's part of the rows' squares)
+  double huge = 0.0;
   for (int64_t x0 = __ldg(a.item_base + blockIdx.y) + (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * kGpw;
        x0 < x_end; x0 += step) {
     const int4 it = x0 + grp < x_end ? __ldg(a.items + x0 + grp) : make_int4(0, 0, 0, 0);
     const int32_t n = it.w >> 16, most = __reduce_max_sync(0xffffffffu, n);
     f2x2 L[NV];
-    u64 l2 = 0ull;  // packed partial sums of |L|^2
-    Sum2 r2, sq;    // of the entries' |R|^2; of e^2
+    if (BY_WORKER) {
+      sums2 = Sum2{};
+      huge = 0.0;
+    }
 #pragma unroll
     for (int k = 0; k < NV; ++k) {
       L[k] = f2x2{0ull, 0ull};
       ldg_f2x2_if(L[k], L4 + (int64_t)it.x * K4 + k * G, n > 0 && (k < NV - 1 || last_on));
-      l2 = fma2(L[k].lo, L[k].lo, l2);
-      l2 = fma2(L[k].hi, L[k].hi, l2);
     }
+    float se = 0.f;
+    u64 sr = 0ull;
     for (int32_t t = 0; t < most; t += U) {
       f2x2 R[U][NV];
       float d[U];
@@ -107,30 +112,43 @@ __global__ void __launch_bounds__(256) objective_kernel(ObjectiveArgs a) {
       for (int off = G / 2; off > 0; off >>= 1)
 #pragma unroll
         for (int u = 0; u < U; ++u) dot[u] += __shfl_xor_sync(0xffffffffu, dot[u], off);
-      float se = 0.f;
-      u64 sr = 0ull;
 #pragma unroll
       for (int u = 0; u < U; ++u)
         if (t + u < n) {
           const float e = d[u] - dot[u];
-          se = fmaf(e, e, se);
+          if (e * e < kHuge) {
+            se = fmaf(e, e, se);
+          } else {  // (a diverging run, NaN among it) beyond what fp32 sums hold
+            huge += (double)e * (double)e;
+          }
           sr = add2(sr, rr[u]);
         }
-      sq.add(pack2(se, 0.f), minus1);
-      r2.add(sr, minus1);
+      if ((t & (8 - U)) == 8 - U || t + U >= most) {
+        sums2.add(pack2(se, sum2(sr)), minus1);
+        se = 0.f;
+        sr = 0ull;
+      }
+    }
+    if (n > 0) {
+      u64 l2 = 0ull;
+#pragma unroll
+      for (int k = 0; k < NV; ++k) {
+        l2 = fma2(L[k].lo, L[k].lo, l2);
+        l2 = fma2(L[k].hi, L[k].hi, l2);
+      }
+      sums2.add(pack2(0.f, (float)n * sum2(l2)), minus1);
     }
     if (BY_WORKER) {
-      double norm = n > 0 ? (double)n * (double)sum2(l2) + r2.total() : 0.0;
+      double e2;
+      float norm = (float)sums2.total(e2);
 #pragma unroll
       for (int off = G / 2; off > 0; off >>= 1) norm += __shfl_xor_sync(0xffffffffu, norm, off);
       if (glane == 0 && n > 0) {
         const int p = it.w & 0xffff;
-        atomicAdd(&sums[p], sq.total());
-        atomicAdd(&sums[a.P + p], sq.total() + (double)a.lambda * norm);
+        e2 += huge;
+        atomicAdd(&sums[p], e2);
+        atomicAdd(&sums[a.P + p], e2 + (double)a.lambda * (double)norm);
       }
-    } else if (n > 0) {
-      s1 += glane == 0 ? sq.total() : 0.0;
-      s2 += (double)n * (double)sum2(l2) + r2.total();
     }
   }
   if (BY_WORKER) {
@@ -140,6 +158,8 @@ __global__ void __launch_bounds__(256) objective_kernel(ObjectiveArgs a) {
       if (sums[a.P + k] != 0.0) atomicAdd(a.out + a.out_stride + k, sums[a.P + k]);
     }
   } else {
+    double s1, s2 = sums2.total(s1);
+    s1 = glane == 0 ? s1 + huge : 0.0;
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) {
       s1 += __shfl_xor_sync(0xffffffffu, s1, off);
