@@ -744,6 +744,7 @@ esspt_status esspt_mf_sgd_clock(esspt_ctx* c, float eta, float lambda, int32_t c
   m.chg_item = c->chg_item;
   m.clock = c->clock;
   m.copy_all_until = c->copy_all_until;
+  m.chained = stream_is_small(c->K, sa.n_warps, c->n_users);
   // SSP and ESSP schedules need only the previous read versions, so the merge
   // computes them; VAP needs version c complete, so it runs after the merge.
   m.do_schedule = c->cfg.model == ESSPT_SSP_LAZY || c->cfg.model == ESSPT_ESSP_EAGER || c->cfg.model == ESSPT_SSP_ROW;

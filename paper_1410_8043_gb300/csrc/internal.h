@@ -149,6 +149,7 @@ struct MergeArgs {
   int32_t *chg, *chg_item;  // see SgdArgs
   int32_t clock, copy_all_until;
   int32_t do_schedule;      // also compute the next clock's read versions
+  int32_t chained;          // start beside the kernel before it
   ScheduleArgs sched;
 };
 
@@ -173,6 +174,8 @@ cudaError_t launch_inc(float* slot, int64_t n_rows, int32_t K, const int32_t* id
 // device, and the shape of its stream.
 cudaError_t launch_sgd_stream(const StreamArgs& a, cudaStream_t st);
 int64_t stream_max_warps(int32_t K);
+// Whether a clock of n_warps warps and n_users users is one block per SM at most.
+bool stream_is_small(int32_t K, int64_t n_warps, int64_t n_users);
 StreamGeometry stream_geometry(int32_t K);
 // Build of a minibatch's stream (setup): the split of its n_items work items
 // over n_warps warps (pre: see LayoutBuild), the steps of the warps (their sum

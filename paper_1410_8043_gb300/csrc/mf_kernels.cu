@@ -105,6 +105,7 @@ __global__ void __launch_bounds__(kStreamWarps * 32, MINB) sgd_stream_kernel(Str
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   float loss = 0.f;
+  await_previous_kernel();
 
   // Half of the warps copy idle rows first, the others last: the copy's DRAM
   // traffic runs beside the other warps' arithmetic.
@@ -578,6 +579,7 @@ __global__ void __launch_bounds__(256, 3) clock_merge_kernel(MergeArgs a) {
   constexpr int kRows = kBatch;                 // replica rows per group in flight
   const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t nth = (int64_t)gridDim.x * blockDim.x;
+  await_previous_kernel();
   if (a.do_schedule)
     for (int64_t p = tid; p < a.sched.P; p += nth) schedule_worker(a.sched, (int32_t)p);
   const int lane = threadIdx.x & 31, glane = lane & (G - 1), grp = lane / G;
@@ -696,6 +698,26 @@ int grid_for(int64_t work_items, int64_t per_block, int max_per_sm) {
   return (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)sm_count() * max_per_sm));
 }
 
+// The SGD kernel starts while the kernel before it, in a run of clocks the
+// merge, drains (see await_previous_kernel); the merge only on clocks of at most
+// one block per SM.  2k x 1k, K = 16: 14.0 us per clock with neither, 10.6 with
+// the first, 8.7 with both.  Larger clocks lose with both (480k x 18k, K = 100:
+// 445 us, 520 with both; 10M x 1M, K = 64: 2480, 2700).
+template <typename Args>
+cudaError_t launch_chained(void (*kernel)(Args), int blocks, int threads, cudaStream_t st, const Args& args,
+                           bool chained) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = chained ? 1 : 0;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)blocks);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.stream = st;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, args);
+}
+
 // Row-group shape for K: G lanes per row (a power of two) and NV float4 slices
 // per lane, G (NV - 1) < K/4 <= G NV; E entries per step and PF steps of gathers
 // ahead (see the kernel); the blocks per SM it is compiled for.  Eight lanes
@@ -724,7 +746,18 @@ auto dispatch_stream(int32_t K, F&& f) {
   return f(StreamShape<32, 4, 1, 1, 4>{});
 }
 
+// Blocks of the stream kernel: warps for the work list, and one per 32 users
+// for the forward copy, up to one resident wave.
+template <typename S>
+int stream_blocks(int64_t n_warps, int64_t n_users) {
+  return grid_for(std::max<int64_t>(n_warps, (n_users + 31) / 32), kStreamWarps, S::MINB);
+}
+
 }  // namespace
+
+bool stream_is_small(int32_t K, int64_t n_warps, int64_t n_users) {
+  return dispatch_stream(K, [&](auto s) { return stream_blocks<decltype(s)>(n_warps, n_users) <= sm_count(); });
+}
 
 int64_t stream_max_warps(int32_t K) {
   return dispatch_stream(K, [](auto s) { return (int64_t)sm_count() * s.MINB * kStreamWarps; });
@@ -752,11 +785,7 @@ cudaError_t launch_sgd_stream(const StreamArgs& c, cudaStream_t st) {
       if (e != cudaSuccess) return e;
       configured = true;
     }
-    // Warps for the work list, and one per 32 users for the forward copy, up
-    // to one resident wave.
-    const int64_t warps = std::max<int64_t>(c.n_warps, (c.a.n_users + 31) / 32);
-    kernel<<<grid_for(warps, kStreamWarps, S::MINB), kStreamWarps * 32, 0, st>>>(c);
-    return cudaGetLastError();
+    return launch_chained(kernel, stream_blocks<S>(c.n_warps, c.a.n_users), kStreamWarps * 32, st, c, true);
   });
 }
 
@@ -810,8 +839,7 @@ cudaError_t launch_clock_merge(const MergeArgs& a, cudaStream_t st) {
     const int64_t unit = S::GPW * (S::NV >= 3 ? 1 : 4 / S::NV);
     const int64_t warps = a.n_popular + a.n_heavy + (a.n_items + unit - 1) / unit;
     const int64_t most = std::max<int64_t>(warps, a.do_schedule ? (a.sched.P + 31) / 32 : 0);
-    clock_merge_kernel<S::G, S::NV><<<grid_for(most, 8, 3), 256, 0, st>>>(a);
-    return cudaGetLastError();
+    return launch_chained(clock_merge_kernel<S::G, S::NV>, grid_for(most, 8, 3), 256, st, a, a.chained != 0);
   });
 }
 

@@ -136,6 +136,15 @@ __device__ __forceinline__ void red_add_f2x2_if(float4* p, u64 lo, u64 hi, bool 
                : "memory");
 }
 
+// Programmatic dependent launch: a kernel launched with it may start while the
+// kernel before it in the stream still runs; it waits here, before its first
+// access to global memory, until that one (and so all before it) has finished
+// and its writes are visible.  Then it lets the next such kernel start.
+__device__ __forceinline__ void await_previous_kernel() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // SplitMix64 (Steele, Lea and Flood, OOPSLA 2014): output n of the sequence
 // whose state starts at s0 is mix64(s0 + n * 0x9E3779B97F4A7C15).
 __host__ __device__ __forceinline__ uint64_t mix64(uint64_t z) {
