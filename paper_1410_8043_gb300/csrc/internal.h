@@ -247,6 +247,7 @@ struct ObjectiveArgs {
   float lambda;
   double* out;
   int64_t out_stride;
+  int32_t parts;  // (set by the launch) parts that an item is taken in
 };
 cudaError_t launch_objective(const ObjectiveArgs& a, cudaStream_t st);
 cudaError_t launch_worker_objective(const ObjectiveArgs& a, cudaStream_t st);

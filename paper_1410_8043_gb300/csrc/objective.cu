@@ -23,7 +23,10 @@ namespace {
 // rounding error kept beside them (two-sum, Knuth, TAOCP vol. 2, 4.2.2) and only
 // at the end in fp64, whose units are few: an fp64 sum per item takes 1.05 ms
 // there.  An entry's fp32 residual carries more error than the eight additions.
+// By worker, where few entries may share a sum, every entry's exact square is
+// added so.
 constexpr float kHuge = 1e36f;
+constexpr int32_t kPart = 8;  // entries of a part of an item
 struct Sum2 {  // two packed fp32 sums and what they lost
   u64 sum = 0ull, lost = 0ull;
   __device__ __forceinline__ void add(u64 x, u64 minus1) {
@@ -58,15 +61,25 @@ __global__ void __launch_bounds__(256) objective_kernel(ObjectiveArgs a) {
   const int64_t x_end = __ldg(a.item_base + blockIdx.y + 1), e_base = __ldg(a.entry_base + blockIdx.y);
   const int32_t* rec_j = a.rec_j + e_base;
   const float* rec_D = a.rec_D + e_base;
-  const int64_t step = (((int64_t)gridDim.x * blockDim.x) >> 5) * kGpw;
+  const uint32_t step = (gridDim.x * blockDim.x) >> 5;
   const u64 minus1 = pack2(-1.f, -1.f);
   // e^2 and what the rows' squares add up to; by worker, of the item at hand.
   Sum2 sums2;  // (e^2, this lane's part of the rows' squares)
   double huge = 0.0;
-  for (int64_t x0 = __ldg(a.item_base + blockIdx.y) + (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * kGpw;
-       x0 < x_end; x0 += step) {
-    const int4 it = x0 + grp < x_end ? __ldg(a.items + x0 + grp) : make_int4(0, 0, 0, 0);
-    const int32_t n = it.w >> 16, most = __reduce_max_sync(0xffffffffu, n);
+  // Units of kGpw items; with a.parts > 1, part by part.
+  const int64_t x_first = __ldg(a.item_base + blockIdx.y);
+  const uint32_t units = (uint32_t)((x_end - x_first + kGpw - 1) / kGpw);
+  for (uint32_t v = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; v < units * a.parts; v += step) {
+    const uint32_t part = a.parts > 1 ? v / units : 0;
+    const int64_t x0 = x_first + (int64_t)(v - part * units) * kGpw;
+    int4 it = x0 + grp < x_end ? __ldg(a.items + x0 + grp) : make_int4(0, 0, 0, 0);
+    int32_t n = it.w >> 16;
+    if (a.parts > 1) {
+      it.y += part * kPart;
+      n = min(max(n - (int32_t)part * kPart, 0), kPart);
+    }
+    const int32_t most = __reduce_max_sync(0xffffffffu, n);
+    if (most == 0) continue;
     f2x2 L[NV];
     if (BY_WORKER) {
       sums2 = Sum2{};
@@ -116,6 +129,12 @@ __global__ void __launch_bounds__(256) objective_kernel(ObjectiveArgs a) {
       for (int u = 0; u < U; ++u)
         if (t + u < n) {
           const float e = d[u] - dot[u];
+          if (BY_WORKER && e * e < kHuge) {
+            const float high = e * e;
+            sums2.add(pack2(high, sum2(rr[u])), minus1);
+            sums2.lost = add2(sums2.lost, pack2(fmaf(e, e, -high), 0.f));
+            continue;
+          }
           if (e * e < kHuge) {
             se = fmaf(e, e, se);
           } else {  // (a diverging run, NaN among it) beyond what fp32 sums hold
@@ -184,19 +203,22 @@ __global__ void __launch_bounds__(256) objective_kernel(ObjectiveArgs a) {
 }
 
 template <bool BY_WORKER>
-cudaError_t run(const ObjectiveArgs& a, cudaStream_t st) {
+cudaError_t run(ObjectiveArgs a, cudaStream_t st) {
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
   auto go = [&](auto g, auto nv) {
-    constexpr int G = decltype(g)::value, NV = decltype(nv)::value;
+    constexpr int G = decltype(g)::value, NV = decltype(nv)::value, kGpw = 32 / G;
     const size_t smem = BY_WORKER ? 2 * sizeof(double) * (size_t)a.P : 0;
-    int dev = 0, sms = 0, per_sm = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess)
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, objective_kernel<G, NV, BY_WORKER>, 256, smem);
-    if (e != cudaSuccess) return e;
-    // Two waves of blocks over the minibatches, no more than their items need.
-    const int64_t need = (a.n_items / a.F + 8 * (32 / G)) / (8 * (32 / G));
-    const int64_t x = std::max<int64_t>(1, std::min<int64_t>(need, 2ll * sms * per_sm / a.F));
+    // About two waves of blocks (four per SM) over the minibatches, no more than
+    // their units need.  With fewer items than the GPU holds groups, an item is
+    // taken in parts of kPart entries, so that a call lasts no longer than the
+    // gathers of one part (20k entries, K = 224: 77 us whole).
+    const int64_t resident = 4ll * sms * 8;
+    a.parts = a.n_items < resident * kGpw ? (kHeavy + kPart - 1) / kPart : 1;
+    const int64_t need = (a.parts * (a.n_items / a.F + kGpw) / kGpw + 7) / 8;
+    const int64_t x = std::max<int64_t>(1, std::min<int64_t>(need, resident / 4 / a.F));
     objective_kernel<G, NV, BY_WORKER><<<dim3((unsigned)x, (unsigned)a.F), 256, smem, st>>>(a);
     return cudaGetLastError();
   };
