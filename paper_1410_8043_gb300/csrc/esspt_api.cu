@@ -416,8 +416,9 @@ esspt_status esspt_get(esspt_ctx* c, int32_t worker, const int32_t* d_row_ids, i
   if ((s = need_schedule(c)) != ESSPT_OK) return s;
   if (worker < 0 || worker >= c->P) return fail(c, ESSPT_EINVAL, "worker out of range");
   if (n < 0 || (n > 0 && (!d_row_ids || !d_out))) return fail(c, ESSPT_EINVAL, "bad row list");
-  int32_t* vmin = reinterpret_cast<int32_t*>(c->status) + kGetMinWord;
-  if (c->rowver) ESSPT_CUDA(c, cudaMemsetAsync(vmin, 0x7f, sizeof(int32_t), c->st));
+  // the oldest row version, where a row-granular GET's caller wants it
+  int32_t* vmin = c->rowver && h_version_out ? reinterpret_cast<int32_t*>(c->status) + kGetMinWord : nullptr;
+  if (vmin) ESSPT_CUDA(c, cudaMemsetAsync(vmin, 0x7f, sizeof(int32_t), c->st));
   ESSPT_CUDA(c, launch_get(c->ring, c->n_rows, c->K, c->nslots, c->v, worker, d_row_ids, n, d_out, c->status,
                            c->rowver, c->clock, c->s, vmin, c->st));
   if (h_version_out) {

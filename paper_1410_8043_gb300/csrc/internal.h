@@ -164,7 +164,7 @@ cudaError_t launch_vap(const float* ring, int64_t slot_floats, int32_t nslots, i
 cudaError_t launch_copy_rows(float* dst, const float* src, int64_t n_floats, cudaStream_t st);
 // GET; with rowver non-null (row-granular SSP at clock c) each row is read at
 // the worker's cached version, refreshed to c-1 first where it is missing or
-// older than c-1-s, and *vmin receives the oldest version read.
+// older than c-1-s, and *vmin (if non-null) receives the oldest version read.
 cudaError_t launch_get(const float* ring, int64_t n_rows, int32_t K, int32_t nslots, const int32_t* v,
                        int32_t worker, const int32_t* ids, int64_t n, float* out, uint32_t* status,
                        int32_t* rowver, int32_t c, int32_t s, int32_t* vmin, cudaStream_t st);

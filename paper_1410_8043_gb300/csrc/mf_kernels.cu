@@ -14,6 +14,7 @@
 #include <algorithm>
 #include <type_traits>
 
+#include "chained.cuh"
 #include "copy_idle.cuh"
 #include "internal.h"
 #include "ptx.cuh"
@@ -698,26 +699,6 @@ int grid_for(int64_t work_items, int64_t per_block, int max_per_sm) {
   return (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)sm_count() * max_per_sm));
 }
 
-// The SGD kernel starts while the kernel before it, in a run of clocks the
-// merge, drains (see await_previous_kernel); the merge only on clocks of at most
-// one block per SM.  2k x 1k, K = 16: 14.0 us per clock with neither, 10.6 with
-// the first, 8.7 with both.  Larger clocks lose with both (480k x 18k, K = 100:
-// 445 us, 520 with both; 10M x 1M, K = 64: 2480, 2700).
-template <typename Args>
-cudaError_t launch_chained(void (*kernel)(Args), int blocks, int threads, cudaStream_t st, const Args& args,
-                           bool chained) {
-  cudaLaunchAttribute at{};
-  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at.val.programmaticStreamSerializationAllowed = chained ? 1 : 0;
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)blocks);
-  cfg.blockDim = dim3((unsigned)threads);
-  cfg.stream = st;
-  cfg.attrs = &at;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, args);
-}
-
 // Row-group shape for K: G lanes per row (a power of two) and NV float4 slices
 // per lane, G (NV - 1) < K/4 <= G NV; E entries per step and PF steps of gathers
 // ahead (see the kernel); the blocks per SM it is compiled for.  Eight lanes
@@ -785,7 +766,12 @@ cudaError_t launch_sgd_stream(const StreamArgs& c, cudaStream_t st) {
       if (e != cudaSuccess) return e;
       configured = true;
     }
-    return launch_chained(kernel, stream_blocks<S>(c.n_warps, c.a.n_users), kStreamWarps * 32, st, c, true);
+    // The SGD kernel starts while the kernel before it, in a run of clocks the
+    // merge, drains; the merge only on clocks of at most one block per SM.
+    // 2k x 1k, K = 16: 14.0 us per clock with neither, 10.6 with the first, 8.7
+    // with both.  Larger clocks lose with both (480k x 18k, K = 100: 445 us, 520
+    // with both; 10M x 1M, K = 64: 2480, 2700).
+    return launch_chained(kernel, stream_blocks<S>(c.n_warps, c.a.n_users), kStreamWarps * 32, st, true, c);
   });
 }
 
@@ -839,7 +825,7 @@ cudaError_t launch_clock_merge(const MergeArgs& a, cudaStream_t st) {
     const int64_t unit = S::GPW * (S::NV >= 3 ? 1 : 4 / S::NV);
     const int64_t warps = a.n_popular + a.n_heavy + (a.n_items + unit - 1) / unit;
     const int64_t most = std::max<int64_t>(warps, a.do_schedule ? (a.sched.P + 31) / 32 : 0);
-    return launch_chained(clock_merge_kernel<S::G, S::NV>, grid_for(most, 8, 3), 256, st, a, a.chained != 0);
+    return launch_chained(clock_merge_kernel<S::G, S::NV>, grid_for(most, 8, 3), 256, st, a.chained != 0, a);
   });
 }
 

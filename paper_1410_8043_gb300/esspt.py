@@ -125,8 +125,10 @@ class Table:
                  device=None, stream=None):
         if not torch.cuda.is_available():
             raise RuntimeError("esspt needs a CUDA device")
-        L = lib()
+        L = self._lib = lib()
         self.device = torch.device(device if device is not None else "cuda")
+        # as the tensors on it name it
+        self._on = self.device if self.device.index is not None else torch.device("cuda", torch.cuda.current_device())
         self.stream = stream if stream is not None else torch.cuda.current_stream(self.device)
         self.cfg = Config(n_rows, K, P, s, MODELS[model], int(phased), essp_max_delay, essp_p,
                           seed & 0xFFFFFFFFFFFFFFFF, ctypes.c_void_p(self.stream.cuda_stream), vap_v0)
@@ -144,6 +146,11 @@ class Table:
         self.n_users = None
 
     # -- plumbing -----------------------------------------------------------
+    def _dev(self, x, dtype) -> torch.Tensor:
+        if isinstance(x, torch.Tensor) and x.dtype is dtype and x.device == self._on and x.is_contiguous():
+            return x  # the usual call: nothing to convert
+        return _dev_tensor(x, dtype, self.device)
+
     def _check(self, st: int) -> None:
         if st != OK:
             raise EssptError(st, lib().esspt_last_error(self._h).decode())
@@ -175,22 +182,30 @@ class Table:
 
     def get(self, worker: int, row_ids, out=None, want_version: bool = False):
         """esspt_get: rows of `worker`'s read version; returns (rows, version or None)."""
-        ids = _dev_tensor(row_ids, torch.int32, self.device)
+        ids = self._dev(row_ids, torch.int32)
         if out is None:
             out = torch.empty((ids.numel(), self.K), dtype=torch.float32, device=self.device)
-        ver = ctypes.c_int32(-1)
-        self._check(lib().esspt_get(self._h, worker, ids.data_ptr(), ids.numel(), out.data_ptr(),
-                                    ctypes.byref(ver) if want_version else None))
         self._keep_ids = ids
-        return out, (ver.value if want_version else None)
+        if not want_version:
+            st = self._lib.esspt_get(self._h, worker, ids.data_ptr(), ids.numel(), out.data_ptr(), None)
+            if st != OK:
+                self._check(st)
+            return out, None
+        ver = ctypes.c_int32(-1)
+        self._check(self._lib.esspt_get(self._h, worker, ids.data_ptr(), ids.numel(), out.data_ptr(),
+                                        ctypes.byref(ver)))
+        return out, ver.value
 
     def inc(self, worker: int, row_ids, deltas) -> None:
         """esspt_inc: additive updates into the version being written."""
-        ids = _dev_tensor(row_ids, torch.int32, self.device)
-        d = _dev_tensor(deltas, torch.float32, self.device)
-        assert d.numel() == ids.numel() * self.K
-        self._check(lib().esspt_inc(self._h, worker, ids.data_ptr(), d.data_ptr(), ids.numel()))
+        ids = self._dev(row_ids, torch.int32)
+        d = self._dev(deltas, torch.float32)
+        n = ids.numel()
+        assert d.numel() == n * self.K
         self._keep_inc = (ids, d)
+        st = self._lib.esspt_inc(self._h, worker, ids.data_ptr(), d.data_ptr(), n)
+        if st != OK:
+            self._check(st)
 
     def clock(self) -> None:
         """esspt_clock: all workers tick."""
