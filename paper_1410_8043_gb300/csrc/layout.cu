@@ -189,9 +189,10 @@ __global__ void iota_kernel(uint32_t* __restrict__ val, int64_t n) {
   for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += stride) val[k] = (uint32_t)k;
 }
 
-// The work list in its final order, and each item's cost.
+// The work list in its final order, and each item's cost (64 bits: a scan adds
+// in its input's type, and the costs of a data set pass 2^31).
 __global__ void place_items_kernel(const int4* __restrict__ raw, const uint32_t* __restrict__ perm, int64_t n,
-                                   int4* __restrict__ items, int32_t* __restrict__ cost) {
+                                   int4* __restrict__ items, int64_t* __restrict__ cost) {
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x <= n; x += stride) {
     if (x == n) {
@@ -280,7 +281,7 @@ ScratchPlan plan(int64_t n_obs, int64_t n_users, int64_t n_items, int32_t F) {
   cub::DeviceScan::ExclusiveSum(nullptr, scan_bytes, (const int32_t*)nullptr, (int64_t*)nullptr, (int)(keys + 1));
   cub::DeviceScan::ExclusiveSum(nullptr, scan2_bytes, (const int32_t*)nullptr, (int32_t*)nullptr,
                                 (int)(n_items + 1));
-  cub::DeviceScan::ExclusiveSum(nullptr, scan3_bytes, (const int32_t*)nullptr, (int64_t*)nullptr, (int)(items + 1));
+  cub::DeviceScan::ExclusiveSum(nullptr, scan3_bytes, (const int64_t*)nullptr, (int64_t*)nullptr, (int)(items + 1));
   p.cub_bytes = std::max(std::max(sort_bytes, scan3_bytes), std::max(scan_bytes, scan2_bytes));
   size_t o = 0;
   auto take = [&o](size_t bytes) {
@@ -423,10 +424,12 @@ cudaError_t build_layout(LayoutBuild& b, cudaStream_t st) {
                                         bits_for((uint64_t)b.F * n_tiles << 7), st);
     if (e != cudaSuccess) return e;
   }
-  place_items_kernel<<<blocks_for(n + 1), 256, 0, st>>>(raw, val_out, n, b.chunk, reinterpret_cast<int32_t*>(key_in));
+  // The costs take the place of both key arrays, side by side and free now: 8 (n + 1) bytes of at least 8 (n_obs + 1).
+  int64_t* cost = reinterpret_cast<int64_t*>(key_in);
+  place_items_kernel<<<blocks_for(n + 1), 256, 0, st>>>(raw, val_out, n, b.chunk, cost);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   tb = p.cub_bytes;
-  return cub::DeviceScan::ExclusiveSum(cub_tmp, tb, reinterpret_cast<int32_t*>(key_in), pre, (int)(n + 1), st);
+  return cub::DeviceScan::ExclusiveSum(cub_tmp, tb, cost, pre, (int)(n + 1), st);
 }
 
 // A round takes gpw * per_step places per step of its longest item.  In a sorted

@@ -149,3 +149,36 @@ def test_get_inc_row_lanes(K, n, model):
         np.testing.assert_array_equal(t.read_table(c).cpu().numpy(), x)
     t.poll()
     t.close()
+
+
+def test_costs_past_31_bits():
+    """380M users' entries, whose costs (6 each, in the order of the work list) pass 2^31 in
+    the second of two minibatches: one entry per user and minibatch, every row of L and R a
+    constant, so every user row of versions 1 and 2 has the same value, computed here.  The
+    gradient's few fp32 roundings are within 1e-6 of values of order 1."""
+    N, M, K, eta, lam = 190_000_000, 1000, 4, 0.01, 0.05
+    if torch.cuda.mem_get_info()[0] < 120 << 30:
+        pytest.skip("needs 120 GB")
+    dev = "cuda"
+    ids = torch.arange(N, dtype=torch.int32, device=dev)
+    i = torch.cat([ids, ids])
+    j = i % M
+    D = torch.full((2 * N,), 3.0, device=dev)
+    mb = torch.cat([torch.zeros(N, dtype=torch.uint8, device=dev), torch.ones(N, dtype=torch.uint8, device=dev)])
+    t = _esspt().Table(N + M, K, 2, 0, model="ssp")
+    t.mf_load(i, j, D, mb, ids % 2, N, 2)
+    del i, j, D, mb, ids
+    rows = torch.full((N + M, K), 0.5, device=dev)
+    t.table_init(rows)
+    L, R = 0.5, 0.5
+    for c in (1, 2):
+        t.mf_sgd_clock(eta, lam, 1)  # cap 1: an item takes the mean of its 190 000 updates
+        e = 3.0 - K * L * R
+        L, R = L + eta * (e * R - lam * L), R + eta * (e * L - lam * R)
+        got = t.read_table(c, out=rows)
+        lo, hi = float(got[:N].min()), float(got[:N].max())
+        assert abs(lo - L) <= 1e-6 and abs(hi - L) <= 1e-6, (c, lo, hi, L)
+        # item rows: 190 000 fp32 additions over replicas of at least 2048 each (test_gpu_parity.py's bar)
+        assert float((got[N:] - R).abs().max()) <= TOL, (c, R)
+    t.poll()
+    t.close()
