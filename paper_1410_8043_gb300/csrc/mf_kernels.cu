@@ -43,9 +43,8 @@ __device__ __forceinline__ float4 f4_add(float4 a, float4 b) {
   return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
 }
 
-__device__ __forceinline__ void flush_loss(double* out, float v, int lane) {
+__device__ __forceinline__ void flush_loss(double* out, double x, int lane) {
   if (out == nullptr) return;
-  double x = (double)v;
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
   if (lane == 0 && x != 0.0) atomicAdd(out, x);
@@ -105,7 +104,16 @@ __global__ void __launch_bounds__(kStreamWarps * 32, MINB) sgd_stream_kernel(Str
   const bool last_on = glane + (NV - 1) * G < K4;  // the lane's last slice lies inside the row
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  float loss = 0.f;
+  // Sum of e^2: of the round, and of the rounds before with the rounding error
+  // kept beside it (two-sum, Knuth, TAOCP vol. 2, 4.2.2): a lane adds thousands
+  // of squares, and one fp32 sum of them was off by 6.5e-7 on 10M x 1M, K = 64.
+  float loss = 0.f, loss_sum = 0.f, loss_lost = 0.f;
+  auto fold_loss = [&]() {
+    const float t = loss_sum + loss, b = t - loss_sum;
+    loss_lost += (loss_sum - (t - b)) + (loss - b);
+    loss_sum = t;
+    loss = 0.f;
+  };
   await_previous_kernel();
 
   // Half of the warps copy idle rows first, the others last: the copy's DRAM
@@ -251,6 +259,7 @@ __global__ void __launch_bounds__(kStreamWarps * 32, MINB) sgd_stream_kernel(Str
     auto step_done = [&]() -> bool {
       if (--left > 0) return false;
       close_round();
+      fold_loss();
       xr += kGpw;
       if (xr >= xb) return true;
       rnd = (rnd + 1) & (kMetaRounds - 1);
@@ -341,7 +350,7 @@ __global__ void __launch_bounds__(kStreamWarps * 32, MINB) sgd_stream_kernel(Str
         if ((hi ? r.y : r.x) != kNoRecord) loss += e * e;
         if (step_done()) break;
       }
-      if (glane % (G / 2) != 0) loss = 0.f;
+      if (glane % (G / 2) != 0) loss_sum = loss_lost = 0.f;
     } else {
       f2x2 Ra[NV], Rb[NV];
 #pragma unroll
@@ -379,7 +388,7 @@ __global__ void __launch_bounds__(kStreamWarps * 32, MINB) sgd_stream_kernel(Str
         if (step(s, Ra, Rb)) break;
         if (step(s + 1, Rb, Ra)) break;
       }
-      if (glane != 0) loss = 0.f;
+      if (glane != 0) loss_sum = loss_lost = 0.f;
     }
     cp_async_wait_all();
     // Hot items: the groups' sums, added once into a replica row of the item
@@ -407,7 +416,8 @@ __global__ void __launch_bounds__(kStreamWarps * 32, MINB) sgd_stream_kernel(Str
     }
   }
   if (!(warp & 1)) copy_idle_users<G, NV>(a, warp, nwarps, lane);
-  flush_loss(a.sq_loss, loss, lane);
+  // (an infinite or NaN sum has no rounding error)
+  flush_loss(a.sq_loss, isfinite(loss_sum) ? (double)loss_sum + (double)loss_lost : (double)loss_sum, lane);
 }
 
 // ---- the stream's build (setup) --------------------------------------------

@@ -182,3 +182,22 @@ def test_costs_past_31_bits():
         assert float((got[N:] - R).abs().max()) <= TOL, (c, R)
     t.poll()
     t.close()
+
+
+@pytest.mark.parametrize("K", [4, 64, 100, 256])
+def test_loss_is_exact_over_long_ranges(K):
+    """Rows of zeros, so that every residual is the value 1 + 2^-8, whose square has 17
+    bits: up to 96 of them are exact in fp32, so the clock's loss is exactly n times it,
+    while one fp32 sum per lane would round from its 128th on (8M entries give a lane
+    hundreds)."""
+    N, M, n = 50_000, 1000, 8_000_000
+    i = torch.arange(n, dtype=torch.int32, device="cuda") % N
+    j = (torch.arange(n, dtype=torch.int32, device="cuda") * 7) % M
+    t = _esspt().Table(N + M, K, 4, 1, model="ssp")
+    t.mf_load(i, j, torch.full((n,), 1 + 2.0**-8, device="cuda"), torch.zeros(n, dtype=torch.uint8, device="cuda"),
+              torch.arange(N, dtype=torch.int32, device="cuda") % 4, N, 1)
+    t.table_init(torch.zeros((N + M, K), device="cuda"))
+    loss = torch.zeros(1, dtype=torch.float64, device="cuda")
+    t.mf_sgd_clock(0.01, 0.05, 20, loss)
+    assert float(loss) == n * (1 + 2.0**-8) ** 2
+    t.close()
