@@ -19,12 +19,11 @@ namespace {
 // 400 bytes per entry out of L2).  One warp per entry, which it replaces, read
 // both rows and reduced three sums per entry: 11.0 ms on 20M entries, K = 100.
 //
-// The squares of up to eight entries are added in fp32, their sums with the
-// rounding error kept beside them (two-sum, Knuth, TAOCP vol. 2, 4.2.2) and only
-// at the end in fp64, whose units are few: an fp64 sum per item takes 1.05 ms
-// there.  An entry's fp32 residual carries more error than the eight additions.
-// By worker, where few entries may share a sum, every entry's exact square is
-// added so.
+// Every entry's exact square (high and low fp32 parts) is added to an fp32 sum
+// with its rounding error kept beside it (two-sum, Knuth, TAOCP vol. 2, 4.2.2);
+// fp64, whose units are few, only at the end: an fp64 sum per item takes 1.05 ms
+// on those 20M entries, this 0.85.  Squares added eight at a time without their
+// rounding errors were 8.7e-10 off on 51k entries, the exact ones 7e-11.
 constexpr float kHuge = 1e36f;
 constexpr int32_t kPart = 8;  // entries of a part of an item
 struct Sum2 {  // two packed fp32 sums and what they lost
@@ -90,16 +89,29 @@ __global__ void __launch_bounds__(256) objective_kernel(ObjectiveArgs a) {
       L[k] = f2x2{0ull, 0ull};
       ldg_f2x2_if(L[k], L4 + (int64_t)it.x * K4 + k * G, n > 0 && (k < NV - 1 || last_on));
     }
-    float se = 0.f;
-    u64 sr = 0ull;
+    // A part's entries by lane, so that no step's rows wait for a load of ids (38k
+    // entries, K = 320, cold caches: 65 us with one load per step, 55 so).
+    const bool by_lane = G >= kPart && a.parts > 1;
+    int32_t lane_j = 0;
+    float lane_d = 0.f;
+    if (by_lane && glane < n) {
+      lane_j = __ldg(rec_j + it.y + glane);
+      lane_d = __ldg(rec_D + it.y + glane);
+    }
     for (int32_t t = 0; t < most; t += U) {
       f2x2 R[U][NV];
       float d[U];
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         const bool on = t + u < n;
-        d[u] = on ? __ldg(rec_D + it.y + t + u) : 0.f;
-        const int64_t j = on ? __ldg(rec_j + it.y + t + u) : 0;
+        int64_t j = 0;
+        if (by_lane) {
+          d[u] = __shfl_sync(0xffffffffu, lane_d, t + u, G);
+          j = __shfl_sync(0xffffffffu, lane_j, t + u, G);
+        } else {
+          d[u] = on ? __ldg(rec_D + it.y + t + u) : 0.f;
+          j = on ? __ldg(rec_j + it.y + t + u) : 0;
+        }
 #pragma unroll
         for (int k = 0; k < NV; ++k) {
           R[u][k] = f2x2{0ull, 0ull};
@@ -129,24 +141,14 @@ __global__ void __launch_bounds__(256) objective_kernel(ObjectiveArgs a) {
       for (int u = 0; u < U; ++u)
         if (t + u < n) {
           const float e = d[u] - dot[u];
-          if (BY_WORKER && e * e < kHuge) {
-            const float high = e * e;
-            sums2.add(pack2(high, sum2(rr[u])), minus1);
-            sums2.lost = add2(sums2.lost, pack2(fmaf(e, e, -high), 0.f));
-            continue;
-          }
-          if (e * e < kHuge) {
-            se = fmaf(e, e, se);
-          } else {  // (a diverging run, NaN among it) beyond what fp32 sums hold
+          float high = e * e, low = fmaf(e, e, -high);
+          if (!(high < kHuge)) {  // (a diverging run, NaN among it) beyond what fp32 sums hold
             huge += (double)e * (double)e;
+            high = low = 0.f;
           }
-          sr = add2(sr, rr[u]);
+          sums2.add(pack2(high, sum2(rr[u])), minus1);
+          sums2.lost = add2(sums2.lost, pack2(low, 0.f));
         }
-      if ((t & (8 - U)) == 8 - U || t + U >= most) {
-        sums2.add(pack2(se, sum2(sr)), minus1);
-        se = 0.f;
-        sr = 0ull;
-      }
     }
     if (n > 0) {
       u64 l2 = 0ull;
@@ -214,7 +216,8 @@ cudaError_t run(ObjectiveArgs a, cudaStream_t st) {
     // About two waves of blocks (four per SM) over the minibatches, no more than
     // their units need.  With fewer items than the GPU holds groups, an item is
     // taken in parts of kPart entries, so that a call lasts no longer than the
-    // gathers of one part (20k entries, K = 224: 77 us whole).
+    // gathers of one part (20k entries, K = 224: 77 us whole, 41 in parts; parts
+    // of 4 the same, of 2 and 32 slower).
     const int64_t resident = 4ll * sms * 8;
     a.parts = a.n_items < resident * kGpw ? (kHeavy + kPart - 1) / kPart : 1;
     const int64_t need = (a.parts * (a.n_items / a.F + kGpw) / kGpw + 7) / 8;
