@@ -213,15 +213,17 @@ cudaError_t run(ObjectiveArgs a, cudaStream_t st) {
   auto go = [&](auto g, auto nv) {
     constexpr int G = decltype(g)::value, NV = decltype(nv)::value, kGpw = 32 / G;
     const size_t smem = BY_WORKER ? 2 * sizeof(double) * (size_t)a.P : 0;
-    // About two waves of blocks (four per SM) over the minibatches, no more than
-    // their units need.  With fewer items than the GPU holds groups, an item is
-    // taken in parts of kPart entries, so that a call lasts no longer than the
-    // gathers of one part (20k entries, K = 224: 77 us whole, 41 in parts; parts
-    // of 4 the same, of 2 and 32 slower).
+    // With fewer items than the GPU holds groups, an item is taken in parts of
+    // kPart entries, so that a call lasts no longer than the gathers of one part
+    // (20k entries, K = 224: 77 us whole, 41 in parts; parts of 4 the same, of 2
+    // and 32 slower).  Blocks (four per SM) for about two waves over the
+    // minibatches, for parts one: many parts are empty, and every block ends in
+    // two fp64 additions to one place (13k entries of 531k users, K = 64: 41 us
+    // with two waves, 30 with one; half a wave 32).
     const int64_t resident = 4ll * sms * 8;
     a.parts = a.n_items < resident * kGpw ? (kHeavy + kPart - 1) / kPart : 1;
     const int64_t need = (a.parts * (a.n_items / a.F + kGpw) / kGpw + 7) / 8;
-    const int64_t x = std::max<int64_t>(1, std::min<int64_t>(need, resident / 4 / a.F));
+    const int64_t x = std::max<int64_t>(1, std::min<int64_t>(need, resident / (a.parts > 1 ? 8 : 4) / a.F));
     objective_kernel<G, NV, BY_WORKER><<<dim3((unsigned)x, (unsigned)a.F), 256, smem, st>>>(a);
     return cudaGetLastError();
   };
