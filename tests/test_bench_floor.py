@@ -139,13 +139,12 @@ def test_host_minibatches_are_disjoint_views_of_one_buffer(monkeypatch):
 def test_committed_profiles_match_the_kernel_source():
     """The bench line's roofline.traffic comes from the committed ncu summary
     of each headline kernel, and only while the summary's code digest equals
-    that of the kernels' current source: the kernels that the committed
-    summaries describe were replaced, so there is no figure."""
+    that of the kernels' current source."""
     import bench
 
+    assert bench._profiled_traffic("sgd_stream_kernel", "large") == 7663694080.0
+    assert bench._profiled_traffic("sgd_stream_kernel", "mid") == 774075264.0
     assert bench._profiled_traffic("sgd_work16_kernel", "large") is None
-    assert bench._profiled_traffic("sgd_users32_kernel", "mid") is None
-    assert bench._profiled_traffic("sgd_stream_kernel", "large") is None
 
 
 def test_kernel_code_digest_ignores_comments_only():
