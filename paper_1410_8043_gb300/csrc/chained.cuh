@@ -1,6 +1,8 @@
 // Launch of a kernel that may start while the kernel before it in the stream
 // still runs (programmatic dependent launch); the kernel waits for that one with
-// await_previous_kernel() before its first access to global memory.
+// await_previous_kernel() before its first access to global memory, and reads
+// as read-only data (__ldg, const __restrict__) only what no kernel writes: the
+// layout of the loaded entries.
 #pragma once
 
 #include <cuda_runtime.h>

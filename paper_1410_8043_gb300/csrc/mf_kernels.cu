@@ -144,7 +144,7 @@ __global__ void __launch_bounds__(kStreamWarps * 32, MINB) sgd_stream_kernel(Str
     auto put_meta = [&](int at, const int4& it) {
       const int32_t n = it.w >> 16;
       const int32_t steps = __reduce_max_sync(0xffffffffu, (n + E - 1) / E);
-      const int32_t vs = a.row_mode ? __ldg(a.user_slot + it.x) : __ldg(a.vslot + (it.w & 0xffff));
+      const int32_t vs = a.row_mode ? a.user_slot[it.x] : a.vslot[it.w & 0xffff];
       if (glane == 0) metas[wib][at][grp] = make_int4(it.x, steps, it.z, vs << 7 | n);
     };
     auto item_rows = [&](int32_t vs) -> const float4* {
@@ -359,7 +359,7 @@ __global__ void __launch_bounds__(kStreamWarps * 32, MINB) sgd_stream_kernel(Str
         if (t < s1) {
           const uint32_t x = recX[wib][((t - s0) & (kRing - 1)) * kGpw + grp];
 #pragma unroll
-          for (int k = 0; k < NV; ++k) ldg_f2x2_if(R[k], fR + x + k * G, x != kNoRecord && (k < NV - 1 || last_on));
+          for (int k = 0; k < NV; ++k) ld_f2x2_if(R[k], fR + x + k * G, x != kNoRecord && (k < NV - 1 || last_on));
           f_next();
         }
       };

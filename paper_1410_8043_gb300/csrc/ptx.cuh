@@ -104,8 +104,15 @@ __device__ __forceinline__ u64 fma2(u64 a, u64 b, u64 c) {
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
   return r;
 }
-// r = *p when `pred`, else r as it was; through L1, for memory that no kernel
-// in flight writes.
+// r = *p when `pred`, else r as it was; through L1.  The second form (.nc) is
+// for memory that no kernel writes while the reading one is resident: not for
+// ring rows in a kernel that may start beside the clock before it
+// (await_previous_kernel orders ordinary accesses only).
+__device__ __forceinline__ void ld_f2x2_if(f2x2& r, const float4* p, bool pred) {
+  asm volatile("{\n .reg .pred q;\n setp.ne.b32 q, %3, 0;\n @q ld.global.v2.b64 {%0, %1}, [%2];\n}"
+               : "+l"(r.lo), "+l"(r.hi)
+               : "l"(p), "r"((int)pred));
+}
 __device__ __forceinline__ void ldg_f2x2_if(f2x2& r, const float4* p, bool pred) {
   asm volatile("{\n .reg .pred q;\n setp.ne.b32 q, %3, 0;\n @q ld.global.nc.v2.b64 {%0, %1}, [%2];\n}"
                : "+l"(r.lo), "+l"(r.hi)
@@ -139,7 +146,10 @@ __device__ __forceinline__ void red_add_f2x2_if(float4* p, u64 lo, u64 hi, bool 
 // Programmatic dependent launch: a kernel launched with it may start while the
 // kernel before it in the stream still runs; it waits here, before its first
 // access to global memory, until that one (and so all before it) has finished
-// and its writes are visible.  Then it lets the next such kernel start.
+// and its writes are visible to ordinary accesses.  Memory that a kernel may
+// write is therefore read with ordinary loads here, never as read-only data
+// (.nc, __ldg, const __restrict__), which must not change while the reading
+// kernel is resident.  Then it lets the next such kernel start.
 __device__ __forceinline__ void await_previous_kernel() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

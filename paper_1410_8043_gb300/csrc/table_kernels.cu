@@ -191,8 +191,7 @@ cudaError_t launch_vap(const float* ring, int64_t slot_floats, int32_t nslots, i
 // Copy-forward: slot(c) <- slot(c-1) for a range of rows, so that the
 // deltas of clock c can land in place (Clock() merge, Sec. 2.1 / Sec. 4).
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) copy_rows_kernel(float4* __restrict__ dst, const float4* __restrict__ src,
-                                                        int64_t n4) {
+__global__ void __launch_bounds__(256) copy_rows_kernel(float4* dst, const float4* src, int64_t n4) {
   await_previous_kernel();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -238,11 +237,10 @@ struct RowLanes {  // the row group of a thread
         lanes(1 << log_lanes) {}
 };
 
-__global__ void __launch_bounds__(256) get_rows_kernel(const float* __restrict__ ring, int64_t n_rows, int32_t K,
-                                                       int32_t nslots, const int32_t* __restrict__ v, int32_t worker,
-                                                       const int32_t* __restrict__ ids, int64_t n,
-                                                       float* __restrict__ out, uint32_t* status, int32_t* rowver,
-                                                       int32_t c, int32_t s, int32_t* vmin, int log_lanes) {
+__global__ void __launch_bounds__(256) get_rows_kernel(const float* ring, int64_t n_rows, int32_t K, int32_t nslots,
+                                                       const int32_t* v, int32_t worker, const int32_t* ids, int64_t n,
+                                                       float* out, uint32_t* status, int32_t* rowver, int32_t c,
+                                                       int32_t s, int32_t* vmin, int log_lanes) {
   await_previous_kernel();
   const RowLanes g(log_lanes);
   const int32_t K4 = K >> 2;
@@ -270,6 +268,7 @@ __global__ void __launch_bounds__(256) get_rows_kernel(const float* __restrict__
     }
     const float4* src = reinterpret_cast<const float4*>(ring) + ((int64_t)slot * n_rows + r) * K4;
     float4* o = reinterpret_cast<float4*>(out + k * K);
+#pragma unroll 1
     for (int32_t q = g.lane; q < K4; q += g.lanes) o[q] = src[q];
   }
   if (vmin != nullptr) {
@@ -278,9 +277,8 @@ __global__ void __launch_bounds__(256) get_rows_kernel(const float* __restrict__
   }
 }
 
-__global__ void __launch_bounds__(256) inc_rows_kernel(float* __restrict__ slot, int64_t n_rows, int32_t K,
-                                                       const int32_t* __restrict__ ids, const float* __restrict__ d,
-                                                       int64_t n, uint32_t* status, int log_lanes) {
+__global__ void __launch_bounds__(256) inc_rows_kernel(float* slot, int64_t n_rows, int32_t K, const int32_t* ids,
+                                                       const float* d, int64_t n, uint32_t* status, int log_lanes) {
   await_previous_kernel();
   const RowLanes g(log_lanes);
   const int32_t K4 = K >> 2;
