@@ -1,6 +1,6 @@
 // The training objective (Sec. 3.1, Sec. 5) over all entries at one table
 // version: sum e^2 and sum [e^2 + lambda (|L_i|^2 + |R_j|^2)], fp32 residuals
-// and row norms, fp64 sums over the work items; whole, or by worker.
+// and row norms, summed to the precision of fp64; whole, or by worker.
 #include <algorithm>
 #include <type_traits>
 
@@ -22,10 +22,22 @@ namespace {
 // Every entry's exact square (high and low fp32 parts) is added to an fp32 sum
 // with its rounding error kept beside it (two-sum, Knuth, TAOCP vol. 2, 4.2.2);
 // fp64, whose units are few, only at the end: an fp64 sum per item takes 1.05 ms
-// on those 20M entries, this 0.85.  Squares added eight at a time without their
-// rounding errors were 8.7e-10 off on 51k entries, the exact ones 7e-11.
-constexpr float kHuge = 1e36f;
+// on those 20M entries, this 0.80.  Squares added eight at a time without their
+// rounding errors were 8.7e-10 off on 51k entries, the exact ones 7e-11.  What
+// fp32 cannot hold so goes to fp64 sums of its own: squares and norms from 1e29
+// on, NaN among them (a lane adds fewer than 2^31 of them, which stay finite
+// below it), and squares whose low part would be subnormal.
+constexpr float kHuge = 1e29f;
+__device__ __forceinline__ bool in_range(float e, float norm) {
+  return fabsf(e) < 3e14f && !(fabsf(e) < 1e-14f && e != 0.f) && norm < kHuge;
+}
 constexpr int32_t kPart = 8;  // entries of a part of an item
+// x + y and its rounding error.
+__device__ __forceinline__ float two_sum(float x, float y, float& err) {
+  const float s = x + y, b = s - x;
+  err = (x - (s - b)) + (y - b);
+  return s;
+}
 struct Sum2 {  // two packed fp32 sums and what they lost
   u64 sum = 0ull, lost = 0ull;
   __device__ __forceinline__ void add(u64 x, u64 minus1) {
@@ -33,14 +45,6 @@ struct Sum2 {  // two packed fp32 sums and what they lost
     const u64 d = add2(fma2(fma2(b, minus1, s), minus1, sum), fma2(b, minus1, x));  // (sum - (s - b)) + (x - b)
     sum = s;
     lost = add2(lost, d);
-  }
-  // The second sum, and the first (an infinite or NaN sum has no rounding error).
-  __device__ __forceinline__ double total(double& first) const {
-    float a, b, c, d;
-    unpack2(sum, a, b);
-    unpack2(lost, c, d);
-    first = isfinite(a) ? (double)a + (double)c : (double)a;
-    return isfinite(b) ? (double)b + (double)d : (double)b;
   }
 };
 
@@ -64,7 +68,7 @@ __global__ void __launch_bounds__(256) objective_kernel(ObjectiveArgs a) {
   const u64 minus1 = pack2(-1.f, -1.f);
   // e^2 and what the rows' squares add up to; by worker, of the item at hand.
   Sum2 sums2;  // (e^2, this lane's part of the rows' squares)
-  double huge = 0.0;
+  double wide_e = 0.0, wide_n = 0.0;  // the same of what fp32 cannot hold
   // Units of kGpw items; with a.parts > 1, part by part.
   const int64_t x_first = __ldg(a.item_base + blockIdx.y);
   const uint32_t units = (uint32_t)((x_end - x_first + kGpw - 1) / kGpw);
@@ -82,7 +86,7 @@ __global__ void __launch_bounds__(256) objective_kernel(ObjectiveArgs a) {
     f2x2 L[NV];
     if (BY_WORKER) {
       sums2 = Sum2{};
-      huge = 0.0;
+      wide_e = wide_n = 0.0;
     }
 #pragma unroll
     for (int k = 0; k < NV; ++k) {
@@ -118,37 +122,45 @@ __global__ void __launch_bounds__(256) objective_kernel(ObjectiveArgs a) {
           ldg_f2x2_if(R[u][k], R4 + j * K4 + k * G, on && (k < NV - 1 || last_on));
         }
       }
-      float dot[U];
-      u64 rr[U];
+      float e[U], norm[U];  // residuals, and this lane's part of |R|^2
 #pragma unroll
       for (int u = 0; u < U; ++u) {
-        u64 p = 0ull;
-        rr[u] = 0ull;
+        u64 p = 0ull, r = 0ull;
 #pragma unroll
         for (int k = 0; k < NV; ++k) {
           p = fma2(L[k].lo, R[u][k].lo, p);
           p = fma2(L[k].hi, R[u][k].hi, p);
-          rr[u] = fma2(R[u][k].lo, R[u][k].lo, rr[u]);
-          rr[u] = fma2(R[u][k].hi, R[u][k].hi, rr[u]);
+          r = fma2(R[u][k].lo, R[u][k].lo, r);
+          r = fma2(R[u][k].hi, R[u][k].hi, r);
         }
-        dot[u] = sum2(p);
+        e[u] = sum2(p);
+        norm[u] = sum2(r);
       }
 #pragma unroll
       for (int off = G / 2; off > 0; off >>= 1)
 #pragma unroll
-        for (int u = 0; u < U; ++u) dot[u] += __shfl_xor_sync(0xffffffffu, dot[u], off);
+        for (int u = 0; u < U; ++u) e[u] += __shfl_xor_sync(0xffffffffu, e[u], off);
+      bool wide = false;
 #pragma unroll
-      for (int u = 0; u < U; ++u)
-        if (t + u < n) {
-          const float e = d[u] - dot[u];
-          float high = e * e, low = fmaf(e, e, -high);
-          if (!(high < kHuge)) {  // (a diverging run, NaN among it) beyond what fp32 sums hold
-            huge += (double)e * (double)e;
-            high = low = 0.f;
+      for (int u = 0; u < U; ++u) {
+        e[u] = t + u < n ? d[u] - e[u] : 0.f;
+        wide |= !in_range(e[u], norm[u]);
+      }
+      if (wide) {  // (one branch for the step: one per entry took 1380 us instead of 802, 20M entries, K = 100)
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          if (!in_range(e[u], norm[u])) {
+            wide_e += (double)e[u] * (double)e[u];
+            wide_n += (double)norm[u];
+            e[u] = norm[u] = 0.f;
           }
-          sums2.add(pack2(high, sum2(rr[u])), minus1);
-          sums2.lost = add2(sums2.lost, pack2(low, 0.f));
-        }
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const float high = e[u] * e[u];
+        sums2.add(pack2(high, norm[u]), minus1);
+        sums2.lost = add2(sums2.lost, pack2(fmaf(e[u], e[u], -high), 0.f));
+      }
     }
     if (n > 0) {
       u64 l2 = 0ull;
@@ -157,18 +169,34 @@ __global__ void __launch_bounds__(256) objective_kernel(ObjectiveArgs a) {
         l2 = fma2(L[k].lo, L[k].lo, l2);
         l2 = fma2(L[k].hi, L[k].hi, l2);
       }
-      sums2.add(pack2(0.f, (float)n * sum2(l2)), minus1);
+      const float l = sum2(l2);
+      float high = (float)n * l, low = fmaf((float)n, l, -high);
+      if (!(high < kHuge)) {
+        wide_n += (double)n * (double)l;
+        high = low = 0.f;
+      }
+      sums2.add(pack2(0.f, high), minus1);
+      sums2.lost = add2(sums2.lost, pack2(0.f, low));
     }
     if (BY_WORKER) {
-      double e2;
-      float norm = (float)sums2.total(e2);
+      float e2, e2_lost, norm, norm_lost;
+      unpack2(sums2.sum, e2, norm);
+      unpack2(sums2.lost, e2_lost, norm_lost);
 #pragma unroll
-      for (int off = G / 2; off > 0; off >>= 1) norm += __shfl_xor_sync(0xffffffffu, norm, off);
+      for (int off = G / 2; off > 0; off >>= 1) {
+        const float lost = __shfl_xor_sync(0xffffffffu, norm_lost, off);
+        float err;
+        norm = two_sum(norm, __shfl_xor_sync(0xffffffffu, norm, off), err);
+        norm_lost += lost + err;
+      }
+      if (__any_sync(0xffffffffu, wide_n != 0.0))
+#pragma unroll
+        for (int off = G / 2; off > 0; off >>= 1) wide_n += __shfl_xor_sync(0xffffffffu, wide_n, off);
       if (glane == 0 && n > 0) {
         const int p = it.w & 0xffff;
-        e2 += huge;
-        atomicAdd(&sums[p], e2);
-        atomicAdd(&sums[a.P + p], e2 + (double)a.lambda * (double)norm);
+        const double sq = (double)e2 + (double)e2_lost + wide_e;
+        atomicAdd(&sums[p], sq);
+        atomicAdd(&sums[a.P + p], sq + (double)a.lambda * ((double)norm + (double)norm_lost + wide_n));
       }
     }
   }
@@ -179,8 +207,11 @@ __global__ void __launch_bounds__(256) objective_kernel(ObjectiveArgs a) {
       if (sums[a.P + k] != 0.0) atomicAdd(a.out + a.out_stride + k, sums[a.P + k]);
     }
   } else {
-    double s1, s2 = sums2.total(s1);
-    s1 = glane == 0 ? s1 + huge : 0.0;
+    float e2, e2_lost, norm, norm_lost;
+    unpack2(sums2.sum, e2, norm);
+    unpack2(sums2.lost, e2_lost, norm_lost);
+    double s1 = glane == 0 ? (double)e2 + (double)e2_lost + wide_e : 0.0;
+    double s2 = (double)norm + (double)norm_lost + wide_n;
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) {
       s1 += __shfl_xor_sync(0xffffffffu, s1, off);

@@ -62,6 +62,66 @@ def test_objective_shapes(K, N, n):
     t.close()
 
 
+def _constant_objective(K, N, n, D, element, P=3):
+    """Objective inputs: every entry's value D (or an array of them); L's first and R's last value `element`, the rest
+    0, so that the residual is the value and every row's square is one product.  Returns whole and by-worker sums."""
+    M, F = 7, 2
+    i = torch.arange(n, dtype=torch.int32, device="cuda") % N
+    rows = torch.zeros((N + M, K), device="cuda")
+    rows[:N, 0] = element
+    rows[N:, K - 1] = element
+    t = _esspt().Table(N + M, K, P, 1, model="ssp")
+    t.mf_load(i, (torch.arange(n, dtype=torch.int32, device="cuda") * 5) % M,
+              torch.as_tensor(D, dtype=torch.float32, device="cuda").expand(n).contiguous(),
+              (torch.arange(n, device="cuda") % F).to(torch.uint8),
+              torch.arange(N, dtype=torch.int32, device="cuda") % P, N, F)
+    t.table_init(rows)
+    out = t.mf_objective(0, 0.5), t.mf_worker_objective_noalloc(0, 0.5)
+    t.close()
+    return out, np.bincount(i.cpu().numpy() % P, minlength=P)
+
+
+# Items taken in parts and taken whole.
+@pytest.mark.parametrize("N,n", [(700, 40_000), (200_000, 4_000_000)])
+@pytest.mark.parametrize("K", [8, 32, 64, 96, 128, 256, 512])
+def test_objective_sums_are_exact(K, N, n):
+    """The value's square has 27 bits (24 in its high fp32 part, one in its low one), a row's |.|^2 24, and both
+    sums keep every bit: each is a multiple of 2^-26 below 2^27, with fewer than 24 bits lost per lane."""
+    x = 1 + 2.0**-11 + 2.0**-13
+    norm = float(np.float32(x) * np.float32(x))
+    assert norm != x * x and norm + 2.0**-26 == x * x
+    ((sq, pen), (wsq, wpen)), cnt = _constant_objective(K, N, n, x, x)
+    assert (sq, pen) == (n * x * x, n * (x * x + norm))
+    assert (wsq == cnt * (x * x)).all() and (wpen == cnt * (x * x + norm)).all()
+
+
+@pytest.mark.parametrize("K", [4, 64, 100])
+@pytest.mark.parametrize("value,element", [(9e17, 0.0), (3e14, 0.0), (1e25, 0.0), (0.0, 9e17), (0.0, 1.5e19),
+                                           (3.0, 3e14), (1e-20, 0.0)])
+def test_objective_beyond_fp32_sums(K, value, element):
+    """Squares whose sum, or themselves, pass what fp32 holds: finite wherever a sum in 64 bits is, to 1e-12."""
+    n, v, a = 2_000_000, float(np.float32(value)), np.float32(element)
+    ((sq, pen), (wsq, wpen)), cnt = _constant_objective(K, 5000, n, value, element)
+    norm = float(a * a)
+    assert np.isfinite(norm)
+    np.testing.assert_allclose([sq, pen], [n * (v * v), n * (v * v + norm)], rtol=1e-12)
+    np.testing.assert_allclose(wsq, cnt * (v * v), rtol=1e-12)
+    np.testing.assert_allclose(wpen, cnt * (v * v + norm), rtol=1e-12)
+
+
+@pytest.mark.parametrize("K", [4, 64, 100])
+@pytest.mark.parametrize("bad", [float("nan"), float("inf"), -float("inf")])
+def test_objective_not_finite(K, bad):
+    """One such value reaches the whole sums and its worker's, and no other worker's."""
+    n, N = 3000, 300
+    D = torch.ones(n)
+    D[7] = bad  # user 7, worker 1 of 3
+    ((sq, pen), (wsq, wpen)), cnt = _constant_objective(K, N, n, D, 0.0)
+    same = np.isnan if np.isnan(bad) else np.isposinf
+    assert same([sq, pen, wsq[1], wpen[1]]).all()
+    assert (wsq[[0, 2]] == cnt[[0, 2]]).all() and (wpen[[0, 2]] == cnt[[0, 2]]).all()
+
+
 # 100 x 4: all norms at once; 120 001 x 100 (48 MB a version, kmax = 4 and 9): the scan, in one launch and two.
 @pytest.mark.parametrize("rows,K,s", [(100, 4, 3), (120_001, 100, 4), (120_001, 100, 9)])
 @pytest.mark.parametrize("seed", [0, 1])
