@@ -153,6 +153,9 @@ struct MergeArgs {
   ScheduleArgs sched;
 };
 
+// Blocks for work_items at per_block each, at most max_per_sm per SM, at least one.
+int grid_for(int64_t work_items, int64_t per_block, int max_per_sm);
+
 // Launchers (return the launch error, if any).
 cudaError_t launch_schedule(const ScheduleArgs& a, cudaStream_t st);
 // VAP: norm[k], k = 1..kmax, is within the bound (as fp32 bits) exactly where
