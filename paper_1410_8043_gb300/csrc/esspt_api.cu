@@ -237,7 +237,7 @@ MfCarve mf_carve(int64_t n_obs, int64_t n_users, int64_t n_items, int32_t F, int
   k.sx = take(sizeof(uint32_t) * k.max_places);
   k.syz = take(2 * sizeof(uint32_t) * k.max_places);
   k.place = take(sizeof(uint32_t) * k.max_chunks);
-  k.steps = take(sizeof(int32_t) * F);
+  k.steps = take(sizeof(int64_t) * F);
   k.uoff = take(sizeof(int32_t) * (size_t)F * (n_users + 1));
   k.mb_base = take(sizeof(int64_t) * (F + 1));
   k.item_cnt = take(sizeof(int32_t) * (size_t)F * n_items);
@@ -270,11 +270,12 @@ bool mf_sizes_ok(const esspt_ctx* c, int64_t n_obs, int64_t n_users, int32_t F) 
   if (!(c && n_obs >= 0 && n_obs < (int64_t)INT32_MAX && n_users > 0 && n_users < c->n_rows && F >= 1 && F <= 255 &&
         (int64_t)F * n_users < (int64_t)INT32_MAX))
     return false;
-  // Item rows (item * K/4 float4) and item replica rows (in whole 32-byte
-  // sectors) stay below 2^31 float4; the merge splits the first with 32 bits.
-  const int64_t n_items = c->n_rows - n_users;
-  return n_items * (c->K / 4) < (int64_t)INT32_MAX &&
-         layout_max_item_reps(n_obs, n_items) * ((c->K + 7) / 8 * 2) < (int64_t)INT32_MAX;
+  // The stream's words offset item rows (item * K/4) and item replica rows
+  // (row * dR_stride4) in float4, unsigned with kNoRecord left over.  The replicas
+  // are held to 2^31 in 32-byte sectors; dR_stride4 pads by a third at most.
+  const int64_t n_items = c->n_rows - n_users, reps = layout_max_item_reps(n_obs, n_items);
+  return n_items * (c->K / 4) < (int64_t)INT32_MAX && reps * ((c->K + 7) / 8 * 2) < (int64_t)INT32_MAX &&
+         reps * dR_stride4(c->K) < (int64_t)kNoRecord;
 }
 
 }  // namespace
@@ -580,7 +581,7 @@ esspt_status esspt_mf_load(esspt_ctx* c, const int32_t* d_i, const int32_t* d_j,
   uint32_t* sx = reinterpret_cast<uint32_t*>(w + k.sx);
   uint32_t* syz = reinterpret_cast<uint32_t*>(w + k.syz);
   uint32_t* place = reinterpret_cast<uint32_t*>(w + k.place);
-  int32_t* steps = reinterpret_cast<int32_t*>(w + k.steps);
+  int64_t* steps = reinterpret_cast<int64_t*>(w + k.steps);
   for (int32_t f = 0; f < F; ++f) {
     const int64_t items = chb[f + 1] - chb[f];
     const int64_t warps = std::min(stream_max_warps(c->K), (items + geo.gpw - 1) / geo.gpw);
@@ -589,14 +590,14 @@ esspt_status esspt_mf_load(esspt_ctx* c, const int32_t* d_i, const int32_t* d_j,
     ESSPT_CUDA(c, launch_stream_partition(b.pre + chb[f], items, warps, part + ptb[f], c->st));
     ESSPT_CUDA(c, launch_stream_steps(b.chunk + chb[f], part + ptb[f], warps, geo, steps + f, c->st));
   }
-  std::vector<int32_t> n_steps((size_t)F);
-  ESSPT_CUDA(c, cudaMemcpyAsync(n_steps.data(), steps, sizeof(int32_t) * F, cudaMemcpyDeviceToHost, c->st));
+  std::vector<int64_t> n_steps((size_t)F);
+  ESSPT_CUDA(c, cudaMemcpyAsync(n_steps.data(), steps, sizeof(int64_t) * F, cudaMemcpyDeviceToHost, c->st));
   ESSPT_CUDA(c, cudaStreamSynchronize(c->st));
   std::vector<int64_t> rcb((size_t)F + 1, 0);
   for (int32_t f = 0; f < F; ++f) {
-    const int64_t places = (int64_t)n_steps[f] * geo.gpw * geo.per_step;
+    const int64_t places = n_steps[f] * geo.gpw * geo.per_step;
     rcb[f + 1] = rcb[f] + places;
-    if (rcb[f + 1] > k.max_places) return fail(c, ESSPT_ECUDA, "internal: stream overflow");
+    if (n_steps[f] > kMaxSteps || rcb[f + 1] > k.max_places) return fail(c, ESSPT_ECUDA, "internal: stream overflow");
     StreamSource src{};
     src.rec_j = b.rec_j + mbb[f];
     src.rec_D = b.rec_D + mbb[f];

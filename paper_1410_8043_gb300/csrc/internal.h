@@ -108,7 +108,7 @@ struct SgdArgs {
 // length within tiles of 2^kTileBits users.
 // Warp w takes items part[w].x .. part[w].y in rounds of gpw (one per row
 // group), per_step entries of an item per step, and its steps are part[w].z ..
-// part[w].w of the minibatch's stream.  A step has gpw * per_step places, those
+// part[w].w (unsigned) of the minibatch's stream.  A step has gpw * per_step places, those
 // of one group side by side.  Place p holds an entry: x[p] = item * K/4, and in
 // yz, per_step y words before per_step z words, y = replica row * dR_stride4
 // (both float4 offsets: of the item's row, and of the row in dR that its update
@@ -119,6 +119,22 @@ constexpr int kStepAlign = 4;  // a warp's first step is a multiple
 struct StreamGeometry {
   int gpw, per_step;
 };
+// A minibatch of nearly 2^31 entries of users with one each has 2^32 places at two
+// entries per step, and steps past 2^31 at one place per step: an item's place
+// word is step * gpw + group, and steps and replica offsets are unsigned.
+__host__ __device__ inline uint32_t place_word(const StreamGeometry& g, int64_t step, int grp) {
+  return (uint32_t)(step * g.gpw + grp);
+}
+// Place of entry k of an item with place word `at`, and where its y word is (the
+// z word follows per_step words later).
+__host__ __device__ inline int64_t record_place(const StreamGeometry& g, uint32_t at, int32_t k) {
+  return ((int64_t)at + (int64_t)(k / g.per_step) * g.gpw) * g.per_step + k % g.per_step;
+}
+__host__ __device__ inline int64_t y_word(const StreamGeometry& g, int64_t place) {
+  return place / g.per_step * g.per_step * 2 + place % g.per_step;
+}
+// The most steps of a minibatch: the SGD kernel looks a few past the last.
+constexpr int64_t kMaxSteps = (int64_t)UINT32_MAX - 64;
 struct StreamArgs {
   SgdArgs a;
   const int4* items;
@@ -182,8 +198,7 @@ bool stream_is_small(int32_t K, int64_t n_warps, int64_t n_users);
 StreamGeometry stream_geometry(int32_t K);
 // Build of a minibatch's stream (setup): the split of its n_items work items
 // over n_warps warps (pre: see LayoutBuild), the steps of the warps (their sum
-// in *total), the places (place[i] = that of item i's first entry), and new
-// values for them.
+// in *total), the places (place[i] = item i's place word), and new values for them.
 struct StreamSource {
   const int32_t* rec_j;
   const float* rec_D;
@@ -194,7 +209,7 @@ struct StreamSource {
 };
 cudaError_t launch_stream_partition(const int64_t* pre, int64_t n_items, int64_t n_warps, int4* part, cudaStream_t st);
 cudaError_t launch_stream_steps(const int4* items, int4* part, int64_t n_warps, const StreamGeometry& g,
-                                int32_t* total, cudaStream_t st);
+                                int64_t* total, cudaStream_t st);
 cudaError_t launch_stream_fill(const int4* items, const int4* part, int64_t n_warps, const StreamGeometry& g,
                                const StreamSource& src, int64_t n_places, uint32_t* x, uint32_t* yz, uint32_t* place,
                                cudaStream_t st);

@@ -120,13 +120,14 @@ __global__ void __launch_bounds__(kStreamWarps * 32, MINB) sgd_stream_kernel(Str
   // traffic runs beside the other warps' arithmetic.
   if (warp & 1) copy_idle_users<G, NV>(a, warp, nwarps, lane);
 
-  int32_t xr = 0, xb = 0, s0 = 0, s1 = 0;
+  int32_t xr = 0, xb = 0;
+  uint32_t s0 = 0, s1 = 0;
   if (warp < c.n_warps) {
     const int4 p0 = __ldg(c.part + warp);
     xr = p0.x;
     xb = p0.y;
-    s0 = p0.z;
-    s1 = p0.w;
+    s0 = (uint32_t)p0.z;
+    s1 = (uint32_t)p0.w;
   }
   if (s0 < s1) {
     const int64_t slot4 = a.n_rows * K4;
@@ -157,7 +158,7 @@ __global__ void __launch_bounds__(kStreamWarps * 32, MINB) sgd_stream_kernel(Str
       for (int k = 0; k < NV; ++k) cp_async16_hint_if(&to[k][lane], row + k * G, on && (k < NV - 1 || last_on), pol);
     };
     // The records of kChunkSteps steps from step s (s - s0 a multiple of it).
-    auto fetch_records = [&](int32_t s) {
+    auto fetch_records = [&](uint32_t s) {
       const int half = (s - s0) & kChunkSteps;
 #pragma unroll
       for (int l0 = 0; l0 < kChunkSteps * kPlaces; l0 += 128) {
@@ -307,7 +308,7 @@ __global__ void __launch_bounds__(kStreamWarps * 32, MINB) sgd_stream_kernel(Str
     }
     if constexpr (E == 2) {
       // Gather the item rows of step t into place q of the ring of rows.
-      auto gather = [&](int32_t t, int q) {
+      auto gather = [&](uint32_t t, int q) {
         if (t < s1) {
           const uint2 x = *reinterpret_cast<const uint2*>(&recX[wib][(((t - s0) & (kRing - 1)) * kGpw + grp) * 2]);
 #pragma unroll
@@ -324,7 +325,7 @@ __global__ void __launch_bounds__(kStreamWarps * 32, MINB) sgd_stream_kernel(Str
       open_round();
       int q = 0;  // place of step s in the ring of rows
       const bool hi = lane & (G / 2);  // this lane ends up with the second entry's dot product
-      for (int32_t s = s0;; ++s) {
+      for (uint32_t s = s0;; ++s) {
         gather(s + PF, q == 0 ? PF : q - 1);
         if (((s - s0) & (kChunkSteps - 1)) == 0 && s > s0) fetch_records(s + kChunkSteps);
         cp_async_commit();
@@ -355,7 +356,7 @@ __global__ void __launch_bounds__(kStreamWarps * 32, MINB) sgd_stream_kernel(Str
       f2x2 Ra[NV], Rb[NV];
 #pragma unroll
       for (int k = 0; k < NV; ++k) Ra[k] = Rb[k] = f2x2{0ull, 0ull};
-      auto gather = [&](int32_t t, f2x2(&R)[NV]) {
+      auto gather = [&](uint32_t t, f2x2(&R)[NV]) {
         if (t < s1) {
           const uint32_t x = recX[wib][((t - s0) & (kRing - 1)) * kGpw + grp];
 #pragma unroll
@@ -366,7 +367,7 @@ __global__ void __launch_bounds__(kStreamWarps * 32, MINB) sgd_stream_kernel(Str
       gather(s0, Ra);
       cp_async_wait_all();
       open_round();
-      auto step = [&](int32_t s, const f2x2(&Rc)[NV], f2x2(&Rn)[NV]) -> bool {
+      auto step = [&](uint32_t s, const f2x2(&Rc)[NV], f2x2(&Rn)[NV]) -> bool {
         if (((s - s0) & (kChunkSteps - 1)) == kChunkSteps - 1) {  // the next step's records, fetched 8 steps ago
           cp_async_wait_all();
           __syncwarp();
@@ -384,7 +385,7 @@ __global__ void __launch_bounds__(kStreamWarps * 32, MINB) sgd_stream_kernel(Str
         }
         return step_done();
       };
-      for (int32_t s = s0;; s += 2) {
+      for (uint32_t s = s0;; s += 2) {
         if (step(s, Ra, Rb)) break;
         if (step(s + 1, Rb, Ra)) break;
       }

@@ -46,54 +46,48 @@ __global__ void __launch_bounds__(256) stream_steps_kernel(const int4* __restric
   if (w >= n_warps) return;
   const int lane = threadIdx.x & 31;
   const int32_t x0 = part[w].x, x1 = part[w].y;
-  int32_t sum = 0;
+  uint32_t sum = 0;
   for (int32_t r = x0 + lane * g.gpw; r < x1; r += 32 * g.gpw) {
     int32_t mx = 0;
     for (int32_t x = r; x < min(r + g.gpw, x1); ++x) mx = max(mx, items[x].w >> 16);
     sum += (mx + g.per_step - 1) / g.per_step;
   }
   sum = __reduce_add_sync(0xffffffffu, sum);
-  if (lane == 0) part[w].z = sum;
+  if (lane == 0) part[w].z = (int32_t)sum;
 }
 // part[w].z, .w = first and end step of warp w; a warp starts at a multiple of
 // kStepAlign steps, so that its records start on 16 bytes.  One block.
-__global__ void __launch_bounds__(1024) stream_offsets_kernel(int4* part, int64_t n_warps, int32_t* total) {
-  __shared__ int32_t sums[1024];
+__global__ void __launch_bounds__(1024) stream_offsets_kernel(int4* part, int64_t n_warps, int64_t* total) {
+  __shared__ int64_t sums[1024];
   const int64_t per = (n_warps + 1023) / 1024, w0 = threadIdx.x * per, w1 = min(n_warps, w0 + per);
-  int32_t sum = 0;
-  for (int64_t w = w0; w < w1; ++w) sum += (part[w].z + kStepAlign - 1) / kStepAlign * kStepAlign;
+  auto aligned = [&](int64_t w) {
+    return ((int64_t)(uint32_t)part[w].z + kStepAlign - 1) / kStepAlign * kStepAlign;
+  };
+  int64_t sum = 0;
+  for (int64_t w = w0; w < w1; ++w) sum += aligned(w);
   sums[threadIdx.x] = sum;
   __syncthreads();
   for (int off = 1; off < 1024; off <<= 1) {
-    const int32_t v = threadIdx.x >= off ? sums[threadIdx.x - off] : 0;
+    const int64_t v = threadIdx.x >= off ? sums[threadIdx.x - off] : 0;
     __syncthreads();
     sums[threadIdx.x] += v;
     __syncthreads();
   }
-  int32_t at = sums[threadIdx.x] - sum;
+  int64_t at = sums[threadIdx.x] - sum;
   for (int64_t w = w0; w < w1; ++w) {
-    const int32_t n = part[w].z;
-    part[w].z = at;
-    part[w].w = at + n;
-    at += (n + kStepAlign - 1) / kStepAlign * kStepAlign;
+    const int64_t n = (uint32_t)part[w].z, next = at + aligned(w);
+    part[w].z = (int32_t)(uint32_t)at;
+    part[w].w = (int32_t)(uint32_t)(at + n);
+    at = next;
   }
   if (threadIdx.x == 1023) *total = sums[1023];
 }
 
 cudaError_t launch_stream_steps(const int4* items, int4* part, int64_t n_warps, const StreamGeometry& g,
-                                int32_t* total, cudaStream_t st) {
+                                int64_t* total, cudaStream_t st) {
   stream_steps_kernel<<<(unsigned)(n_warps / 8 + 1), 256, 0, st>>>(items, part, n_warps, g);
   stream_offsets_kernel<<<1, 1024, 0, st>>>(part, n_warps, total);
   return cudaGetLastError();
-}
-
-// Place of entry k of an item whose first entry's place is `at`, and where its
-// y and z words are.
-__device__ __forceinline__ int64_t record_place(const StreamGeometry& g, int64_t at, int32_t k) {
-  return at + (int64_t)(k / g.per_step) * g.gpw * g.per_step + k % g.per_step;
-}
-__device__ __forceinline__ int64_t y_word(const StreamGeometry& g, int64_t place) {
-  return place / g.per_step * g.per_step * 2 + place % g.per_step;
 }
 
 // The records of a minibatch (x and yz hold kNoRecord everywhere on entry) and
@@ -106,13 +100,13 @@ __global__ void __launch_bounds__(256) stream_fill_kernel(const int4* __restrict
   if (w >= n_warps) return;
   const int lane = threadIdx.x & 31, G = 32 / g.gpw, grp = lane / G, l = lane & (G - 1);
   const int4 p = part[w];
-  int64_t s = p.z;
+  int64_t s = (uint32_t)p.z;
   for (int32_t x0 = p.x; x0 < p.y; x0 += g.gpw) {
     const int32_t i = x0 + grp;
     const int4 it = i < p.y ? items[i] : make_int4(0, 0, -2, 0);
     const int32_t n = it.w >> 16;
-    const int64_t at = (s * g.gpw + grp) * g.per_step;
-    if (l == 0 && n > 0) place[i] = (uint32_t)at;
+    const uint32_t at = place_word(g, s, grp);
+    if (l == 0 && n > 0) place[i] = at;
     for (int32_t k = l; k < n; k += G) {
       const int32_t t = it.y + k, j = src.rec_j[t];
       const int32_t e0 = src.item_rep[j], e1 = src.item_rep[j + 1];  // extra replicas of j: e1 - e0 (reps - 1)
@@ -147,7 +141,7 @@ __global__ void __launch_bounds__(256) stream_refill_kernel(const int4* __restri
   const int64_t stride = ((int64_t)gridDim.x * blockDim.x) >> 3;
   for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 3; i < n_items; i += stride) {
     const int4 it = items[i];
-    const int64_t at = place[i];
+    const uint32_t at = place[i];
     for (int32_t k = threadIdx.x & 7; k < it.w >> 16; k += 8)
       yz[y_word(g, record_place(g, at, k)) + g.per_step] = __float_as_uint(D[it.y + k]);
   }
@@ -170,7 +164,7 @@ __global__ void __launch_bounds__(256) row_refresh_kernel(RowRefreshArgs a) {
   const int64_t stride = ((int64_t)gridDim.x * blockDim.x) >> 3;
   for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 3; i < a.n_items; i += stride) {
     const int4 it = __ldg(a.items + i);
-    const int64_t at = __ldg(a.place + i);
+    const uint32_t at = __ldg(a.place + i);
     int32_t* V = a.rowver + (int64_t)(it.w & 0xffff) * a.n_rows;
     if ((threadIdx.x & 7) == 0) {
       int32_t v = V[it.x];
