@@ -237,6 +237,7 @@ MfCarve mf_carve(int64_t n_obs, int64_t n_users, int64_t n_items, int32_t F, int
   k.sx = take(sizeof(uint32_t) * k.max_places);
   k.syz = take(2 * sizeof(uint32_t) * k.max_places);
   k.place = take(sizeof(uint32_t) * k.max_chunks);
+  o = std::max(o, k.sx + layout_stage_bytes(n_obs, n_users, F));  // the load uses the stream's memory before
   k.steps = take(sizeof(int64_t) * F);
   k.uoff = take(sizeof(int32_t) * (size_t)F * (n_users + 1));
   k.mb_base = take(sizeof(int64_t) * (F + 1));
@@ -245,7 +246,7 @@ MfCarve mf_carve(int64_t n_obs, int64_t n_users, int64_t n_items, int32_t F, int
   k.dR = take(sizeof(float4) * (size_t)k.dR_rows * dR_stride4(K));
   k.wuser = take(sizeof(int32_t) * n_users);
   k.wbase = take(sizeof(int32_t) * (P + 1));
-  k.chunk = take(sizeof(int4) * k.max_chunks);
+  k.chunk = take(layout_chunk_bytes(n_obs, n_users, F));
   k.chunk_base = take(sizeof(int64_t) * (F + 1));
   k.heavy = take(sizeof(int4) * k.max_heavy);
   k.heavy_base = take(sizeof(int64_t) * (F + 1));
@@ -541,6 +542,7 @@ esspt_status esspt_mf_load(esspt_ctx* c, const int32_t* d_i, const int32_t* d_j,
   b.max_heavy = k.max_heavy;
   b.wuser = reinterpret_cast<int32_t*>(w + k.wuser);
   b.wbase = reinterpret_cast<int32_t*>(w + k.wbase);
+  b.stream_mem = w + k.sx;
   b.scratch = d_scratch;
   b.scratch_bytes = scratch_bytes;
   b.status = c->status;
@@ -587,7 +589,7 @@ esspt_status esspt_mf_load(esspt_ctx* c, const int32_t* d_i, const int32_t* d_j,
     const int64_t warps = std::min(stream_max_warps(c->K), (items + geo.gpw - 1) / geo.gpw);
     ptb[f + 1] = ptb[f] + warps;
     if (ptb[f + 1] > k.part_rows) return fail(c, ESSPT_ECUDA, "internal: work split overflow");
-    ESSPT_CUDA(c, launch_stream_partition(b.pre + chb[f], items, warps, part + ptb[f], c->st));
+    ESSPT_CUDA(c, launch_stream_partition(b.pre + chb[f], items, warps, geo, part + ptb[f], c->st));
     ESSPT_CUDA(c, launch_stream_steps(b.chunk + chb[f], part + ptb[f], warps, geo, steps + f, c->st));
   }
   std::vector<int64_t> n_steps((size_t)F);

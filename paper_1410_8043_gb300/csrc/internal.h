@@ -207,7 +207,8 @@ struct StreamSource {
   int64_t n_items;
   int32_t K, dR_ld;
 };
-cudaError_t launch_stream_partition(const int64_t* pre, int64_t n_items, int64_t n_warps, int4* part, cudaStream_t st);
+cudaError_t launch_stream_partition(const int64_t* pre, int64_t n_items, int64_t n_warps, const StreamGeometry& g,
+                                    int4* part, cudaStream_t st);
 cudaError_t launch_stream_steps(const int4* items, int4* part, int64_t n_warps, const StreamGeometry& g,
                                 int64_t* total, cudaStream_t st);
 cudaError_t launch_stream_fill(const int4* items, const int4* part, int64_t n_warps, const StreamGeometry& g,
@@ -290,21 +291,24 @@ struct LayoutBuild {
   int32_t* item_rep;    // [n_items+1]
   int4* popular;        // [max_popular] items with extra replicas (see MergeArgs), in no order
   uint32_t* n_popular;  // their number
-  int4* chunk;          // [max_chunks] work items (see StreamArgs)
+  int4* chunk;          // [max_chunks] work items (see StreamArgs); before that 3 words per item of the build's
   int64_t* chunk_base;  // [F+1]
   int4* heavy;          // [max_heavy]
   int64_t* heavy_base;  // [F+1]
   int32_t* wuser;       // [n_users] users by worker, ascending within a worker
   int32_t* wbase;       // [P+1] first of each worker's users
   int64_t max_chunks, max_heavy;
-  // scratch
+  // scratch, and the stream's memory, which is free until the stream is filled
   void* scratch;
   size_t scratch_bytes;
-  const int64_t* pre;   // out, in the scratch: [items+1] summed cost of the items before each
+  void* stream_mem;     // layout_stage_bytes
+  const int64_t* pre;   // out, in stream_mem: [items+1] summed cost of the items before each
   uint32_t* status;
 };
 
 size_t layout_scratch_bytes(int64_t n_obs, int64_t n_users, int64_t n_items, int32_t F);
+size_t layout_stage_bytes(int64_t n_obs, int64_t n_users, int32_t F);
+size_t layout_chunk_bytes(int64_t n_obs, int64_t n_users, int32_t F);
 int64_t layout_max_chunks(int64_t n_obs, int32_t F, int64_t n_users);
 int64_t layout_max_heavy(int64_t n_obs, int32_t F);
 int64_t layout_max_popular(int64_t n_obs);

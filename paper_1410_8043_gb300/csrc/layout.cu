@@ -10,6 +10,8 @@
 
 #include <cub/device/device_radix_sort.cuh>
 #include <cub/device/device_scan.cuh>
+#include <thrust/iterator/counting_iterator.h>
+#include <thrust/iterator/transform_iterator.h>
 
 #include "internal.h"
 
@@ -189,20 +191,23 @@ __global__ void iota_kernel(uint32_t* __restrict__ val, int64_t n) {
   for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += stride) val[k] = (uint32_t)k;
 }
 
-// The work list in its final order, and each item's cost (64 bits: a scan adds
-// in its input's type, and the costs of a data set pass 2^31).
+// The work list in its final order.
 __global__ void place_items_kernel(const int4* __restrict__ raw, const uint32_t* __restrict__ perm, int64_t n,
-                                   int4* __restrict__ items, int64_t* __restrict__ cost) {
+                                   int4* __restrict__ items) {
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x <= n; x += stride) {
-    if (x == n) {
-      cost[x] = 0;
-      continue;
-    }
-    const int4 it = raw[perm[x]];
-    items[x] = it;
-    cost[x] = (it.w >> 16) + kItemCost;
-  }
+  for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < n; x += stride) items[x] = raw[perm[x]];
+}
+
+// Cost of item x (64 bits: a scan adds in its input's type, and the costs of a
+// data set pass 2^31); 0 past the last.
+struct ItemCost {
+  const int4* items;
+  int64_t n;
+  __host__ __device__ int64_t operator()(int64_t x) const { return x < n ? (items[x].w >> 16) + kItemCost : 0; }
+};
+cudaError_t scan_costs(void* tmp, size_t& bytes, const int4* items, int64_t n, int64_t* pre, cudaStream_t st) {
+  const auto cost = thrust::make_transform_iterator(thrust::counting_iterator<int64_t>(0), ItemCost{items, n});
+  return cub::DeviceScan::ExclusiveSum(tmp, bytes, cost, pre, (int)(n + 1), st);
 }
 
 // The items with extra replicas.
@@ -265,23 +270,26 @@ int blocks_for(int64_t n) {
   return (int)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, (int64_t)sms * 16));
 }
 
+int64_t max_items(int64_t n_obs, int64_t n_users, int32_t F) {  // an item holds an entry or more
+  return std::min(n_obs, layout_max_chunks(n_obs, F, n_users));
+}
+
 struct ScratchPlan {
-  size_t key_in, key_out, val_in, val_out, cnt, off, nch, choff, hflag, hoff, hextra, hext, ireps, raw, pre, cub, total;
+  size_t val_out, cnt, nch, off, choff, hflag, hoff, hextra, ireps, cub, total;
   size_t cub_bytes;
 };
 
 ScratchPlan plan(int64_t n_obs, int64_t n_users, int64_t n_items, int32_t F) {
   ScratchPlan p{};
   const int64_t keys = (int64_t)F * n_users;
-  const int64_t items = std::min(n_obs, layout_max_chunks(n_obs, F, n_users));  // an item holds an entry or more
   size_t sort_bytes = 0, scan_bytes = 0, scan2_bytes = 0, scan3_bytes = 0;
-  cub::DeviceRadixSort::SortPairs(nullptr, sort_bytes, (const uint32_t*)nullptr, (uint32_t*)nullptr,
-                                  (const uint32_t*)nullptr, (uint32_t*)nullptr, (int)std::max<int64_t>(std::max(n_obs, n_users), 1), 0,
-                                  32);
+  cub::DoubleBuffer<uint32_t> none(nullptr, nullptr);
+  cub::DeviceRadixSort::SortPairs(nullptr, sort_bytes, none, none,
+                                  (int)std::max<int64_t>(std::max(n_obs, n_users), 1), 0, 32);
   cub::DeviceScan::ExclusiveSum(nullptr, scan_bytes, (const int32_t*)nullptr, (int64_t*)nullptr, (int)(keys + 1));
   cub::DeviceScan::ExclusiveSum(nullptr, scan2_bytes, (const int32_t*)nullptr, (int32_t*)nullptr,
                                 (int)(n_items + 1));
-  cub::DeviceScan::ExclusiveSum(nullptr, scan3_bytes, (const int64_t*)nullptr, (int64_t*)nullptr, (int)(items + 1));
+  scan_costs(nullptr, scan3_bytes, nullptr, max_items(n_obs, n_users, F), nullptr, nullptr);
   p.cub_bytes = std::max(std::max(sort_bytes, scan3_bytes), std::max(scan_bytes, scan2_bytes));
   size_t o = 0;
   auto take = [&o](size_t bytes) {
@@ -289,24 +297,28 @@ ScratchPlan plan(int64_t n_obs, int64_t n_users, int64_t n_items, int32_t F) {
     o += align256(bytes);
     return at;
   };
-  p.key_in = take(sizeof(uint32_t) * (n_obs + 1));
-  p.key_out = take(sizeof(uint32_t) * n_obs);
-  p.val_in = take(sizeof(uint32_t) * n_obs);
   p.val_out = take(sizeof(uint32_t) * n_obs);
   p.cnt = take(sizeof(int32_t) * (keys + 1));
-  p.off = take(sizeof(int64_t) * (keys + 1));
   p.nch = take(sizeof(int32_t) * (keys + 1));
+  p.off = take(sizeof(int64_t) * (keys + 1));  // then the extra replica rows before each heavy user
   p.choff = take(sizeof(int64_t) * (keys + 1));
   p.hflag = take(sizeof(int32_t) * (keys + 1));
   p.hoff = take(sizeof(int64_t) * (keys + 1));
   p.hextra = take(sizeof(int32_t) * (keys + 1));
-  p.hext = take(sizeof(int64_t) * (keys + 1));
   p.ireps = take(sizeof(int32_t) * (n_items + 1));
-  p.raw = take(sizeof(int4) * items);
-  p.pre = take(sizeof(int64_t) * (items + 1));
   p.cub = take(p.cub_bytes);
   p.total = o;
   return p;
+}
+
+// The build's sorts in memory that the load has in hand for later: both buffers
+// of the keys and one of the ids of n entries or items.
+struct SortPlan {
+  size_t key_in, key_out, val_in, total;
+};
+SortPlan sort_plan(int64_t n) {
+  const size_t words = align256(sizeof(uint32_t) * (size_t)n);
+  return SortPlan{0, words, 2 * words, 3 * words};
 }
 
 int bits_for(uint64_t max_key) {
@@ -315,10 +327,34 @@ int bits_for(uint64_t max_key) {
   return b;
 }
 
+// Sorts n pairs on the keys' low bits, stable, between the two buffers of each
+// (sorting into separate ones takes 8 bytes a pair more): ids in vals[0] on entry,
+// sorted in *sorted, which is vals[0] or vals[1].
+cudaError_t sort_ids(void* tmp, size_t bytes, uint32_t* key0, uint32_t* key1, uint32_t* val0, uint32_t* val1, int64_t n,
+                     int bits, uint32_t** sorted, uint32_t** sorted_keys, cudaStream_t st) {
+  cub::DoubleBuffer<uint32_t> keys(key0, key1), vals(val0, val1);
+  const cudaError_t e = cub::DeviceRadixSort::SortPairs(tmp, bytes, keys, vals, (int)n, 0, bits, st);
+  *sorted = vals.Current();
+  *sorted_keys = keys.Current();
+  return e;
+}
+
 }  // namespace
 
 size_t layout_scratch_bytes(int64_t n_obs, int64_t n_users, int64_t n_items, int32_t F) {
   return plan(n_obs, n_users, n_items, F).total;
+}
+
+// In the stream's memory: the sort of the entries, then the work items in user
+// order, then their summed costs.
+size_t layout_stage_bytes(int64_t n_obs, int64_t n_users, int32_t F) {
+  const int64_t items = max_items(n_obs, n_users, F);
+  return std::max(sort_plan(n_obs).total, align256(std::max(sizeof(int4) * items, sizeof(int64_t) * (items + 1))));
+}
+// In the work list's: the sort of the items.
+size_t layout_chunk_bytes(int64_t n_obs, int64_t n_users, int32_t F) {
+  const int64_t items = max_items(n_obs, n_users, F);
+  return std::max(sort_plan(items).total, sizeof(int4) * (size_t)layout_max_chunks(n_obs, F, n_users));
 }
 
 // A heavy segment has n > kHeavy >= kChunk entries and ceil(n/kChunk) < 2n/kChunk chunks.
@@ -342,9 +378,11 @@ cudaError_t build_layout(LayoutBuild& b, cudaStream_t st) {
   const ScratchPlan p = plan(b.n_obs, b.n_users, b.n_items, b.F);
   if (b.scratch_bytes < p.total) return cudaErrorInvalidValue;
   char* s = static_cast<char*>(b.scratch);
-  uint32_t* key_in = reinterpret_cast<uint32_t*>(s + p.key_in);
-  uint32_t* key_out = reinterpret_cast<uint32_t*>(s + p.key_out);
-  uint32_t* val_in = reinterpret_cast<uint32_t*>(s + p.val_in);
+  const SortPlan q = sort_plan(b.n_obs);
+  char* m = static_cast<char*>(b.stream_mem);
+  uint32_t* key_in = reinterpret_cast<uint32_t*>(m + q.key_in);
+  uint32_t* key_out = reinterpret_cast<uint32_t*>(m + q.key_out);
+  uint32_t* val_in = reinterpret_cast<uint32_t*>(m + q.val_in);
   uint32_t* val_out = reinterpret_cast<uint32_t*>(s + p.val_out);
   int32_t* cnt = reinterpret_cast<int32_t*>(s + p.cnt);
   int64_t* off = reinterpret_cast<int64_t*>(s + p.off);
@@ -353,10 +391,11 @@ cudaError_t build_layout(LayoutBuild& b, cudaStream_t st) {
   int32_t* hflag = reinterpret_cast<int32_t*>(s + p.hflag);
   int64_t* hoff = reinterpret_cast<int64_t*>(s + p.hoff);
   int32_t* hextra = reinterpret_cast<int32_t*>(s + p.hextra);
-  int64_t* hext = reinterpret_cast<int64_t*>(s + p.hext);
+  int64_t* hext = off;
   int32_t* ireps = reinterpret_cast<int32_t*>(s + p.ireps);
   void* cub_tmp = s + p.cub;
   const int64_t keys = (int64_t)b.F * b.n_users;
+  uint32_t *perm = nullptr, *sorted = nullptr;
   cudaError_t e;
 
   for (void* z : {(void*)cnt, (void*)nch, (void*)hflag, (void*)hextra})
@@ -366,11 +405,10 @@ cudaError_t build_layout(LayoutBuild& b, cudaStream_t st) {
                                                   b.item_cnt);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if (b.n_obs > 0) {
-    size_t tb = p.cub_bytes;
-    e = cub::DeviceRadixSort::SortPairs(cub_tmp, tb, key_in, key_out, val_in, val_out, (int)b.n_obs, 0,
-                                        bits_for((uint64_t)keys), st);
+    e = sort_ids(cub_tmp, p.cub_bytes, key_in, key_out, val_in, val_out, b.n_obs, bits_for((uint64_t)keys), &perm,
+                 &sorted, st);
     if (e != cudaSuccess) return e;
-    gather_kernel<<<blocks_for(b.n_obs), 256, 0, st>>>(val_out, b.n_obs, b.i, b.j, b.D, b.rec_u, b.rec_j, b.rec_D);
+    gather_kernel<<<blocks_for(b.n_obs), 256, 0, st>>>(perm, b.n_obs, b.i, b.j, b.D, b.rec_u, b.rec_j, b.rec_D);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   size_t tb = p.cub_bytes;
@@ -396,8 +434,12 @@ cudaError_t build_layout(LayoutBuild& b, cudaStream_t st) {
   if (b.n_obs > 0 && (e = build_hot(b, st)) != cudaSuccess) return e;
   // The work list, then its order: by tile of users and length, ties in user
   // order (the sort is stable).  The sort buffers of the entries are free now.
-  int4* raw = reinterpret_cast<int4*>(s + p.raw);
-  int64_t* pre = reinterpret_cast<int64_t*>(s + p.pre);
+  int4* raw = static_cast<int4*>(b.stream_mem);
+  int64_t* pre = static_cast<int64_t*>(b.stream_mem);
+  const SortPlan qi = sort_plan(max_items(b.n_obs, b.n_users, b.F));
+  key_in = reinterpret_cast<uint32_t*>(reinterpret_cast<char*>(b.chunk) + qi.key_in);
+  key_out = reinterpret_cast<uint32_t*>(reinterpret_cast<char*>(b.chunk) + qi.key_out);
+  val_in = reinterpret_cast<uint32_t*>(reinterpret_cast<char*>(b.chunk) + qi.val_in);
   const int64_t n_tiles = (b.n_users >> kTileBits) + 1;
   heavy_kernel<<<blocks_for(keys + 1), 256, 0, st>>>(
       choff, nch, hoff, hext, b.uoff, b.worker, b.n_users, b.F, raw, key_in, val_in, n_tiles, b.chunk_base,
@@ -408,42 +450,49 @@ cudaError_t build_layout(LayoutBuild& b, cudaStream_t st) {
   if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return e;
   if (n > std::min(b.n_obs, b.max_chunks)) return cudaErrorInvalidValue;
   b.pre = pre;
-  // Users by worker (cnt and nch, [F n_users + 1] each, are free now).
+  // Users by worker (cnt, nch and hflag, [F n_users + 1] each, are free now).
   uint32_t* ids = reinterpret_cast<uint32_t*>(cnt);
-  uint32_t* sorted = reinterpret_cast<uint32_t*>(nch);
+  uint32_t* worker = reinterpret_cast<uint32_t*>(hflag);
+  uint32_t* wuser = reinterpret_cast<uint32_t*>(b.wuser);
   iota_kernel<<<blocks_for(b.n_users), 256, 0, st>>>(ids, b.n_users);
-  tb = p.cub_bytes;
-  e = cub::DeviceRadixSort::SortPairs(cub_tmp, tb, reinterpret_cast<const uint32_t*>(b.worker), sorted, ids,
-                                      reinterpret_cast<uint32_t*>(b.wuser), (int)b.n_users, 0, bits_for(b.P), st);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  e = cudaMemcpyAsync(worker, b.worker, sizeof(int32_t) * b.n_users, cudaMemcpyDeviceToDevice, st);
+  if (e != cudaSuccess) return e;
+  e = sort_ids(cub_tmp, p.cub_bytes, worker, reinterpret_cast<uint32_t*>(nch), ids, wuser, b.n_users, bits_for(b.P), &perm,
+               &sorted, st);
+  if (e == cudaSuccess && perm != wuser)
+    e = cudaMemcpyAsync(wuser, perm, sizeof(uint32_t) * b.n_users, cudaMemcpyDeviceToDevice, st);
   if (e != cudaSuccess) return e;
   worker_bases_kernel<<<b.P / 256 + 1, 256, 0, st>>>(sorted, b.n_users, b.P, b.wbase);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if (n > 0) {
-    tb = p.cub_bytes;
-    e = cub::DeviceRadixSort::SortPairs(cub_tmp, tb, key_in, key_out, val_in, val_out, (int)n, 0,
-                                        bits_for((uint64_t)b.F * n_tiles << 7), st);
+    e = sort_ids(cub_tmp, p.cub_bytes, key_in, key_out, val_in, val_out, n, bits_for((uint64_t)b.F * n_tiles << 7), &perm,
+                 &sorted, st);
+    // (the work list is written where the other buffers are)
+    if (e == cudaSuccess && perm != val_out)
+      e = cudaMemcpyAsync(val_out, perm, sizeof(uint32_t) * n, cudaMemcpyDeviceToDevice, st);
     if (e != cudaSuccess) return e;
   }
-  // The costs take the place of both key arrays, side by side and free now: 8 (n + 1) bytes of at least 8 (n_obs + 1).
-  int64_t* cost = reinterpret_cast<int64_t*>(key_in);
-  place_items_kernel<<<blocks_for(n + 1), 256, 0, st>>>(raw, val_out, n, b.chunk, cost);
+  place_items_kernel<<<blocks_for(n), 256, 0, st>>>(raw, val_out, n, b.chunk);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   tb = p.cub_bytes;
-  return cub::DeviceScan::ExclusiveSum(cub_tmp, tb, cost, pre, (int)(n + 1), st);
+  return scan_costs(cub_tmp, tb, b.chunk, n, pre, st);
 }
 
-// A round takes gpw * per_step places per step of its longest item.  In a sorted
-// run its longest item is no longer than any of the round before it, so all but
-// two rounds per run cost no more than the entries of the round before, each
-// rounded up to whole steps; those two cost at most kHeavy entries' steps.  A
-// run ends with a tile or a warp; a warp's first step is aligned.
+// A round takes gpw * per_step places per step of its longest item, and the
+// warps take whole rounds: those of a minibatch are its items gpw at a time, the
+// last one partial.  With each item's entries rounded up to whole steps, a round's
+// empty places are at most (gpw - 1) times the rise and fall of the lengths in it.
+// Over a minibatch the lengths rise only from one tile of users to the next, so
+// rise and fall add up to less than 2 kHeavy per tile, and to less than twice the
+// entries.  A warp's first step is aligned.
 int64_t layout_max_places(int64_t n_obs, int64_t n_users, int32_t F, const StreamGeometry& g, int64_t max_warps) {
-  const int64_t items = std::min(n_obs, layout_max_chunks(n_obs, F, n_users));
-  const int64_t warps = std::min((int64_t)F * max_warps, items);
-  const int64_t runs = (int64_t)F * ((n_users >> kTileBits) + 1) + warps;
-  const int64_t step = (int64_t)g.gpw * g.per_step;
-  return std::min(step * n_obs, n_obs + (items + g.gpw * warps) * (g.per_step - 1) +
-                                    2 * runs * g.gpw * (kHeavy + g.per_step)) + kStepAlign * step * (warps + F);
+  const int64_t items = max_items(n_obs, n_users, F);
+  const int64_t warps = std::min((int64_t)F * max_warps, items / g.gpw + F);
+  const int64_t tiles = (int64_t)F * ((n_users >> kTileBits) + 1), step = (int64_t)g.gpw * g.per_step;
+  const int64_t uneven = std::min(2 * kHeavy * tiles, 2 * (n_obs + items * (g.per_step - 1)));
+  const int64_t places = n_obs + items * (g.per_step - 1) + (g.gpw - 1) * uneven + F * g.gpw * (kHeavy + g.per_step);
+  return std::min(step * n_obs, places) + kStepAlign * step * (warps + F);
 }
 
 cudaError_t launch_stage_check(const int32_t* su, const int32_t* sj, const int32_t* suoff, const int32_t* ru,

@@ -10,13 +10,18 @@ namespace esspt {
 
 // Warp w of n_warps takes items [part[w].x, part[w].y), the shares balanced by
 // cost: pre[x] is the summed cost of the items before x (over all minibatches).
+// They are whole rounds but for the minibatch's last, so that the empty places of
+// partial rounds do not add up over the warps; one round each where that is all.
 __global__ void __launch_bounds__(256) stream_partition_kernel(const int64_t* __restrict__ pre, int32_t n_items,
-                                                               int32_t n_warps, int4* __restrict__ part) {
+                                                               int32_t n_warps, int32_t gpw,
+                                                               int4* __restrict__ part) {
   const int32_t w = blockIdx.x * blockDim.x + threadIdx.x;
   if (w > n_warps) return;
   int32_t lo = 0, hi = n_items;
   if (w == n_warps) {
     lo = n_items;
+  } else if ((int64_t)n_warps * gpw >= n_items) {
+    lo = w * gpw;
   } else {
     const int64_t target = pre[0] + (int64_t)((double)(pre[n_items] - pre[0]) * w / n_warps);
     while (lo < hi) {
@@ -27,15 +32,16 @@ __global__ void __launch_bounds__(256) stream_partition_kernel(const int64_t* __
         lo = m + 1;
       }
     }
+    lo = (int32_t)min((int64_t)n_items, ((int64_t)lo + gpw / 2) / gpw * gpw);
   }
   if (w < n_warps) part[w].x = lo;
   if (w > 0) part[w - 1].y = lo;
 }
 
-cudaError_t launch_stream_partition(const int64_t* pre, int64_t n_items, int64_t n_warps, int4* part,
-                                    cudaStream_t st) {
+cudaError_t launch_stream_partition(const int64_t* pre, int64_t n_items, int64_t n_warps, const StreamGeometry& g,
+                                    int4* part, cudaStream_t st) {
   stream_partition_kernel<<<(unsigned)(n_warps / 256 + 1), 256, 0, st>>>(pre, (int32_t)n_items, (int32_t)n_warps,
-                                                                        part);
+                                                                        g.gpw, part);
   return cudaGetLastError();
 }
 
