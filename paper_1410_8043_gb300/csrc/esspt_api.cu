@@ -209,9 +209,19 @@ bool is_host_ptr(const void* p) {
 }
 
 struct MfCarve {
-  size_t rec_u, rec_j, rec_D, sx, syz, place, steps, uoff, mb_base, item_cnt, item_rep, dR, wuser, wbase, chunk, chunk_base, heavy, heavy_base, dL,
-      user_slot, row_x, chg, chg_item, popular, n_popular, hot_item, part, total;
+  size_t rec_u, rec_j, rec_D, sx, syz, place, uoff, bases, item_cnt, item_rep, dR, wuser, wbase, chunk, heavy, dL, user_slot,
+      row_x, chg, chg_item, popular, hot_item, part, total;
   int64_t max_chunks, max_heavy, dR_rows, dL_rows, part_rows, max_places;
+};
+
+// What the host reads back of a load, side by side in 64-bit words: the first
+// entry, work item, heavy user, warp and place of each minibatch (and the ends),
+// the steps of each, the number of popular items, and the status word.
+struct Bases {
+  int64_t entry, item, heavy, part, place, steps, n_popular, status, words;
+  explicit Bases(int32_t F)
+      : entry(0), item(F + 1), heavy(2 * (F + 1)), part(3 * (F + 1)), place(4 * (F + 1)), steps(5 * (F + 1)),
+        n_popular(steps + F), status(n_popular + 1), words(status + 1) {}
 };
 
 // Persistent MF workspace: entries laid out by (minibatch, user), per-minibatch
@@ -238,18 +248,15 @@ MfCarve mf_carve(int64_t n_obs, int64_t n_users, int64_t n_items, int32_t F, int
   k.syz = take(2 * sizeof(uint32_t) * k.max_places);
   k.place = take(sizeof(uint32_t) * k.max_chunks);
   o = std::max(o, k.sx + layout_stage_bytes(n_obs, n_users, F));  // the load uses the stream's memory before
-  k.steps = take(sizeof(int64_t) * F);
   k.uoff = take(sizeof(int32_t) * (size_t)F * (n_users + 1));
-  k.mb_base = take(sizeof(int64_t) * (F + 1));
+  k.bases = take(sizeof(int64_t) * Bases(F).words);
   k.item_cnt = take(sizeof(int32_t) * (size_t)F * n_items);
   k.item_rep = take(sizeof(int32_t) * (n_items + 1));
   k.dR = take(sizeof(float4) * (size_t)k.dR_rows * dR_stride4(K));
   k.wuser = take(sizeof(int32_t) * n_users);
   k.wbase = take(sizeof(int32_t) * (P + 1));
   k.chunk = take(layout_chunk_bytes(n_obs, n_users, F));
-  k.chunk_base = take(sizeof(int64_t) * (F + 1));
   k.heavy = take(sizeof(int4) * k.max_heavy);
-  k.heavy_base = take(sizeof(int64_t) * (F + 1));
   k.dL = take(sizeof(float) * (size_t)k.dL_rows * K);
   // Row-granular SSP: per-clock user slots and x words of the stream.
   k.user_slot = row_mode ? take(sizeof(int32_t) * n_users) : o;
@@ -258,7 +265,6 @@ MfCarve mf_carve(int64_t n_obs, int64_t n_users, int64_t n_items, int32_t F, int
   k.chg = take(sizeof(int32_t) * n_users);
   k.chg_item = take(sizeof(int32_t) * n_items);
   k.popular = take(sizeof(int4) * layout_max_popular(n_obs));
-  k.n_popular = take(sizeof(uint32_t));
   k.hot_item = uses_hot(K) ? take(sizeof(int32_t) * (size_t)F * kHot) : o;
   // A minibatch uses at most one warp per work item.
   k.part_rows = std::min((int64_t)F * stream_max_warps(K), k.max_chunks);
@@ -528,16 +534,18 @@ esspt_status esspt_mf_load(esspt_ctx* c, const int32_t* d_i, const int32_t* d_j,
   b.rec_j = reinterpret_cast<int32_t*>(w + k.rec_j);
   b.rec_D = reinterpret_cast<float*>(w + k.rec_D);
   b.uoff = reinterpret_cast<int32_t*>(w + k.uoff);
-  b.mb_base = reinterpret_cast<int64_t*>(w + k.mb_base);
+  const Bases at(F);
+  int64_t* bases = reinterpret_cast<int64_t*>(w + k.bases);
+  b.mb_base = bases + at.entry;
   b.item_cnt = reinterpret_cast<int32_t*>(w + k.item_cnt);
   b.item_rep = reinterpret_cast<int32_t*>(w + k.item_rep);
   b.hot_item = uses_hot(c->K) ? reinterpret_cast<int32_t*>(w + k.hot_item) : nullptr;
   b.chunk = reinterpret_cast<int4*>(w + k.chunk);
-  b.chunk_base = reinterpret_cast<int64_t*>(w + k.chunk_base);
+  b.chunk_base = bases + at.item;
   b.heavy = reinterpret_cast<int4*>(w + k.heavy);
   b.popular = reinterpret_cast<int4*>(w + k.popular);
-  b.n_popular = reinterpret_cast<uint32_t*>(w + k.n_popular);
-  b.heavy_base = reinterpret_cast<int64_t*>(w + k.heavy_base);
+  b.n_popular = reinterpret_cast<uint32_t*>(bases + at.n_popular);
+  b.heavy_base = bases + at.heavy;
   b.max_chunks = k.max_chunks;
   b.max_heavy = k.max_heavy;
   b.wuser = reinterpret_cast<int32_t*>(w + k.wuser);
@@ -563,55 +571,56 @@ esspt_status esspt_mf_load(esspt_ctx* c, const int32_t* d_i, const int32_t* d_j,
   ESSPT_CUDA(c, cudaMemsetAsync(b.rec_u + n_obs, 0, 16, c->st));
   ESSPT_CUDA(c, cudaMemsetAsync(b.rec_j + n_obs, 0, 16, c->st));
   ESSPT_CUDA(c, cudaMemsetAsync(b.rec_D + n_obs, 0, 16, c->st));
+  ESSPT_CUDA(c, cudaMemsetAsync(bases, 0, sizeof(int64_t) * at.words, c->st));
   ESSPT_CUDA(c, build_layout(b, c->st));
-  std::vector<int64_t> mbb((size_t)F + 1), chb((size_t)F + 1), hvb((size_t)F + 1);
-  ESSPT_CUDA(c, cudaMemcpyAsync(mbb.data(), b.mb_base, sizeof(int64_t) * (F + 1), cudaMemcpyDeviceToHost, c->st));
-  ESSPT_CUDA(c, cudaMemcpyAsync(chb.data(), b.chunk_base, sizeof(int64_t) * (F + 1), cudaMemcpyDeviceToHost, c->st));
-  uint32_t n_popular = 0;
-  ESSPT_CUDA(c, cudaMemcpyAsync(&n_popular, b.n_popular, sizeof n_popular, cudaMemcpyDeviceToHost, c->st));
-  ESSPT_CUDA(c, cudaMemcpyAsync(hvb.data(), b.heavy_base, sizeof(int64_t) * (F + 1), cudaMemcpyDeviceToHost, c->st));
-  ESSPT_CUDA(c, cudaMemcpyAsync(&bits, c->status, sizeof bits, cudaMemcpyDeviceToHost, c->st));
-  ESSPT_CUDA(c, cudaStreamSynchronize(c->st));
-  if (chb[F] > k.max_chunks || hvb[F] > k.max_heavy || (bits & kErrInput)) {
-    ESSPT_CUDA(c, cudaMemsetAsync(c->status, 0, sizeof(uint32_t), c->st));
-    return fail(c, ESSPT_ECUDA, "internal: chunk list overflow");
-  }
-  // Split each minibatch's work items over the warps of the SGD kernel.
+  // The stream that the SGD kernel takes each minibatch's work items in.
   const StreamGeometry geo = stream_geometry(c->K);
-  std::vector<int64_t> ptb((size_t)F + 1, 0);
   int4* part = reinterpret_cast<int4*>(w + k.part);
   uint32_t* sx = reinterpret_cast<uint32_t*>(w + k.sx);
   uint32_t* syz = reinterpret_cast<uint32_t*>(w + k.syz);
   uint32_t* place = reinterpret_cast<uint32_t*>(w + k.place);
-  int64_t* steps = reinterpret_cast<int64_t*>(w + k.steps);
-  for (int32_t f = 0; f < F; ++f) {
-    const int64_t items = chb[f + 1] - chb[f];
-    const int64_t warps = std::min(stream_max_warps(c->K), (items + geo.gpw - 1) / geo.gpw);
-    ptb[f + 1] = ptb[f] + warps;
-    if (ptb[f + 1] > k.part_rows) return fail(c, ESSPT_ECUDA, "internal: work split overflow");
-    ESSPT_CUDA(c, launch_stream_partition(b.pre + chb[f], items, warps, geo, part + ptb[f], c->st));
-    ESSPT_CUDA(c, launch_stream_steps(b.chunk + chb[f], part + ptb[f], warps, geo, steps + f, c->st));
-  }
-  std::vector<int64_t> n_steps((size_t)F);
-  ESSPT_CUDA(c, cudaMemcpyAsync(n_steps.data(), steps, sizeof(int64_t) * F, cudaMemcpyDeviceToHost, c->st));
+  StreamBuild sb{};
+  sb.items = b.chunk;
+  sb.item_base = b.chunk_base;
+  sb.entry_base = b.mb_base;
+  sb.pre = b.pre;
+  sb.status = c->status;
+  sb.F = F;
+  sb.max_items = b.n_work;
+  sb.max_warps = stream_max_warps(c->K);
+  sb.g = geo;
+  sb.rec_j = b.rec_j;
+  sb.rec_D = b.rec_D;
+  sb.item_rep = b.item_rep;
+  sb.hot_item = b.hot_item;
+  sb.n_items = n_items;
+  sb.K = c->K;
+  sb.dR_ld = dR_stride4(c->K);
+  sb.max_places = k.max_places;
+  sb.part = part;
+  sb.part_base = bases + at.part;
+  sb.place_base = bases + at.place;
+  sb.steps = bases + at.steps;
+  sb.x = sx;
+  sb.yz = syz;
+  sb.place = place;
+  ESSPT_CUDA(c, launch_stream_build(sb, c->st));
+  std::vector<int64_t> h((size_t)at.words);
+  ESSPT_CUDA(c, cudaMemcpyAsync(bases + at.status, c->status, sizeof(uint32_t), cudaMemcpyDeviceToDevice, c->st));
+  ESSPT_CUDA(c, cudaMemcpyAsync(h.data(), bases, sizeof(int64_t) * at.words, cudaMemcpyDeviceToHost, c->st));
   ESSPT_CUDA(c, cudaStreamSynchronize(c->st));
-  std::vector<int64_t> rcb((size_t)F + 1, 0);
-  for (int32_t f = 0; f < F; ++f) {
-    const int64_t places = n_steps[f] * geo.gpw * geo.per_step;
-    rcb[f + 1] = rcb[f] + places;
-    if (n_steps[f] > kMaxSteps || rcb[f + 1] > k.max_places) return fail(c, ESSPT_ECUDA, "internal: stream overflow");
-    StreamSource src{};
-    src.rec_j = b.rec_j + mbb[f];
-    src.rec_D = b.rec_D + mbb[f];
-    src.item_rep = b.item_rep;
-    src.hot_item = b.hot_item ? b.hot_item + (int64_t)f * kHot : nullptr;
-    src.n_items = n_items;
-    src.K = c->K;
-    src.dR_ld = dR_stride4(c->K);
-    ESSPT_CUDA(c, launch_stream_fill(b.chunk + chb[f], part + ptb[f], ptb[f + 1] - ptb[f], geo, src, places,
-                                     sx + rcb[f], syz + 2 * rcb[f], place + chb[f], c->st));
+  auto words = [&](int64_t first) {
+    return std::vector<int64_t>(h.begin() + first, h.begin() + first + F + 1);
+  };
+  const std::vector<int64_t> mbb = words(at.entry), chb = words(at.item), hvb = words(at.heavy), ptb = words(at.part),
+                             rcb = words(at.place);
+  if (chb[F] > k.max_chunks || hvb[F] > k.max_heavy || (h[at.status] & kErrInput)) {
+    ESSPT_CUDA(c, cudaMemsetAsync(c->status, 0, sizeof(uint32_t), c->st));
+    return fail(c, ESSPT_ECUDA, "internal: chunk list overflow");
   }
-  ESSPT_CUDA(c, cudaStreamSynchronize(c->st));
+  if (ptb[F] > k.part_rows) return fail(c, ESSPT_ECUDA, "internal: work split overflow");
+  if (rcb[F] > k.max_places || *std::max_element(h.begin() + at.steps, h.begin() + at.steps + F) > kMaxSteps)
+    return fail(c, ESSPT_ECUDA, "internal: stream overflow");
   c->part = part;
   c->part_base = ptb;
   c->n_users = n_users;
@@ -647,7 +656,7 @@ esspt_status esspt_mf_load(esspt_ctx* c, const int32_t* d_i, const int32_t* d_j,
   c->chg_item = reinterpret_cast<int32_t*>(w + k.chg_item);
   ESSPT_CUDA(c, cudaMemsetAsync(c->chg_item, 0, sizeof(int32_t) * (size_t)n_items, c->st));
   c->popular = b.popular;
-  c->n_popular = n_popular;
+  c->n_popular = h[at.n_popular];
   // rows changed before this load are not tracked
   c->copy_all_until = c->clock + c->s + 1;
   c->mb_base = mbb;

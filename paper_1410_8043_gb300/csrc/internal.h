@@ -196,24 +196,31 @@ int64_t stream_max_warps(int32_t K);
 // Whether a clock of n_warps warps and n_users users is one block per SM at most.
 bool stream_is_small(int32_t K, int64_t n_warps, int64_t n_users);
 StreamGeometry stream_geometry(int32_t K);
-// Build of a minibatch's stream (setup): the split of its n_items work items
-// over n_warps warps (pre: see LayoutBuild), the steps of the warps (their sum
-// in *total), the places (place[i] = item i's place word), and new values for them.
-struct StreamSource {
+// Build of the streams of all minibatches (setup), in four launches: the split of
+// each one's work items over its warps, the steps of the warps, the records and
+// their places (place[i] = item i's place word).  Nothing is written where status
+// holds an error or a stream passes its limits, which the caller checks.
+struct StreamBuild {
+  const int4* items;
+  const int64_t *item_base, *entry_base;  // [F+1] first item and entry of each minibatch
+  const int64_t* pre;                     // see LayoutBuild
+  const uint32_t* status;
+  int32_t F;
+  int64_t max_items, max_warps;           // of one minibatch at most
+  StreamGeometry g;
   const int32_t* rec_j;
   const float* rec_D;
   const int32_t* item_rep;
-  const int32_t* hot_item;  // [kHot] or null
+  const int32_t* hot_item;                // [F][kHot] or null
   int64_t n_items;
   int32_t K, dR_ld;
+  int64_t max_places;
+  int4* part;
+  int64_t *part_base, *place_base, *steps;  // out: [F+1], [F+1] first warp and place, [F] steps
+  uint32_t *x, *yz, *place;
 };
-cudaError_t launch_stream_partition(const int64_t* pre, int64_t n_items, int64_t n_warps, const StreamGeometry& g,
-                                    int4* part, cudaStream_t st);
-cudaError_t launch_stream_steps(const int4* items, int4* part, int64_t n_warps, const StreamGeometry& g,
-                                int64_t* total, cudaStream_t st);
-cudaError_t launch_stream_fill(const int4* items, const int4* part, int64_t n_warps, const StreamGeometry& g,
-                               const StreamSource& src, int64_t n_places, uint32_t* x, uint32_t* yz, uint32_t* place,
-                               cudaStream_t st);
+cudaError_t launch_stream_build(const StreamBuild& b, cudaStream_t st);
+// New values for the places of a minibatch.
 cudaError_t launch_stream_refill(const int4* items, const uint32_t* place, int64_t n_items, const StreamGeometry& g,
                                  const float* D, uint32_t* yz, cudaStream_t st);
 // Row-granular SSP, before the SGD kernels of clock c: refresh the cached
@@ -290,7 +297,7 @@ struct LayoutBuild {
   int32_t* item_cnt;    // [F][n_items]
   int32_t* item_rep;    // [n_items+1]
   int4* popular;        // [max_popular] items with extra replicas (see MergeArgs), in no order
-  uint32_t* n_popular;  // their number
+  uint32_t* n_popular;  // their number (0 on entry)
   int4* chunk;          // [max_chunks] work items (see StreamArgs); before that 3 words per item of the build's
   int64_t* chunk_base;  // [F+1]
   int4* heavy;          // [max_heavy]
@@ -302,6 +309,7 @@ struct LayoutBuild {
   void* scratch;
   size_t scratch_bytes;
   void* stream_mem;     // layout_stage_bytes
+  int64_t n_work;       // out: work items
   const int64_t* pre;   // out, in stream_mem: [items+1] summed cost of the items before each
   uint32_t* status;
 };

@@ -427,7 +427,6 @@ cudaError_t build_layout(LayoutBuild& b, cudaStream_t st) {
   tb = p.cub_bytes;
   if ((e = cub::DeviceScan::ExclusiveSum(cub_tmp, tb, ireps, b.item_rep, (int)(b.n_items + 1), st)) != cudaSuccess)
     return e;
-  if ((e = cudaMemsetAsync(b.n_popular, 0, sizeof(uint32_t), st)) != cudaSuccess) return e;
   popular_kernel<<<blocks_for(b.n_items), 256, 0, st>>>(b.item_rep, b.n_items, layout_max_popular(b.n_obs), b.popular,
                                                        b.n_popular, b.status);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
@@ -450,6 +449,7 @@ cudaError_t build_layout(LayoutBuild& b, cudaStream_t st) {
   if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return e;
   if (n > std::min(b.n_obs, b.max_chunks)) return cudaErrorInvalidValue;
   b.pre = pre;
+  b.n_work = n;
   // Users by worker (cnt, nch and hflag, [F n_users + 1] each, are free now).
   uint32_t* ids = reinterpret_cast<uint32_t*>(cnt);
   uint32_t* worker = reinterpret_cast<uint32_t*>(hflag);

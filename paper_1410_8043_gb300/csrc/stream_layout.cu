@@ -8,63 +8,82 @@
 
 namespace esspt {
 
-// Warp w of n_warps takes items [part[w].x, part[w].y), the shares balanced by
-// cost: pre[x] is the summed cost of the items before x (over all minibatches).
-// They are whole rounds but for the minibatch's last, so that the empty places of
-// partial rounds do not add up over the warps; one round each where that is all.
-__global__ void __launch_bounds__(256) stream_partition_kernel(const int64_t* __restrict__ pre, int32_t n_items,
-                                                               int32_t n_warps, int32_t gpw,
-                                                               int4* __restrict__ part) {
-  const int32_t w = blockIdx.x * blockDim.x + threadIdx.x;
+// Warps of a minibatch: at most one per round of its items.
+__device__ __forceinline__ int64_t warps_of(const StreamBuild& b, int32_t f) {
+  const int64_t items = __ldg(b.item_base + f + 1) - __ldg(b.item_base + f);
+  return min(b.max_warps, (items + b.g.gpw - 1) / b.g.gpw);
+}
+
+// Warp w of minibatch blockIdx.y's takes items [part[w].x, part[w].y), the shares
+// balanced by cost: pre[x] is the summed cost of the items before x (over all
+// minibatches).  They are whole rounds but for the minibatch's last, so that the
+// empty places of partial rounds do not add up over the warps; one round each
+// where that is all.
+__global__ void __launch_bounds__(256) stream_partition_kernel(StreamBuild b) {
+  const int32_t f = blockIdx.y, gpw = b.g.gpw;
+  __shared__ int64_t first;
+  if (threadIdx.x == 0) {
+    first = 0;
+    for (int32_t k = 0; k < f; ++k) first += warps_of(b, k);
+    if (blockIdx.x == 0) {
+      b.part_base[f] = first;
+      if (f == b.F - 1) b.part_base[b.F] = first + warps_of(b, f);
+    }
+  }
+  __syncthreads();
+  const int64_t x0 = __ldg(b.item_base + f), n_items = __ldg(b.item_base + f + 1) - x0, n_warps = warps_of(b, f);
+  const int64_t* pre = b.pre + x0;
+  int4* part = b.part + first;
+  const int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (w > n_warps) return;
-  int32_t lo = 0, hi = n_items;
+  int64_t lo = 0, hi = n_items;
   if (w == n_warps) {
     lo = n_items;
-  } else if ((int64_t)n_warps * gpw >= n_items) {
+  } else if (n_warps * gpw >= n_items) {
     lo = w * gpw;
   } else {
     const int64_t target = pre[0] + (int64_t)((double)(pre[n_items] - pre[0]) * w / n_warps);
     while (lo < hi) {
-      const int32_t m = lo + (hi - lo) / 2;
+      const int64_t m = lo + (hi - lo) / 2;
       if (pre[m] >= target) {
         hi = m;
       } else {
         lo = m + 1;
       }
     }
-    lo = (int32_t)min((int64_t)n_items, ((int64_t)lo + gpw / 2) / gpw * gpw);
+    lo = min(n_items, (lo + gpw / 2) / gpw * gpw);
   }
-  if (w < n_warps) part[w].x = lo;
-  if (w > 0) part[w - 1].y = lo;
+  if (w < n_warps) part[w].x = (int32_t)lo;
+  if (w > 0) part[w - 1].y = (int32_t)lo;
 }
 
-cudaError_t launch_stream_partition(const int64_t* pre, int64_t n_items, int64_t n_warps, const StreamGeometry& g,
-                                    int4* part, cudaStream_t st) {
-  stream_partition_kernel<<<(unsigned)(n_warps / 256 + 1), 256, 0, st>>>(pre, (int32_t)n_items, (int32_t)n_warps,
-                                                                        g.gpw, part);
-  return cudaGetLastError();
-}
-
-// Steps of every warp of a minibatch, in part[w].z for now.
-__global__ void __launch_bounds__(256) stream_steps_kernel(const int4* __restrict__ items, int4* part,
-                                                           int64_t n_warps, StreamGeometry g) {
-  const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (w >= n_warps) return;
+// Steps of every warp, in part[w].z for now.
+__global__ void __launch_bounds__(256) stream_steps_kernel(StreamBuild b) {
+  const int32_t f = blockIdx.y;
+  const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5, first = __ldg(b.part_base + f);
+  if (w >= __ldg(b.part_base + f + 1) - first || (*b.status & kErrInput) != 0u) return;
   const int lane = threadIdx.x & 31;
-  const int32_t x0 = part[w].x, x1 = part[w].y;
+  const int4* items = b.items + __ldg(b.item_base + f);
+  int4* part = b.part + first + w;
+  const int64_t x0 = part->x, x1 = part->y;
   uint32_t sum = 0;
-  for (int32_t r = x0 + lane * g.gpw; r < x1; r += 32 * g.gpw) {
+  for (int64_t r = x0 + lane * b.g.gpw; r < x1; r += 32 * b.g.gpw) {
     int32_t mx = 0;
-    for (int32_t x = r; x < min(r + g.gpw, x1); ++x) mx = max(mx, items[x].w >> 16);
-    sum += (mx + g.per_step - 1) / g.per_step;
+    for (int64_t x = r; x < min(r + b.g.gpw, x1); ++x) mx = max(mx, items[x].w >> 16);
+    sum += (mx + b.g.per_step - 1) / b.g.per_step;
   }
   sum = __reduce_add_sync(0xffffffffu, sum);
-  if (lane == 0) part[w].z = (int32_t)sum;
+  if (lane == 0) part->z = (int32_t)sum;
 }
+
 // part[w].z, .w = first and end step of warp w; a warp starts at a multiple of
-// kStepAlign steps, so that its records start on 16 bytes.  One block.
-__global__ void __launch_bounds__(1024) stream_offsets_kernel(int4* part, int64_t n_warps, int64_t* total) {
+// kStepAlign steps, so that its records start on 16 bytes.  One block per
+// minibatch.
+__global__ void __launch_bounds__(1024) stream_offsets_kernel(StreamBuild b) {
   __shared__ int64_t sums[1024];
+  const int32_t f = blockIdx.x;
+  int4* part = b.part + __ldg(b.part_base + f);
+  const int64_t n_warps = __ldg(b.part_base + f + 1) - __ldg(b.part_base + f);
   const int64_t per = (n_warps + 1023) / 1024, w0 = threadIdx.x * per, w1 = min(n_warps, w0 + per);
   auto aligned = [&](int64_t w) {
     return ((int64_t)(uint32_t)part[w].z + kStepAlign - 1) / kStepAlign * kStepAlign;
@@ -86,56 +105,78 @@ __global__ void __launch_bounds__(1024) stream_offsets_kernel(int4* part, int64_
     part[w].w = (int32_t)(uint32_t)(at + n);
     at = next;
   }
-  if (threadIdx.x == 1023) *total = sums[1023];
+  if (threadIdx.x == 1023) b.steps[f] = sums[1023];
 }
 
-cudaError_t launch_stream_steps(const int4* items, int4* part, int64_t n_warps, const StreamGeometry& g,
-                                int64_t* total, cudaStream_t st) {
-  stream_steps_kernel<<<(unsigned)(n_warps / 8 + 1), 256, 0, st>>>(items, part, n_warps, g);
-  stream_offsets_kernel<<<1, 1024, 0, st>>>(part, n_warps, total);
-  return cudaGetLastError();
-}
-
-// The records of a minibatch (x and yz hold kNoRecord everywhere on entry) and
-// the place of every item's first entry.  One warp per warp of the kernel.
-__global__ void __launch_bounds__(256) stream_fill_kernel(const int4* __restrict__ items,
-                                                          const int4* __restrict__ part, int64_t n_warps,
-                                                          StreamGeometry g, StreamSource src, uint32_t* __restrict__ x,
-                                                          uint32_t* __restrict__ yz, uint32_t* __restrict__ place) {
-  const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (w >= n_warps) return;
+// The records of minibatch blockIdx.y, empty places among them, and the place of
+// every item's first entry.  One warp per warp of the kernel.
+__global__ void __launch_bounds__(256) stream_fill_kernel(StreamBuild b) {
+  const int32_t f = blockIdx.y, K4 = b.K / 4;
+  const StreamGeometry g = b.g;
+  __shared__ int64_t first;
+  if (threadIdx.x == 0) {
+    first = 0;
+    for (int32_t k = 0; k < f; ++k) first += __ldg(b.steps + k) * g.gpw * g.per_step;
+    if (blockIdx.x == 0) {
+      b.place_base[f] = first;
+      if (f == b.F - 1) b.place_base[b.F] = first + __ldg(b.steps + f) * g.gpw * g.per_step;
+    }
+  }
+  __syncthreads();
+  const int64_t steps = __ldg(b.steps + f), w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (w >= __ldg(b.part_base + f + 1) - __ldg(b.part_base + f)) return;
+  if ((*b.status & kErrInput) != 0u || steps > kMaxSteps || first + steps * g.gpw * g.per_step > b.max_places) return;
   const int lane = threadIdx.x & 31, G = 32 / g.gpw, grp = lane / G, l = lane & (G - 1);
-  const int4 p = part[w];
+  const int64_t x_first = __ldg(b.item_base + f), e_first = __ldg(b.entry_base + f);
+  const int4* items = b.items + x_first;
+  const int32_t* rec_j = b.rec_j + e_first;
+  const float* rec_D = b.rec_D + e_first;
+  uint32_t *x = b.x + first, *yz = b.yz + 2 * first, *place = b.place + x_first;
+  int32_t hot[kHot];
+#pragma unroll
+  for (int h = 0; h < kHot; ++h) hot[h] = b.hot_item != nullptr ? __ldg(b.hot_item + (int64_t)f * kHot + h) : -1;
+  const int4 p = b.part[__ldg(b.part_base + f) + w];
   int64_t s = (uint32_t)p.z;
-  for (int32_t x0 = p.x; x0 < p.y; x0 += g.gpw) {
-    const int32_t i = x0 + grp;
+  for (int64_t x0 = p.x; x0 < p.y; x0 += g.gpw) {
+    const int64_t i = x0 + grp;
     const int4 it = i < p.y ? items[i] : make_int4(0, 0, -2, 0);
     const int32_t n = it.w >> 16;
+    const int32_t most = __reduce_max_sync(0xffffffffu, (n + g.per_step - 1) / g.per_step);
     const uint32_t at = place_word(g, s, grp);
     if (l == 0 && n > 0) place[i] = at;
-    for (int32_t k = l; k < n; k += G) {
-      const int32_t t = it.y + k, j = src.rec_j[t];
-      const int32_t e0 = src.item_rep[j], e1 = src.item_rep[j + 1];  // extra replicas of j: e1 - e0 (reps - 1)
-      const int32_t q = t & (e1 - e0);                               // reps is a power of two
-      uint32_t y = (uint32_t)(q == 0 ? j : src.n_items + e0 + q - 1) * (uint32_t)src.dR_ld;
-      if (src.hot_item != nullptr)
+    for (int32_t k = l; k < most * g.per_step; k += G) {
+      uint32_t xw = kNoRecord, y = kNoRecord, z = kNoRecord;
+      if (k < n) {
+        const int32_t t = it.y + k, j = rec_j[t];
+        const int32_t e0 = b.item_rep[j], e1 = b.item_rep[j + 1];  // extra replicas of j: e1 - e0 (reps - 1)
+        const int32_t q = t & (e1 - e0);                           // reps is a power of two
+        xw = (uint32_t)j * (uint32_t)K4;
+        y = (uint32_t)(q == 0 ? j : b.n_items + e0 + q - 1) * (uint32_t)b.dR_ld;
+#pragma unroll
         for (int h = 0; h < kHot; ++h)
-          if (src.hot_item[h] == j) y = 2u * h + 1u;
-      const int64_t to = record_place(g, at, k);
-      x[to] = (uint32_t)j * (uint32_t)(src.K / 4);
-      yz[y_word(g, to)] = y;
-      yz[y_word(g, to) + g.per_step] = __float_as_uint(src.rec_D[t]);
+          if (hot[h] == j) y = 2u * h + 1u;
+        z = __float_as_uint(rec_D[t]);
+      }
+      const int64_t to = record_place(g, at, k), to_y = y_word(g, to);
+      x[to] = xw;
+      yz[to_y] = y;
+      yz[to_y + g.per_step] = z;
     }
-    s += __reduce_max_sync(0xffffffffu, (n + g.per_step - 1) / g.per_step);
+    s += most;
   }
 }
-cudaError_t launch_stream_fill(const int4* items, const int4* part, int64_t n_warps, const StreamGeometry& g,
-                               const StreamSource& src, int64_t n_places, uint32_t* x, uint32_t* yz, uint32_t* place,
-                               cudaStream_t st) {
-  cudaError_t e = cudaMemsetAsync(x, 0xff, sizeof(uint32_t) * n_places, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(yz, 0xff, 2 * sizeof(uint32_t) * n_places, st);
-  if (e != cudaSuccess || n_warps <= 0) return e;
-  stream_fill_kernel<<<(unsigned)((n_warps + 7) / 8), 256, 0, st>>>(items, part, n_warps, g, src, x, yz, place);
+
+cudaError_t launch_stream_build(const StreamBuild& b, cudaStream_t st) {
+  const int64_t warps = std::min(b.max_warps, (b.max_items + b.g.gpw - 1) / b.g.gpw);
+  const unsigned F = (unsigned)b.F;
+  stream_partition_kernel<<<dim3((unsigned)(warps / 256 + 1), F), 256, 0, st>>>(b);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  stream_steps_kernel<<<dim3((unsigned)(warps / 8 + 1), F), 256, 0, st>>>(b);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  stream_offsets_kernel<<<F, 1024, 0, st>>>(b);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  stream_fill_kernel<<<dim3((unsigned)(warps / 8 + 1), F), 256, 0, st>>>(b);
   return cudaGetLastError();
 }
 
