@@ -127,7 +127,8 @@ __global__ void __launch_bounds__(256) vap_scan_kernel(const float4* __restrict_
     if (t >= last) return;
     const int32_t k = k1 - (int32_t)(t / pieces);
     const float4* old = ring + (int64_t)((c - 1 - k) % nslots) * slot4;
-    const int64_t q0 = (int64_t)(t % pieces) * kVapPiece + threadIdx.x;
+    const uint32_t p = t % pieces;  // taken from both ends in turn
+    const int64_t q0 = (int64_t)((p & 1u) ? pieces - 1u - p / 2u : p / 2u) * kVapPiece + threadIdx.x;
     bool breaks = false;
     float4 x[kVapLoads], y[kVapLoads];
 #pragma unroll
@@ -161,7 +162,12 @@ cudaError_t launch_vap(const float* ring, int64_t slot_floats, int32_t nslots, i
   if ((double)fb > bound) fb = std::nextafterf(fb, 0.f);
   const int64_t slot4 = slot_floats / 4, pieces = (slot4 + kVapPiece - 1) / kVapPiece;
   // The scan saves up to kmax - 1 tables of traffic and costs its tickets, about
-  // 10 us (4 MB table, kmax = 6: 17 us against 7 for all norms at once).
+  // 10 us (4 MB table, kmax = 6: 17 us against 7 for all norms at once).  Its worst
+  // case is one element, far from both ends of the table, that breaks every
+  // candidate: each is read nearly whole, 2 kmax tables where the norms read kmax +
+  // 1 (the newest version's from L2).  48 MB table, whole CLOCK, norms against scan:
+  // kmax = 4: 67 us, 40 with the stalest version in bound, 47 broken at an end of
+  // the table, 62 in its middle; kmax = 8: 112, 41, 92, 127.
   if ((kmax - 1) * slot_floats * 4 < (128 << 20)) {
     const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((slot4 + 255) / 256, (int64_t)sms * 8));
     for (int32_t k0 = 1; k0 <= kmax; k0 += kVapBatch) {
