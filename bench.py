@@ -47,13 +47,22 @@ def kernel_code_digest(text: str) -> str:
     return hashlib.sha256(code.encode()).hexdigest()[:16]
 
 
+# the SGD kernel, the forward copy in it, and the inline PTX of both
+KERNEL_SOURCES = ("mf_kernels.cu", "copy_idle.cuh", "ptx.cuh")
+
+
+def kernel_source_digest() -> str:
+    """Digest of the code of KERNEL_SOURCES together."""
+    csrc = os.path.join(ROOT, "paper_1410_8043_gb300", "csrc")
+    return kernel_code_digest("\n".join(open(os.path.join(csrc, f)).read() for f in KERNEL_SOURCES))
+
+
 def _profiled_traffic(kernel: str, workload: str):
     """DRAM bytes per launch of `kernel` on `workload` from its committed ncu
     summary profiles/<kernel>_<workload>.md, or None when there is none or the
     kernels' code changed since the capture."""
-    src = os.path.join(ROOT, "paper_1410_8043_gb300", "csrc", "mf_kernels.cu")
     try:
-        digest = kernel_code_digest(open(src).read())
+        digest = kernel_source_digest()
     except OSError:
         return None
     for path in [os.path.join(ROOT, "profiles", f"{kernel}_{workload}.md")]:
@@ -181,20 +190,21 @@ def replica_throughput(world, ratings: float, ms: float) -> float:
 
 
 class FloorModel:
-    """Compulsory HBM bytes of the SGD kernels of one clock (minibatch b, read
-    versions v): 12 B per entry (i, j, D); the merge of every user row (read
-    version c-1, write version c); each user row read at a stale version
-    (v != c-1) by a user with entries; each distinct (item, stale version)
-    row read.  Item rows of version c-1 count as resident (the previous
-    clock's merge just wrote them).  Counted with torch on `device` (the
-    distinct pairs by sorting), one minibatch at a time.
+    """Compulsory HBM bytes of the SGD kernel of one clock (minibatch b, read
+    versions v): 12 B per entry (i, j, D); the merge of the user rows that it
+    writes (read version c-1, write version c); each of these rows read at a
+    stale version (v != c-1) by a user with entries; the row of each heavy user
+    (more than 96 entries: the Clock() merge writes it, in the next kernel);
+    each distinct (item, stale version) row read.  Item rows of version c-1 count
+    as resident (the previous clock's merge just wrote them).  Counted with torch
+    on `device` (the distinct pairs by sorting), one minibatch at a time.
 
-    An idle user row unchanged over the last s+2 clocks is not merged (its ring
+    An idle user row unchanged over the last s+2 clocks is not written (its ring
     slot already holds it), and each user has a 4-byte change-clock word, read
-    for idle users and written for active ones: counted for 32 < K <= 64, where
-    the workloads have many idle users (at other widths the count is an upper
-    bound: mid has 14 of 480k idle).  `bytes` must then see every clock from the
-    table's version 0 in order."""
+    for idle users and written for active ones.  `bytes` must therefore see every
+    clock from the table's version 0 in order."""
+
+    HEAVY = 96  # entries in a minibatch past which a user is heavy
 
     def __init__(self, w, data, wp, mb, device="cpu"):
         import torch
@@ -206,25 +216,24 @@ class FloorModel:
         self.mb = torch.as_tensor(np.ascontiguousarray(mb)).to(self.dev)
         self.wp = torch.as_tensor(np.ascontiguousarray(wp)).to(self.dev).long()
         self._b = None
-        self.skip = 32 < w.K <= 64
-        self.chg = torch.zeros(w.n_users, dtype=torch.int64, device=self.dev) if self.skip else None
+        self.chg = torch.zeros(w.n_users, dtype=torch.int64, device=self.dev)
         self.last_c = 0
 
     def _minibatch(self, b):
-        """(entries, worker of each user with entries, distinct worker*M + item
-        pairs, users with entries) of minibatch b."""
+        """(entries, worker of each light user with entries, distinct worker*M +
+        item pairs, users with entries, heavy users) of minibatch b."""
         import torch
 
         if self._b != b:
             idx = torch.nonzero(self.mb == b).squeeze(1)
             ui = self.i[idx].long()
             jj = self.j[idx].long()
-            users = torch.unique(ui)
-            uw = self.wp[users]
+            users, cnt = torch.unique(ui, return_counts=True)
+            uw = self.wp[users[cnt <= self.HEAVY]]
             pj = torch.unique(self.wp[ui] * self.w.n_items + jj)
-            self._cache = (int(idx.numel()), uw, pj, users)
+            self._cache = (int(idx.numel()), uw, pj, users, int((cnt > self.HEAVY).sum()))
             self._b = b
-            del idx, ui, jj, users
+            del idx, ui, jj, users, cnt
         return self._cache
 
     def bytes(self, c, v):
@@ -232,25 +241,21 @@ class FloorModel:
 
         w = self.w
         b = (c - 1) % w.F
-        n, uw, pj, active = self._minibatch(b)
+        n, uw, pj, active, heavy = self._minibatch(b)
         vt = torch.as_tensor(np.ascontiguousarray(v, dtype=np.int64)).to(self.dev)
         stale = vt != (c - 1)
         users = int(stale[uw].sum())
         p = pj // w.n_items
         sp = stale[p]
         items = int(torch.unique(vt[p[sp]] * w.n_items + (pj[sp] % w.n_items)).numel())
-        merged = w.n_users
-        words = 0
-        if self.skip:
-            assert c == self.last_c + 1, "the work-list floor needs every clock in order"
-            self.last_c = c
-            idle = torch.ones(w.n_users, dtype=torch.bool, device=self.dev)
-            idle[active] = False
-            skipped = int((idle & (c - self.chg >= w.s + 2)).sum())
-            merged = w.n_users - skipped
-            words = 4 * w.n_users
-            self.chg[active] = c
-        return 12 * n + 8 * w.K * merged + words + 4 * w.K * (users + items), n
+        assert c == self.last_c + 1, "the floor needs every clock in order"
+        self.last_c = c
+        idle = torch.ones(w.n_users, dtype=torch.bool, device=self.dev)
+        idle[active] = False
+        skipped = int((idle & (c - self.chg >= w.s + 2)).sum())
+        self.chg[active] = c
+        merged = w.n_users - skipped - heavy
+        return 12 * n + 8 * w.K * merged + 4 * w.n_users + 4 * w.K * (users + heavy + items), n
 
 
 def _model_launches(w, c):
@@ -268,11 +273,13 @@ def _stage_overlapped(t, w, host_mb, W, K, stream, copy_stream, loss_d, loss_h):
     """K clocks through the public API with host inputs: minibatch of clock
     c+1 is copied from pinned host memory on `copy_stream` while clock c runs
     on `stream`; each clock's squared loss is copied back to pinned host
-    memory.  Returns (start event on `stream`, h2d bytes, d2h bytes)."""
+    memory.  Returns (start event on `stream`, h2d bytes, d2h bytes, the event
+    pairs around each minibatch's staging)."""
     import torch
 
     F = w.F
-    staged = [torch.cuda.Event() for _ in range(K)]
+    begun = [torch.cuda.Event(enable_timing=True) for _ in range(K)]
+    staged = [torch.cuda.Event(enable_timing=True) for _ in range(K)]
     done = [torch.cuda.Event() for _ in range(K)]
     h2d = d2h = 0
 
@@ -284,6 +291,7 @@ def _stage_overlapped(t, w, host_mb, W, K, stream, copy_stream, loss_d, loss_h):
         if k - F >= 0:
             copy_stream.wait_event(done[k - F])
         u, j, D, uoff = host_mb[b]
+        begun[k].record(copy_stream)
         t.mf_stage_minibatch(b, u, j, D, uoff, stream=copy_stream)
         staged[k].record(copy_stream)
         h2d += 4 * (u.numel() + j.numel() + D.numel() + uoff.numel())
@@ -301,7 +309,23 @@ def _stage_overlapped(t, w, host_mb, W, K, stream, copy_stream, loss_d, loss_h):
             loss_h[k:k + 1].copy_(loss_d[k:k + 1], non_blocking=True)
         d2h += 8
         done[k].record(stream)
-    return start, h2d, d2h
+    return start, h2d, d2h, list(zip(begun, staged))
+
+
+def huge_page_bytes(address: int, smaps: str = "/proc/self/smaps") -> int:
+    """Bytes in huge pages of the mapping that holds `address` (0 if unknown)."""
+    try:
+        inside = False
+        for line in open(smaps):
+            head = line.split()[0]
+            if "-" in head and not head.endswith(":"):
+                lo, hi = (int(x, 16) for x in head.split("-"))
+                inside = lo <= address < hi
+            elif inside and head == "AnonHugePages:":
+                return int(line.split()[1]) * 1024
+    except (OSError, ValueError, IndexError):
+        pass
+    return 0
 
 
 class HostBuffer:
@@ -312,7 +336,7 @@ class HostBuffer:
     address translation on the host link, and tens of GB of small pages
     overflow it: copies from a 26 GB set of ordinary pinned buffers slowed from
     2.5 ms to 4-20 ms each.  With huge pages every copy ran at the link's
-    speed.  Falls back to torch's pinned allocator if registration fails."""
+    speed; `kind` says how much of it the kernel granted.  Falls back to torch's pinned allocator if registration fails."""
 
     def __init__(self, n_int32: int):
         import mmap
@@ -331,7 +355,7 @@ class HostBuffer:
                 raise RuntimeError("cudaHostRegister failed")
             self.mm, self.arr, self.nbytes = mm, arr, nbytes
             self.tensor = torch.from_numpy(arr[:n_int32])
-            self.kind = "huge-page mapping registered with CUDA"
+            self.kind = f"mapping registered with CUDA, {huge_page_bytes(arr.ctypes.data) / nbytes:.2f} of it in huge pages"
         except Exception:
             self.tensor = torch.empty(n_int32, dtype=torch.int32, pin_memory=True)
             self.kind = "torch pinned memory"
@@ -366,6 +390,25 @@ def _export_host_minibatches(t, w, need):
         o += 3 * n + w.n_users + 1
         out[b] = t.mf_export_minibatch(b, out=(u, j, D, uoff))
     return out, buf
+
+
+def _copy_times(host_mb, need, dev, stream):
+    """Milliseconds of copying each minibatch's host arrays to the device, alone."""
+    import torch
+
+    out = []
+    into = [torch.empty(max(host_mb[b][k].numel() for b in need), dtype=host_mb[need[0]][k].dtype, device=dev)
+            for k in range(4)]
+    with torch.cuda.stream(stream):
+        for b in need:
+            a, z = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record(stream)
+            for x, y in zip(host_mb[b], into):
+                y[: x.numel()].copy_(x, non_blocking=True)
+            z.record(stream)
+            z.synchronize()
+            out.append(a.elapsed_time(z))
+    return out
 
 
 def measure(args, w, dev, world, rank, local):
@@ -461,7 +504,7 @@ def measure(args, w, dev, world, rank, local):
     t.poll()
     _barrier(world)
     wall0 = time.time()
-    e0, h2d, d2h = _stage_overlapped(t, w, host_mb, W, K, stream, copy_stream, loss_d, loss_h)
+    e0, h2d, d2h, stages = _stage_overlapped(t, w, host_mb, W, K, stream, copy_stream, loss_d, loss_h)
     e1 = torch.cuda.Event(enable_timing=True)
     e1.record(stream)
     torch.cuda.synchronize(dev)
@@ -471,6 +514,8 @@ def measure(args, w, dev, world, rank, local):
     e2e_ms = _max_over_ranks(world, e2e_ms)
     e2e_value = total_ratings / (e2e_ms / 1e3)
     t.poll()
+    stage_ms = [a.elapsed_time(b_) for a, b_ in stages]
+    copy_ms = _copy_times(host_mb, need, dev, copy_stream)
     del host_mb
     host_kind = host_buf.kind
     host_buf.close()
@@ -516,7 +561,11 @@ def measure(args, w, dev, world, rank, local):
         },
         "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": h2d // K, "d2h_bytes_per_step": d2h // K,
                 "copies": "minibatch of clock c+1 staged on a second stream while clock c runs",
-                "host_memory": host_kind},
+                "host_memory": host_kind,
+                # staging a minibatch during the timed clocks (copies, new values into the stream, check),
+                # and the same bytes copied alone afterwards
+                "stage_ms": {"median": statistics.median(stage_ms), "max": max(stage_ms)},
+                "copy_ms": {"median": statistics.median(copy_ms), "max": max(copy_ms)}},
         # per clock: the SGD kernel and the Clock() merge (which also computes the
         # next schedule), plus the read model's own kernels
         "gpu_launches": int(sum(_sgd_launches() + _model_launches(w, c) for c in range(W + 1, W + K + 1))),

@@ -7,18 +7,21 @@ from gen import make_mf_data, minibatch_labels, shard_users
 
 
 def _brute_floor(w, d, wp, mb, c, v):
-    """12 B per entry; 8K bytes per user row (read c-1, write c); 4K bytes per
-    stale user row read and per distinct (item, stale version) read."""
+    """12 B per entry; 8K bytes per row of a user of at most 96 entries (read c-1,
+    write c); 4K bytes per stale row of these read, per row of a user of more, and
+    per distinct (item, stale version) read; a 4-byte word per user."""
     b = (c - 1) % w.F
     idx = np.flatnonzero(mb == b)
-    total = 12 * idx.size + 8 * w.K * w.n_users
+    heavy = np.bincount(d.i[idx], minlength=w.n_users) > 96
+    total = 12 * idx.size + 4 * w.n_users + 8 * w.K * int((~heavy).sum()) + 4 * w.K * int(heavy.sum())
     users = set()
     items = set()
     for k in idx:
         u, j = int(d.i[k]), int(d.j[k])
         ver = int(v[wp[u]])
         if ver != c - 1:
-            users.add(u)
+            if not heavy[u]:
+                users.add(u)
             items.add((j, ver))
     return total + 4 * w.K * (len(users) + len(items)), idx.size
 
@@ -39,9 +42,39 @@ def test_floor_model_matches_brute_force():
         assert m.bytes(c, v) == _brute_floor(w, d, wp, mb, c, v)
 
 
+def test_floor_model_leaves_heavy_rows_to_the_merge():
+    """Users of more than 96 entries in a minibatch: the SGD kernel reads their rows and the merge writes them."""
+    import bench
+    from gen.workloads import Workload
+
+    d = make_mf_data(n_users=40, n_items=30, n_obs=4000, K=8, seed=6, truth_rank=2, user_dist="zipf", user_a=1.0)
+    w = Workload("t", 40, 30, 4000, K=8, P=3, F=2, s=2, model="ssp", clocks=5, eta=0.01, lam=0.05, cap=0)
+    wp, mb = shard_users(40, 3, 7), minibatch_labels(4000, 2, 8)
+    cnt = np.bincount(d.i[mb == 0], minlength=40)
+    assert (cnt > 96).sum() > 2 and ((cnt > 0) & (cnt <= 96)).sum() > 2
+    m = bench.FloorModel(w, d, wp, mb)
+    rng = np.random.default_rng(3)
+    for c in range(1, 6):
+        v = rng.integers(max(0, c - 1 - w.s), c, size=3).astype(np.int32)
+        base, n = _brute_floor(w, d, wp, mb, c, v)
+        got, n_got = m.bytes(c, v)
+        idle = 40 - np.unique(d.i).size  # never active: skipped once they are in every slot
+        assert n_got == n and got == base - (8 * w.K * idle if c >= w.s + 2 else 0)
+
+
+def test_huge_page_bytes(tmp_path):
+    import bench
+
+    f = tmp_path / "smaps"
+    f.write_text("1000-3000 rw-p 00000000 00:00 0\nSize: 8 kB\nAnonHugePages:      4 kB\n"
+                 "7f0000000000-7f0000400000 rw-p 00000000 00:00 0 \nSize: 4096 kB\nAnonHugePages:   2048 kB\n")
+    assert bench.huge_page_bytes(0x7F0000000010, str(f)) == 2048 * 1024
+    assert bench.huge_page_bytes(0x2FFF, str(f)) == 4096 and bench.huge_page_bytes(0x3000, str(f)) == 0
+    assert bench.huge_page_bytes(0x1000, str(tmp_path / "none")) == 0
+
+
 def test_floor_model_work_list_skips_unchanged_idle_rows():
-    """On the work-list path (K 36..64) an idle user row unchanged over the last
-    s+2 clocks is not merged; every user has a 4-byte change-clock word."""
+    """An idle user row unchanged over the last s+2 clocks is not written."""
     import bench
     from gen.workloads import Workload
 
@@ -62,7 +95,7 @@ def test_floor_model_work_list_skips_unchanged_idle_rows():
         skipped = int(np.sum(~active & (c - chg >= s + 2)))
         assert skipped > 0 or c < s + 2
         chg[active] = c
-        assert got == (base - 8 * K * skipped + 4 * N, n), c
+        assert got == (base - 8 * K * skipped, n), c
 
 
 def test_model_launch_counts():
