@@ -571,8 +571,9 @@ namespace {
 // ahead (see the kernel); the blocks per SM it is compiled for.  Eight lanes
 // read 128 consecutive bytes per load, a whole line; wider groups only where
 // NV = 4 slices per lane do not hold the row.  Measured (us per clock):
-//   K = 32, 200k x 30k: PF 2 with 7 blocks 84, PF 1 with 8 blocks 89, 6 blocks
-//     82; one entry per step 86..93;
+//   K = 32, 200k x 30k: PF 2 with 6 blocks 68..75 over three inputs, with 7 (it
+//     spills) 74..78, PF 1 with 7 blocks 74..77; one entry per step more; K = 28,
+//     1M x 100k: 197, 195, 195;
 //   K = 48, 300k x 40k: PF 1 with 5 blocks 107, PF 2 with 4 blocks 114; one
 //     entry per step 108..118; 10M x 1M, K = 64: 2630, 2650; 2720..2810;
 //   K = 100, 480k x 18k: 4 blocks 441..450, 3 blocks 470, 5 blocks spill (785).
@@ -584,7 +585,7 @@ template <typename F>
 auto dispatch_stream(int32_t K, F&& f) {
   const int32_t K4 = K / 4;
   if (K4 <= 4) return f(StreamShape<4, 1, 2, 2, 6>{});
-  if (K4 <= 8) return f(StreamShape<8, 1, 2, 2, 7>{});
+  if (K4 <= 8) return f(StreamShape<8, 1, 2, 2, 6>{});
   if (K4 <= 16) return f(StreamShape<8, 2, 2, 1, 5, kHot>{});
   if (K4 <= 24) return f(StreamShape<8, 3, 1, 1, 5>{});
   if (K4 <= 32) return f(StreamShape<8, 4, 1, 1, 4>{});

@@ -175,8 +175,8 @@ def test_committed_profiles_match_the_kernel_source():
     that of the kernels' current source."""
     import bench
 
-    assert bench._profiled_traffic("sgd_stream_kernel", "large") == 7664658560.0
-    assert bench._profiled_traffic("sgd_stream_kernel", "mid") == 773927552.0
+    assert bench._profiled_traffic("sgd_stream_kernel", "large") == 7663310080.0
+    assert bench._profiled_traffic("sgd_stream_kernel", "mid") == 777274368.0
     assert bench._profiled_traffic("sgd_work16_kernel", "large") is None
 
 
