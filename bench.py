@@ -438,7 +438,7 @@ def measure(args, w, dev, world, rank, local):
     for c in range(1, W + K + 1):
         v, clk = t.read_schedule()
         assert clk == c
-        fb, n = model.bytes(c, v)  # every clock: the work-list floor follows the rows' history
+        fb, n = model.bytes(c, v)  # every clock: the floor follows the rows' history
         if c > W:
             floors.append(fb)
             counts.append(n)

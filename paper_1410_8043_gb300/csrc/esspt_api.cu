@@ -445,7 +445,7 @@ esspt_status esspt_inc(esspt_ctx* c, int32_t worker, const int32_t* d_row_ids, c
   if (n < 0 || (n > 0 && (!d_row_ids || !d_deltas))) return fail(c, ESSPT_EINVAL, "bad row list");
   if ((s = ensure_acc(c)) != ESSPT_OK) return s;
   ESSPT_CUDA(c, launch_inc(slot_ptr(c, c->clock), c->n_rows, c->K, d_row_ids, d_deltas, n, c->status, c->st));
-  // INC changes rows the work-list path does not track: copy every idle row
+  // INC changes rows that `chg` does not track: copy every idle row
   // until the changed version has gone round the ring.
   c->copy_all_until = std::max(c->copy_all_until, c->clock + c->s + 1);
   return ESSPT_OK;

@@ -48,8 +48,11 @@ struct Sum2 {  // two packed fp32 sums and what they lost
   }
 };
 
+// Four blocks per SM, as the grid is sized for, where that spills nothing.  Left
+// to the compiler some shapes take 66..72 registers and lose a block: 1.5M
+// entries, K = 512, 286 us against 239 so; 9M, K = 64, 239 against 205.
 template <int G, int NV, bool BY_WORKER>
-__global__ void __launch_bounds__(256) objective_kernel(ObjectiveArgs a) {
+__global__ void __launch_bounds__(256, G == 8 && NV == 1 ? 3 : 4) objective_kernel(ObjectiveArgs a) {
   constexpr int kGpw = 32 / G, U = NV >= 3 ? 2 : NV == 2 || G == 4 ? 4 : 8;
   extern __shared__ double sums[];  // BY_WORKER: sum e^2 at [p], penalised sum at [P + p]
   if (BY_WORKER) {

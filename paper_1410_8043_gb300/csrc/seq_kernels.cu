@@ -2,9 +2,11 @@
 // entries in order and reads L_i and R_j from its read version plus its own
 // updates of this clock so far, as the per-entry SGD of Sec. 3.1 runs inside
 // a worker (Sec. 5); the workers' summed changes then join the Clock() merge.
-// Within a clock the entries of one worker form one dependent chain, so the
-// parallelism is one warp per worker: this is a semantic variant, not the
-// data-parallel hot path.
+// An entry depends on the worker's earlier entries of the same user and of the
+// same item.  One warp per worker takes them all in turn, though entries that
+// share neither could go side by side (64k entries, K = 64, 16 workers: about
+// 4000 entries per worker, 230..330 of them in the longest chain of dependent
+// ones): this is a semantic variant, not the data-parallel hot path.
 #include <algorithm>
 #include <type_traits>
 
@@ -34,7 +36,7 @@ constexpr int kFirst = 1, kLast = 2, kRepeat = 4;
 // Blocks [0, P): worker p's chain, walked by warp 0, its queue filled by warp 1.
 // Blocks from P on copy the idle users' rows.
 //
-// The chain's length bounds it, so it holds as little as it can: the dot
+// The length of the walk bounds it, so an entry holds as little as it can: the dot
 // product and two fused updates.  The rows of the read version (item's, user's
 // at its first entry, and the base row at its last) come by cp.async AHEAD
 // entries early, the worker's change to the item's row in registers three

@@ -154,9 +154,8 @@ def test_staleness_models_and_cap(s, model, cap):
 @pytest.mark.parametrize("K", [32, 40, 64])
 def test_heavy_users_chunk_path(K):
     """Users with far more than 96 entries in a minibatch (Zipf(1.5) users) go
-    through the chunked kernels (for K = 40 and 64 as items of the work-list
-    kernel, beside the light users and the forward copy of idle users);
-    results must not change."""
+    in chunks, as items of the SGD kernel beside the light users and the forward
+    copy of idle users; results must not change."""
     d = make_mf_data(n_users=400, n_items=300, n_obs=40000, K=K, seed=9, user_dist="zipf", user_a=1.5,
                      truth_rank=4, truth_var=0.5, noise_var=0.1, init_var=0.05)
     mb = minibatch_labels(40000, 2, 7)
@@ -171,7 +170,7 @@ def test_popular_items_with_extra_replicas(K):
     """Items popular enough for extra replica rows (one per 2048 entries of
     their largest minibatch, a power of two, at most 64), here 1 to 64 of
     them, beside heavy users, idle users and (for K = 48, 64) the two hot
-    items that the work-list kernel sums per warp.  The item merge must add
+    items that the SGD kernel sums per warp.  The item merge must add
     every replica and clear it for the next clock."""
     n = 400_000
     d = make_mf_data(n_users=3000, n_items=40, n_obs=n, K=K, seed=11, user_dist="zipf", user_a=1.2,
@@ -191,8 +190,8 @@ def test_popular_items_with_extra_replicas(K):
 @pytest.mark.parametrize("K", [16, 64, 100])
 def test_rows_that_no_entry_names(K):
     """Users and items that no entry names keep their initial rows, bit for bit,
-    in every version, through more clocks than the ring has slots (so the
-    work-list path also skips their forward copies)."""
+    in every version, through more clocks than the ring has slots (so their
+    forward copies are skipped too)."""
     d = make_mf_data(n_users=400, n_items=90, n_obs=12000, K=K, seed=21, item_dist="zipf", item_a=1.0,
                      truth_rank=4, truth_var=0.5, noise_var=0.1, init_var=0.05)
     d.i = (d.i % 390).astype(np.int32)  # users 390..399 and items 80..89 have no entries
@@ -487,7 +486,7 @@ def test_short_workspaces_are_refused():
 
 @pytest.mark.parametrize("K", [40, 64])
 def test_idle_rows_skipped_across_the_ring(K):
-    """Work-list path, many clocks at s = 1 and 6 minibatches: most user rows
+    """Many clocks at s = 1 and 6 minibatches: most user rows
     are idle for more than s+2 clocks in a row, so their forward copy is
     skipped (the ring slot already holds them).  Every clock against the
     oracle; then an INC on an idle row must survive the following clocks."""

@@ -53,7 +53,7 @@ def test_row_cache_tiny_every_clock(s):
 
 @pytest.mark.parametrize("K", [16, 48, 100, 132])
 def test_row_cache_row_widths(K):
-    """The generic, work-list, one-slice-per-lane and wide-row SGD kernels in row mode."""
+    """Four row shapes of the SGD kernel in row mode."""
     d = make_mf_data(n_users=300, n_items=120, n_obs=6000, K=K, seed=K + 1, truth_rank=4, truth_var=0.5,
                      noise_var=0.1, init_var=0.05)
     _run_pair(d, shard_users(300, 5, 1), minibatch_labels(6000, 3, 2), P=5, s=2, F=3, eta=0.02, lam=0.05, cap=0,
@@ -72,7 +72,7 @@ def test_row_cache_heavy_users(K):
 @pytest.mark.parametrize("K", [64, 100])
 def test_row_cache_popular_items(K):
     """Popular items with many replica rows (and, at K = 64, the hot items that
-    the work-list kernel sums per warp) while each worker reads its own cached
+    the SGD kernel sums per warp) while each worker reads its own cached
     version of every row; 6 clocks, sparse minibatches so rows age."""
     n = 200_000
     d = make_mf_data(n_users=2000, n_items=40, n_obs=n, K=K, seed=51, user_dist="zipf", user_a=1.2,

@@ -65,8 +65,8 @@ def test_vap_tiny_every_clock(v0):
 
 @pytest.mark.parametrize("K,v0", [(48, 0.6), (64, 0.6), (100, 0.8)])
 def test_vap_wide_rows_every_clock(K, v0):
-    """VAP on the work-list path (K = 48, 64) and on the one-slice-per-lane
-    kernel (K = 100), Zipf items, a hot-row cap: schedule bit-exact and every
+    """VAP on rows gathered through shared memory (K = 48, 64) and through
+    registers (K = 100), Zipf items, a hot-row cap: schedule bit-exact and every
     parameter within tolerance for 12 clocks, reads of every staleness 0..3."""
     from gen import make_mf_data, minibatch_labels, shard_users
 
