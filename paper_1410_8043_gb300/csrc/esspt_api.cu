@@ -43,6 +43,7 @@ struct esspt_ctx {
   int32_t* user_slot = nullptr;  // row-granular SSP: [n_users] per-clock ring slot of each user row
   int4 *chunk = nullptr, *heavy = nullptr, *popular = nullptr;
   int64_t n_popular = 0;
+  int32_t longest = 0;  // entries of the longest work item
   std::vector<int64_t> mb_base, chunk_base, heavy_base;
   int64_t *d_mb_base = nullptr, *d_chunk_base = nullptr;
   int4* part = nullptr;               // split of each minibatch's work items over the warps
@@ -216,12 +217,13 @@ struct MfCarve {
 
 // What the host reads back of a load, side by side in 64-bit words: the first
 // entry, work item, heavy user, warp and place of each minibatch (and the ends),
-// the steps of each, the number of popular items, and the status word.
+// the steps of each, the number of popular items, the longest work item and the
+// status word.
 struct Bases {
-  int64_t entry, item, heavy, part, place, steps, n_popular, status, words;
+  int64_t entry, item, heavy, part, place, steps, n_popular, longest, status, words;
   explicit Bases(int32_t F)
       : entry(0), item(F + 1), heavy(2 * (F + 1)), part(3 * (F + 1)), place(4 * (F + 1)), steps(5 * (F + 1)),
-        n_popular(steps + F), status(n_popular + 1), words(status + 1) {}
+        n_popular(steps + F), longest(n_popular + 1), status(longest + 1), words(status + 1) {}
 };
 
 // Persistent MF workspace: entries laid out by (minibatch, user), per-minibatch
@@ -307,6 +309,8 @@ esspt_status mf_view(esspt_ctx* c, int32_t version, ObjectiveArgs* a, cudaStream
   a->entry_base = c->d_mb_base;
   a->rec_j = c->rec_j;
   a->rec_D = c->rec_D;
+  a->n_obs = c->n_obs;
+  a->longest = c->longest;
   *st = c->st;
   return ESSPT_OK;
 }
@@ -545,6 +549,7 @@ esspt_status esspt_mf_load(esspt_ctx* c, const int32_t* d_i, const int32_t* d_j,
   b.heavy = reinterpret_cast<int4*>(w + k.heavy);
   b.popular = reinterpret_cast<int4*>(w + k.popular);
   b.n_popular = reinterpret_cast<uint32_t*>(bases + at.n_popular);
+  b.longest = reinterpret_cast<uint32_t*>(bases + at.longest);
   b.heavy_base = bases + at.heavy;
   b.max_chunks = k.max_chunks;
   b.max_heavy = k.max_heavy;
@@ -657,6 +662,7 @@ esspt_status esspt_mf_load(esspt_ctx* c, const int32_t* d_i, const int32_t* d_j,
   ESSPT_CUDA(c, cudaMemsetAsync(c->chg_item, 0, sizeof(int32_t) * (size_t)n_items, c->st));
   c->popular = b.popular;
   c->n_popular = h[at.n_popular];
+  c->longest = (int32_t)h[at.longest];
   // rows changed before this load are not tracked
   c->copy_all_until = c->clock + c->s + 1;
   c->mb_base = mbb;

@@ -273,7 +273,9 @@ struct ObjectiveArgs {
   float lambda;
   double* out;
   int64_t out_stride;
-  int32_t parts;  // (set by the launch) parts that an item is taken in
+  int64_t n_obs;        // entries, and those of the longest item
+  int32_t longest;
+  int32_t part, parts;  // (set by the launch) entries of a part, and parts of an item
 };
 cudaError_t launch_objective(const ObjectiveArgs& a, cudaStream_t st);
 cudaError_t launch_worker_objective(const ObjectiveArgs& a, cudaStream_t st);
@@ -298,6 +300,7 @@ struct LayoutBuild {
   int32_t* item_rep;    // [n_items+1]
   int4* popular;        // [max_popular] items with extra replicas (see MergeArgs), in no order
   uint32_t* n_popular;  // their number (0 on entry)
+  uint32_t* longest;    // entries of the longest work item (0 on entry)
   int4* chunk;          // [max_chunks] work items (see StreamArgs); before that 3 words per item of the build's
   int64_t* chunk_base;  // [F+1]
   int4* heavy;          // [max_heavy]

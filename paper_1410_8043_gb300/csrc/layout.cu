@@ -112,10 +112,12 @@ __global__ void heavy_kernel(const int64_t* __restrict__ choff, const int32_t* _
                              uint32_t* __restrict__ key, uint32_t* __restrict__ val, int64_t n_tiles,
                              int64_t* __restrict__ chunk_base, int64_t max_chunks, int4* __restrict__ heavy,
                              int64_t* __restrict__ heavy_base, int64_t max_heavy, int64_t max_user_reps,
-                             uint32_t* status) {
+                             uint32_t* longest, uint32_t* status) {
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   const int64_t total = (int64_t)F * n_users;
+  int32_t most = 0;
   auto put = [&](int64_t at, int64_t b, int64_t u, int32_t beg, int32_t dst, int32_t n) {
+    most = max(most, n);
     chunk[at] = make_int4((int32_t)u, beg, dst, n << 16 | worker[u]);
     key[at] = (uint32_t)(b * n_tiles + (u >> kTileBits)) << 7 | (uint32_t)(127 - n);
     val[at] = (uint32_t)at;
@@ -151,6 +153,8 @@ __global__ void heavy_kernel(const int64_t* __restrict__ choff, const int32_t* _
     chunk_base[b] = choff[b * n_users];
     heavy_base[b] = hoff[b * n_users];
   }
+  most = __reduce_max_sync(0xffffffffu, most);
+  if ((threadIdx.x & 31) == 0 && most > 0) atomicMax(longest, (uint32_t)most);
 }
 
 // Extra replica rows of every item (replicas - 1) from its largest minibatch
@@ -442,7 +446,8 @@ cudaError_t build_layout(LayoutBuild& b, cudaStream_t st) {
   const int64_t n_tiles = (b.n_users >> kTileBits) + 1;
   heavy_kernel<<<blocks_for(keys + 1), 256, 0, st>>>(
       choff, nch, hoff, hext, b.uoff, b.worker, b.n_users, b.F, raw, key_in, val_in, n_tiles, b.chunk_base,
-      std::min(b.n_obs, b.max_chunks), b.heavy, b.heavy_base, b.max_heavy, layout_max_user_reps(b.n_obs), b.status);
+      std::min(b.n_obs, b.max_chunks), b.heavy, b.heavy_base, b.max_heavy, layout_max_user_reps(b.n_obs), b.longest,
+      b.status);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   int64_t n = 0;
   if ((e = cudaMemcpyAsync(&n, choff + keys, sizeof n, cudaMemcpyDeviceToHost, st)) != cudaSuccess) return e;

@@ -22,7 +22,7 @@ namespace {
 // Every entry's exact square (high and low fp32 parts) is added to an fp32 sum
 // with its rounding error kept beside it (two-sum, Knuth, TAOCP vol. 2, 4.2.2);
 // fp64, whose units are few, only at the end: an fp64 sum per item takes 1.05 ms
-// on those 20M entries, this 0.80.  Squares added eight at a time without their
+// on those 20M entries, this 0.77.  Squares added eight at a time without their
 // rounding errors were 8.7e-10 off on 51k entries, the exact ones 7e-11.  What
 // fp32 cannot hold so goes to fp64 sums of its own: squares and norms from 1e29
 // on, NaN among them (a lane adds fewer than 2^31 of them, which stay finite
@@ -31,7 +31,10 @@ constexpr float kHuge = 1e29f;
 __device__ __forceinline__ bool in_range(float e, float norm) {
   return fabsf(e) < 3e14f && !(fabsf(e) < 1e-14f && e != 0.f) && norm < kHuge;
 }
-constexpr int32_t kPart = 8;  // entries of a part of an item
+// Rows of a group in flight.
+template <int G, int NV>
+constexpr int kInFlight = NV >= 3 ? 2 : NV == 2 || G == 4 ? 4 : 8;
+constexpr int32_t kPart = 8;  // entries of a part of an item at most
 // x + y and its rounding error.
 __device__ __forceinline__ float two_sum(float x, float y, float& err) {
   const float s = x + y, b = s - x;
@@ -48,12 +51,14 @@ struct Sum2 {  // two packed fp32 sums and what they lost
   }
 };
 
-// Four blocks per SM, as the grid is sized for, where that spills nothing.  Left
-// to the compiler some shapes take 66..72 registers and lose a block: 1.5M
-// entries, K = 512, 286 us against 239 so; 9M, K = 64, 239 against 205.
+// Four blocks per SM, as the grid is sized for, where that spills nothing and, by
+// worker, leaves both rows of a step in flight.  1.5M entries, us: K = 512 286
+// with what the compiler takes (66..72 registers), 228 so; by worker at K = 128
+// and 256 139 and 198 with four, 117 and 177 with three (9M: 319 and 540 with
+// four, 331 and 577 with three).
 template <int G, int NV, bool BY_WORKER>
-__global__ void __launch_bounds__(256, G == 8 && NV == 1 ? 3 : 4) objective_kernel(ObjectiveArgs a) {
-  constexpr int kGpw = 32 / G, U = NV >= 3 ? 2 : NV == 2 || G == 4 ? 4 : 8;
+__global__ void __launch_bounds__(256, (G == 8 && NV == 1) || (BY_WORKER && NV == 4 && G < 32) ? 3 : 4) objective_kernel(ObjectiveArgs a) {
+  constexpr int kGpw = 32 / G, U = kInFlight<G, NV>;
   extern __shared__ double sums[];  // BY_WORKER: sum e^2 at [p], penalised sum at [P + p]
   if (BY_WORKER) {
     for (int k = threadIdx.x; k < 2 * a.P; k += blockDim.x) sums[k] = 0.0;
@@ -72,17 +77,17 @@ __global__ void __launch_bounds__(256, G == 8 && NV == 1 ? 3 : 4) objective_kern
   // e^2 and what the rows' squares add up to; by worker, of the item at hand.
   Sum2 sums2;  // (e^2, this lane's part of the rows' squares)
   double wide_e = 0.0, wide_n = 0.0;  // the same of what fp32 cannot hold
-  // Units of kGpw items; with a.parts > 1, part by part.
+  // Units of kGpw items, or of a part of each.
   const int64_t x_first = __ldg(a.item_base + blockIdx.y);
   const uint32_t units = (uint32_t)((x_end - x_first + kGpw - 1) / kGpw);
-  for (uint32_t v = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; v < units * a.parts; v += step) {
-    const uint32_t part = a.parts > 1 ? v / units : 0;
+  for (uint32_t v = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; v < units * max(a.parts, 1); v += step) {
+    const uint32_t part = a.parts > 0 ? v / units : 0;
     const int64_t x0 = x_first + (int64_t)(v - part * units) * kGpw;
     int4 it = x0 + grp < x_end ? __ldg(a.items + x0 + grp) : make_int4(0, 0, 0, 0);
     int32_t n = it.w >> 16;
-    if (a.parts > 1) {
-      it.y += part * kPart;
-      n = min(max(n - (int32_t)part * kPart, 0), kPart);
+    if (a.parts > 0) {
+      it.y += part * a.part;
+      n = min(max(n - (int32_t)part * a.part, 0), a.part);
     }
     const int32_t most = __reduce_max_sync(0xffffffffu, n);
     if (most == 0) continue;
@@ -96,33 +101,26 @@ __global__ void __launch_bounds__(256, G == 8 && NV == 1 ? 3 : 4) objective_kern
       L[k] = f2x2{0ull, 0ull};
       ldg_f2x2_if(L[k], L4 + (int64_t)it.x * K4 + k * G, n > 0 && (k < NV - 1 || last_on));
     }
-    // A part's entries by lane, so that no step's rows wait for a load of ids (38k
-    // entries, K = 320, cold caches: 65 us with one load per step, 55 so).
-    const bool by_lane = G >= kPart && a.parts > 1;
     int32_t lane_j = 0;
     float lane_d = 0.f;
-    if (by_lane && glane < n) {
-      lane_j = __ldg(rec_j + it.y + glane);
-      lane_d = __ldg(rec_D + it.y + glane);
-    }
+#pragma unroll 1
     for (int32_t t = 0; t < most; t += U) {
+      // The next G entries by lane, so that no step's rows wait for a load of ids (9M
+      // entries, K = 32 and 64: 241 and 205 us with one load per step, 197 and 184 so).
+      if ((t & (G - 1)) == 0 && t + glane < n) {
+        lane_j = __ldg(rec_j + it.y + t + glane);
+        lane_d = __ldg(rec_D + it.y + t + glane);
+      }
       f2x2 R[U][NV];
       float d[U];
 #pragma unroll
       for (int u = 0; u < U; ++u) {
-        const bool on = t + u < n;
-        int64_t j = 0;
-        if (by_lane) {
-          d[u] = __shfl_sync(0xffffffffu, lane_d, t + u, G);
-          j = __shfl_sync(0xffffffffu, lane_j, t + u, G);
-        } else {
-          d[u] = on ? __ldg(rec_D + it.y + t + u) : 0.f;
-          j = on ? __ldg(rec_j + it.y + t + u) : 0;
-        }
+        d[u] = __shfl_sync(0xffffffffu, lane_d, t + u, G);
+        const int64_t j = __shfl_sync(0xffffffffu, lane_j, t + u, G);
 #pragma unroll
         for (int k = 0; k < NV; ++k) {
           R[u][k] = f2x2{0ull, 0ull};
-          ldg_f2x2_if(R[u][k], R4 + j * K4 + k * G, on && (k < NV - 1 || last_on));
+          ldg_f2x2_if(R[u][k], R4 + j * K4 + k * G, t + u < n && (k < NV - 1 || last_on));
         }
       }
       float e[U], norm[U];  // residuals, and this lane's part of |R|^2
@@ -247,17 +245,25 @@ cudaError_t run(ObjectiveArgs a, cudaStream_t st) {
   auto go = [&](auto g, auto nv) {
     constexpr int G = decltype(g)::value, NV = decltype(nv)::value, kGpw = 32 / G;
     const size_t smem = BY_WORKER ? 2 * sizeof(double) * (size_t)a.P : 0;
-    // With fewer items than the GPU holds groups, an item is taken in parts of
-    // kPart entries, so that a call lasts no longer than the gathers of one part
-    // (20k entries, K = 224: 77 us whole, 41 in parts; parts of 4 the same, of 2
-    // and 32 slower).  Blocks (four per SM) for about two waves over the
-    // minibatches, for parts one: many parts are empty, and every block ends in
-    // two fp64 additions to one place (13k entries of 531k users, K = 64: 41 us
-    // with two waves, 30 with one; half a wave 32).
-    const int64_t resident = 4ll * sms * 8;
-    a.parts = a.n_items < resident * kGpw ? (kHeavy + kPart - 1) / kPart : 1;
-    const int64_t need = (a.parts * (a.n_items / a.F + kGpw) / kGpw + 7) / 8;
-    const int64_t x = std::max<int64_t>(1, std::min<int64_t>(need, resident / (a.parts > 1 ? 8 : 4) / a.F));
+    // With fewer items than the GPU holds groups, or some of them far longer than a
+    // group's share of the entries, an item is taken in parts, so that a call lasts
+    // no longer than the gathers of one part (20k entries, K = 224: 77 us whole, 41
+    // in parts of 8; 13k entries in 8k items, some of 96, K = 512: 66 and 40).
+    // A warp then looks at units * parts / resident units, most of them empty.  The
+    // parts are of 2 entries where one look per warp takes them all, else of 4 or 8
+    // (1k entries, K = 100: 13 us of kernel in parts of 8, 8 of 2).  Blocks (four per
+    // SM) for about two waves over the minibatches where there is work for them, for
+    // parts one: every block ends in two fp64 additions to one place (13k entries of
+    // 531k users, K = 64: 41 us with two waves, 30 with one; half a wave 32).
+    const int64_t resident = 4ll * sms * 8, groups = resident * kGpw, units = a.n_items / kGpw + a.F;
+    auto parts_of = [&](int32_t part) { return (a.longest + part - 1) / part; };
+    const int64_t share = a.n_obs / groups, steps = (std::max<int64_t>(a.longest, share) - share) / kInFlight<G, NV>;
+    const bool in_parts = a.n_items < groups || units * parts_of(kPart) / resident < steps;
+    a.part = 2;
+    while (a.part < kPart && units * parts_of(a.part) > resident) a.part *= 2;
+    a.parts = in_parts ? parts_of(a.part) : 0;
+    const int64_t need = ((in_parts ? a.parts : 1) * (a.n_items / a.F + kGpw) / kGpw + 7) / 8, wave = resident / 8 / a.F;
+    const int64_t x = std::max<int64_t>(1, std::min<int64_t>(need, in_parts || need < 4 * wave ? wave : 2 * wave));
     objective_kernel<G, NV, BY_WORKER><<<dim3((unsigned)x, (unsigned)a.F), 256, smem, st>>>(a);
     return cudaGetLastError();
   };

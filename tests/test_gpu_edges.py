@@ -62,11 +62,13 @@ def test_objective_shapes(K, N, n):
     t.close()
 
 
-def _constant_objective(K, N, n, D, element, P=3):
+def _constant_objective(K, N, n, D, element, P=3, long=0):
     """Objective inputs: every entry's value D (or an array of them); L's first and R's last value `element`, the rest
-    0, so that the residual is the value and every row's square is one product.  Returns whole and by-worker sums."""
+    0, so that the residual is the value and every row's square is one product.  The first `long` entries are of two
+    users.  Returns whole and by-worker sums."""
     M, F = 7, 2
     i = torch.arange(n, dtype=torch.int32, device="cuda") % N
+    i[:long] %= 2
     rows = torch.zeros((N + M, K), device="cuda")
     rows[:N, 0] = element
     rows[N:, K - 1] = element
@@ -81,16 +83,16 @@ def _constant_objective(K, N, n, D, element, P=3):
     return out, np.bincount(i.cpu().numpy() % P, minlength=P)
 
 
-# Items taken in parts and taken whole.
-@pytest.mark.parametrize("N,n", [(700, 40_000), (200_000, 4_000_000)])
+# Items taken in parts (few items, of 2, 8 and 96 entries), whole, and in parts as some are far longer than the others.
+@pytest.mark.parametrize("N,n,long", [(40, 120, 0), (700, 40_000, 0), (3, 3000, 0), (200_000, 4_000_000, 0), (30_000, 40_000, 700)])
 @pytest.mark.parametrize("K", [8, 32, 64, 96, 128, 256, 512])
-def test_objective_sums_are_exact(K, N, n):
+def test_objective_sums_are_exact(K, N, n, long):
     """The value's square has 27 bits (24 in its high fp32 part, one in its low one), a row's |.|^2 24, and both
     sums keep every bit: each is a multiple of 2^-26 below 2^27, with fewer than 24 bits lost per lane."""
     x = 1 + 2.0**-11 + 2.0**-13
     norm = float(np.float32(x) * np.float32(x))
     assert norm != x * x and norm + 2.0**-26 == x * x
-    ((sq, pen), (wsq, wpen)), cnt = _constant_objective(K, N, n, x, x)
+    ((sq, pen), (wsq, wpen)), cnt = _constant_objective(K, N, n, x, x, long=long)
     assert (sq, pen) == (n * x * x, n * (x * x + norm))
     assert (wsq == cnt * (x * x)).all() and (wpen == cnt * (x * x + norm)).all()
 
