@@ -51,15 +51,14 @@ struct Sum2 {  // two packed fp32 sums and what they lost
   }
 };
 
-// Four blocks per SM, as the grid is sized for, where that spills nothing and, by
-// worker, leaves both rows of a step in flight.  1.5M entries, us: K = 512 286
-// with what the compiler takes (66..72 registers), 228 so; by worker at K = 128
-// and 256 139 and 198 with four, 117 and 177 with three (9M: 319 and 540 with
-// four, 331 and 577 with three).
+// Four blocks per SM, as the grid is sized for, where that spills nothing.  1.5M
+// entries, us: K = 512 286 with what the compiler takes (66..72 registers), 228 so.
+// By worker at K = 100..128 three (1.5M entries, K = 128: 141 with four, 110).
 template <int G, int NV, bool BY_WORKER>
-__global__ void __launch_bounds__(256, (G == 8 && NV == 1) || (BY_WORKER && NV == 4 && G < 32) ? 3 : 4) objective_kernel(ObjectiveArgs a) {
+__global__ void __launch_bounds__(256, G == 8 && (NV == 1 || (BY_WORKER && NV == 4)) ? 3 : 4)
+    objective_kernel(ObjectiveArgs a) {
   constexpr int kGpw = 32 / G, U = kInFlight<G, NV>;
-  extern __shared__ double sums[];  // BY_WORKER: sum e^2 at [p], penalised sum at [P + p]
+  extern __shared__ double sums[];  // BY_WORKER: sum e^2 at [p], of the rows' squares at [P + p]
   if (BY_WORKER) {
     for (int k = threadIdx.x; k < 2 * a.P; k += blockDim.x) sums[k] = 0.0;
     __syncthreads();
@@ -76,7 +75,40 @@ __global__ void __launch_bounds__(256, (G == 8 && NV == 1) || (BY_WORKER && NV =
   const u64 minus1 = pack2(-1.f, -1.f);
   // e^2 and what the rows' squares add up to; by worker, of the item at hand.
   Sum2 sums2;  // (e^2, this lane's part of the rows' squares)
-  double wide_e = 0.0, wide_n = 0.0;  // the same of what fp32 cannot hold
+  double wide_e = 0.0, wide_n = 0.0;  // the same of what fp32 cannot hold, and whether there is any
+  bool wide = false;
+  // BY_WORKER: the sums of the group's last items, one per lane: the fp64 units are
+  // as long with an instruction for one lane as for all (190k entries, one or two
+  // per item, K = 496: 200 us with fp64 sums for each item in turn, 133 so).
+  float kept_e = 0.f, kept_el = 0.f, kept_n = 0.f, kept_nl = 0.f;
+  int kept_p = -1, kept = 0;
+  auto flush = [&]() {
+    const double sq = (double)kept_e + (double)kept_el, norms = (double)kept_n + (double)kept_nl;
+    // Few places, which many lanes would add to in turn: one addition per worker (the
+    // same case with 1, 2 and 3 workers: 203, 176, 164 us without; 139, 152, 154; with
+    // 8 workers 152, and 190 so).
+    if (a.P <= 3) {
+      for (unsigned left = __ballot_sync(0xffffffffu, kept_p >= 0); left != 0u;) {
+        const int p = __shfl_sync(0xffffffffu, kept_p, __ffs(left) - 1);
+        double x = kept_p == p ? sq : 0.0, y = kept_p == p ? norms : 0.0;
+#pragma unroll 1
+        for (int off = 16; off > 0; off >>= 1) {
+          x += __shfl_xor_sync(0xffffffffu, x, off);
+          y += __shfl_xor_sync(0xffffffffu, y, off);
+        }
+        if (lane == 0) {
+          atomicAdd(&sums[p], x);
+          atomicAdd(&sums[a.P + p], y);
+        }
+        left &= ~__ballot_sync(0xffffffffu, kept_p == p);
+      }
+    } else if (kept_p >= 0) {
+      atomicAdd(&sums[kept_p], sq);
+      atomicAdd(&sums[a.P + kept_p], norms);
+    }
+    kept_p = -1;
+    kept = 0;
+  };
   // Units of kGpw items, or of a part of each.
   const int64_t x_first = __ldg(a.item_base + blockIdx.y);
   const uint32_t units = (uint32_t)((x_end - x_first + kGpw - 1) / kGpw);
@@ -91,23 +123,24 @@ __global__ void __launch_bounds__(256, (G == 8 && NV == 1) || (BY_WORKER && NV =
     }
     const int32_t most = __reduce_max_sync(0xffffffffu, n);
     if (most == 0) continue;
-    f2x2 L[NV];
-    if (BY_WORKER) {
-      sums2 = Sum2{};
-      wide_e = wide_n = 0.0;
+    if (BY_WORKER) sums2 = Sum2{};
+    int32_t lane_j = 0;  // the next G entries by lane
+    float lane_d = 0.f;
+    if (glane < n) {
+      lane_j = __ldg(rec_j + it.y + glane);
+      lane_d = __ldg(rec_D + it.y + glane);
     }
+    f2x2 L[NV];
 #pragma unroll
     for (int k = 0; k < NV; ++k) {
       L[k] = f2x2{0ull, 0ull};
       ldg_f2x2_if(L[k], L4 + (int64_t)it.x * K4 + k * G, n > 0 && (k < NV - 1 || last_on));
     }
-    int32_t lane_j = 0;
-    float lane_d = 0.f;
 #pragma unroll 1
     for (int32_t t = 0; t < most; t += U) {
-      // The next G entries by lane, so that no step's rows wait for a load of ids (9M
-      // entries, K = 32 and 64: 241 and 205 us with one load per step, 197 and 184 so).
-      if ((t & (G - 1)) == 0 && t + glane < n) {
+      // By lane, so that no step's rows wait for a load of ids (9M entries, K = 32 and
+      // 64: 241 and 205 us with one load per step, 197 and 184 so).
+      if (t > 0 && (t & (G - 1)) == 0 && t + glane < n) {
         lane_j = __ldg(rec_j + it.y + t + glane);
         lane_d = __ldg(rec_D + it.y + t + glane);
       }
@@ -141,19 +174,20 @@ __global__ void __launch_bounds__(256, (G == 8 && NV == 1) || (BY_WORKER && NV =
       for (int off = G / 2; off > 0; off >>= 1)
 #pragma unroll
         for (int u = 0; u < U; ++u) e[u] += __shfl_xor_sync(0xffffffffu, e[u], off);
-      bool wide = false;
+      bool odd = false;
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         e[u] = t + u < n ? d[u] - e[u] : 0.f;
-        wide |= !in_range(e[u], norm[u]);
+        odd |= !in_range(e[u], norm[u]);
       }
-      if (wide) {  // (one branch for the step: one per entry took 1380 us instead of 802, 20M entries, K = 100)
+      if (odd) {  // (one branch for the step: one per entry took 1380 us instead of 802, 20M entries, K = 100)
 #pragma unroll
         for (int u = 0; u < U; ++u)
           if (!in_range(e[u], norm[u])) {
             wide_e += (double)e[u] * (double)e[u];
             wide_n += (double)norm[u];
             e[u] = norm[u] = 0.f;
+            wide = true;
           }
       }
 #pragma unroll
@@ -175,6 +209,7 @@ __global__ void __launch_bounds__(256, (G == 8 && NV == 1) || (BY_WORKER && NV =
       if (!(high < kHuge)) {
         wide_n += (double)n * (double)l;
         high = low = 0.f;
+        wide = true;
       }
       sums2.add(pack2(0.f, high), minus1);
       sums2.lost = add2(sums2.lost, pack2(0.f, low));
@@ -190,22 +225,33 @@ __global__ void __launch_bounds__(256, (G == 8 && NV == 1) || (BY_WORKER && NV =
         norm = two_sum(norm, __shfl_xor_sync(0xffffffffu, norm, off), err);
         norm_lost += lost + err;
       }
-      if (__any_sync(0xffffffffu, wide_n != 0.0))
-#pragma unroll
+      if (glane == kept && n > 0) {
+        kept_e = e2;
+        kept_el = e2_lost;
+        kept_n = norm;
+        kept_nl = norm_lost;
+        kept_p = it.w & 0xffff;
+      }
+      if (++kept == G) flush();
+      if (__any_sync(0xffffffffu, wide)) {
+#pragma unroll 1
         for (int off = G / 2; off > 0; off >>= 1) wide_n += __shfl_xor_sync(0xffffffffu, wide_n, off);
-      if (glane == 0 && n > 0) {
-        const int p = it.w & 0xffff;
-        const double sq = (double)e2 + (double)e2_lost + wide_e;
-        atomicAdd(&sums[p], sq);
-        atomicAdd(&sums[a.P + p], sq + (double)a.lambda * ((double)norm + (double)norm_lost + wide_n));
+        if (glane == 0 && n > 0) {
+          atomicAdd(&sums[it.w & 0xffff], wide_e);
+          atomicAdd(&sums[a.P + (it.w & 0xffff)], wide_n);
+        }
+        wide_e = wide_n = 0.0;
+        wide = false;
       }
     }
   }
   if (BY_WORKER) {
+    flush();
     __syncthreads();
     for (int k = threadIdx.x; k < a.P; k += blockDim.x) {
-      if (sums[k] != 0.0) atomicAdd(a.out + k, sums[k]);
-      if (sums[a.P + k] != 0.0) atomicAdd(a.out + a.out_stride + k, sums[a.P + k]);
+      const double sq = sums[k], pen = sq + (double)a.lambda * sums[a.P + k];
+      if (sq != 0.0) atomicAdd(a.out + k, sq);
+      if (pen != 0.0) atomicAdd(a.out + a.out_stride + k, pen);
     }
   } else {
     float e2, e2_lost, norm, norm_lost;
