@@ -80,8 +80,9 @@ constexpr int kMetaRounds = 8;    // rounds in the ring of item metadata
 //   wider rows (E = 1): in registers, one step ahead.  Their 256..2048 bytes
 //     per entry through shared memory as well would make the SM's load/store
 //     data path the limit (480k x 18k, K = 100: 480 us per clock against 440).
-//     What bounds them is the SM's outgoing port: an entry's reduction leaves
-//     at 32 bytes per cycle.
+//     What bounds them is the SM's outgoing port, busy in 86% of the cycles that
+//     L1 is active (K = 100): 12.5 of an entry's 21 cycles there are its reduction,
+//     at 32 bytes per cycle, the rest row requests, entries and user rows.
 template <int G, int NV, int E, int PF, int MINB, int HOT>
 __global__ void __launch_bounds__(kStreamWarps * 32, MINB) sgd_stream_kernel(StreamArgs c) {
   constexpr int kGpw = 32 / G;
