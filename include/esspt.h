@@ -234,7 +234,8 @@ esspt_status esspt_mf_sgd_clock_sequential(esspt_ctx* ctx, float eta, float lamb
 /* Objective of Sec. 3.1 / Sec. 5 at table version `version` over ALL loaded
  * entries: *h_sq = sum e^2 (squared loss) and
  * *h_pen = sum [e^2 + lambda (|L_i|^2 + |R_j|^2)] (l2-penalised, per entry).
- * fp32 residuals, fp64 sums.  Uses `d_scratch` (device, 2 doubles).
+ * fp32 residuals and row norms, summed to the precision of fp64.  Uses
+ * `d_scratch` (device, 2 doubles).
  * Synchronises. */
 esspt_status esspt_mf_objective(esspt_ctx* ctx, int32_t version, float lambda, double* d_scratch,
                                 double* h_sq, double* h_pen);
